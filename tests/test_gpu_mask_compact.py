@@ -130,6 +130,31 @@ def test_group_mask_tie_at_the_cut(lib):
         assert np.array_equal(oracle.compact_group([r[0] for r in recs], k), np.array(want, np.int32))
 
 
+@pytest.mark.parametrize("I,n_lists,W", [(4097, 2, 1), (5121, 37, 1), (9000, 2, 1), (20000, 2, 1), (40000, 2, 2), (3000, 60, 3),
+                                         (1500, 2, 16), (16384, 2, 9)])
+def test_lists_and_records_spread_over_ctas(lib, I, n_lists, W):
+    """Long lists are divided over a cluster's CTAs (with ties on both sides of a boundary), many records go to the CTAs
+    of a cluster in turn, lists beyond the register limit are read again on every pass."""
+    recs = [adversarial_records(I, n_lists, 70 + w) for w in range(W)]
+    for r in recs:
+        r[0, I // 3:I // 2] = r[0, 10]
+    for k in (1, I // 5, I // 2, I - 1):
+        votes = (W + 1) // 2
+        out_idx, out_cnt, status = run_compact(lib, I, recs, lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, n_lists, k=k, min_votes=votes)
+        assert status == 0
+        check_lists(out_idx, out_cnt, [oracle.compact_scores([r[i] for r in recs] if W > 1 else recs[0][i], oracle.RULE_TOPK, k=k,
+                                                             min_votes=votes) for i in range(n_lists)])
+    if W > 1:
+        out_idx, out_cnt, status = run_compact(lib, I, recs, lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_GROUP, n_lists, k=I // 3)
+        assert status == 0
+        check_lists(out_idx, out_cnt, [oracle.compact_group([r[i] for r in recs], I // 3) for i in range(n_lists)])
+    else:
+        m = (recs[0] > 0.7).astype(np.uint8)
+        out_idx, out_cnt, status = run_compact(lib, I, [m], lib.RM_SRC_BOOL_U8, lib.RM_REDUCE_NONE, n_lists)
+        assert status == 0
+        check_lists(out_idx, out_cnt, [np.flatnonzero(m[i]) for i in range(n_lists)])
+
+
 def test_truncation_is_reported_not_fatal(lib):
     I = 512
     m = np.ones((1, I), dtype=np.uint8)

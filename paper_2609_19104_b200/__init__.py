@@ -1,17 +1,22 @@
 """Python binding of the rmuscle C-ABI library (activation-masked gated MLP of an action expert on B200).
 
 The binding only marshals arguments: every tensor is a torch CUDA tensor whose data pointer is handed to the
-`extern "C"` entry point of the same name, on torch's current stream.  There is no CPU path: loading fails with
-an error when the CUDA library has not been built (`python -m paper_2609_19104_b200.build`).
+`extern "C"` entry point of the same name, on torch's current stream.  The calls of a control loop go through a small
+CPython module (csrc/rm_python.cpp: a call's marshalling through ctypes took longer on the host than the shorter kernels
+take on the GPU), set-up and diagnostics through ctypes.  There is no CPU path: loading fails with an error when the CUDA
+library has not been built (`python -m paper_2609_19104_b200.build`).
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional, Sequence
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "librmuscle.so")
+MODULE_PATH = os.path.join(_PKG, "_rmuscle.so")
 
 RM_OK = 0
 RM_ERR_INVALID_ARG, RM_ERR_SHAPE, RM_ERR_ALIGN, RM_ERR_WORKSPACE = -1, -2, -3, -4
@@ -53,6 +58,7 @@ class rm_mask_src(ctypes.Structure):
 
 
 _lib = None
+_native = None
 
 
 def load_library() -> ctypes.CDLL:
@@ -97,8 +103,23 @@ def load_library() -> ctypes.CDLL:
     lib.rm_status_string.restype = ctypes.c_char_p
     for name in EXPORTS:
         getattr(lib, name)
+    _load_module()
     _lib = lib
     return lib
+
+
+def _load_module() -> None:
+    """Loads the CPython module next to the library (it links against that same file)."""
+    global _native
+    if not os.path.exists(MODULE_PATH):
+        raise ImportError(f"{MODULE_PATH} is missing: build it with `python -m paper_2609_19104_b200.build`")
+    import torch
+    loader = importlib.machinery.ExtensionFileLoader("_rmuscle", MODULE_PATH)
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_rmuscle", MODULE_PATH, loader=loader))
+    loader.exec_module(mod)
+    # (a torch without CUDA has neither; nothing but Context, which refuses to exist there, would call them)
+    mod.init(getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None))
+    _native = mod
 
 
 def status_string(code: int) -> str:
@@ -123,9 +144,8 @@ def rm_sparse_mlp_static(packed_layer, x, residual, idx, count_dev, y, T: int, H
     """One masked MLP layer without a context, a workspace or any allocation: the scratch is a fixed array inside the
     library (T * I <= 1,048,576).  For callers that may not allocate device memory.  Calls that overlap on the GPU
     share that array and must be serialised; make the first call on a device outside stream capture."""
-    lib = load_library()
-    _check(lib.rm_sparse_mlp_static(_ptr(packed_layer), _ptr(x), _ptr(residual), _ptr(idx), _ptr(count_dev), _ptr(y),
-                                    int(T), int(H), int(I), _stream()), "rm_sparse_mlp_static")
+    load_library()
+    _check(_native.sparse_mlp_static(packed_layer, x, residual, idx, count_dev, y, T, H, I), "rm_sparse_mlp_static")
     return y
 
 
@@ -141,12 +161,17 @@ class Context:
         desc = rm_model_desc(L, H, I, T_max, B_max, RM_ACT_GELU_TANH)
         self._h = ctypes.c_void_p()
         _check(self.lib.rm_create(ctypes.byref(self._h), ctypes.byref(desc)), "rm_create")
+        self._hv = self._h.value
         self._ws = None
+        self._ws_bytes = 0
+        self._ws_need = {}                                         # (B, T) -> bytes; R_max -> bytes of the Context Cache
+        self._ctx_ws, self._ctx_ws_bytes = None, 0
 
     def close(self) -> None:
         if getattr(self, "_h", None) is not None and self._h.value:
             self.lib.rm_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._hv = 0
 
     def __del__(self):
         try:
@@ -167,7 +192,20 @@ class Context:
         need = self.workspace_bytes(B, T)
         if self._ws is None or self._ws.numel() < need:
             self._ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
+            self._ws_bytes = self._ws.numel()
         return self._ws
+
+    def _scratch(self, B: int, T: int, ws):
+        """(workspace, its bytes) of a call: the caller's, or the cached one."""
+        if ws is not None:
+            return ws, ws.numel()
+        key = (B, T)
+        need = self._ws_need.get(key)
+        if need is None:
+            need = self._ws_need[key] = self.workspace_bytes(max(B, 1), max(T, 1))
+        if self._ws is None or self._ws_bytes < need:
+            self.workspace(max(B, 1), max(T, 1))
+        return self._ws, self._ws_bytes
 
     def rm_set_option(self, name: str, value: int) -> None:
         _check(self.lib.rm_set_option(self._h, name.encode(), int(value)), f"rm_set_option({name})")
@@ -199,30 +237,31 @@ class Context:
     def rm_mask_compact(self, records: Sequence, kind: int, reduce: int, idx_out, count_out, stride: int, *,
                         n_lists: int, threshold: float = 0.0, k: int = 0, min_votes: int = 1, scale=None,
                         scale_per_list: bool = False, I: Optional[int] = None):
-        W = len(records)
-        arr = (ctypes.c_void_p * max(W, 1))(*[_ptr(r) for r in records])
-        src = rm_mask_src(kind, reduce, float(threshold), int(k), W, int(min_votes),
-                          ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p)), _ptr(scale), int(bool(scale_per_list)),
-                          int(n_lists), self.I if I is None else int(I))
-        _check(self.lib.rm_mask_compact(self._h, ctypes.byref(src), _ptr(idx_out), _ptr(count_out), int(stride),
-                                        _stream()), "rm_mask_compact")
+        rc = _native.mask_compact(self._hv, records, kind, reduce, threshold, k, min_votes, scale, scale_per_list, n_lists,
+                                  self.I if I is None else I, idx_out, count_out, stride)
+        if rc != RM_OK:
+            raise RmError(rc, "rm_mask_compact")
 
     def rm_context_drift(self, x, x_ref, P: int, score_out):
         """Eq. 2: per-row drift score of the current FFN input against the reference input."""
-        _check(self.lib.rm_context_drift(self._h, _ptr(x), _ptr(x_ref), int(P), _ptr(score_out), _stream()),
-               "rm_context_drift")
+        _check(_native.context_drift(self._hv, x, x_ref, P, score_out), "rm_context_drift")
         return score_out
 
     def rm_context_ffn(self, Wg, Wu, Wd, x, rows, count_dev, P: int, S: int, R_max: int, y_ref, y_out, ws=None):
         """Eq. 3: recompute the listed visual rows and the S always-recomputed rows, keep y_ref elsewhere."""
-        import torch
-        need = int(self.lib.rm_context_workspace_bytes(self._h, int(R_max)))
         if ws is None:
-            if getattr(self, "_ctx_ws", None) is None or self._ctx_ws.numel() < need:
-                self._ctx_ws = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda")
+            need = self._ws_need.get(R_max)
+            if need is None:
+                need = self._ws_need[R_max] = int(self.lib.rm_context_workspace_bytes(self._h, int(R_max)))
             ws = self._ctx_ws
-        _check(self.lib.rm_context_ffn(self._h, _ptr(Wg), _ptr(Wu), _ptr(Wd), _ptr(x), _ptr(rows), _ptr(count_dev), int(P),
-                                       int(S), int(R_max), _ptr(y_ref), _ptr(y_out), _ptr(ws), int(ws.numel()), _stream()),
+            if ws is None or self._ctx_ws_bytes < need:
+                import torch
+                ws = self._ctx_ws = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda")
+                self._ctx_ws_bytes = ws.numel()
+            ws_bytes = self._ctx_ws_bytes
+        else:
+            ws_bytes = ws.numel()
+        _check(_native.context_ffn(self._hv, Wg, Wu, Wd, x, rows, count_dev, P, S, R_max, y_ref, y_out, ws, ws_bytes),
                "rm_context_ffn")
         return y_out
 
@@ -252,10 +291,9 @@ class Context:
     def rm_sparse_mlp(self, packed_layer, x, residual, idx, count_dev, y, record_out=None, record_scale=None,
                       T: Optional[int] = None, ws=None):
         T = int(x.shape[0]) if T is None else T
-        ws = self.workspace(1, max(T, 1)) if ws is None else ws
-        _check(self.lib.rm_sparse_mlp(self._h, _ptr(packed_layer), _ptr(x), _ptr(residual), _ptr(idx),
-                                      _ptr(count_dev), _ptr(y), _ptr(record_out), _ptr(record_scale), T, _ptr(ws),
-                                      int(ws.numel()), _stream()), "rm_sparse_mlp")
+        ws, ws_bytes = self._scratch(1, T, ws)
+        _check(_native.sparse_mlp(self._hv, packed_layer, x, residual, idx, count_dev, y, record_out, record_scale, T, ws,
+                                  ws_bytes), "rm_sparse_mlp")
         return y
 
     def _layer_ptrs(self, packed_layers):
@@ -264,11 +302,9 @@ class Context:
     def rm_action_expert_step(self, packed_layers, r_in, idx, count_dev, stride: int, r_out, records_out=None,
                               record_scale=None, B: int = 1, T: Optional[int] = None, ws=None):
         T = int(r_in.shape[-2]) if T is None else T
-        ws = self.workspace(max(B, 1), max(T, 1)) if ws is None else ws
-        _check(self.lib.rm_action_expert_step(self._h, self._layer_ptrs(packed_layers), _ptr(r_in), _ptr(idx),
-                                              _ptr(count_dev), int(stride), _ptr(r_out), _ptr(records_out),
-                                              _ptr(record_scale), B, T, _ptr(ws), int(ws.numel()), _stream()),
-               "rm_action_expert_step")
+        ws, ws_bytes = self._scratch(B, T, ws)
+        _check(_native.step(self._hv, packed_layers, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T, ws,
+                            ws_bytes), "rm_action_expert_step")
         return r_out
 
     def rm_action_expert_step_ex(self, packed_layers, r_in, idx, count_dev, stride: int, r_out, anchor_mode: int,
@@ -276,23 +312,17 @@ class Context:
                                  record_scale=None, B: int = 1, T: Optional[int] = None, ws=None):
         """The step with the anchor-relative update (Eq. 4): y_anchor [L,B,T,H], h_anchor [L,B,I,h_stride] fp32."""
         T = int(r_in.shape[-2]) if T is None else T
-        ws = self.workspace(max(B, 1), max(T, 1)) if ws is None else ws
-        _check(self.lib.rm_action_expert_step_ex(self._h, self._layer_ptrs(packed_layers), _ptr(r_in), _ptr(idx),
-                                                 _ptr(count_dev), int(stride), _ptr(r_out), _ptr(records_out),
-                                                 _ptr(record_scale), B, T, int(anchor_mode), _ptr(y_anchor),
-                                                 _ptr(h_anchor), int(h_stride), _ptr(out_gate), _ptr(ws),
-                                                 int(ws.numel()), _stream()),
-               "rm_action_expert_step_ex")
+        ws, ws_bytes = self._scratch(B, T, ws)
+        _check(_native.step_ex(self._hv, packed_layers, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T,
+                               anchor_mode, y_anchor, h_anchor, h_stride, out_gate, ws, ws_bytes), "rm_action_expert_step_ex")
         return r_out
 
     def rm_action_expert_step_host(self, packed_layers, r_in_host, idx, count_dev, stride: int, r_out_host,
                                    B: int = 1, T: Optional[int] = None, ws=None):
         """r_in_host / r_out_host are CPU tensors (pinned for asynchronous copies); returns after the result landed."""
         T = int(r_in_host.shape[-2]) if T is None else T
-        ws = self.workspace(max(B, 1), max(T, 1)) if ws is None else ws
-        _check(self.lib.rm_action_expert_step_host(self._h, self._layer_ptrs(packed_layers), _ptr(r_in_host),
-                                                   _ptr(idx), _ptr(count_dev), int(stride), _ptr(r_out_host), B, T,
-                                                   _ptr(ws), int(ws.numel()), _stream()),
+        ws, ws_bytes = self._scratch(B, T, ws)
+        _check(_native.step_host(self._hv, packed_layers, r_in_host, idx, count_dev, stride, r_out_host, B, T, ws, ws_bytes),
                "rm_action_expert_step_host")
         return r_out_host
 

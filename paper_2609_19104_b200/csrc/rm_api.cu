@@ -100,14 +100,15 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     // against 38 us per layer).
     c->stream_min_tiles = desc->H == 2048 ? 64 : 48;
     c->d_status = nullptr;
-    cudaDeviceProp prop;
-    if (cudaGetDevice(&c->device) != cudaSuccess || cudaGetDeviceProperties(&prop, c->device) != cudaSuccess ||
+    int major = 0;                         // (two attributes: cudaGetDeviceProperties takes milliseconds)
+    if (cudaGetDevice(&c->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device) != cudaSuccess ||
         cudaMalloc(&c->d_status, 256) != cudaSuccess || cudaMemset(c->d_status, 0, 256) != cudaSuccess) {
         if (c->d_status) cudaFree(c->d_status);
         delete c;
         return RM_ERR_CUDA;
     }
-    c->sm_count = prop.multiProcessorCount;
     c->path = 0;
     c->use_pdl = 1;
     c->npc_target = 64;
@@ -126,7 +127,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->persist_sync = nullptr;
     c->persist_sync_dirty = 0;
     for (int b = 0; b < 16; ++b) c->persist_sync_base[b] = c->persist_copy_base[b] = 0;
-    if (prop.major == 10) { rm_fused_init(c); rm_persist_init(c); }   // failure leaves the portable path in charge
+    if (major == 10) { rm_fused_init(c); rm_persist_init(c); }   // failure leaves the portable path in charge
     cudaGetLastError();
     *out = c;
     return RM_OK;

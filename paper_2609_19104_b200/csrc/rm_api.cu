@@ -56,6 +56,21 @@ inline void* persist_ws(const rm_ctx* ctx, void* ws, int B, int T) {
     return static_cast<char*>(ws) + 4 * r_bytes + align_up(rm_ref_workspace_bytes(ctx, B, T), 256);
 }
 
+// The slice kernel (variant 6): where the tcgen05 kernels do not reach (widths other than 1024 and 2048, chunks of more than
+// 64 tokens), instead of the CUDA-core kernels.  One step of 12 layers of 1536/6144 with 25 % of the neurons and 51 tokens:
+// 291 us against 9360.
+inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
+    if (ctx->path == 1 || !rm_slice_supported(ctx, B, T, record)) return false;
+    return ctx->variant_override == 6 || (ctx->path == 0 && !rm_fused_supported(ctx, B, T));
+}
+
+// the slice kernel's buffers in a workspace of (B, T)
+inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, int T) {
+    const size_t r_bytes = align_up((size_t)B * T * ctx->g.H * sizeof(float), 256);
+    for (int i = 0; i < 3; ++i) sa.rot[i] = reinterpret_cast<float*>(static_cast<char*>(ws) + i * r_bytes);
+    sa.ctrl = reinterpret_cast<int*>(static_cast<char*>(persist_ws(ctx, ws, B, T)) + align_up(rm_persist_workspace_bytes(ctx), 256));
+}
+
 // The streaming variant (whole tiles per CTA) pays off only when a launch has about one 64-neuron tile per SM (one SM
 // gathers at most ~38 GB/s with 16-byte cp.async and adds at most ~20 GB/s with red.global, so a tile costs it
 // ~25 us); below that the cluster kernels, which spread a tile over 8 SMs, win.  H = 1024 only: at H = 2048 the
@@ -121,13 +136,14 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->fused_blocks_per_sm = 0;
     c->last_variant = 0;
     c->persist_clusters = 0;
+    c->slice_clusters = 0;
     c->persist_max_b = 1;
     c->persist_prefetch_kb = 0;
     c->persist_xbuf = nullptr;
     c->persist_sync = nullptr;
     c->persist_sync_dirty = 0;
     for (int b = 0; b < 16; ++b) c->persist_sync_base[b] = c->persist_copy_base[b] = 0;
-    if (major == 10) { rm_fused_init(c); rm_persist_init(c); }   // failure leaves the portable path in charge
+    if (major == 10) { rm_fused_init(c); rm_persist_init(c); rm_slice_init(c); }   // failure leaves the portable path in charge
     cudaGetLastError();
     *out = c;
     return RM_OK;
@@ -148,7 +164,8 @@ size_t rm_workspace_bytes(const rm_ctx* ctx, int B, int T) {
     if (!ctx || B < 1 || T < 1) return 0;
     // three rotating residual-stream buffers, the host variant's staging buffer, then the portable path's scratch
     size_t r_bytes = align_up((size_t)B * T * ctx->g.H * sizeof(float), 256);
-    return 4 * r_bytes + align_up(rm_ref_workspace_bytes(ctx, B, T), 256) + rm_persist_workspace_bytes(ctx);
+    return 4 * r_bytes + align_up(rm_ref_workspace_bytes(ctx, B, T), 256) + align_up(rm_persist_workspace_bytes(ctx), 256) +
+           rm_slice_workspace_bytes(ctx, B, T);
 }
 
 int rm_pack_weights(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, void* packed_out,
@@ -275,6 +292,25 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
     a.T = T;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t r_bytes = align_up((size_t)T * ctx->g.H * sizeof(float), 256);
+    if (use_slice(ctx, 1, T, record_out != nullptr)) {
+        const void* one[1] = {packed_layer};
+        rm_step_args sa{};
+        sa.packed_layers = one;
+        sa.L = 1;
+        sa.r = y;
+        sa.r_in = residual;
+        sa.idx = idx;
+        sa.count = count_dev;
+        sa.list_cap = ctx->g.I;
+        sa.record = record_out;
+        sa.record_scale = record_scale;
+        sa.B = 1;
+        sa.T = T;
+        sa.x_ext = x;
+        slice_buffers(ctx, sa, ws, 1, T);
+        ctx->last_variant = 6;
+        return rm_launch_step_slice(ctx, sa, s);
+    }
     if (use_fused(ctx, 1, T)) {
         // y accumulates the CTAs' partial sums with atomics: start it from the residual (or zero)
         if (y != residual) {
@@ -333,7 +369,8 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     const size_t n_bytes = (size_t)B * T * g.H * sizeof(float);
     const size_t r_bytes = align_up(n_bytes, 256);
     char* layer_ws = static_cast<char*>(ws) + 4 * r_bytes;
-    if (use_persist(ctx, B, T, count_dev != nullptr, true)) {
+    const bool slice = use_slice(ctx, B, T, records_out != nullptr);
+    if (slice || use_persist(ctx, B, T, count_dev != nullptr, true)) {
         // the whole step in one launch: the layers add into r_out in place (the kernel starts it as a copy of r_in)
         rm_step_args sa{};
         sa.packed_layers = packed_layers;
@@ -356,6 +393,11 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
         sa.h_anchor = an.h;
         sa.h_stride = an.h_stride;
         sa.gate = an.gate;
+        if (slice) {
+            slice_buffers(ctx, sa, ws, B, T);
+            ctx->last_variant = 6;
+            return rm_launch_step_slice(ctx, sa, s);
+        }
         ctx->last_variant = 5;
         return rm_launch_step_persist(ctx, sa, persist_ws(ctx, ws, B, T), s);
     }
@@ -535,7 +577,7 @@ int rm_set_option(rm_ctx* ctx, const char* name, int value) {
         if (value < 0) return RM_ERR_INVALID_ARG;
         ctx->count_hint = value;
     } else if (n == "variant") {
-        if (value < 0 || value > 5) return RM_ERR_INVALID_ARG;
+        if (value < 0 || value > 6) return RM_ERR_INVALID_ARG;
         ctx->variant_override = value;
     } else if (n == "persist_prefetch_kb") {
         if (value < 0 || value > 4096) return RM_ERR_INVALID_ARG;
@@ -567,6 +609,7 @@ int rm_get_info(const rm_ctx* ctx, const char* name, int* out) {
     else if (n == "fused_blocks_per_sm") *out = ctx->fused_blocks_per_sm;
     else if (n == "sm_count") *out = ctx->sm_count;
     else if (n == "persist_clusters") *out = ctx->persist_clusters;
+    else if (n == "slice_clusters") *out = ctx->slice_clusters;
     else if (n == "last_variant") *out = ctx->last_variant;
     else if (n == "path") *out = ctx->path;
     else if (n == "status_detail") *out = ctx->status_detail;

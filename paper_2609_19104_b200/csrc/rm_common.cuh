@@ -46,6 +46,7 @@ struct rm_ctx {
     int variant_override;                  // 0 auto, 1 lean kernel, 2 kernel with a dedicated staging buffer
     int last_variant;                      // kernel family of the last layer or step launched (see rm_get_info)
     // whole-step kernel (rm_mlp_persist.cu)
+    int slice_clusters;                    // co-resident 8-CTA clusters of the slice kernel (0: unavailable)
     int persist_clusters;                  // co-resident 8-CTA clusters of the whole-step kernel (0: unavailable)
     int persist_prefetch_kb;               // weight KB a CTA of the whole-step kernel may ask into L2 ahead of its loaders
     int persist_max_b;                     // largest batch the whole-step kernel is chosen for when the variant is automatic
@@ -170,7 +171,14 @@ struct rm_step_args {
     float* h_anchor;                       // [L,B,I,h_stride]
     int64_t h_stride;
     const float* gate;                     // [L,B,H] output gate, or NULL
+    float* rot[3];                         // slice kernel: [B,T,H] buffers of the layers in between
+    int* ctrl;                             // slice kernel: control block
 };
+// Slice kernel: every layer of a step in one launch, any H up to 2048, any T (rm_mlp_slice.cu)
+int rm_slice_init(rm_ctx* ctx);
+bool rm_slice_supported(const rm_ctx* ctx, int B, int T, bool record);
+size_t rm_slice_workspace_bytes(const rm_ctx* ctx, int B, int T);
+int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s);
 int rm_persist_init(rm_ctx* ctx);
 bool rm_persist_supported(const rm_ctx* ctx, int B, int T);
 size_t rm_persist_workspace_bytes(const rm_ctx* ctx);

@@ -58,7 +58,7 @@ inline void* persist_ws(const rm_ctx* ctx, void* ws, int B, int T) {
 
 // The slice kernel (variant 6): where the tcgen05 kernels do not reach (widths other than 1024 and 2048, chunks of more than
 // 64 tokens), instead of the CUDA-core kernels.  One step of 12 layers of 1536/6144 with 25 % of the neurons and 51 tokens:
-// 291 us against 9360.
+// 244 us against 9360.
 inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
     if (ctx->path == 1 || !rm_slice_supported(ctx, B, T, record)) return false;
     return ctx->variant_override == 6 || (ctx->path == 0 && !rm_fused_supported(ctx, B, T));
@@ -313,10 +313,10 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
     }
     if (use_fused(ctx, 1, T)) {
         // y accumulates the CTAs' partial sums with atomics: start it from the residual (or zero)
+        // (a kernel of its own, so that the layer's CTAs can set up and gather their first weights while it runs)
         if (y != residual) {
-            if (residual) RM_CUDA_TRY(cudaMemcpyAsync(y, residual, (size_t)T * ctx->g.H * sizeof(float),
-                                                      cudaMemcpyDeviceToDevice, s));
-            else RM_CUDA_TRY(cudaMemsetAsync(y, 0, (size_t)T * ctx->g.H * sizeof(float), s));
+            const int rc = rm_launch_copy(ctx, y, residual, (size_t)T * ctx->g.H, false, s);
+            if (rc != RM_OK) return rc;
         }
         if (use_persist(ctx, 1, T, count_dev != nullptr, false)) {
             // the whole-step kernel on a stack of one layer whose input is the caller's x
@@ -344,7 +344,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
             ctx->last_variant = 4;
             return rm_launch_layer_stream(ctx, a, nullptr, false, s);
         }
-        return rm_launch_layer_fused(ctx, a, nullptr, false, false, s);
+        return rm_launch_layer_fused(ctx, a, nullptr, false, ctx->use_pdl && y != residual, s);
     }
     if (ctx->path == 2) return RM_ERR_UNSUPPORTED;
     ctx->last_variant = 0;
@@ -520,6 +520,19 @@ int rm_action_expert_step_ex(rm_ctx* ctx, const void* const* packed_layers, cons
                        static_cast<cudaStream_t>(stream), an);
 }
 
+// The device's address of a pinned host buffer, or NULL (pageable, not host memory, or not 16-byte aligned)
+static void* pinned_device_pointer(const void* p, size_t bytes) {
+    cudaPointerAttributes first, last;
+    if (!rm_aligned16(p) || cudaPointerGetAttributes(&first, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&last, static_cast<const char*>(p) + bytes - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const bool whole = first.type == cudaMemoryTypeHost && last.type == cudaMemoryTypeHost && first.devicePointer &&
+                       static_cast<char*>(last.devicePointer) - static_cast<char*>(first.devicePointer) == (ptrdiff_t)(bytes - 1);
+    return whole && rm_aligned16(first.devicePointer) ? first.devicePointer : nullptr;
+}
+
 int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, const float* r_in_host,
                                const int32_t* idx, const int32_t* count_dev, int64_t stride, float* r_out_host, int B,
                                int T, void* ws, size_t ws_bytes, rm_stream_t stream) {
@@ -538,10 +551,23 @@ int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, co
     const size_t n_bytes = (size_t)B * T * ctx->g.H * sizeof(float);
     // the fourth residual-stream buffer of the workspace is the staging copy
     float* stage = reinterpret_cast<float*>(static_cast<char*>(ws) + 3 * align_up(n_bytes, 256));
-    RM_CUDA_TRY(cudaMemcpyAsync(stage, r_in_host, n_bytes, cudaMemcpyHostToDevice, s));
+    // pinned buffers are copied by a kernel (rm_launch_copy), others by the copy engine
+    const float* in_dev = static_cast<const float*>(pinned_device_pointer(r_in_host, n_bytes));
+    float* out_dev = static_cast<float*>(pinned_device_pointer(r_out_host, n_bytes));
+    if (in_dev) {
+        const int rc = rm_launch_copy(ctx, stage, in_dev, n_bytes / sizeof(float), false, s);
+        if (rc != RM_OK) return rc;
+    } else {
+        RM_CUDA_TRY(cudaMemcpyAsync(stage, r_in_host, n_bytes, cudaMemcpyHostToDevice, s));
+    }
     int rc = step_device(ctx, packed_layers, stage, idx, count_dev, stride, stage, nullptr, nullptr, B, T, ws, s);
     if (rc != RM_OK) return rc;
-    RM_CUDA_TRY(cudaMemcpyAsync(r_out_host, stage, n_bytes, cudaMemcpyDeviceToHost, s));
+    if (out_dev) {
+        rc = rm_launch_copy(ctx, out_dev, stage, n_bytes / sizeof(float), ctx->use_pdl != 0, s);
+        if (rc != RM_OK) return rc;
+    } else {
+        RM_CUDA_TRY(cudaMemcpyAsync(r_out_host, stage, n_bytes, cudaMemcpyDeviceToHost, s));
+    }
     RM_CUDA_TRY(cudaStreamSynchronize(s));
     return RM_OK;
 }

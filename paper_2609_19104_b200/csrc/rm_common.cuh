@@ -101,6 +101,7 @@ __device__ __forceinline__ float rm_gelu_tanh(float g) {
 // ---- kernels implemented in the other translation units (host launchers)
 int rm_launch_pack(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, void* packed, float* colnorm,
                    cudaStream_t s);
+int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, size_t n, bool pdl, cudaStream_t s);
 int rm_launch_gather_rows(rm_ctx* ctx, const void* packed, const int32_t* idx, const int32_t* count, int64_t cap,
                           void* out, cudaStream_t s);
 // Context Cache (row-sparse dense FFN on the tensor cores)

@@ -484,6 +484,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     cluster_sync();
     tc_fence_after();
     const uint32_t tmem = *g_tmem;
+    pdl_launch_dependents();                                       // (a dependent waits for this grid's end: its CTAs are resident by then)
     // r starts as a copy of r_in: cluster 0's CTA j copies column slice j of every episode and counts itself on the
     // episode's copy counter; nobody adds into r before the 8 copies are counted
     const int pre = a.r_in != a.r ? CS : 0;

@@ -3,12 +3,13 @@
 // Clusters of 8 CTAs, all co-resident (one CTA per SM).  CTA j of a cluster owns column slice j (Hs = H/8 columns of the
 // model width) for BOTH projections, so a neuron's slice -- gate, up and down piece side by side in the packed layout -- is
 // read once, by one CTA, as two contiguous bulk copies.  The active list of a layer is cut over the clusters; a cluster
-// walks its run in rounds of 8 OPN neurons:
-//   gate/up : partial sums over the slice's columns, [16 rows = 8 gate + 8 up] x tokens per warp tile, by mma.sync
-//             (m16n8k16, bf16 in, fp32 accumulators in registers)
-//   owner   : neuron q of the round belongs to CTA q / OPN.  The partial sums travel to it as bulk copies between the
-//             CTAs' shared memories, counted on its mbarrier; it adds the 8 slices' sums, applies gelu_tanh(g) * u, splits h
-//             into a bf16 pair hi + lo (relative error 2^-17) and copies its rows to the other CTAs' h tiles
+// walks its run in rounds of up to 14 tiles of 8 neurons:
+//   gate/up : partial sums over the slice's columns, [8 gate rows, 8 up rows] x tokens, by mma.sync (m16n8k16, bf16 in, fp32
+//             accumulators in registers)
+//   owner   : tile i of the round belongs to CTA i mod 8.  The partial sums travel to it as bulk copies between the
+//             CTAs' shared memories (laid out in the weight stage that the products have just read), counted on its
+//             mbarrier; it adds the 8 slices' sums, applies gelu_tanh(g) * u, splits h into a bf16 pair hi + lo (relative error
+//             2^-17) and copies its rows to the other CTAs' h tiles
 //   down    : [tokens] x [the slice's columns], accumulated in registers over the rounds of the item, then added to the
 //             fp32 residual stream with red.global.add
 // A layer's adds go into a buffer of their own (three in turn, cleared one layer ahead); the residual itself is added by
@@ -34,14 +35,18 @@ using namespace sm100;
 namespace {
 
 constexpr int CS = 8;                  // CTAs per cluster = column slices of the packed layout
-constexpr int SN = 16;                 // neurons per weight stage
+constexpr int TN = 8;                  // neurons of a tile: 8 gate rows and 8 up rows make one 16-row operand
+constexpr int SN = 2 * TN;             // neurons of a weight stage
 constexpr int MAX_ITEMS = 512;         // layers x episodes of one launch
 constexpr int MAXL = 64, MAXB = 64;
 constexpr int NTHREADS = 640;          // warps 0-7: normalisation and gate/up (group A); 8-15: owner, down, adds (group B);
-constexpr int W_B = 8, W_G = 16;   // 16 / 17: loaders of the gate/up and of the down pieces
+constexpr int W_B = 8, W_G = 16;       // 16 / 17: loaders of the gate/up and of the down pieces
 constexpr int HPITCH = 272;            // bytes of an h row: 64 tokens hi, 64 tokens lo, 16 to spread the banks
+constexpr int P_SRC = 4096;            // partial sums of a tile from one CTA: [8-token tile][neuron][token pair] (gate, gate, up, up)
+constexpr int P_SLOT = CS * P_SRC;
 constexpr int SSB = 4;                 // buffers of the row sums of squares: a CTA can be two items ahead of another
 constexpr int MAX_STAGES = 16;
+constexpr int EXACT_STAGES = 7;        // of the 128-column slice
 
 // control block in the workspace, in ints: [0,1] launch epoch, [2] CTAs that have left, [3] abort flag; then lines of 32 ints:
 // per (episode, slice) the CTAs that have set up the first output buffer, and the CTAs that have added their part
@@ -50,41 +55,31 @@ __host__ __device__ constexpr int ctrl_init(int e, int j) { return CTRL_LINE * (
 __host__ __device__ constexpr int ctrl_done(int e, int j) { return CTRL_LINE * (2 + (e * CS + j) * 2); }
 __host__ __device__ constexpr size_t ctrl_bytes(int B) { return (size_t)CTRL_LINE * (1 + 2 * CS * B) * sizeof(int); }
 
-// ---- shared-memory layout (computed by the host, a kernel argument: constants cost no registers)
+// ---- shared memory.  ts: tiles that one CTA may own per round (a round has up to 8 ts tiles)
 struct Lay {
-    int xp, gp, dp;                    // row pitches: x tile, gate|up pieces, down pieces (odd multiples of 16 bytes: eight rows
-                                       // of an ldmatrix fall into different banks)
-    int ks, n_a, n_b;                  // 16-column steps of the slice; 8-token tiles of the two token halves
-    int p_src, p_buf, stg_warp;        // partial sums: bytes from one source, of one buffer, of one warp's outgoing pieces
-    int h_buf, g_stage, d_stage;
-    int off_p, off_stg, off_h, off_ss, off_item, off_bar, off_x, off_g, off_d, total;
+    int ks, xp, gp, dp;                // 16-column steps of the slice; row pitches: x tile, gate|up pieces, down pieces (odd multiples
+                                       // of 16 bytes: eight rows of an ldmatrix fall into different banks)
+    int g_stage, d_stage, stages;
+    int off_ss, off_x, off_p, off_h, off_g, off_d, off_item, total;
 };
-inline Lay make_layout(int Hs, int T, int opn, int stages) {
-    Lay y;
-    const int t8 = (T + 7) / 8;
+__host__ __device__ constexpr Lay make_layout(int Hs, int ts, int stages) {
+    Lay y{};
     y.ks = (Hs + 15) / 16;
     y.xp = y.ks * 32 + 16;
     y.gp = Hs * 4 + 16;
     y.dp = (Hs / 8) % 2 ? Hs * 2 : Hs * 2 + 16;
-    y.n_a = (t8 + 1) / 2;
-    y.n_b = t8 - y.n_a;
-    y.p_src = opn * t8 * 64;
-    y.p_buf = CS * y.p_src;
-    y.stg_warp = 2 * 8 * y.n_a * 64;
-    y.h_buf = CS * opn * HPITCH;
-    y.g_stage = SN * y.gp;
+    // (a gate/up stage that has been used holds the two warps' outgoing partial sums, 8 KB)
+    y.g_stage = SN * y.gp > 8192 ? SN * y.gp : 8192;
     y.d_stage = SN * y.dp + 32;        // (an odd last pair of column tiles reads 16 bytes past the last row)
-    int o = 0;
-    y.off_bar = o;   o += 512;
-    y.off_item = o;  o += MAX_ITEMS * 16;
-    y.off_ss = o;    o += SSB * CS * 64 * 4;
-    y.off_x = o;     o += 64 * y.xp;
-    y.off_p = o;     o += 2 * y.p_buf;
-    y.off_stg = o;   o += 8 * y.stg_warp;
-    y.off_h = o;     o += 2 * y.h_buf;
-    y.off_g = o;     o += stages * y.g_stage;
-    y.off_d = o;     o += stages * y.d_stage;
-    y.total = o + 128;
+    y.stages = stages;
+    y.off_ss = 512;                    // (the barriers of the rings in front of it)
+    y.off_x = y.off_ss + SSB * CS * 64 * 4;
+    y.off_p = y.off_x + 64 * y.xp;
+    y.off_h = y.off_p + ts * P_SLOT;
+    y.off_g = y.off_h + ts * CS * TN * HPITCH;
+    y.off_d = y.off_g + stages * y.g_stage;
+    y.off_item = y.off_d + stages * y.d_stage;
+    y.total = y.off_item + MAX_ITEMS * 16 + 128;
     return y;
 }
 
@@ -107,7 +102,6 @@ struct SArgs {
     int nb;                            // episodes of the caller
     int n_sub;                         // token chunks per episode: "episode" e of the kernel is chunk e % n_sub of e / n_sub
     int T_all;                         // tokens per episode of the caller (T: tokens per chunk; the last one may hold fewer)
-    int stages;                        // weight stages of each ring
     int anchor_mode;                   // Eq. 4 (EQ4 instantiation): RM_ANCHOR_*
     float* y_anchor;                   // [L,B,T,H]
     float* h_anchor;                   // [L,B,I,h_stride]
@@ -200,48 +194,56 @@ __device__ __forceinline__ bool barrier_or(int id, int count, bool pred) {
 struct Item { int start, n, parts_share, target; };                // parts | share << 8 | takes part << 16; target: arrivals
                                                                    // on the episode's counter that complete the layer before
 
-// NG: 8-column tiles of the slice per down warp (four column groups), so Hs <= 32 NG.  OPN: neurons per owner and round.  With
-// OPN = 4 (wide slices, whose stages are large) rounds alternate between two teams of four gate/up warps.
-template <int NG, int OPN, bool EQ4>
+// A cluster's run of n neurons is tiles of 8, cut into rounds of at most `most` tiles, as even as they come: round r of nrd
+// starts at neuron pos and has nr.
+__device__ __forceinline__ int round_count(int n, int most) { return ((n + TN - 1) / TN + most - 1) / most; }
+__device__ __forceinline__ void round_span(int n, int r, int nrd, int& pos, int& nr) {
+    if (nrd == 1) { pos = 0; nr = n; return; }
+    const int tiles = (n + TN - 1) / TN, a = tiles * r / nrd, b = tiles * (r + 1) / nrd;
+    pos = a * TN;
+    nr = (b * TN < n ? b * TN : n) - pos;
+}
+
+// HS: columns of a slice (0: any, from the arguments -- the address arithmetic then costs instructions in every phase).  NG:
+// 8-column tiles of the slice per down warp (four column groups), so Hs <= 32 NG.  TS: tiles a CTA may own per round.
+template <int HS, int NG, int TS, bool EQ4>
 __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constant__ SArgs a) {
     // registers: 640 threads x 96 at launch; the four warps of the loaders give most of theirs to the two groups
-    constexpr int REGS_L = 32, REGS_A = 104, REGS_B = 120;
+    constexpr int REGS_L = 32, REGS_A = NG == 4 ? 120 : 104, REGS_B = NG == 4 ? 104 : 120;
     static_assert(REGS_L * 128 + (REGS_A + REGS_B) * 256 <= 96 * NTHREADS, "more registers than the block is launched with");
-    constexpr int TEAMS = 8 / OPN, RN = CS * OPN, MAXV = 2 * NG;
+    constexpr int MAXV = 2 * NG;
+    constexpr Lay LC = make_layout(HS ? HS : 128, TS, EXACT_STAGES);
+#define LY(field) (HS ? LC.field : a.lay.field)
+    const int Hs = HS ? HS : a.Hs, H = CS * Hs, NST = LY(stages);
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 127u) & ~127u;
     unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
-    const Lay& y = a.lay;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int j = (int)cluster_ctarank(), c = (int)cluster_id_x(), NC = (int)cluster_count_x();
-    const int Hs = a.Hs, H = CS * Hs, T = a.T, L = a.L, B = a.B, I = a.I, NST = a.stages;
-    const int n_items = L * B;
+    const int j = (int)cluster_ctarank();
+    const int n_items = a.L * a.B;
     const int anchor_mode = EQ4 ? a.anchor_mode : (int)RM_ANCHOR_NONE;
-    const uint32_t bar0 = base + y.off_bar;
-    auto g_full = [&](int s) { return bar0 + 8 * s; };
-    auto g_empty = [&](int s) { return bar0 + 128 + 8 * s; };
-    auto d_full = [&](int s) { return bar0 + 256 + 8 * s; };
-    auto d_empty = [&](int s) { return bar0 + 384 - 0 + 8 * s; };
-    // (the remaining barriers and flags live behind the sums of squares' buffers, in the item table's last entry)
-    Item* items = reinterpret_cast<Item*>(gbase + y.off_item);
-    float* sSS = reinterpret_cast<float*>(gbase + y.off_ss);
-    __shared__ __align__(8) unsigned long long sBar[2 + 2 + 2 + SSB];
+    auto g_full = [&](int s) { return base + 8 * s; };
+    auto g_empty = [&](int s) { return base + 128 + 8 * s; };
+    auto d_full = [&](int s) { return base + 256 + 8 * s; };
+    auto d_empty = [&](int s) { return base + 384 + 8 * s; };
+    Item* items = reinterpret_cast<Item*>(gbase + LY(off_item));
+    float* sSS = reinterpret_cast<float*>(gbase + LY(off_ss));
+    __shared__ __align__(8) unsigned long long sBar[4 + SSB];
     __shared__ int sAbortW, sSeen;
-    auto p_full = [&](int b) { return smem_u32(&sBar[b]); };
-    auto h_full = [&](int b) { return smem_u32(&sBar[2 + b]); };
-    auto h_free = [&](int b) { return smem_u32(&sBar[4 + b]); };
-    auto ss_bar = [&](int b) { return smem_u32(&sBar[6 + b]); };
+    auto p_full = [&](int b) { return smem_u32(&sBar[b]); };       // per owned tile of a round
+    const uint32_t h_full = smem_u32(&sBar[2]), h_free = smem_u32(&sBar[3]);
+    auto ss_bar = [&](int b) { return smem_u32(&sBar[4 + b]); };
     volatile int* sAbort = &sAbortW;
 
     // ---- set-up
-    if (blockIdx.x == 0) {                 // the launch's counters, then its epoch
-        for (int e = tid; e < B * CS * 2; e += NTHREADS) a.ctrl[CTRL_LINE * (1 + e)] = 0;
+    if (blockIdx.x == 0) {                 // the launch's counters, then (below) its epoch
+        for (int e = tid; e < a.B * CS * 2; e += NTHREADS) a.ctrl[CTRL_LINE * (1 + e)] = 0;
         if (tid == 0) { a.ctrl[2] = 0; a.ctrl[3] = 0; }
         __threadfence();
     }
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) { mbar_init(g_full(s), 1); mbar_init(g_empty(s), 2); mbar_init(d_full(s), 1); mbar_init(d_empty(s), 8); }
-        for (int b = 0; b < 2; ++b) { mbar_init(p_full(b), 1); mbar_init(h_full(b), 1); mbar_init(h_free(b), CS * 8); }
+        mbar_init(p_full(0), 1); mbar_init(p_full(1), 1); mbar_init(h_full, 1); mbar_init(h_free, CS * 8);
         for (int b = 0; b < SSB; ++b) mbar_init(ss_bar(b), 1);
         fence_mbar_init();
         *sAbort = 0;
@@ -250,63 +252,60 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
     {
         // counts, then this cluster's part of every item.  The lists of a layer's episodes, laid end to end, are cut evenly
         // over the clusters: cluster k takes positions [S k / NC, S (k + 1) / NC) of the S = sum of the counts.
-        const int cap = (int)(a.list_cap < (int64_t)I ? a.list_cap : (int64_t)I);
-        for (int it = tid; it < n_items; it += NTHREADS) {
-            const int l = it / B, e = it - l * B, b = e / a.n_sub;
-            int k = I;
+        const int c = (int)cluster_id_x(), NC = (int)cluster_count_x(), B = a.B;
+        const int cap = (int)(a.list_cap < (int64_t)a.I ? a.list_cap : (int64_t)a.I);
+        const int it = tid, l = it / B, e = it - l * B;            // (n_items <= 512 < NTHREADS)
+        if (it < n_items) {
+            int k = a.I;
             if (a.count) {
-                k = a.count[(size_t)b * a.count_b_stride + l];
+                k = a.count[(size_t)(e / a.n_sub) * a.count_b_stride + l];
                 if (k < 0 || k > cap) { rm_set_status(a.status, RM_ERR_INDEX); k = k < 0 ? 0 : cap; }
             }
             items[it].n = k;
         }
         __syncthreads();
-        Item mine[1];
-        for (int it0 = 0; it0 < n_items; it0 += NTHREADS) {        // (n_items <= 512 < NTHREADS: one pass)
-            const int it = it0 + tid;
-            if (it < n_items) {
-                const int l = it / B, e = it - l * B, K = items[it].n;
-                unsigned S = 0, P = 0;
-                for (int b2 = 0; b2 < B; ++b2) {
-                    const unsigned K2 = (unsigned)items[l * B + b2].n;
-                    S += K2;
-                    P += b2 < e ? K2 : 0u;
-                }
-                Item r{0, 0, 0, 0};
-                if (K == 0) {
-                    r.parts_share = 1 | (e % NC == c ? 1 << 16 : 0);
-                } else {
-                    int parts = 0, share = 0;
-                    for (int k = 0; k < NC; ++k) {
-                        const unsigned lo = S * (unsigned)k / (unsigned)NC, hi = S * (unsigned)(k + 1) / (unsigned)NC;
-                        const unsigned x0 = lo > P ? lo : P, x1 = hi < P + K ? hi : P + K;
-                        if (x1 > x0) {
-                            if (k == c) { r.start = (int)(x0 - P); r.n = (int)(x1 - x0); share = parts; }
-                            ++parts;
-                        }
+        Item r{0, 0, 0, 0};
+        if (it < n_items) {
+            const unsigned K = (unsigned)items[it].n;
+            unsigned S = 0, P = 0;
+            for (int b2 = 0; b2 < B; ++b2) {
+                const unsigned K2 = (unsigned)items[l * B + b2].n;
+                S += K2;
+                P += b2 < e ? K2 : 0u;
+            }
+            if (K == 0) {
+                r.parts_share = 1 | (e % NC == c ? 1 << 16 : 0);
+            } else {
+                int parts = 0, share = 0;
+                for (int k = 0; k < NC; ++k) {
+                    const unsigned lo = S * (unsigned)k / (unsigned)NC, hi = S * (unsigned)(k + 1) / (unsigned)NC;
+                    const unsigned x0 = lo > P ? lo : P, x1 = hi < P + K ? hi : P + K;
+                    if (x1 > x0) {
+                        if (k == c) { r.start = (int)(x0 - P); r.n = (int)(x1 - x0); share = parts; }
+                        ++parts;
                     }
-                    r.parts_share = parts | share << 8 | (r.n > 0 ? 1 << 16 : 0);
                 }
-                mine[0] = r;
+                r.parts_share = parts | share << 8 | (r.n > 0 ? 1 << 16 : 0);
             }
         }
         __syncthreads();
-        if (tid < n_items) items[tid] = mine[0];
+        if (it < n_items) items[it] = r;
         __syncthreads();
         if (tid < B) {
             int t = 0;
-            for (int l = 0; l < L; ++l) {
-                items[l * B + tid].target = t;
-                t += items[l * B + tid].parts_share & 0xff;
+            for (int l2 = 0; l2 < a.L; ++l2) {
+                items[l2 * B + tid].target = t;
+                t += items[l2 * B + tid].parts_share & 0xff;
             }
         }
     }
     // x rows past T, columns past Hs, and weight slots that no copy has filled yet have to hold finite numbers: zeros
-    for (int e = tid; e < 64 * y.xp / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + y.off_x)[e] = make_uint4(0u, 0u, 0u, 0u);
-    for (int e = tid; e < (y.total - 128 - y.off_g) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + y.off_g)[e] = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = tid; e < 64 * LY(xp) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_x))[e] = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = tid; e < (LY(off_item) - LY(off_g)) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_g))[e] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async_smem();
     __syncthreads();
     cluster_sync();                        // peers' shared memory and barriers are live from here on
+    pdl_launch_dependents();               // (a dependent waits for this grid's end: its CTAs are resident by then)
     if (blockIdx.x == 0 && tid == 0) {
         __threadfence();
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(a.ctrl), "l"(a.epoch) : "memory");
@@ -318,196 +317,220 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         gave_up = wait_slow(bar, parity, line, a, sAbort);
     };
 #define WAIT(bar, parity) wait_at((bar), (parity), __LINE__)
+    // One round of tests for up to 32 barriers, a lane each (a test takes ~200 clocks to come back), for a whole warp
+    auto wait_lanes = [&](bool active, uint32_t bar, uint32_t parity, int line) {
+        if (__all_sync(0xffffffffu, !active || gave_up || mbar_test_wait(bar, parity))) return;
+        if (active && !gave_up) gave_up = wait_slow(bar, parity, line, a, sAbort);
+        gave_up = __any_sync(0xffffffffu, gave_up);
+    };
     // first token row (of the caller's [B, T_all]) and tokens of episode e
     auto row0_of = [&](int e) {
-        if (a.n_sub == 1) return (size_t)e * T;
+        if (a.n_sub == 1) return (size_t)e * a.T;
         const int b = e / a.n_sub, s = e - b * a.n_sub;
-        return (size_t)b * a.T_all + (size_t)s * T;
+        return (size_t)b * a.T_all + (size_t)s * a.T;
     };
     auto tokens_of = [&](int e) {
-        if (a.n_sub == 1) return T;
-        const int s = e % a.n_sub, left = a.T_all - s * T;
-        return left < T ? left : T;
+        if (a.n_sub == 1) return a.T;
+        const int s = e % a.n_sub, left = a.T_all - s * a.T;
+        return left < a.T ? left : a.T;
     };
     auto list_of = [&](int l, int e) { return a.idx ? a.idx + (size_t)(a.n_sub == 1 ? e : e / a.n_sub) * a.idx_b_stride + (size_t)l * a.idx_l_stride : nullptr; };
-    auto out_of = [&](int l) { return l == L - 1 ? a.r_out : a.rot[l % 3]; };
+    auto out_of = [&](int l) { return l == a.L - 1 ? a.r_out : a.rot[l % 3]; };
+    const int most = 8 * TS < 2 * NST ? 8 * TS : 2 * NST;          // tiles per round: every one of its stages fits the ring
 
     if (warp >= W_G) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_L));
         if (warp < W_G + 2) {
-        // ================================================================ loaders: a stage is the pieces of 16 neurons, one
-        // bulk copy per neuron; they run as far ahead as the ring lets them (the lists are known before the step starts)
-        const bool is_g = warp == W_G;
-        const uint32_t ring = base + (is_g ? y.off_g : y.off_d), bytes = (uint32_t)Hs * (is_g ? 4u : 2u);
-        const int pitch = is_g ? y.gp : y.dp, stage_bytes = is_g ? y.g_stage : y.d_stage;
-        const uint32_t full0 = is_g ? g_full(0) : d_full(0), empty0 = is_g ? g_empty(0) : d_empty(0);
-        int slot = 0;
-        uint32_t pass = 0;
-        for (int it = 0, l = 0, e = 0; it < n_items && !gave_up; ++it, (++e == B ? (e = 0, ++l) : 0)) {
-            const Item w = items[it];
-            if (w.n == 0) continue;
-            const int32_t* list = list_of(l, e);
-            const __nv_bfloat16* src = a.packed[l] + (size_t)j * 3 * Hs + (is_g ? 0 : 2 * Hs);
-            auto neuron = [&](int k) {
-                int n = -1;
-                if (lane < SN && k + lane < w.n) {
-                    n = list ? __ldg(list + w.start + k + lane) : w.start + k + lane;
-                    if (n < 0 || n >= I) { rm_set_status(a.status, RM_ERR_INDEX); n = -1; }
+            // ============================================================ loaders: a stage is the pieces of two tiles, one bulk
+            // copy per neuron; they run as far ahead as the ring lets them (the lists are known before the step starts)
+            const bool is_g = warp == W_G;
+            // (8 columns past an up piece meet zeros of x in the last 16-column step: they have to be numbers, and the stage has
+            // held partial sums since it was cleared -- so the copy goes on into the down piece)
+            const uint32_t ring = base + (is_g ? LY(off_g) : LY(off_d)), bytes = (uint32_t)Hs * (is_g ? 4u : 2u) + (is_g && Hs % 16 ? 16u : 0u);
+            const int pitch = is_g ? LY(gp) : LY(dp), stage_bytes = is_g ? LY(g_stage) : LY(d_stage);
+            const uint32_t full0 = is_g ? g_full(0) : d_full(0), empty0 = is_g ? g_empty(0) : d_empty(0);
+            int slot = 0;
+            uint32_t pass = 0;
+            for (int it = 0, l = 0, e = 0; it < n_items && !gave_up; ++it, (++e == a.B ? (e = 0, ++l) : 0)) {
+                const Item w = items[it];
+                if (w.n == 0) continue;
+                const int32_t* list = list_of(l, e);
+                const __nv_bfloat16* src = a.packed[l] + (size_t)j * 3 * Hs + (is_g ? 0 : 2 * Hs);
+                const int nrd = round_count(w.n, most);
+                for (int r = 0; r < nrd && !gave_up; ++r) {
+                    int pos, nr;
+                    round_span(w.n, r, nrd, pos, nr);
+                    auto neuron = [&](int k) {
+                        int n = -1;
+                        if (lane < SN && k + lane < nr) {
+                            n = w.start + pos + k + lane;
+                            if (list) n = __ldg(list + n);
+                            if (n < 0 || n >= a.I) { rm_set_status(a.status, RM_ERR_INDEX); n = -1; }
+                        }
+                        return n;
+                    };
+                    int n = neuron(0);
+                    for (int k = 0; k < nr && !gave_up; k += SN) {
+                        const int next = neuron(k + SN);           // (asked for before this stage's wait)
+                        if (pass > 0) WAIT(empty0 + 8 * slot, (pass - 1) & 1);
+                        const uint32_t m = __ballot_sync(0xffffffffu, n >= 0);
+                        if (lane == 0) mbar_arrive_expect_tx(full0 + 8 * slot, (uint32_t)__popc(m) * bytes);
+                        __syncwarp();
+                        if (n >= 0) bulk_load(ring + slot * stage_bytes + lane * pitch, src + (size_t)n * 3 * H, bytes, full0 + 8 * slot);
+                        n = next;
+                        if (++slot == NST) { slot = 0; ++pass; }
+                        gave_up = __any_sync(0xffffffffu, gave_up);
+                    }
                 }
-                return n;
-            };
-            int n = neuron(0);
-            for (int k = 0; k < w.n && !gave_up; k += SN) {
-                const int next = neuron(k + SN);                   // (asked for before this stage's wait)
-                if (pass > 0) WAIT(empty0 + 8 * slot, (pass - 1) & 1);
-                const uint32_t m = __ballot_sync(0xffffffffu, n >= 0);
-                if (lane == 0) mbar_arrive_expect_tx(full0 + 8 * slot, (uint32_t)__popc(m) * bytes);
-                __syncwarp();
-                if (n >= 0) bulk_load(ring + slot * stage_bytes + lane * pitch, src + (size_t)n * 3 * H, bytes, full0 + 8 * slot);
-                n = next;
-                if (++slot == NST) { slot = 0; ++pass; }
-                gave_up = __any_sync(0xffffffffu, gave_up);
             }
-        }
         }
     } else if (warp < W_B) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_A));
         // ================================================================ group A: x of an item, then its gate/up products
-        const int team = TEAMS == 2 ? warp >> 2 : 0, mp = TEAMS == 2 ? (warp >> 1) & 1 : warp >> 1, nh = warp & 1;
-        const int cnt = nh ? y.n_b : y.n_a, nt0 = nh ? y.n_a : 0;  // this warp's 8-token tiles
+        const int mp = warp >> 1, nh = warp & 1;                   // gate/up: pair of tiles mp, mp + 4 of a round; token half
+        const int t8 = (a.T + 7) / 8, cnt = nh ? (t8 > 4 ? t8 - 4 : 0) : (t8 < 4 ? t8 : 4);
         const int t = tid >> 2, q = tid & 3, n4 = Hs / 4;          // normalisation: token row, every fourth float4 of its slice
-        const uint32_t a_lane = (lane & 7) * y.gp + ((lane >> 3) & 1) * 2 * Hs + (lane >> 4) * 16;
-        const uint32_t x_lane = base + y.off_x + (nt0 * 8 + ((lane >> 4) << 3) + (lane & 7)) * y.xp + ((lane >> 3) & 1) * 16;
-        unsigned char* stg = gbase + y.off_stg + warp * y.stg_warp;
-        const uint32_t s_stg = base + y.off_stg + warp * y.stg_warp;
+        const uint32_t a_lane = base + LY(off_g) + (lane & 7) * LY(gp) + ((lane >> 3) & 1) * 2 * Hs + (lane >> 4) * 16;
+        const uint32_t x_lane = base + LY(off_x) + (nh * 32 + ((lane >> 4) << 3) + (lane & 7)) * LY(xp) + ((lane >> 3) & 1) * 16;
         uint32_t R = 0;                                            // rounds before this one
         int g_slot = 0, ni = 0, pi = 0;                            // ring slot of the round's first stage; items so far
         uint32_t g_pass = 0;
-        for (int it = 0, l = 0, e = 0; it < n_items; ++it, (++e == B ? (e = 0, ++l) : 0)) {
+        for (int it = 0, l = 0, e = 0; it < n_items; ++it, (++e == a.B ? (e = 0, ++l) : 0)) {
             const Item w = items[it];
             if (!(w.parts_share >> 16)) continue;
             const int Te = tokens_of(e);
-            const size_t row = row0_of(e) + t;
+            const float4* src = reinterpret_cast<const float4*>((l == 0 ? a.r_in : out_of(l - 1)) + (row0_of(e) + t) * H + (size_t)j * Hs) + q;
             // ---- every cluster has added its part of the layer before to this slice (one thread looks)
             if (tid == 0 && !gave_up) {
                 if (pi == 0) gave_up = epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
                 if (l > 0 && !gave_up) gave_up = counter_wait(a.ctrl + ctrl_done(e, j), w.target, __LINE__, a, sAbort);
                 asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(&sSeen)), "r"(pi + 1) : "memory");
             }
-            if (w.n == 0) { ++pi; continue; }                      // (nothing selected: group B passes the residual on)
+            ++pi;
             if (barrier_or(1, 256, gave_up || *sAbort)) break;
-            const bool ext = a.x_ext != nullptr;
-            float4 v[MAXV];
-            float ss = 0.f;
-            if (!ext) {
-                const float4* src = reinterpret_cast<const float4*>((l == 0 ? a.r_in : out_of(l - 1)) + row * H + (size_t)j * Hs);
+            if (w.n == 0) continue;                                // (nothing selected: group B passes the residual on)
+            // ---- x tile: [token][column] bf16
+            if (a.x_ext) {
+                const uint4* xs = reinterpret_cast<const uint4*>(a.x_ext + (row0_of(e) + t) * H + (size_t)j * Hs);
 #pragma unroll
-                for (int i = 0; i < MAXV; ++i)
-                    v[i] = t < Te && q + 4 * i < n4 ? __ldcg(src + q + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = 0; i < MAXV / 2; ++i)
+                    if (t < Te && q + 4 * i < Hs / 8) *reinterpret_cast<uint4*>(gbase + LY(off_x) + t * LY(xp) + (q + 4 * i) * 16) = xs[q + 4 * i];
+            } else {
+                float4 v[MAXV];
+                float ss = 0.f;
+#pragma unroll
+                for (int i = 0; i < MAXV; ++i) v[i] = t < Te && (HS || q + 4 * i < n4) ? __ldcg(src + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int i = 0; i < MAXV; ++i) {
                     ss = fmaf(v[i].x, v[i].x, ss); ss = fmaf(v[i].y, v[i].y, ss);
                     ss = fmaf(v[i].z, v[i].z, ss); ss = fmaf(v[i].w, v[i].w, ss);
                 }
-                {
-                    // all-gather of the row sums of squares over the cluster: lane q of a row sends to CTAs q and q + 4
-                    ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-                    ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-                    const uint32_t bar = ss_bar(ni & (SSB - 1)), at = smem_u32(sSS + ((ni & (SSB - 1)) * CS + j) * 64 + t);
-                    if (tid == 0) mbar_arrive_expect_tx(bar, CS * 64 * 4);
-                    st_async_f32(map_to_rank(at, q), ss, map_to_rank(bar, q));
-                    st_async_f32(map_to_rank(at, q + 4), ss, map_to_rank(bar, q + 4));
-                }
-            }
-            // ---- x tile: [token][column] bf16
-            if (ext) {
-                const uint4* src = reinterpret_cast<const uint4*>(a.x_ext + row * H + (size_t)j * Hs);
-#pragma unroll
-                for (int i = 0; i < MAXV / 2; ++i)
-                    if (t < Te && q + 4 * i < Hs / 8) *reinterpret_cast<uint4*>(gbase + y.off_x + t * y.xp + (q + 4 * i) * 16) = src[q + 4 * i];
-            } else {
-                const float* sums = sSS + (ni & (SSB - 1)) * CS * 64 + t;
-                WAIT(ss_bar(ni & (SSB - 1)), (ni / SSB) & 1);
-                float tot = 0.f;
-#pragma unroll
-                for (int s = 0; s < CS; ++s) tot += sums[s * 64];
-                const float inv = 1.0f / sqrtf(tot / (float)H + 1e-6f);
+                // all-gather of the row sums of squares over the cluster: lane q of a row sends to CTAs q and q + 4
+                ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+                ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+                const int sb = ni & (SSB - 1);
+                const uint32_t bar = ss_bar(sb), at = smem_u32(sSS) + ((sb * 64 + t) * CS + j) * 4;
+                if (tid == 0) mbar_arrive_expect_tx(bar, CS * 64 * 4);
+                st_async_f32(map_to_rank(at, q), ss, map_to_rank(bar, q));
+                st_async_f32(map_to_rank(at, q + 4), ss, map_to_rank(bar, q + 4));
+                WAIT(bar, (ni / SSB) & 1);
+                const float4* sums = reinterpret_cast<const float4*>(sSS + (sb * 64 + t) * CS);
+                const float4 s0 = sums[0], s1 = sums[1];
+                const float tot = ((s0.x + s0.y) + (s0.z + s0.w)) + ((s1.x + s1.y) + (s1.z + s1.w));
+                const float inv = __frsqrt_rn(tot / (float)H + 1e-6f);
+                unsigned char* xr = gbase + LY(off_x) + t * LY(xp) + q * 8;
 #pragma unroll
                 for (int i = 0; i < MAXV; ++i) {
-                    if (q + 4 * i >= n4) continue;                 // (rows past Te: v = 0, so x = 0)
+                    if (!HS && q + 4 * i >= n4) continue;          // (rows past Te: v = 0, so x = 0)
                     const __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x * inv, v[i].y * inv);
                     const __nv_bfloat162 hi = __floats2bfloat162_rn(v[i].z * inv, v[i].w * inv);
                     uint2 u;
                     u.x = *reinterpret_cast<const uint32_t*>(&lo);
                     u.y = *reinterpret_cast<const uint32_t*>(&hi);
-                    *reinterpret_cast<uint2*>(gbase + y.off_x + t * y.xp + (q + 4 * i) * 8) = u;
+                    *reinterpret_cast<uint2*>(xr + i * 32) = u;
                 }
+                ++ni;
             }
-            ++ni;
-            ++pi;
-            if (barrier_or(1, 256, gave_up || *sAbort)) break;
-            // ---- gate/up: warp (mp, nh) multiplies stage mp of a round (two row tiles) with half of the tokens
-            for (int pos = 0; pos < w.n; pos += RN, ++R) {
-                const int nr = w.n - pos < RN ? w.n - pos : RN, ns = (nr + SN - 1) / SN;
-                if (TEAMS == 1 || (int)(R & 1) == team) {
-                    const bool act = mp < ns;
+            named_barrier(1, 256);
+            // ---- gate/up: warp (mp, nh) multiplies the pairs of tiles mp and mp + 4 of a round with its half of the tokens
+            const int nrd = round_count(w.n, most);
+            for (int r = 0; r < nrd; ++r, ++R) {
+                int pos, nr;
+                round_span(w.n, r, nrd, pos, nr);
+                const int tiles = (nr + TN - 1) / TN, pairs = (tiles + 1) / 2;
+                {
+                    const int p = mp + 4 * lane;                   // lane u looks at the stage of this warp's pair u
+                    int slot = g_slot + p;
+                    uint32_t ps = g_pass;
+                    if (slot >= NST) { slot -= NST; ++ps; }
+                    wait_lanes(lane < TS && p < pairs, g_full(slot), ps & 1, __LINE__);
+                }
+                int held = -1;                                     // stage that this warp's outgoing sums still lie in
+#pragma unroll 1
+                for (int u = 0; u < TS; ++u) {
+                    const int p = mp + 4 * u;
+                    if (p >= pairs) break;
+                    int slot = g_slot + p;
+                    if (slot >= NST) slot -= NST;
                     float acc[2][4][4];
-                    if (act) {
-                        int slot = g_slot + mp;
-                        uint32_t ps = g_pass;
-                        if (slot >= NST) { slot -= NST; ++ps; }
 #pragma unroll
-                        for (int u = 0; u < 2; ++u)
+                    for (int m = 0; m < 2; ++m)
 #pragma unroll
-                            for (int n = 0; n < 4; ++n) acc[u][n][0] = acc[u][n][1] = acc[u][n][2] = acc[u][n][3] = 0.f;
-                        WAIT(g_full(slot), ps & 1);
-                        const uint32_t ga = base + y.off_g + slot * y.g_stage + a_lane, gb = ga + 8 * y.gp;
-#pragma unroll 2
-                        for (int ks = 0; ks < y.ks; ++ks) {
-                            uint32_t A0[4], A1[4], X0[4], X1[4];
-                            ldm4(ga + ks * 32, A0);
-                            ldm4(gb + ks * 32, A1);
-                            ldm4(x_lane + ks * 32, X0);
-                            if (cnt > 2) ldm4(x_lane + 16 * y.xp + ks * 32, X1);
-                            mma16816(acc[0][0], A0, X0[0], X0[1]);
-                            mma16816(acc[1][0], A1, X0[0], X0[1]);
-                            if (cnt > 1) { mma16816(acc[0][1], A0, X0[2], X0[3]); mma16816(acc[1][1], A1, X0[2], X0[3]); }
-                            if (cnt > 2) { mma16816(acc[0][2], A0, X1[0], X1[1]); mma16816(acc[1][2], A1, X1[0], X1[1]); }
-                            if (cnt > 3) { mma16816(acc[0][3], A0, X1[2], X1[3]); mma16816(acc[1][3], A1, X1[2], X1[3]); }
-                        }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(g_empty(slot));
+                        for (int n = 0; n < 4; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+                    const uint32_t ga = a_lane + slot * LY(g_stage);
+#pragma unroll 4
+                    for (int ks = 0; ks < LY(ks); ++ks) {
+                        uint32_t A0[4], A1[4], X0[4], X1[4];
+                        ldm4(ga + ks * 32, A0);
+                        ldm4(x_lane + ks * 32, X0);
+                        ldm4(ga + 8 * LY(gp) + ks * 32, A1);
+                        if (cnt > 2) ldm4(x_lane + 16 * LY(xp) + ks * 32, X1);
+                        mma16816(acc[0][0], A0, X0[0], X0[1]);
+                        if (cnt > 1) mma16816(acc[0][1], A0, X0[2], X0[3]);
+                        mma16816(acc[1][0], A1, X0[0], X0[1]);
+                        if (cnt > 1) mma16816(acc[1][1], A1, X0[2], X0[3]);
+                        if (cnt > 2) { mma16816(acc[0][2], A0, X1[0], X1[1]); mma16816(acc[1][2], A1, X1[0], X1[1]); }
+                        if (cnt > 3) { mma16816(acc[0][3], A0, X1[2], X1[3]); mma16816(acc[1][3], A1, X1[2], X1[3]); }
                     }
-                    // every owner has used up the partial sums of two rounds ago: h of that round is complete here
-                    if (R >= 2) WAIT(h_full(R & 1), ((R >> 1) - 1) & 1);
-                    if (act && cnt > 0) {
-                        bulk_wait_read_all();                      // this warp's pieces of its previous round have left
+                    // both warps of the pair have read the stage: it holds their outgoing sums now, 4 KB each
+                    named_barrier(3 + mp, 64);
+                    if (held >= 0) {                               // (the previous pair's sums have left by now)
+                        bulk_wait_read_all();
                         __syncwarp();
-                        // [row tile][neuron][token pair] (gate, gate, up, up)
+                        if (lane == 0) mbar_arrive(g_empty(held));
+                    }
+                    held = slot;
+                    const int out = LY(off_g) + slot * LY(g_stage) + nh * 4096;
+                    unsigned char* d = gbase + out + lane * 16;
 #pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            unsigned char* d = stg + (u * 8 + (lane >> 2)) * (cnt * 64) + (lane & 3) * 16;
+                    for (int m = 0; m < 2; ++m)
 #pragma unroll
-                            for (int n = 0; n < 4; ++n)
-                                if (n < cnt) *reinterpret_cast<float4*>(d + n * 64) = make_float4(acc[u][n][0], acc[u][n][1], acc[u][n][2], acc[u][n][3]);
-                        }
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        constexpr int OPT = 8 / OPN;               // owners per row tile
-                        if (lane < 2 * OPT) {
-                            const int o = 2 * OPT * mp + lane;     // owner; its neurons are OPN o .. of the round
-                            if (o * OPN < nr && !gave_up) {
-                                const uint32_t piece = (uint32_t)OPN * cnt * 64;
-                                const uint32_t dst = base + y.off_p + (R & 1) * y.p_buf + j * y.p_src + nh * (OPN * y.n_a * 64);
-                                bulk_copy_to_peer(map_to_rank(dst, o), s_stg + lane * piece, piece, map_to_rank(p_full(R & 1), o));
-                            }
-                        }
-                        // (the lanes' copies are waited for by the lanes that issued them)
-                        if (lane < 2 * OPT) bulk_commit();
+                        for (int n = 0; n < 4; ++n)
+                            if (n < cnt) *reinterpret_cast<float4*>(d + m * 2048 + n * 512) = make_float4(acc[m][n][0], acc[m][n][1], acc[m][n][2], acc[m][n][3]);
+                    fence_proxy_async_smem();
+                    // every owner has used up the sums of the round before: h of that round is complete here
+                    if (R >= 1 && u == 0) WAIT(h_full, (R - 1) & 1);
+                    __syncwarp();
+                    const int tile = 2 * p + lane;                 // lanes 0 and 1 send a tile each
+                    if (lane < 2 && tile < tiles && cnt > 0 && !gave_up) {
+                        const int o = tile & 7, s = tile >> 3;     // its owner, and which of the owner's tiles it is
+                        bulk_copy_to_peer(map_to_rank(base + LY(off_p) + s * P_SLOT + j * P_SRC + nh * 2048, o), base + out + lane * 2048,
+                                          (uint32_t)cnt * 512u, map_to_rank(p_full(s), o));
+                        bulk_commit();
                     }
                 }
-                g_slot += ns;
+                if (held >= 0) {
+                    bulk_wait_read_all();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(g_empty(held));
+                } else if (R >= 1) {
+                    WAIT(h_full, (R - 1) & 1);                     // (a warp follows every phase: parity tells two apart)
+                }
+                g_slot += pairs;
                 if (g_slot >= NST) { g_slot -= NST; ++g_pass; }
+                // A parity tells a phase from the one before it only.  A ring slot's phases belong to different warps, and copies
+                // complete in any order: no warp looks at a slot's next phase before every warp has seen its own in this round.
+                if (r + 1 < nrd) named_barrier(1, 256);
             }
         }
         bulk_wait_read_all();
@@ -517,25 +540,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         const int bt = tid - W_B * 32, bw = warp - W_B;
         const int th = bw & 1, cg = bw >> 1;                       // token half and column group of this warp's down products
         const int pairs = (Hs / 8 + 1) / 2, gpp = (pairs + 3) / 4; // pairs of 8-column tiles: of the slice, of a group
-        const int cp0 = cg * gpp, cpn = pairs - cp0 < gpp ? pairs - cp0 : gpp;
-        const int t16 = (T + 15) / 16, mh = (t16 + 1) / 2, m0 = th * mh, mcnt = t16 - m0 < mh ? t16 - m0 : mh;
-        const int np = (y.n_a + y.n_b) * 4, na = y.n_a * 4;        // token pairs; of the first half
-        const uint32_t h_lane = base + y.off_h + ((lane & 7) + ((lane >> 4) & 1) * 8) * HPITCH + (m0 * 16 + ((lane >> 3) & 1) * 8) * 2;
-        const uint32_t d_lane = ((lane & 7) + ((lane >> 3) & 1) * 8) * y.dp + (cp0 * 16 + (lane >> 4) * 8) * 2;
+        const int cp0 = cg * gpp, cpn = HS ? NG / 2 : (pairs - cp0 < gpp ? pairs - cp0 : gpp);
+        const int t16 = (a.T + 15) / 16, mh = (t16 + 1) / 2, m0 = th * mh, mcnt = t16 - m0 < mh ? t16 - m0 : mh;
+        const int np = (a.T + 7) / 8 * 4;                          // token pairs
+        const uint32_t h_lane = base + LY(off_h) + ((lane & 7) + ((lane >> 4) & 1) * 8) * HPITCH + (m0 * 16 + ((lane >> 3) & 1) * 8) * 2;
+        const uint32_t d_lane = base + LY(off_d) + ((lane & 7) + ((lane >> 3) & 1) * 8) * LY(dp) + (cp0 * 16 + (lane >> 4) * 8) * 2;
         uint32_t R = 0, p_par = 0, d_pass = 0;
         int d_slot = 0, pi = 0;
         bool stop = false;
-        for (int it = 0, l = 0, e = 0; it < n_items && !stop; ++it, (++e == B ? (e = 0, ++l) : 0)) {
+        for (int it = 0, l = 0, e = 0; it < n_items && !stop; ++it, (++e == a.B ? (e = 0, ++l) : 0)) {
             const Item w = items[it];
             if (!(w.parts_share >> 16)) continue;
             const int Te = tokens_of(e), b = a.n_sub == 1 ? e : e / a.n_sub, nb = a.nb;
-            const size_t tok0 = (size_t)(e - b * a.n_sub) * T;     // first token of the chunk inside its episode
+            const size_t tok0 = (size_t)(e - b * a.n_sub) * a.T;   // first token of the chunk inside its episode
             const int32_t* list = list_of(l, e);
-            float acc[2][NG][4];
-#pragma unroll
-            for (int m = 0; m < 2; ++m)
-#pragma unroll
-                for (int n = 0; n < NG; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
             // ---- while group A prepares x: this cluster's share of the layer's residual (+ gate * y_a in an update step) and
             // of the clearing of the next layer's output buffer.  Both need the layer before to be complete, which group A's
             // first thread has seen.
@@ -569,10 +587,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (l > 0) red_add_v4(out, r.x, r.y, r.z, r.w);
                     else if (out != in + o || !a.x_ext) *reinterpret_cast<float4*>(out) = r;
-                    if (l + 1 < L) *reinterpret_cast<float4*>(out_of(l + 1) + o) = zero;
+                    if (l + 1 < a.L) *reinterpret_cast<float4*>(out_of(l + 1) + o) = zero;
                     if (EQ4 && anchor_mode == RM_ANCHOR_WRITE) {
                         if (l == 0) *reinterpret_cast<float4*>(a.y_anchor + o) = zero;
-                        if (l + 1 < L) *reinterpret_cast<float4*>(a.y_anchor + (l + 1) * layer + o) = zero;
+                        if (l + 1 < a.L) *reinterpret_cast<float4*>(a.y_anchor + (l + 1) * layer + o) = zero;
                     }
                 }
             }
@@ -580,55 +598,60 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                 stop = barrier_or(2, 256, gave_up || *sAbort);
                 if (bt == 0 && !stop) red_release_gpu(a.ctrl + ctrl_init(e, j), 1);
             }
-            const int rounds = (w.n + RN - 1) / RN;
-            for (int r = 0; r <= rounds && w.n > 0 && !stop; ++r) {
-                if (r < rounds) {
-                    // ---- owner work of round r: warp i has this CTA's neuron i, lane = token pair
-                    const uint32_t Rr = R + r, buf = Rr & 1;
-                    const int pos = r * RN, nr = w.n - pos < RN ? w.n - pos : RN, ns = (nr + SN - 1) / SN;
-                    const int n_own = (nr + OPN - 1) / OPN;
-                    const bool own = j < n_own;
-                    const int qn = j * OPN + bw;
-                    int n = -1;
-                    if (own && bw < OPN && qn < nr) {
-                        n = list ? __ldg(list + w.start + pos + qn) : w.start + pos + qn;
-                        if (n < 0 || n >= I) n = -1;               // (reported by the loaders)
-                    }
-                    float2 ha = make_float2(0.f, 0.f);
-                    float2* hap = nullptr;
-                    if (EQ4 && anchor_mode != RM_ANCHOR_NONE && n >= 0 && 2 * lane < Te) {
-                        hap = reinterpret_cast<float2*>(a.h_anchor + (((size_t)l * nb + b) * I + n) * a.h_stride + tok0) + lane;
-                        if (anchor_mode == RM_ANCHOR_UPDATE) ha = __ldcg(hap);
-                    }
+            float acc[2][NG][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int n = 0; n < NG; ++n) acc[m][n][0] = acc[m][n][1] = acc[m][n][2] = acc[m][n][3] = 0.f;
+            const int nrd = round_count(w.n, most);
+            for (int r = 0; r < nrd; ++r, ++R) {
+                int pos, nr;
+                round_span(w.n, r, nrd, pos, nr);
+                const int tiles = (nr + TN - 1) / TN;
+                const int own = j < tiles ? (j + 8 < tiles ? 2 : 1) : 0;               // this CTA's tiles: j, j + 8
+                if (bt < own) mbar_arrive_expect_tx(p_full(bt), (uint32_t)np * (CS * TN * 16));
+                unsigned char* hb = gbase + LY(off_h);
+#pragma unroll 1
+                for (int s = 0; s < own || s == 0; ++s) {
+                    // ---- owner work: warp i has neuron i of the tile, lane = token pair
                     float h0 = 0.f, h1 = 0.f;
-                    if (own) {
-                        if (bt == 0) mbar_arrive_expect_tx(p_full(buf), (uint32_t)y.p_buf);
-                        WAIT(p_full(buf), (p_par >> buf) & 1u);
-                        p_par ^= 1u << buf;
-                        if (bw < OPN && lane < np) {
-                            const unsigned char* p = gbase + y.off_p + buf * y.p_buf +
-                                                     (lane < na ? bw * (na * 16) + lane * 16 : OPN * na * 16 + bw * ((np - na) * 16) + (lane - na) * 16);
-                            float4 s = *reinterpret_cast<const float4*>(p);
+                    if (s < own) {
+                        const int qn = (j + 8 * s) * TN + bw;
+                        int n = -1;
+                        if (qn < nr) {
+                            n = w.start + pos + qn;
+                            if (list) n = __ldg(list + n);
+                            if (n < 0 || n >= a.I) n = -1;         // (reported by the loaders)
+                        }
+                        float2 ha = make_float2(0.f, 0.f);
+                        float2* hap = nullptr;
+                        if (EQ4 && anchor_mode != RM_ANCHOR_NONE && n >= 0 && 2 * lane < Te) {
+                            hap = reinterpret_cast<float2*>(a.h_anchor + (((size_t)l * nb + b) * a.I + n) * a.h_stride + tok0) + lane;
+                            if (anchor_mode == RM_ANCHOR_UPDATE) ha = __ldcg(hap);
+                        }
+                        WAIT(p_full(s), (p_par >> s) & 1u);
+                        p_par ^= 1u << s;
+                        if (lane < np) {
+                            const unsigned char* p = gbase + LY(off_p) + s * P_SLOT + (lane >> 2) * 512 + bw * 64 + (lane & 3) * 16;
+                            float4 v = *reinterpret_cast<const float4*>(p);
 #pragma unroll
                             for (int k = 1; k < CS; ++k) {
-                                const float4 o = *reinterpret_cast<const float4*>(p + k * y.p_src);
-                                s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+                                const float4 o = *reinterpret_cast<const float4*>(p + k * P_SRC);
+                                v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
                             }
-                            if (n >= 0) {
-                                // GeLU-tanh(g) = g / (1 + exp(-2 z)), z = sqrt(2/pi) (g + 0.044715 g^3)
-                                const float e0 = __expf(-1.5957691216057308f * (s.x + 0.044715f * s.x * s.x * s.x));
-                                const float e1 = __expf(-1.5957691216057308f * (s.y + 0.044715f * s.y * s.y * s.y));
-                                if (2 * lane < Te) h0 = __fdividef(s.x, 1.0f + e0) * s.z;
-                                if (2 * lane + 1 < Te) h1 = __fdividef(s.y, 1.0f + e1) * s.w;
-                            }
+                            // GeLU-tanh(g) = g / (1 + exp(-2 z)), z = sqrt(2/pi) (g + 0.044715 g^3)
+                            const float e0 = __expf(-1.5957691216057308f * (v.x + 0.044715f * v.x * v.x * v.x));
+                            const float e1 = __expf(-1.5957691216057308f * (v.y + 0.044715f * v.y * v.y * v.y));
+                            if (n >= 0 && 2 * lane < Te) h0 = __fdividef(v.x, 1.0f + e0) * v.z;
+                            if (n >= 0 && 2 * lane + 1 < Te) h1 = __fdividef(v.y, 1.0f + e1) * v.w;
                         }
-                        if (a.record && bw < OPN) {
+                        if (a.record) {
                             float rec = fabsf(h0) + fabsf(h1);
 #pragma unroll
                             for (int d = 16; d > 0; d >>= 1) rec += __shfl_xor_sync(0xffffffffu, rec, d);
                             if (lane == 0 && n >= 0) {
-                                const float sc = a.record_scale ? a.record_scale[(size_t)l * I + n] : 1.f;
-                                a.record[(size_t)b * a.rec_b_stride + (size_t)l * I + n] = a.record_scale ? rec * sc : rec;
+                                const float sc = a.record_scale ? a.record_scale[(size_t)l * a.I + n] : 1.f;
+                                a.record[(size_t)b * a.rec_b_stride + (size_t)l * a.I + n] = a.record_scale ? rec * sc : rec;
                             }
                         }
                         if (EQ4 && hap) {
@@ -637,61 +660,63 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                             else { h0 -= ha.x; h1 -= 2 * lane + 1 < Te ? ha.y : 0.f; }
                         }
                     }
-                    // every CTA of the cluster is done with this h buffer's previous round
-                    if (Rr >= 2) WAIT(h_free(buf), ((Rr >> 1) - 1) & 1);
-                    unsigned char* hb = gbase + y.off_h + buf * y.h_buf;
-                    if (own && bw < OPN) {
+                    // every CTA of the cluster is done with the h tile of the round before
+                    if (s == 0 && R >= 1) WAIT(h_free, (R - 1) & 1);
+                    if (s < own) {
                         const __nv_bfloat162 hi = __floats2bfloat162_rn(h0, h1);
                         const float2 hf = __bfloat1622float2(hi);
                         const __nv_bfloat162 lo = __floats2bfloat162_rn(h0 - hf.x, h1 - hf.y);
-                        *reinterpret_cast<__nv_bfloat162*>(hb + qn * HPITCH + lane * 4) = hi;
-                        *reinterpret_cast<__nv_bfloat162*>(hb + qn * HPITCH + 128 + lane * 4) = lo;
+                        unsigned char* hr = hb + ((j + 8 * s) * TN + bw) * HPITCH + lane * 4;
+                        *reinterpret_cast<__nv_bfloat162*>(hr) = hi;
+                        *reinterpret_cast<__nv_bfloat162*>(hr + 128) = lo;
                     }
-                    for (int z = n_own * OPN * 16 + bt; z < ns * SN * 16; z += 256)      // rows of the last stage that nobody owns
-                        *reinterpret_cast<uint4*>(hb + (z >> 4) * HPITCH + (z & 15) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    if (s == 0 && (tiles & 1) && bt < TN * 16)     // the last stage's second half, which nobody owns
+                        *reinterpret_cast<uint4*>(hb + (tiles * TN + (bt >> 4)) * HPITCH + (bt & 15) * 16) = make_uint4(0u, 0u, 0u, 0u);
                     fence_proxy_async_smem();
                     stop = barrier_or(2, 256, gave_up || *sAbort);
-                    if (bt == 32) mbar_arrive_expect_tx(h_full(buf), (uint32_t)(n_own - (own ? 1 : 0)) * (OPN * HPITCH));
-                    if (own && bt < CS && bt != j && !stop) {
-                        const uint32_t src = base + y.off_h + buf * y.h_buf + j * OPN * HPITCH;
-                        bulk_copy_to_peer(map_to_rank(src, bt), src, OPN * HPITCH, map_to_rank(h_full(buf), bt));
+                    if (bt == 32 && (s + 1 == own || own == 0)) mbar_arrive_expect_tx(h_full, (uint32_t)(tiles - own) * (TN * HPITCH));
+                    if (s < own && bt < CS && bt != j && !stop) {
+                        const uint32_t from = base + LY(off_h) + (j + 8 * s) * TN * HPITCH;
+                        bulk_copy_to_peer(map_to_rank(from, bt), from, TN * HPITCH, map_to_rank(h_full, bt));
                     }
                 }
-                if (r > 0 && !stop) {
-                    // ---- down products of round r - 1
-                    const uint32_t Rr = R + r - 1, buf = Rr & 1;
-                    const int nr = w.n - (r - 1) * RN < RN ? w.n - (r - 1) * RN : RN, ns = (nr + SN - 1) / SN;
-                    WAIT(h_full(buf), (Rr >> 1) & 1);
-                    for (int s = 0; s < ns; ++s) {
-                        WAIT(d_full(d_slot), d_pass & 1);
-                        const uint32_t ha = h_lane + buf * y.h_buf + s * SN * HPITCH, wd = base + y.off_d + d_slot * y.d_stage + d_lane;
-                        uint32_t Ah[2][4], Al[2][4];
+                if (stop) break;
+                // ---- down products of the round
+                const int ns = (tiles + 1) / 2;
+                {
+                    int slot = d_slot + lane;                      // lane s looks at stage s, lane 31 at the h tile
+                    uint32_t ps = d_pass;
+                    if (slot >= NST) { slot -= NST; ++ps; }
+                    wait_lanes(lane < ns || lane == 31, lane == 31 ? h_full : d_full(slot), lane == 31 ? R & 1 : ps & 1, __LINE__);
+                }
+#pragma unroll 1
+                for (int s = 0; s < ns; ++s) {
+                    const uint32_t ha = h_lane + s * SN * HPITCH, wd = d_lane + d_slot * LY(d_stage);
+                    uint32_t Ah[2][4], Al[2][4], Bw[NG / 2][4];
+#pragma unroll
+                    for (int n = 0; n < NG / 2; ++n)
+                        if (HS || n < cpn) ldm4t(wd + n * 32, Bw[n]);
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+                        if (m < mcnt) { ldm4t(ha + m * 32, Ah[m]); ldm4t(ha + 128 + m * 32, Al[m]); }
+#pragma unroll
+                    for (int hl = 0; hl < 2; ++hl)
 #pragma unroll
                         for (int m = 0; m < 2; ++m)
-                            if (m < mcnt) { ldm4t(ha + m * 32, Ah[m]); ldm4t(ha + 128 + m * 32, Al[m]); }
+                            if (m < mcnt) {
 #pragma unroll
-                        for (int n = 0; n < NG / 2; ++n)
-                            if (n < cpn) {
-                                uint32_t Bw[4];
-                                ldm4t(wd + n * 32, Bw);
-#pragma unroll
-                                for (int m = 0; m < 2; ++m)
-                                    if (m < mcnt) {
-                                        mma16816(acc[m][2 * n], Ah[m], Bw[0], Bw[1]);
-                                        mma16816(acc[m][2 * n + 1], Ah[m], Bw[2], Bw[3]);
-                                        mma16816(acc[m][2 * n], Al[m], Bw[0], Bw[1]);
-                                        mma16816(acc[m][2 * n + 1], Al[m], Bw[2], Bw[3]);
+                                for (int n = 0; n < NG / 2; ++n)
+                                    if (HS || n < cpn) {
+                                        mma16816(acc[m][2 * n], hl ? Al[m] : Ah[m], Bw[n][0], Bw[n][1]);
+                                        mma16816(acc[m][2 * n + 1], hl ? Al[m] : Ah[m], Bw[n][2], Bw[n][3]);
                                     }
                             }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(d_empty(d_slot));
-                        if (++d_slot == NST) { d_slot = 0; ++d_pass; }
-                    }
                     __syncwarp();
-                    if (lane < CS) arrive_remote(map_to_rank(h_free(buf), lane));
+                    if (lane == 0) mbar_arrive(d_empty(d_slot));
+                    if (++d_slot == NST) { d_slot = 0; ++d_pass; }
                 }
+                if (lane < CS) arrive_remote(map_to_rank(h_free, lane));
             }
-            R += rounds;
             if (stop) break;
             // ---- the item's sums are complete: into the output buffer of the layer (the first layer's has to be set up by
             // every cluster before)
@@ -729,6 +754,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         }
     }
 #undef WAIT
+#undef LY
     __syncthreads();
     if (*sAbort) {
         // a wait gave up somewhere: copies into this CTA's shared memory may still be in flight although nobody waits for
@@ -747,9 +773,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
 // ---- host side
 constexpr int SMEM_MAX = 232448 - 1024;                            // (1 KB for the static part)
 
-template <int NG, int OPN, bool EQ4>
+template <int HS, int NG, int TS, bool EQ4>
 int configure(int smem) {
-    RM_CUDA_TRY(cudaFuncSetAttribute(slice_kernel<NG, OPN, EQ4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    RM_CUDA_TRY(cudaFuncSetAttribute(slice_kernel<HS, NG, TS, EQ4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     return RM_OK;
 }
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int clusters, int smem, cudaStream_t s) {
@@ -764,36 +790,37 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cluste
     cfg.attrs = at;
     cfg.numAttrs = 1;
 }
-template <int NG, int OPN>
+template <int HS, int NG, int TS>
 int query(int* out) {
-    int rc = configure<NG, OPN, false>(SMEM_MAX);
-    if (rc == RM_OK) rc = configure<NG, OPN, true>(SMEM_MAX);
+    int rc = configure<HS, NG, TS, false>(SMEM_MAX);
+    if (rc == RM_OK) rc = configure<HS, NG, TS, true>(SMEM_MAX);
     if (rc != RM_OK) return rc;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cluster_config(cfg, at, 32, SMEM_MAX, nullptr);
-    RM_CUDA_TRY(cudaOccupancyMaxActiveClusters(out, slice_kernel<NG, OPN, true>, &cfg));
+    RM_CUDA_TRY(cudaOccupancyMaxActiveClusters(out, slice_kernel<HS, NG, TS, true>, &cfg));
     return RM_OK;
 }
-template <int NG, int OPN, bool EQ4>
+template <int HS, int NG, int TS, bool EQ4>
 int launch(rm_ctx* ctx, const SArgs& a, int clusters, int smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cluster_config(cfg, at, clusters, smem, s);
-    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, slice_kernel<NG, OPN, EQ4>, a));
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, slice_kernel<HS, NG, TS, EQ4>, a));
     ctx->launches++;
     return RM_OK;
 }
 
-inline bool narrow(int Hs) { return Hs <= 128; }
+inline int tiles_per_owner(int Hs) { return Hs <= 128 ? 2 : 1; }
 
-// Stages of each weight ring that fit beside the other buffers, at most MAX_STAGES
-int ring_stages(int Hs, int T) {
-    const int opn = narrow(Hs) ? 8 : 4;
+// The layout with as many stages of each weight ring as fit beside the other buffers, at most MAX_STAGES
+Lay layout_of(int Hs) {
+    if (Hs == 128) return make_layout(128, 2, EXACT_STAGES);
     int st = MAX_STAGES;
-    while (st > 0 && make_layout(Hs, T, opn, st).total > SMEM_MAX) --st;
-    return st;
+    while (st > 0 && make_layout(Hs, tiles_per_owner(Hs), st).total > SMEM_MAX) --st;
+    return make_layout(Hs, tiles_per_owner(Hs), st);
 }
+static_assert(make_layout(128, 2, EXACT_STAGES).total <= SMEM_MAX, "the buffers of the 128-column slice exceed a CTA's shared memory");
 // A chunk of more than 64 tokens is cut into equal parts (multiples of 8 tokens): tokens are independent of one another
 void cut_tokens(int T, int& n_sub, int& part) {
     n_sub = (T + 63) / 64;
@@ -809,9 +836,9 @@ unsigned long long next_epoch() {
 int rm_slice_init(rm_ctx* ctx) {
     ctx->slice_clusters = 0;
     const int Hs = ctx->g.Hs;
-    if (Hs > 256 || ring_stages(Hs, 64) < 4) return RM_OK;
+    if (Hs > 256 || layout_of(Hs).stages < 4) return RM_OK;
     int n = 0;
-    const int rc = narrow(Hs) ? query<4, 8>(&n) : query<8, 4>(&n);
+    const int rc = Hs == 128 ? query<128, 4, 2>(&n) : Hs < 128 ? query<0, 4, 2>(&n) : query<0, 8, 1>(&n);
     if (rc == RM_OK) ctx->slice_clusters = n;
     return rc;
 }
@@ -867,7 +894,6 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     a.n_sub = n_sub;
     a.nb = sa.B;
     a.T_all = sa.T;
-    a.stages = ring_stages(g.Hs, part);
     a.anchor_mode = sa.anchor_mode;
     a.y_anchor = sa.y_anchor;
     a.h_anchor = sa.h_anchor;
@@ -876,8 +902,9 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     int nc = ctx->slice_clusters;
     if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < nc) nc = ctx->max_clusters_override;
     const bool eq4 = sa.anchor_mode != RM_ANCHOR_NONE || sa.gate != nullptr;
-    a.lay = make_layout(g.Hs, part, narrow(g.Hs) ? 8 : 4, a.stages);
+    a.lay = layout_of(g.Hs);
     const int smem = a.lay.total;
-    if (narrow(g.Hs)) return eq4 ? launch<4, 8, true>(ctx, a, nc, smem, s) : launch<4, 8, false>(ctx, a, nc, smem, s);
-    return eq4 ? launch<8, 4, true>(ctx, a, nc, smem, s) : launch<8, 4, false>(ctx, a, nc, smem, s);
+    if (g.Hs == 128) return eq4 ? launch<128, 4, 2, true>(ctx, a, nc, smem, s) : launch<128, 4, 2, false>(ctx, a, nc, smem, s);
+    if (g.Hs < 128) return eq4 ? launch<0, 4, 2, true>(ctx, a, nc, smem, s) : launch<0, 4, 2, false>(ctx, a, nc, smem, s);
+    return eq4 ? launch<0, 8, 1, true>(ctx, a, nc, smem, s) : launch<0, 8, 1, false>(ctx, a, nc, smem, s);
 }

@@ -1,6 +1,7 @@
 // rm_pack_weights: one-off repacking of a layer into the neuron-major layout (see rm_geom in rm_common.cuh),
 // and the per-neuron down-projection column norm ||Wd[:,n]||_2, the weight factor of Eq. 1.
 #include "rm_common.cuh"
+#include "rm_sm100.cuh"
 
 namespace {
 
@@ -80,7 +81,34 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
     for (int e = lane; e < row_u4; e += 32) out[(size_t)p * row_u4 + e] = src[e];
 }
 
+// dst = src (src NULL: zeros), n4 float4.  Either side may be pinned host memory: a step's 209 KB (51 x 1024 fp32) cross
+// PCIe in one kernel with every load in flight at once, where the copy engine's start-up and its hand-over to and from
+// the kernel in the same stream cost about 7 us per direction.
+__global__ void __launch_bounds__(256) copy_kernel(float4* dst, const float4* src, size_t n4) {
+    sm100::pdl_launch_dependents();        // a kernel behind this one may set up
+    sm100::pdl_wait();                     // (launched as a dependent: the kernel in front writes src)
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256)
+        dst[i] = src ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 }  // namespace
+
+// A multiple of 4 floats, 16-byte aligned on both sides
+int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, size_t n, bool pdl, cudaStream_t s) {
+    const size_t n4 = n / 4, ctas = (n4 + 255) / 256;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ctas < 592 ? ctas : 592));
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, copy_kernel, reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n4));
+    ctx->launches++;
+    return RM_OK;
+}
 
 int rm_launch_gather_rows(rm_ctx* ctx, const void* packed, const int32_t* idx, const int32_t* count, int64_t cap,
                           void* out, cudaStream_t s) {

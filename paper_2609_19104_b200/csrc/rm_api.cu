@@ -41,7 +41,7 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool steps) {
     if (ctx->path == 1 || !rm_persist_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 5) return true;
-    if (ctx->variant_override != 0 || B > ctx->persist_max_b || !steps) return false;
+    if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b || !steps) return false;
     const long long I = ctx->g.I, K = masked ? rm_effective_count_hint(ctx) : I;
     if (ctx->g.H == 2048) {
         if (K <= 0) return true;
@@ -64,6 +64,17 @@ inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
     return ctx->variant_override == 6 || (ctx->path == 0 && !rm_fused_supported(ctx, B, T));
 }
 
+// The sweep kernel (variant 7): dense steps of one episode.
+inline bool use_sweep(const rm_ctx* ctx, int B, int T, bool dense) {
+    if (ctx->path == 1 || !dense || !rm_sweep_supported(ctx, B, T)) return false;
+    if (ctx->variant_override == 7) return true;
+    return false;
+}
+inline void* sweep_ws(const rm_ctx* ctx, void* ws, int B, int T) {
+    char* p = static_cast<char*>(persist_ws(ctx, ws, B, T)) + align_up(rm_persist_workspace_bytes(ctx), 256) + rm_slice_workspace_bytes(ctx, B, T);
+    return reinterpret_cast<void*>(align_up(reinterpret_cast<size_t>(p), 1024));
+}
+
 // the slice kernel's buffers in a workspace of (B, T)
 inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, int T) {
     const size_t r_bytes = align_up((size_t)B * T * ctx->g.H * sizeof(float), 256);
@@ -81,7 +92,7 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, bool anchor_write = false) {
     if (ctx->path == 1 || !rm_stream_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 4) return true;
-    if (ctx->variant_override != 0 && ctx->variant_override != 5) return false;   // 5: a call the whole-step kernel does not cover
+    if (ctx->variant_override != 0 && ctx->variant_override != 5 && ctx->variant_override != 7) return false;   // 5, 7: a call the whole-step kernel does not cover
     const int per_episode = masked ? rm_effective_count_hint(ctx) : ctx->g.I;
     if (per_episode <= 0) return false;
     const long long tiles = (long long)((per_episode + 63) / 64) * B;
@@ -142,6 +153,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->persist_xbuf = nullptr;
     c->persist_sync = nullptr;
     c->persist_sync_dirty = 0;
+    for (int l = 0; l < 64; ++l) c->sweep_key[l] = nullptr;
     for (int b = 0; b < 16; ++b) c->persist_sync_base[b] = c->persist_copy_base[b] = 0;
     if (major == 10) { rm_fused_init(c); rm_persist_init(c); rm_slice_init(c); }   // failure leaves the portable path in charge
     cudaGetLastError();
@@ -165,7 +177,7 @@ size_t rm_workspace_bytes(const rm_ctx* ctx, int B, int T) {
     // three rotating residual-stream buffers, the host variant's staging buffer, then the portable path's scratch
     size_t r_bytes = align_up((size_t)B * T * ctx->g.H * sizeof(float), 256);
     return 4 * r_bytes + align_up(rm_ref_workspace_bytes(ctx, B, T), 256) + align_up(rm_persist_workspace_bytes(ctx), 256) +
-           rm_slice_workspace_bytes(ctx, B, T);
+           align_up(rm_slice_workspace_bytes(ctx, B, T), 1024) + 1024 + rm_sweep_workspace_bytes(ctx);
 }
 
 int rm_pack_weights(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, void* packed_out,
@@ -370,7 +382,8 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     const size_t r_bytes = align_up(n_bytes, 256);
     char* layer_ws = static_cast<char*>(ws) + 4 * r_bytes;
     const bool slice = use_slice(ctx, B, T, records_out != nullptr);
-    if (slice || use_persist(ctx, B, T, count_dev != nullptr, true)) {
+    const bool sweep = !slice && use_sweep(ctx, B, T, !idx && !count_dev && an.mode == RM_ANCHOR_NONE && !an.gate);
+    if (slice || sweep || use_persist(ctx, B, T, count_dev != nullptr, true)) {
         // the whole step in one launch: the layers add into r_out in place (the kernel starts it as a copy of r_in)
         rm_step_args sa{};
         sa.packed_layers = packed_layers;
@@ -393,6 +406,10 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
         sa.h_anchor = an.h;
         sa.h_stride = an.h_stride;
         sa.gate = an.gate;
+        if (sweep) {
+            ctx->last_variant = 7;
+            return rm_launch_step_sweep(ctx, sa, sweep_ws(ctx, ws, B, T), s);
+        }
         if (slice) {
             slice_buffers(ctx, sa, ws, B, T);
             ctx->last_variant = 6;
@@ -603,7 +620,7 @@ int rm_set_option(rm_ctx* ctx, const char* name, int value) {
         if (value < 0) return RM_ERR_INVALID_ARG;
         ctx->count_hint = value;
     } else if (n == "variant") {
-        if (value < 0 || value > 6) return RM_ERR_INVALID_ARG;
+        if (value < 0 || value > 7) return RM_ERR_INVALID_ARG;
         ctx->variant_override = value;
     } else if (n == "persist_prefetch_kb") {
         if (value < 0 || value > 4096) return RM_ERR_INVALID_ARG;

@@ -55,6 +55,8 @@ struct rm_ctx {
     int persist_sync_base[16];             // their values after the launches so far
     int persist_copy_base[16];             // the same for the counters of the r_in -> r copies
     int persist_sync_dirty;                // a launch may have left them at an unknown count: clear before the next one
+    const void* sweep_key[64];             // layers whose tensor maps the sweep kernel has (NULL: none yet)
+    alignas(64) unsigned char sweep_maps[64 * 128];
     alignas(64) unsigned char persist_tm[128];   // CUtensorMap of the clusters' x copies in the workspace
 };
 
@@ -180,6 +182,10 @@ int rm_slice_init(rm_ctx* ctx);
 bool rm_slice_supported(const rm_ctx* ctx, int B, int T, bool record);
 size_t rm_slice_workspace_bytes(const rm_ctx* ctx, int B, int T);
 int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s);
+// Sweep kernel: dense steps of one episode, every layer in one launch, no clusters (rm_mlp_sweep.cu)
+bool rm_sweep_supported(const rm_ctx* ctx, int B, int T);
+size_t rm_sweep_workspace_bytes(const rm_ctx* ctx);
+int rm_launch_step_sweep(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStream_t s);
 int rm_persist_init(rm_ctx* ctx);
 bool rm_persist_supported(const rm_ctx* ctx, int B, int T);
 size_t rm_persist_workspace_bytes(const rm_ctx* ctx);
@@ -187,4 +193,6 @@ int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaSt
 int rm_persist_debug_stamps(long long* host_out, int n);
 // Tiled tensor map (a 128-byte CUtensorMap, 64-byte aligned) of an fp32 residual buffer [B, T, H] with boxes of
 // box_rows token rows x 128 columns of one episode, not swizzled: the target of the kernels' bulk adds.
+// Tiled tensor map of a bf16 matrix [rows, cols], boxes of box_rows x 64 columns, 128-byte swizzle, 256-byte L2 promotion
+int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows);
 int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int box_rows);

@@ -28,9 +28,11 @@
 #include <chrono>
 
 #include "rm_common.cuh"
+#include "rm_grid.cuh"
 #include "rm_sm100.cuh"
 
 using namespace sm100;
+using namespace grid;
 
 namespace {
 
@@ -48,9 +50,8 @@ constexpr int SSB = 4;                 // buffers of the row sums of squares: a 
 constexpr int MAX_STAGES = 16;
 constexpr int EXACT_STAGES = 7;        // of the 128-column slice
 
-// control block in the workspace, in ints: [0,1] launch epoch, [2] CTAs that have left, [3] abort flag; then lines of 32 ints:
-// per (episode, slice) the CTAs that have set up the first output buffer, and the CTAs that have added their part
-constexpr int CTRL_LINE = 32;
+// the control block's counters, lines of 32 ints: per (episode, slice) the CTAs that have set up the first output buffer, and the
+// CTAs that have added their part
 __host__ __device__ constexpr int ctrl_init(int e, int j) { return CTRL_LINE * (1 + (e * CS + j) * 2); }
 __host__ __device__ constexpr int ctrl_done(int e, int j) { return CTRL_LINE * (2 + (e * CS + j) * 2); }
 __host__ __device__ constexpr size_t ctrl_bytes(int B) { return (size_t)CTRL_LINE * (1 + 2 * CS * B) * sizeof(int); }
@@ -127,68 +128,11 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ void red_add_v2(float* p, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
 }
-__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void red_release_gpu(int* p, int v) {
-    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 // (relaxed: it only says that this CTA's reads of a buffer are over; the values have been used by then.  A release at cluster
 // scope waits for every earlier store and add, an acquire at cluster scope empties the L1 cache)
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// ---- bounded waits.  Both return true when the waiter has to give up: the wait ran out (status RM_ERR_TIMEOUT with the
-// wait's source line and the CTA), or this CTA or the grid is aborting.
-__device__ __forceinline__ void report_timeout(const SArgs& a, volatile int* abort_cta, int line) {
-    rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
-    *abort_cta = 1;
-    atomicExch(a.ctrl + 3, 1);
-}
-__device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, const SArgs& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 22); ++i) {
-        if (mbar_try_wait(bar, parity)) return false;
-        if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && (*abort_cta || ((i & 16383u) == 16383u && ld_acquire_gpu(a.ctrl + 3) == 1))) {
-            *abort_cta = 1;
-            return true;
-        }
-    }
-    report_timeout(a, abort_cta, line);
-    return true;
-}
-__device__ __forceinline__ bool counter_wait(const int* counter, int target, int line, const SArgs& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 21); ++i) {
-        if (ld_acquire_gpu(counter) >= target) return false;
-        if ((i & 255u) == 255u && (*abort_cta || ld_acquire_gpu(a.ctrl + 3) == 1)) { *abort_cta = 1; return true; }
-    }
-    report_timeout(a, abort_cta, line);
-    return true;
-}
-__device__ __forceinline__ bool epoch_wait(const int* ctrl, unsigned long long epoch, int line, const SArgs& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 21); ++i) {
-        unsigned long long v;
-        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctrl) : "memory");
-        if (v == epoch) return false;
-        if ((i & 255u) == 255u && *abort_cta) return true;
-    }
-    rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
-    *abort_cta = 1;
-    return true;
-}
-__device__ __forceinline__ bool barrier_or(int id, int count, bool pred) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "barrier.cta.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r) : "r"((uint32_t)pred), "r"(id), "r"(count) : "memory");
-    return r != 0;
-}
-
 // What a cluster does for one (layer, episode): n neurons of the list from position `start` (0: another cluster's, or an
 // empty list whose residual this cluster passes on), `share` of `parts` of the item's token rows.
 struct Item { int start, n, parts_share, target; };                // parts | share << 8 | takes part << 16; target: arrivals
@@ -307,8 +251,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
     cluster_sync();                        // peers' shared memory and barriers are live from here on
     pdl_launch_dependents();               // (a dependent waits for this grid's end: its CTAs are resident by then)
     if (blockIdx.x == 0 && tid == 0) {
-        __threadfence();
-        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(a.ctrl), "l"(a.epoch) : "memory");
+        epoch_publish(a.ctrl, a.epoch);
     }
 
     bool gave_up = false;
@@ -764,9 +707,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
     }
     cluster_sync();                        // no CTA leaves while a peer may still write into its shared memory
     if (tid == 0 && !epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort)) {
-        // the last CTA to leave takes the epoch back, so that a captured launch can be replayed
-        if (atomicAdd(a.ctrl + 2, 1) == (int)gridDim.x - 1)
-            asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(a.ctrl), "l"(0ull) : "memory");
+        epoch_leave(a.ctrl);
     }
 }
 
@@ -826,10 +767,6 @@ void cut_tokens(int T, int& n_sub, int& part) {
     n_sub = (T + 63) / 64;
     part = n_sub == 1 ? T : ((T + n_sub - 1) / n_sub + 7) / 8 * 8;
 }
-unsigned long long next_epoch() {
-    static std::atomic<unsigned long long> n{(unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() << 20 | 1u};
-    return n.fetch_add(2);                                         // (odd: never 0)
-}
 
 }  // namespace
 
@@ -841,6 +778,11 @@ int rm_slice_init(rm_ctx* ctx) {
     const int rc = Hs == 128 ? query<128, 4, 2>(&n) : Hs < 128 ? query<0, 4, 2>(&n) : query<0, 8, 1>(&n);
     if (rc == RM_OK) ctx->slice_clusters = n;
     return rc;
+}
+
+unsigned long long rm_next_epoch() {
+    static std::atomic<unsigned long long> n{(unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() << 20 | 1u};
+    return n.fetch_add(2);
 }
 
 bool rm_slice_supported(const rm_ctx* ctx, int B, int T, bool record) {
@@ -884,7 +826,7 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     a.rec_b_stride = sa.rec_b_stride;
     a.record_scale = sa.record_scale;
     a.ctrl = sa.ctrl;
-    a.epoch = next_epoch();
+    a.epoch = rm_next_epoch();
     a.status = ctx->d_status;
     a.L = sa.L;
     a.B = sa.B * n_sub;

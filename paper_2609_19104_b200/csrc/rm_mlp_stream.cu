@@ -577,7 +577,8 @@ EncodeTiledFn encode_fn() {
 }
 
 // bf16 matrix [rows, cols] row-major, boxes of box_rows x 64 columns (128 bytes), 128-byte swizzle
-int make_map(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+int make_map(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows,
+             CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return RM_ERR_UNSUPPORTED;
     cuuint64_t dims[2] = {cols, rows};
@@ -585,7 +586,7 @@ int make_map(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uin
     cuuint32_t box[2] = {64, box_rows};
     cuuint32_t es[2] = {1, 1};
     const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, promotion,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? RM_OK : RM_ERR_CUDA;
 }
@@ -650,6 +651,11 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
 
 int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int box_rows) {
     return make_map_out(static_cast<CUtensorMap*>(tensor_map), ptr, (uint64_t)B, (uint64_t)T, (uint64_t)H, (uint32_t)box_rows);
+}
+
+int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows) {
+    return make_map(static_cast<CUtensorMap*>(tensor_map), ptr, (uint64_t)rows, (uint64_t)cols, (uint32_t)box_rows,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
 int rm_stream_debug_stamps(long long* host_out) {

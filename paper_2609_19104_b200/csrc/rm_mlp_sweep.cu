@@ -1,0 +1,465 @@
+// Sweep kernel: ONE launch runs every layer of a dense denoising step of one episode as two sweeps over the layer's weights,
+// spread over all SMs (one CTA per SM, all co-resident, no clusters).
+//
+//   gate/up : CTA p owns the neurons of units [U p / G, U (p+1) / G) (a unit is 16 neurons, at most 8 units a CTA) over the
+//             whole width H: D_gate[128 x 64 tokens] and D_up in tensor memory, so a thread of the epilogue finds gate and up of its neuron in
+//             the same lane; GeLU-tanh(g) * u, activation record, h as a bf16 pair hi + lo to global memory (4 KB per unit)
+//   down    : CTA = (column slice j of 8, K split s): D2[H/8 columns x (hi | lo tokens)] over the units [U s / S, U (s+1) / S), then
+//             added to the residual stream with red.global.add
+//   between : a CTA waits only for the producers of its own units of h (a flag each); the rows of the next layer are
+//             normalised by one CTA per token row once every CTA has added its part, and x is shared by all.
+//
+// What bounds a dense layer of 2048/16384 is HBM: 201 MB, 31 us at the measured copy rate.  The cluster kernels hold it to 3.5
+// TB/s on 120 of the SMs: 16-byte gathers (a dense pass has none to do), and the stream stops at every layer boundary with
+// 128 KB per CTA loaded ahead.  Here the weights arrive as tensor-map boxes of 16 rows x 64 columns into a ring of 160 KB per
+// CTA (23 MB over the chip) that a loader warp keeps full across the boundaries: it depends on nothing but ring space.
+// @MEASURED@
+//
+// Every wait is bounded (rm_grid.cuh).
+#include <cuda.h>
+
+#include <mutex>
+
+#include "rm_common.cuh"
+#include "rm_grid.cuh"
+#include "rm_sm100.cuh"
+
+using namespace sm100;
+using namespace grid;
+
+namespace {
+
+constexpr int UN = 16;                 // neurons of a unit
+constexpr int MAXU = 8;                // units of a CTA in the gate/up sweep (128 accumulator lanes)
+constexpr int NTOK = 64, MAXL = 64;
+constexpr int NSL = 8;                 // column slices of the packed layout
+constexpr int WSTAGE = 32768, NWS = 5; // weight ring
+constexpr int ASTAGE = 16384, NAS = 4; // activation ring: x (8 KB used) or h (4 units)
+constexpr int NTHREADS = 352;          // warps 0-7 epilogue and normalisation, 8 weights, 9 activations, 10 issuer
+constexpr int OFF_A = NWS * WSTAGE, OFF_MISC = OFF_A + NAS * ASTAGE;
+constexpr int SMEM = OFF_MISC + 2048 + 1024;
+constexpr int TMEM_COLS = 512, D2_COL = 128;                       // D_gate at 0, D_up at 64, D2 from 128 (128 columns per 128-column block)
+
+// control block: [CTRL_LINE] token rows normalised, [2 CTRL_LINE] CTAs that have added their part (both cumulative over the
+// layers), then a line of 8 ints per CTA: layers whose h it has written
+constexpr int C_X = CTRL_LINE, C_Y = 2 * CTRL_LINE, C_H = 3 * CTRL_LINE;
+constexpr size_t CTRL_BYTES = (C_H + 8 * 1024) * sizeof(int);
+
+struct WArgs {
+    const float* r_in;                 // [T,H]
+    float* r;                          // [T,H]: r_L on exit
+    unsigned char* x;                  // [H/64][64 rows x 128 bytes]: shared-memory images of x
+    unsigned char* h;                  // [U][hi, lo][16 rows x 128 bytes]
+    float* record;                     // [L, I] or NULL
+    const float* record_scale;         // [L, I] or NULL
+    int* ctrl;
+    unsigned long long epoch;
+    int* status;
+    int L, T, I, U, S;                 // U units, S splits of them in the down sweep (S * 8 CTAs)
+};
+struct WMaps { CUtensorMap m[MAXL]; };
+
+// CTA p's units [u0, u1) of the U when they are cut evenly into n parts
+__device__ __forceinline__ void cut(int U, int n, int p, int& u0, int& u1) {
+    u0 = (int)((unsigned)U * (unsigned)p / (unsigned)n);
+    u1 = (int)((unsigned)U * (unsigned)(p + 1) / (unsigned)n);
+}
+
+template <int HS>
+__global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constant__ WArgs a, const __grid_constant__ WMaps maps) {
+    constexpr int H = NSL * HS, KB = H / 64, NCB = HS / 64, NMB = HS / 128;
+    extern __shared__ unsigned char smem_dyn[];
+    const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
+    unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
+    const uint32_t bar0 = base + OFF_MISC;
+    auto w_full = [&](int s) { return bar0 + 8 * s; };
+    auto w_empty = [&](int s) { return bar0 + 64 + 8 * s; };
+    auto a_full = [&](int s) { return bar0 + 128 + 8 * s; };
+    auto a_empty = [&](int s) { return bar0 + 192 + 8 * s; };
+    const uint32_t d1_full = bar0 + 256, d2_full = bar0 + 264, s_tmem = bar0 + 272;
+    volatile uint32_t* g_tmem = reinterpret_cast<volatile uint32_t*>(gbase + OFF_MISC + 272);
+    volatile int* sAbort = reinterpret_cast<volatile int*>(gbase + OFF_MISC + 276);
+    float* sPart = reinterpret_cast<float*>(gbase + OFF_MISC + 288);       // 8 partial sums of a row
+    float* sRec = reinterpret_cast<float*>(gbase + OFF_MISC + 512);        // record sums of the second token half
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c = (int)blockIdx.x, G = (int)gridDim.x;
+    const int T = a.T, L = a.L, U = a.U;
+    int u0, u1;                                                    // this CTA's units of the gate/up sweep
+    cut(U, G, c, u0, u1);
+    const int nu = u1 - u0;
+    const int js = c % NSL, sp = c / NSL;                          // column slice and split of the down sweep
+    int k0 = 0, k1 = 0;
+    if (sp < a.S) cut(U, a.S, sp, k0, k1);
+    const int nk = k1 - k0, nst = (nk + 3) / 4;                    // units, stages (4 units) of the down sweep
+    const int n_add = a.S * NSL;                                   // CTAs that add (S <= U: every split has units)
+
+    if (c == 0) {
+        for (int e = tid; e < C_H + 8 * G; e += NTHREADS)
+            if (e >= 2) a.ctrl[e] = 0;
+        __threadfence();
+    }
+    if (tid == 0) {
+        for (int s = 0; s < NWS; ++s) { mbar_init(w_full(s), 1); mbar_init(w_empty(s), 1); }
+        for (int s = 0; s < NAS; ++s) { mbar_init(a_full(s), 1); mbar_init(a_empty(s), 1); }
+        mbar_init(d1_full, 1); mbar_init(d2_full, 1);
+        fence_mbar_init();
+        *sAbort = 0;
+    }
+    if (warp == 10) tmem_alloc(s_tmem, TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *g_tmem;
+    pdl_launch_dependents();               // (a dependent waits for this grid's end)
+    if (c == 0 && tid == 0) epoch_publish(a.ctrl, a.epoch);
+
+    bool gave_up = false;
+    auto wait_at = [&](uint32_t bar, uint32_t parity, int line) {
+        if (gave_up || mbar_test_wait(bar, parity)) return;
+        gave_up = wait_slow(bar, parity, line, a, sAbort);
+    };
+#define WAIT(bar, parity) wait_at((bar), (parity), __LINE__)
+
+    if (warp == 8) {
+        // ================================================================ weights: nothing to wait for but ring space
+        int ws = 0;
+        uint32_t pass = 0;
+        auto acquire = [&](uint32_t bytes) {
+            if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
+            gave_up = __any_sync(0xffffffffu, gave_up);
+            if (lane == 0 && !gave_up) mbar_arrive_expect_tx(w_full(ws), bytes);
+            __syncwarp();
+        };
+        auto advance = [&]() { if (++ws == NWS) { ws = 0; ++pass; } };
+        for (int l = 0; l < L && !gave_up; ++l) {
+            const CUtensorMap* tm = &maps.m[l];
+            for (int kb = 0; kb < KB && nu > 0 && !gave_up; ++kb) {
+                acquire((uint32_t)nu * 4096u);
+                // lane = (unit, gate or up): 16 rows x 64 columns each
+                const int x0 = (kb / NCB) * 3 * HS + (kb % NCB) * 64 + (lane & 1) * HS, u = lane >> 1;
+                if (u < nu && !gave_up) tma_load_2d(base + ws * WSTAGE + (lane & 1) * 16384 + u * 2048, tm, x0, (u0 + u) * UN, w_full(ws));
+                advance();
+            }
+            for (int s = 0; s < nst && !gave_up; ++s) {
+                const int ku = nk - 4 * s < 4 ? nk - 4 * s : 4;
+                acquire((uint32_t)ku * NCB * 2048u);
+                // lane = (column block, unit)
+                const int cb = lane >> 2, u = lane & 3;
+                if (cb < NCB && u < ku && !gave_up)
+                    tma_load_2d(base + ws * WSTAGE + cb * 8192 + u * 2048, tm, js * 3 * HS + 2 * HS + cb * 64, (k0 + 4 * s + u) * UN, w_full(ws));
+                advance();
+            }
+        }
+    } else if (warp == 9) {
+        // ================================================================ activations: x blocks once the layer's x is complete, h units
+        // once their producers have written them
+        int as = 0;
+        uint32_t pass = 0;
+        auto acquire = [&](uint32_t bytes) {
+            if (pass > 0) WAIT(a_empty(as), (pass - 1) & 1);
+            gave_up = __any_sync(0xffffffffu, gave_up);
+            if (lane == 0 && !gave_up) mbar_arrive_expect_tx(a_full(as), bytes);
+            __syncwarp();
+        };
+        auto advance = [&]() { if (++as == NAS) { as = 0; ++pass; } };
+        if (lane == 0) gave_up = epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
+        gave_up = __any_sync(0xffffffffu, gave_up);
+        for (int l = 0; l < L && !gave_up; ++l) {
+            if (nu > 0) {
+                if (lane == 0) gave_up = counter_wait(a.ctrl + C_X, T * (l + 1), __LINE__, a, sAbort);
+                gave_up = __any_sync(0xffffffffu, gave_up);
+                fence_proxy_async_global();
+                for (int kb = 0; kb < KB && !gave_up; ++kb) {
+                    acquire((uint32_t)T * 128u);
+                    if (lane == 0 && !gave_up) bulk_load(base + OFF_A + as * ASTAGE, a.x + (size_t)kb * 8192, (uint32_t)T * 128u, a_full(as));
+                    advance();
+                }
+            }
+            if (nk > 0 && !gave_up) {
+                int p0 = (int)((unsigned)k0 * (unsigned)G / (unsigned)U);      // first producer of units from k0 on
+                for (int q0, q1; p0 > 0; --p0) { cut(U, G, p0 - 1, q0, q1); if (q1 <= k0) break; }
+                for (int p = p0 + lane; p < G; p += 32) {
+                    int q0, q1;
+                    cut(U, G, p, q0, q1);
+                    if (q0 >= k1) break;
+                    if (q1 > q0 && q1 > k0 && !gave_up) gave_up = counter_wait(a.ctrl + C_H + 8 * p, l + 1, __LINE__, a, sAbort);
+                }
+                gave_up = __any_sync(0xffffffffu, gave_up);
+                fence_proxy_async_global();
+                for (int s = 0; s < nst && !gave_up; ++s) {
+                    const int ku = nk - 4 * s < 4 ? nk - 4 * s : 4;
+                    acquire((uint32_t)ku * 4096u);
+                    const int u = lane >> 1, lo = lane & 1;
+                    if (u < ku && !gave_up)
+                        bulk_load(base + OFF_A + as * ASTAGE + lo * 8192 + u * 2048, a.h + (size_t)(k0 + 4 * s + u) * 4096 + lo * 2048, 2048u, a_full(as));
+                    advance();
+                }
+            }
+        }
+    } else if (warp == 10) {
+        // ================================================================ issuer: the whole warp runs the loop, one elected lane issues; the
+        // next stage's barriers are tested behind the current stage's products
+        constexpr uint32_t IDESC_G = idesc_bf16_f32(128, NTOK, false, false), IDESC_D = idesc_bf16_f32(128, 2 * NTOK, true, true);
+        const uint64_t desc_k = smem_desc_sw128(0, 16, 1024), desc_mn = smem_desc_sw128(0, 8192, 1024);
+        int ws = 0, as = 0;
+        uint32_t wph = 0, aph = 0;
+        bool w_ok = false, a_ok = false;
+        auto ready = [&]() {
+            if (!w_ok) WAIT(w_full(ws), wph);
+            if (!a_ok) WAIT(a_full(as), aph);
+            gave_up = __any_sync(0xffffffffu, gave_up);
+            tc_fence_after();
+        };
+        auto advance = [&]() {
+            if (++ws == NWS) { ws = 0; wph ^= 1; }
+            if (++as == NAS) { as = 0; aph ^= 1; }
+            const uint32_t m = mbar_test_wait_2(w_full(ws), wph, a_full(as), aph);
+            w_ok = __all_sync(0xffffffffu, m & 1u);
+            a_ok = __all_sync(0xffffffffu, (m >> 1) & 1u);
+        };
+        for (int l = 0; l < L && !gave_up; ++l) {
+            if (nu > 0) {
+                for (int kb = 0; kb < KB && !gave_up; ++kb) {
+                    ready();
+                    if (gave_up) break;
+                    const uint32_t wt = base + ws * WSTAGE, xt = base + OFF_A + as * ASTAGE;
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) {
+                            const uint64_t bx = desc_k | desc_addr(xt + ks * 32);
+                            mma_bf16_ss(tmem, desc_k | desc_addr(wt + ks * 32), bx, IDESC_G, (kb | ks) != 0);
+                            mma_bf16_ss(tmem + NTOK, desc_k | desc_addr(wt + 16384 + ks * 32), bx, IDESC_G, (kb | ks) != 0);
+                        }
+                        mma_commit(w_empty(ws));
+                        mma_commit(a_empty(as));
+                        if (kb == KB - 1) mma_commit(d1_full);
+                    }
+                    __syncwarp();
+                    advance();
+                }
+            }
+            for (int s = 0; s < nst && !gave_up; ++s) {
+                ready();
+                if (gave_up) break;
+                const int ku = nk - 4 * s < 4 ? nk - 4 * s : 4;
+                const uint32_t wt = base + ws * WSTAGE, ht = base + OFF_A + as * ASTAGE;
+                if (elect_one()) {
+                    for (int ks = 0; ks < ku; ++ks) {
+                        const uint64_t bh = desc_mn | desc_addr(ht + ks * 2048);
+#pragma unroll
+                        for (int mb = 0; mb < NMB; ++mb)
+                            mma_bf16_ss(tmem + D2_COL + mb * 2 * NTOK, desc_mn | desc_addr(wt + mb * 16384 + ks * 2048), bh, IDESC_D, (s | ks) != 0);
+                    }
+                    mma_commit(w_empty(ws));
+                    mma_commit(a_empty(as));
+                    if (s == nst - 1) mma_commit(d2_full);
+                }
+                __syncwarp();
+                advance();
+            }
+        }
+    } else {
+        // ================================================================ epilogue: normalisation, GLU, adds
+        const int q4 = warp & 3, ch = warp >> 2;                   // tensor-memory lane quarter; token half (gate/up)
+        const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
+        bool stop = false;
+        if (tid == 0) gave_up = epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
+        for (int l = 0; l < L && !stop; ++l) {
+            // ---- x rows c, c + G, ... of the layer
+            if (c < T) {
+                if (tid == 0 && l > 0 && !gave_up) gave_up = counter_wait(a.ctrl + C_Y, n_add * l, __LINE__, a, sAbort);
+                stop = barrier_or(1, 256, gave_up || *sAbort);
+                if (stop) break;
+                int rows = 0;
+                for (int t = c; t < T; t += G, ++rows) {
+                    const float4* src = reinterpret_cast<const float4*>((l == 0 ? a.r_in : a.r) + (size_t)t * H) + tid;
+                    float4 v[H / 1024];
+                    float ss = 0.f;
+#pragma unroll
+                    for (int i = 0; i < H / 1024; ++i) v[i] = __ldcg(src + 256 * i);
+#pragma unroll
+                    for (int i = 0; i < H / 1024; ++i) {
+                        ss = fmaf(v[i].x, v[i].x, ss); ss = fmaf(v[i].y, v[i].y, ss);
+                        ss = fmaf(v[i].z, v[i].z, ss); ss = fmaf(v[i].w, v[i].w, ss);
+                    }
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
+                    if (rows > 0) named_barrier(1, 256);           // (sPart of the row before has been read)
+                    if (lane == 0) sPart[warp] = ss;
+                    named_barrier(1, 256);
+                    float tot = 0.f;
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) tot += sPart[w];
+                    const float inv = 1.0f / sqrtf(tot / (float)H + 1e-6f);
+#pragma unroll
+                    for (int i = 0; i < H / 1024; ++i) {
+                        const int col = 4 * (tid + 256 * i);
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x * inv, v[i].y * inv);
+                        const __nv_bfloat162 hi = __floats2bfloat162_rn(v[i].z * inv, v[i].w * inv);
+                        uint2 u;
+                        u.x = *reinterpret_cast<const uint32_t*>(&lo);
+                        u.y = *reinterpret_cast<const uint32_t*>(&hi);
+                        *reinterpret_cast<uint2*>(a.x + (size_t)(col >> 6) * 8192 + t * 128 + ((((col & 63) >> 3) ^ (t & 7)) << 4) + (col & 7) * 2) = u;
+                        if (l == 0 && a.r != a.r_in) reinterpret_cast<float4*>(a.r + (size_t)t * H)[tid + 256 * i] = v[i];
+                    }
+                }
+                fence_proxy_async_global();
+                named_barrier(1, 256);
+                if (tid == 0) red_release_gpu(a.ctrl + C_X, rows);
+            }
+            // ---- h of this CTA's neurons
+            if (nu > 0) {
+                const int row = q4 * 32 + lane, n = u0 * UN + row; // lane of the accumulators = neuron
+                WAIT(d1_full, l & 1);
+                tc_fence_after();
+                float g[32], u[32];
+                tmem_ld32(tmem + ch * 32 + lane_off, g);
+                tmem_ld32(tmem + NTOK + ch * 32 + lane_off, u);
+                tc_fence_before();
+                float rec = 0.f;
+                if (row < nu * UN) {
+                    unsigned char* hp = a.h + (size_t)(u0 + (row >> 4)) * 4096 + (row & 15) * 128;
+                    // in stages, so that the exponentials and divisions of different tokens overlap
+                    float e[32];
+#pragma unroll
+                    for (int t = 0; t < 32; ++t) e[t] = __expf(-1.5957691216057308f * (g[t] + 0.044715f * g[t] * g[t] * g[t]));
+#pragma unroll
+                    for (int t = 0; t < 32; ++t) e[t] = __fdividef(g[t], 1.0f + e[t]);
+#pragma unroll
+                    for (int t = 0; t < 32; ++t) {
+                        e[t] = n < a.I && ch * 32 + t < T ? e[t] * u[t] : 0.f;
+                        rec += fabsf(e[t]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        uint32_t hi[4], lo[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float f0 = e[8 * k + 2 * i], f1 = e[8 * k + 2 * i + 1];
+                            const __nv_bfloat162 h2 = __floats2bfloat162_rn(f0, f1);
+                            const float2 hf = __bfloat1622float2(h2);
+                            const __nv_bfloat162 l2 = __floats2bfloat162_rn(f0 - hf.x, f1 - hf.y);
+                            hi[i] = *reinterpret_cast<const uint32_t*>(&h2);
+                            lo[i] = *reinterpret_cast<const uint32_t*>(&l2);
+                        }
+                        const int off = ((ch * 4 + k) ^ (row & 7)) << 4;
+                        *reinterpret_cast<uint4*>(hp + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        *reinterpret_cast<uint4*>(hp + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                    }
+                    if (ch == 1) sRec[row] = rec;
+                }
+                fence_proxy_async_global();
+                stop = barrier_or(1, 256, gave_up || *sAbort);
+                if (stop) break;
+                if (tid == 0) st_release_gpu(a.ctrl + C_H + 8 * c, l + 1);
+                if (a.record && ch == 0 && row < nu * UN && n < a.I) {
+                    rec += sRec[row];
+                    a.record[(size_t)l * a.I + n] = a.record_scale ? rec * a.record_scale[(size_t)l * a.I + n] : rec;
+                }
+            }
+            // ---- this CTA's [columns of the slice x tokens] sums of the down sweep
+            if (nk > 0) {
+                WAIT(d2_full, l & 1);
+                tc_fence_after();
+                const int mb = NMB == 2 ? ch : 0, t0 = NMB == 2 ? 0 : ch * 32, t1 = NMB == 2 ? NTOK : t0 + 32;
+                float* rb = a.r + (size_t)js * HS + mb * 128 + q4 * 32 + lane;
+                const uint32_t d2 = tmem + D2_COL + mb * 2 * NTOK + lane_off;
+                if (!gave_up) {
+#pragma unroll 1
+                    for (int t = t0; t < t1 && t < T; t += 8) {
+                        float hi[8], lo[8];
+                        tmem_ld8(d2 + t, hi);
+                        tmem_ld8(d2 + NTOK + t, lo);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (t + i < T) red_add_f32(rb + (size_t)(t + i) * H, hi[i] + lo[i]);
+                    }
+                }
+                tc_fence_before();
+                stop = barrier_or(1, 256, gave_up || *sAbort);
+                if (stop) break;
+                if (tid == 0) red_release_gpu(a.ctrl + C_Y, 1);
+            }
+        }
+    }
+#undef WAIT
+    tc_fence_before();
+    __syncthreads();
+    if (*sAbort) {
+        // a wait gave up somewhere: copies into this CTA's shared memory may still be in flight although nobody waits for them
+        for (int i = 0; i < 64; ++i) __nanosleep(4000);
+        __syncthreads();
+    }
+    if (warp == 10) tmem_dealloc(tmem, TMEM_COLS);
+    if (tid == 0 && !epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort)) epoch_leave(a.ctrl);
+}
+
+// ---- host side
+inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+template <int HS>
+int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s) {
+    static rm_smem_configured configured = {};
+    if (!configured.covers(ctx->device, SMEM)) {
+        RM_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<HS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
+        configured.set(ctx->device, SMEM);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = SMEM;
+    cfg.stream = s;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<HS>, a, maps));
+    ctx->launches++;
+    return RM_OK;
+}
+inline int units(int I) { return (I + UN - 1) / UN; }
+inline int grid_size(const rm_ctx* ctx) { return ctx->sm_count < 1024 ? ctx->sm_count : 1024; }
+
+}  // namespace
+
+bool rm_sweep_supported(const rm_ctx* ctx, int B, int T) {
+    const int H = ctx->g.H, G = grid_size(ctx);
+    return (H == 1024 || H == 2048) && ctx->fused_clusters > 0 && B == 1 && T >= 1 && T <= NTOK && ctx->g.L <= MAXL && G >= NSL &&
+           units(ctx->g.I) <= MAXU * G;
+}
+
+size_t rm_sweep_workspace_bytes(const rm_ctx* ctx) {
+    if (!rm_sweep_supported(ctx, 1, 1)) return 0;
+    return align_up(CTRL_BYTES, 1024) + (size_t)(ctx->g.H / 64) * 8192 + (size_t)units(ctx->g.I) * 4096;
+}
+
+// Dense steps of one episode (no lists, no anchor state)
+int rm_launch_step_sweep(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStream_t s) {
+    const rm_geom& g = ctx->g;
+    WMaps* maps = reinterpret_cast<WMaps*>(ctx->sweep_maps);       // (encoded again only for layers whose address has changed)
+    static_assert(sizeof(WMaps) == sizeof(ctx->sweep_maps), "the context holds the tensor maps");
+    for (int l = 0; l < sa.L; ++l) {
+        if (ctx->sweep_key[l] == sa.packed_layers[l]) continue;
+        const int rc = rm_make_weight_map(&maps->m[l], sa.packed_layers[l], g.I, 3 * g.H, UN);
+        if (rc != RM_OK) return rc;
+        ctx->sweep_key[l] = sa.packed_layers[l];
+    }
+    WArgs a{};
+    a.r_in = sa.r_in ? sa.r_in : sa.r;
+    a.r = sa.r;
+    unsigned char* w = static_cast<unsigned char*>(ws);
+    a.ctrl = reinterpret_cast<int*>(w);
+    w += align_up(CTRL_BYTES, 1024);
+    a.x = w;
+    w += (size_t)(g.H / 64) * 8192;
+    a.h = w;
+    a.record = sa.record;
+    a.record_scale = sa.record_scale;
+    a.epoch = rm_next_epoch();
+    a.status = ctx->d_status;
+    a.L = sa.L;
+    a.T = sa.T;
+    a.I = g.I;
+    a.U = units(g.I);
+    int G = grid_size(ctx);
+    if (ctx->max_clusters_override > 0 && ctx->max_clusters_override * NSL < G && a.U <= MAXU * ctx->max_clusters_override * NSL)
+        G = ctx->max_clusters_override * NSL;
+    a.S = G / NSL < a.U ? G / NSL : a.U;
+    return g.H == 1024 ? launch<128>(ctx, a, *maps, G, s) : launch<256>(ctx, a, *maps, G, s);
+}

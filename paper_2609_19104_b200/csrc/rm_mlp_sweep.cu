@@ -2,8 +2,9 @@
 // spread over all SMs (one CTA per SM, all co-resident, no clusters).
 //
 //   gate/up : CTA p owns the neurons of units [U p / G, U (p+1) / G) (a unit is 16 neurons, at most 8 units a CTA) over the
-//             whole width H: D_gate[128 x 64 tokens] and D_up in tensor memory, so a thread of the epilogue finds gate and up of its neuron in
-//             the same lane; GeLU-tanh(g) * u, activation record, h as a bf16 pair hi + lo to global memory (4 KB per unit)
+//             whole width H: D1[128 x 64 tokens] per 4 units in tensor memory, a unit's 16 gate rows and 16 up rows in the lanes of
+//             one warp (they meet by shuffle); GeLU-tanh(g) * u, activation record, h as a bf16 pair hi + lo to global memory
+//             (4 KB per unit)
 //   down    : CTA = (column slice j of 8, K split s): D2[H/8 columns x (hi | lo tokens)] over the units [U s / S, U (s+1) / S), then
 //             added to the residual stream with red.global.add
 //   between : a CTA waits only for the producers of its own units of h (a flag each); the rows of the next layer are
@@ -34,11 +35,11 @@ constexpr int MAXU = 8;                // units of a CTA in the gate/up sweep (1
 constexpr int NTOK = 64, MAXL = 64;
 constexpr int NSL = 8;                 // column slices of the packed layout
 constexpr int WSTAGE = 32768, NWS = 5; // weight ring
-constexpr int ASTAGE = 16384, NAS = 4; // activation ring: x (8 KB used) or h (4 units)
+constexpr int ASTAGE = 16384, NAS = 4; // activation ring: two 64-column blocks of x, or 4 units of h (hi, lo)
 constexpr int NTHREADS = 352;          // warps 0-7 epilogue and normalisation, 8 weights, 9 activations, 10 issuer
 constexpr int OFF_A = NWS * WSTAGE, OFF_MISC = OFF_A + NAS * ASTAGE;
 constexpr int SMEM = OFF_MISC + 2048 + 1024;
-constexpr int TMEM_COLS = 512, D2_COL = 128;                       // D_gate at 0, D_up at 64, D2 from 128 (128 columns per 128-column block)
+constexpr int TMEM_COLS = 512, D2_COL = 128;                       // D1 at 0 and 64, D2 from 128 (128 columns per 128-column block)
 
 // control block: [CTRL_LINE] token rows normalised, [2 CTRL_LINE] CTAs that have added their part (both cumulative over the
 // layers), then a line of 8 ints per CTA: layers whose h it has written
@@ -91,6 +92,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
     int k0 = 0, k1 = 0;
     if (sp < a.S) cut(U, a.S, sp, k0, k1);
     const int nk = k1 - k0, nst = (nk + 3) / 4;                    // units, stages (4 units) of the down sweep
+    // a gate/up stage holds one 64-column block of 8 units, or two of 4 units when no CTA has more
+    const int kps = U <= 4 * G ? 2 : 1, nga = nu > 0 ? KB / kps : 0;       // column blocks per stage, stages of the gate/up sweep
+    // Every CTA reads all of x.  Each starts at another column block: with all of them asking for the same block at the same
+    // time a block took ~0.5 us (layer of 1024/4096: 7.6 us for 16 blocks)
+    const int rot = c % (KB / kps);
     const int n_add = a.S * NSL;                                   // CTAs that add (S <= U: every split has units)
 
     if (c == 0) {
@@ -121,35 +127,35 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
 #define WAIT(bar, parity) wait_at((bar), (parity), __LINE__)
 
     if (warp == 8) {
-        // ================================================================ weights: nothing to wait for but ring space
+        // ================================================================ weights: nothing to wait for but ring space.  A lane per
+        // box.  (Lanes 16-31 asking the boxes of a later stage into L2 meanwhile: 740 -> 1090 us; the copy engine handles a 2 KB box in
+        // ~60 clocks, prefetch or not, which is close to what the stream itself needs)
         int ws = 0;
         uint32_t pass = 0;
-        auto acquire = [&](uint32_t bytes) {
-            if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
-            gave_up = __any_sync(0xffffffffu, gave_up);
-            if (lane == 0 && !gave_up) mbar_arrive_expect_tx(w_full(ws), bytes);
-            __syncwarp();
-        };
-        auto advance = [&]() { if (++ws == NWS) { ws = 0; ++pass; } };
-        for (int l = 0; l < L && !gave_up; ++l) {
-            const CUtensorMap* tm = &maps.m[l];
-            for (int kb = 0; kb < KB && nu > 0 && !gave_up; ++kb) {
-                acquire((uint32_t)nu * 4096u);
-                // lane = (unit, gate or up): 16 rows x 64 columns each
-                const int x0 = (kb / NCB) * 3 * HS + (kb % NCB) * 64 + (lane & 1) * HS, u = lane >> 1;
-                if (u < nu && !gave_up) tma_load_2d(base + ws * WSTAGE + (lane & 1) * 16384 + u * 2048, tm, x0, (u0 + u) * UN, w_full(ws));
-                advance();
+        for (int l = 0; l < L && !gave_up; ++l)
+            for (int s = 0; s < nga + nst && !gave_up; ++s) {
+                int x, y = -1, dst;                                // box (y < 0: none), its place in the stage
+                if (s < nga) {
+                    // lane = (column block of the stage, unit, gate or up): 16 rows x 64 columns each
+                    const int sr = (s + rot) % nga, u = kps == 1 ? lane >> 1 : (lane >> 1) & 3, kb = kps == 1 ? sr : 2 * sr + (lane >> 3);
+                    if (lane < 16 && u < nu) y = (u0 + u) * UN;
+                    x = (kb / NCB) * 3 * HS + (kb % NCB) * 64 + (lane & 1) * HS;
+                    dst = lane * 2048;
+                } else {
+                    const int st = s - nga, cb = lane >> 2, u = lane & 3;
+                    if (cb < NCB && 4 * st + u < nk) y = (k0 + 4 * st + u) * UN;
+                    x = js * 3 * HS + 2 * HS + cb * 64;
+                    dst = cb * 8192 + u * 2048;
+                }
+                const uint32_t bytes = 2048u * __popc(__ballot_sync(0xffffffffu, y >= 0));
+                if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
+                gave_up = __any_sync(0xffffffffu, gave_up);
+                if (gave_up) break;
+                if (lane == 0) mbar_arrive_expect_tx(w_full(ws), bytes);
+                __syncwarp();
+                if (y >= 0) tma_load_2d(base + ws * WSTAGE + dst, &maps.m[l], x, y, w_full(ws));
+                if (++ws == NWS) { ws = 0; ++pass; }
             }
-            for (int s = 0; s < nst && !gave_up; ++s) {
-                const int ku = nk - 4 * s < 4 ? nk - 4 * s : 4;
-                acquire((uint32_t)ku * NCB * 2048u);
-                // lane = (column block, unit)
-                const int cb = lane >> 2, u = lane & 3;
-                if (cb < NCB && u < ku && !gave_up)
-                    tma_load_2d(base + ws * WSTAGE + cb * 8192 + u * 2048, tm, js * 3 * HS + 2 * HS + cb * 64, (k0 + 4 * s + u) * UN, w_full(ws));
-                advance();
-            }
-        }
     } else if (warp == 9) {
         // ================================================================ activations: x blocks once the layer's x is complete, h units
         // once their producers have written them
@@ -169,9 +175,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                 if (lane == 0) gave_up = counter_wait(a.ctrl + C_X, T * (l + 1), __LINE__, a, sAbort);
                 gave_up = __any_sync(0xffffffffu, gave_up);
                 fence_proxy_async_global();
-                for (int kb = 0; kb < KB && !gave_up; ++kb) {
-                    acquire((uint32_t)T * 128u);
-                    if (lane == 0 && !gave_up) bulk_load(base + OFF_A + as * ASTAGE, a.x + (size_t)kb * 8192, (uint32_t)T * 128u, a_full(as));
+                for (int kp = 0; kp < KB / 2 && !gave_up; ++kp) {
+                    acquire((uint32_t)T * 256u);
+                    const int kb = (2 * kp + rot * kps + lane) % KB;
+                    if (lane < 2 && !gave_up) bulk_load(base + OFF_A + as * ASTAGE + lane * 8192, a.x + (size_t)kb * 8192, (uint32_t)T * 128u, a_full(as));
                     advance();
                 }
             }
@@ -204,42 +211,70 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
         int ws = 0, as = 0;
         uint32_t wph = 0, aph = 0;
         bool w_ok = false, a_ok = false;
-        auto ready = [&]() {
-            if (!w_ok) WAIT(w_full(ws), wph);
+        auto w_ready = [&]() { if (!w_ok) WAIT(w_full(ws), wph); };
+        auto a_ready = [&]() {
             if (!a_ok) WAIT(a_full(as), aph);
             gave_up = __any_sync(0xffffffffu, gave_up);
             tc_fence_after();
         };
-        auto advance = [&]() {
-            if (++ws == NWS) { ws = 0; wph ^= 1; }
-            if (++as == NAS) { as = 0; aph ^= 1; }
+        // (a test takes ~200 clocks to come back: one for both rings, behind the products of the stage in front)
+        auto next = [&](bool w, bool x) {
+            if (w && ++ws == NWS) { ws = 0; wph ^= 1; }
+            if (x && ++as == NAS) { as = 0; aph ^= 1; }
             const uint32_t m = mbar_test_wait_2(w_full(ws), wph, a_full(as), aph);
-            w_ok = __all_sync(0xffffffffu, m & 1u);
-            a_ok = __all_sync(0xffffffffu, (m >> 1) & 1u);
+            if (w) w_ok = __all_sync(0xffffffffu, m & 1u);
+            if (x) a_ok = __all_sync(0xffffffffu, (m >> 1) & 1u);
         };
         for (int l = 0; l < L && !gave_up; ++l) {
-            if (nu > 0) {
-                for (int kb = 0; kb < KB && !gave_up; ++kb) {
-                    ready();
-                    if (gave_up) break;
-                    const uint32_t wt = base + ws * WSTAGE, xt = base + OFF_A + as * ASTAGE;
+            for (int kp = 0; kp < KB / 2 && nu > 0 && !gave_up; ++kp) {        // two column blocks: one stage of x, one or two of weights
+                a_ready();
+                w_ready();
+                gave_up = __any_sync(0xffffffffu, gave_up);
+                if (gave_up) break;
+                const uint32_t xt = base + OFF_A + as * ASTAGE;
+                if (kps == 2) {
+                    const uint32_t wt = base + ws * WSTAGE;
                     if (elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) {
-                            const uint64_t bx = desc_k | desc_addr(xt + ks * 32);
-                            mma_bf16_ss(tmem, desc_k | desc_addr(wt + ks * 32), bx, IDESC_G, (kb | ks) != 0);
-                            mma_bf16_ss(tmem + NTOK, desc_k | desc_addr(wt + 16384 + ks * 32), bx, IDESC_G, (kb | ks) != 0);
+                        for (int k8 = 0; k8 < 8; ++k8) {
+                            const int o = (k8 >> 2), ks = k8 & 3;
+                            mma_bf16_ss(tmem, desc_k | desc_addr(wt + o * 16384 + ks * 32), desc_k | desc_addr(xt + o * 8192 + ks * 32), IDESC_G, (kp | k8) != 0);
                         }
                         mma_commit(w_empty(ws));
                         mma_commit(a_empty(as));
-                        if (kb == KB - 1) mma_commit(d1_full);
+                        if (kp == KB / 2 - 1) mma_commit(d1_full);
                     }
                     __syncwarp();
-                    advance();
+                    next(true, true);
+                } else {
+#pragma unroll 1
+                    for (int o = 0; o < 2; ++o) {
+                        if (o == 1) {
+                            w_ready();
+                            gave_up = __any_sync(0xffffffffu, gave_up);
+                            if (gave_up) break;
+                            tc_fence_after();
+                        }
+                        const uint32_t wt = base + ws * WSTAGE;
+                        if (elect_one()) {
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks) {
+                                const uint64_t bx = desc_k | desc_addr(xt + o * 8192 + ks * 32);
+                                mma_bf16_ss(tmem, desc_k | desc_addr(wt + ks * 32), bx, IDESC_G, (kp | o | ks) != 0);
+                                if (nu > 4) mma_bf16_ss(tmem + NTOK, desc_k | desc_addr(wt + 16384 + ks * 32), bx, IDESC_G, (kp | o | ks) != 0);
+                            }
+                            mma_commit(w_empty(ws));
+                            if (o == 1) mma_commit(a_empty(as));
+                            if (o == 1 && kp == KB / 2 - 1) mma_commit(d1_full);
+                        }
+                        __syncwarp();
+                        next(true, o == 1);
+                    }
                 }
             }
             for (int s = 0; s < nst && !gave_up; ++s) {
-                ready();
+                w_ready();
+                a_ready();
                 if (gave_up) break;
                 const int ku = nk - 4 * s < 4 ? nk - 4 * s : 4;
                 const uint32_t wt = base + ws * WSTAGE, ht = base + OFF_A + as * ASTAGE;
@@ -255,7 +290,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     if (s == nst - 1) mma_commit(d2_full);
                 }
                 __syncwarp();
-                advance();
+                next(true, true);
             }
         }
     } else {
@@ -309,29 +344,40 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
             }
             // ---- h of this CTA's neurons
             if (nu > 0) {
-                const int row = q4 * 32 + lane, n = u0 * UN + row; // lane of the accumulators = neuron
+                // lanes 0-15 of a warp hold the gate rows of unit q4 (q4 + 4), lanes 16-31 its up rows, for the 32 tokens of half
+                // ch: the gate lane finishes the first 16 of them, the up lane the last 16
+                const bool isup = lane >= 16;
+                const int nl = lane & 15, tb = ch * 32 + (isup ? 16 : 0);      // neuron of the unit; first token of this lane
                 WAIT(d1_full, l & 1);
                 tc_fence_after();
-                float g[32], u[32];
-                tmem_ld32(tmem + ch * 32 + lane_off, g);
-                tmem_ld32(tmem + NTOK + ch * 32 + lane_off, u);
-                tc_fence_before();
-                float rec = 0.f;
-                if (row < nu * UN) {
-                    unsigned char* hp = a.h + (size_t)(u0 + (row >> 4)) * 4096 + (row & 15) * 128;
+                float rec[2] = {0.f, 0.f};
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const int unit = 4 * v + q4;
+                    if (unit >= nu) break;
+                    float d[32], g[16];
+                    tmem_ld32(tmem + v * NTOK + ch * 32 + lane_off, d);
                     // in stages, so that the exponentials and divisions of different tokens overlap
-                    float e[32];
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) e[t] = __expf(-1.5957691216057308f * (g[t] + 0.044715f * g[t] * g[t] * g[t]));
-#pragma unroll
-                    for (int t = 0; t < 32; ++t) e[t] = __fdividef(g[t], 1.0f + e[t]);
-#pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        e[t] = n < a.I && ch * 32 + t < T ? e[t] * u[t] : 0.f;
-                        rec += fabsf(e[t]);
+                    for (int t = 0; t < 16; ++t) {
+                        const float got = __shfl_xor_sync(0xffffffffu, isup ? d[t] : d[16 + t], 16);
+                        g[t] = isup ? got : d[t];
+                        d[t] = isup ? d[16 + t] : got;             // up
                     }
+                    float e[16];
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
+                    for (int t = 0; t < 16; ++t) e[t] = __expf(-1.5957691216057308f * (g[t] + 0.044715f * g[t] * g[t] * g[t]));
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) e[t] = __fdividef(g[t], 1.0f + e[t]);
+                    const bool real = (u0 + unit) * UN + nl < a.I;
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) {
+                        e[t] = real && tb + t < T ? e[t] * d[t] : 0.f;
+                        rec[v] += fabsf(e[t]);
+                    }
+                    unsigned char* hp = a.h + (size_t)(u0 + unit) * 4096 + nl * 128;
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
                         uint32_t hi[4], lo[4];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
@@ -342,19 +388,28 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                             hi[i] = *reinterpret_cast<const uint32_t*>(&h2);
                             lo[i] = *reinterpret_cast<const uint32_t*>(&l2);
                         }
-                        const int off = ((ch * 4 + k) ^ (row & 7)) << 4;
+                        const int off = (((tb >> 3) + k) ^ (nl & 7)) << 4;
                         *reinterpret_cast<uint4*>(hp + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                         *reinterpret_cast<uint4*>(hp + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     }
-                    if (ch == 1) sRec[row] = rec;
+                    if (a.record) {
+                        rec[v] += __shfl_xor_sync(0xffffffffu, rec[v], 16);
+                        if (ch == 1 && !isup) sRec[unit * UN + nl] = rec[v];
+                    }
                 }
+                tc_fence_before();
                 fence_proxy_async_global();
                 stop = barrier_or(1, 256, gave_up || *sAbort);
                 if (stop) break;
                 if (tid == 0) st_release_gpu(a.ctrl + C_H + 8 * c, l + 1);
-                if (a.record && ch == 0 && row < nu * UN && n < a.I) {
-                    rec += sRec[row];
-                    a.record[(size_t)l * a.I + n] = a.record_scale ? rec * a.record_scale[(size_t)l * a.I + n] : rec;
+                if (a.record && ch == 0 && !isup) {
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int unit = 4 * v + q4, n = (u0 + unit) * UN + nl;
+                        if (unit >= nu || n >= a.I) continue;
+                        const float r = rec[v] + sRec[unit * UN + nl];
+                        a.record[(size_t)l * a.I + n] = a.record_scale ? r * a.record_scale[(size_t)l * a.I + n] : r;
+                    }
                 }
             }
             // ---- this CTA's [columns of the slice x tokens] sums of the down sweep

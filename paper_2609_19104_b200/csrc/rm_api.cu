@@ -35,7 +35,7 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 // kernel's with every 64-neuron tile beyond 15; the whole-step kernel grows evenly with K and has a fixed cost of
 // ~10-15 us per layer.  So, with K the caller's count hint (the whole layer for a dense pass): at H = 1024 from 23.5 %
 // of the neurons upwards; at H = 2048 from 5 % upwards, except where the streaming kernel's single wave is nearly full
-// (47 % of the neurons up to 148 tiles).  Without a hint at H = 2048 it is chosen as well (it adapts to the counts on
+// (7700 neurons up to 148 tiles).  Without a hint at H = 2048 it is chosen as well (it adapts to the counts on
 // the device), at H = 1024 the lean kernel.  Batches stay with the streaming kernel.  `steps`: a whole stack (false:
 // the one-layer entry, which would pay the kernel's set-up for a single layer).
 inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool steps) {
@@ -46,7 +46,7 @@ inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool steps
     if (ctx->g.H == 2048) {
         if (K <= 0) return true;
         if (K * 100 < I * 5) return false;
-        return !(K * 100 > I * 47 && (K + 63) / 64 <= ctx->sm_count);
+        return !(K > 7700 && (K + 63) / 64 <= ctx->sm_count);
     }
     return K > 0 && K * 1000 >= I * 235;
 }
@@ -64,11 +64,13 @@ inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
     return ctx->variant_override == 6 || (ctx->path == 0 && !rm_fused_supported(ctx, B, T));
 }
 
-// The sweep kernel (variant 7): dense steps of one episode.
+// The sweep kernel (variant 7): dense steps of one episode, where a cluster of the whole-step kernel would walk more than one
+// tile of 256 neurons per layer.  us per step of 18 layers, 51 tokens, whole-step / sweep: H = 1024, I = 3000: 213 / 248,
+// 3500: 220 / 263, 4096: 282 / 255, 6000: 309 / 279; H = 2048, I = 8000: 540 / 430, 16384: 1085 / 750.
 inline bool use_sweep(const rm_ctx* ctx, int B, int T, bool dense) {
     if (ctx->path == 1 || !dense || !rm_sweep_supported(ctx, B, T)) return false;
-    if (ctx->variant_override == 7) return true;
-    return false;
+    if (ctx->variant_override != 0) return ctx->variant_override == 7;
+    return ctx->g.I > 256 * ctx->persist_clusters;
 }
 inline void* sweep_ws(const rm_ctx* ctx, void* ws, int B, int T) {
     char* p = static_cast<char*>(persist_ws(ctx, ws, B, T)) + align_up(rm_persist_workspace_bytes(ctx), 256) + rm_slice_workspace_bytes(ctx, B, T);
@@ -382,7 +384,7 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     const size_t r_bytes = align_up(n_bytes, 256);
     char* layer_ws = static_cast<char*>(ws) + 4 * r_bytes;
     const bool slice = use_slice(ctx, B, T, records_out != nullptr);
-    const bool sweep = !slice && use_sweep(ctx, B, T, !idx && !count_dev && an.mode == RM_ANCHOR_NONE && !an.gate);
+    const bool sweep = !slice && use_sweep(ctx, B, T, !idx && !count_dev && an.mode != RM_ANCHOR_UPDATE);
     if (slice || sweep || use_persist(ctx, B, T, count_dev != nullptr, true)) {
         // the whole step in one launch: the layers add into r_out in place (the kernel starts it as a copy of r_in)
         rm_step_args sa{};

@@ -56,7 +56,7 @@ struct rm_ctx {
     int persist_copy_base[16];             // the same for the counters of the r_in -> r copies
     int persist_sync_dirty;                // a launch may have left them at an unknown count: clear before the next one
     const void* sweep_key[64];             // layers whose tensor maps the sweep kernel has (NULL: none yet)
-    alignas(64) unsigned char sweep_maps[64 * 128];
+    alignas(64) unsigned char sweep_maps[2 * 64 * 128];
     alignas(64) unsigned char persist_tm[128];   // CUtensorMap of the clusters' x copies in the workspace
 };
 
@@ -193,6 +193,7 @@ int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaSt
 int rm_persist_debug_stamps(long long* host_out, int n);
 // Tiled tensor map (a 128-byte CUtensorMap, 64-byte aligned) of an fp32 residual buffer [B, T, H] with boxes of
 // box_rows token rows x 128 columns of one episode, not swizzled: the target of the kernels' bulk adds.
-// Tiled tensor map of a bf16 matrix [rows, cols], boxes of box_rows x 64 columns, 128-byte swizzle, 256-byte L2 promotion
-int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows);
+// Tiled tensor map of a bf16 matrix [rows, cols], boxes of box_rows x 64 columns, 128-byte swizzle, 256-byte L2 promotion.
+// pair_stride: boxes of box_rows x 2 x 64 columns, the second 64 that many columns further on (0: none)
+int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows, int pair_stride);
 int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int box_rows);

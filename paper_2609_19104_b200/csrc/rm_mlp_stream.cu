@@ -653,9 +653,19 @@ int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int
     return make_map_out(static_cast<CUtensorMap*>(tensor_map), ptr, (uint64_t)B, (uint64_t)T, (uint64_t)H, (uint32_t)box_rows);
 }
 
-int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows) {
-    return make_map(static_cast<CUtensorMap*>(tensor_map), ptr, (uint64_t)rows, (uint64_t)cols, (uint32_t)box_rows,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+int rm_make_weight_map(void* tensor_map, const void* ptr, int rows, int cols, int box_rows, int pair_stride) {
+    CUtensorMap* tm = static_cast<CUtensorMap*>(tensor_map);
+    if (!pair_stride) return make_map(tm, ptr, (uint64_t)rows, (uint64_t)cols, (uint32_t)box_rows, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return RM_ERR_UNSUPPORTED;
+    cuuint64_t dims[3] = {(cuuint64_t)(cols - pair_stride), 2, (cuuint64_t)rows};
+    cuuint64_t strides[2] = {pair_stride * sizeof(__nv_bfloat16), (cuuint64_t)cols * sizeof(__nv_bfloat16)};
+    cuuint32_t box[3] = {64, 2, (cuuint32_t)box_rows};
+    cuuint32_t es[3] = {1, 1, 1};
+    const CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? RM_OK : RM_ERR_CUDA;
 }
 
 int rm_stream_debug_stamps(long long* host_out) {

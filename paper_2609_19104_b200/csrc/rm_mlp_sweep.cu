@@ -2,8 +2,8 @@
 // spread over all SMs (one CTA per SM, all co-resident, no clusters).
 //
 //   gate/up : CTA p owns the neurons of units [U p / G, U (p+1) / G) (a unit is 16 neurons, at most 8 units a CTA) over the
-//             whole width H: D1[128 x 64 tokens] per 4 units in tensor memory, a unit's 16 gate rows and 16 up rows in the lanes of
-//             one warp (they meet by shuffle); GeLU-tanh(g) * u, activation record, h as a bf16 pair hi + lo to global memory
+//             whole width H: D1[128 x 64 tokens] per 4 units in tensor memory, the gate and the up row of a neuron in neighbouring
+//             lanes (they meet by shuffle); GeLU-tanh(g) * u, activation record, h as a bf16 pair hi + lo to global memory
 //             (4 KB per unit)
 //   down    : CTA = (column slice j of 8, K split s): D2[H/8 columns x (hi | lo tokens)] over the units [U s / S, U (s+1) / S), then
 //             added to the residual stream with red.global.add
@@ -12,9 +12,10 @@
 //
 // What bounds a dense layer of 2048/16384 is HBM: 201 MB, 31 us at the measured copy rate.  The cluster kernels hold it to 3.5
 // TB/s on 120 of the SMs: 16-byte gathers (a dense pass has none to do), and the stream stops at every layer boundary with
-// 128 KB per CTA loaded ahead.  Here the weights arrive as tensor-map boxes of 16 rows x 64 columns into a ring of 160 KB per
+// 128 KB per CTA loaded ahead.  Here the weights arrive as tensor-map boxes of 4 or 8 KB into a ring of 160 KB per
 // CTA (23 MB over the chip) that a loader warp keeps full across the boundaries: it depends on nothing but ring space.
-// @MEASURED@
+// us per step, 51 tokens, 18 layers, sweep / before: 2048/16384 750 / 1085, 2048/8000 430 / 618, 1024/4096 254 / 284.  What is left
+// over HBM time is the chain between the sweeps (~7 us a layer, of which the ring covers ~4).
 //
 // Every wait is bounded (rm_grid.cuh).
 #include <cuda.h>
@@ -57,8 +58,14 @@ struct WArgs {
     unsigned long long epoch;
     int* status;
     int L, T, I, U, S;                 // U units, S splits of them in the down sweep (S * 8 CTAs)
+    // anchor step of Eq. 4 and output gate (EQ4 instantiation)
+    float* y_anchor;                   // [L,T,H] or NULL
+    float* h_anchor;                   // [L,I,h_stride]
+    int64_t h_stride;
+    const float* gate;                 // [L,H] or NULL
 };
-struct WMaps { CUtensorMap m[MAXL]; };
+// Per layer: `gu` a box of 16 neurons x (gate, up) x 64 columns (row 2 i gate, 2 i + 1 up of neuron i), `dn` 64 neurons x 64 columns
+struct WMaps { CUtensorMap gu[MAXL], dn[MAXL]; };
 
 // CTA p's units [u0, u1) of the U when they are cut evenly into n parts
 __device__ __forceinline__ void cut(int U, int n, int p, int& u0, int& u1) {
@@ -66,7 +73,7 @@ __device__ __forceinline__ void cut(int U, int n, int p, int& u0, int& u1) {
     u1 = (int)((unsigned)U * (unsigned)(p + 1) / (unsigned)n);
 }
 
-template <int HS>
+template <int HS, bool EQ4>
 __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constant__ WArgs a, const __grid_constant__ WMaps maps) {
     constexpr int H = NSL * HS, KB = H / 64, NCB = HS / 64, NMB = HS / 128;
     extern __shared__ unsigned char smem_dyn[];
@@ -134,26 +141,33 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
         uint32_t pass = 0;
         for (int l = 0; l < L && !gave_up; ++l)
             for (int s = 0; s < nga + nst && !gave_up; ++s) {
-                int x, y = -1, dst;                                // box (y < 0: none), its place in the stage
+                bool box;
+                int x, y, dst;                                     // this lane's box and its place in the stage
+                uint32_t bytes;
                 if (s < nga) {
-                    // lane = (column block of the stage, unit, gate or up): 16 rows x 64 columns each
-                    const int sr = (s + rot) % nga, u = kps == 1 ? lane >> 1 : (lane >> 1) & 3, kb = kps == 1 ? sr : 2 * sr + (lane >> 3);
-                    if (lane < 16 && u < nu) y = (u0 + u) * UN;
-                    x = (kb / NCB) * 3 * HS + (kb % NCB) * 64 + (lane & 1) * HS;
-                    dst = lane * 2048;
+                    // lane = (column block of the stage, unit)
+                    const int sr = (s + rot) % nga, u = kps == 1 ? lane : lane & 3, kb = kps == 1 ? sr : 2 * sr + (lane >> 2);
+                    box = lane < 8 && u < nu;
+                    y = (u0 + u) * UN;
+                    x = (kb / NCB) * 3 * HS + (kb % NCB) * 64;
+                    dst = lane * 4096;
+                    bytes = 4096u * kps * nu;
                 } else {
-                    const int st = s - nga, cb = lane >> 2, u = lane & 3;
-                    if (cb < NCB && 4 * st + u < nk) y = (k0 + 4 * st + u) * UN;
-                    x = js * 3 * HS + 2 * HS + cb * 64;
-                    dst = cb * 8192 + u * 2048;
+                    box = lane < NCB;                              // (the last stage may bring rows that nothing multiplies)
+                    y = (k0 + 4 * (s - nga)) * UN;
+                    x = js * 3 * HS + 2 * HS + lane * 64;
+                    dst = lane * 8192;
+                    bytes = 8192u * NCB;
                 }
-                const uint32_t bytes = 2048u * __popc(__ballot_sync(0xffffffffu, y >= 0));
                 if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
                 gave_up = __any_sync(0xffffffffu, gave_up);
                 if (gave_up) break;
                 if (lane == 0) mbar_arrive_expect_tx(w_full(ws), bytes);
                 __syncwarp();
-                if (y >= 0) tma_load_2d(base + ws * WSTAGE + dst, &maps.m[l], x, y, w_full(ws));
+                if (box) {
+                    if (s < nga) tma_load_3d(base + ws * WSTAGE + dst, &maps.gu[l], x, 0, y, w_full(ws));
+                    else tma_load_2d(base + ws * WSTAGE + dst, &maps.dn[l], x, y, w_full(ws));
+                }
                 if (++ws == NWS) { ws = 0; ++pass; }
             }
     } else if (warp == 9) {
@@ -335,6 +349,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                         u.x = *reinterpret_cast<const uint32_t*>(&lo);
                         u.y = *reinterpret_cast<const uint32_t*>(&hi);
                         *reinterpret_cast<uint2*>(a.x + (size_t)(col >> 6) * 8192 + t * 128 + ((((col & 63) >> 3) ^ (t & 7)) << 4) + (col & 7) * 2) = u;
+                        if (EQ4 && a.y_anchor)                     // (the sums start from zero: they are added behind x)
+                            reinterpret_cast<float4*>(a.y_anchor + ((size_t)l * T + t) * H)[tid + 256 * i] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (l == 0 && a.r != a.r_in) reinterpret_cast<float4*>(a.r + (size_t)t * H)[tid + 256 * i] = v[i];
                     }
                 }
@@ -344,10 +360,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
             }
             // ---- h of this CTA's neurons
             if (nu > 0) {
-                // lanes 0-15 of a warp hold the gate rows of unit q4 (q4 + 4), lanes 16-31 its up rows, for the 32 tokens of half
+                // lanes 2 i, 2 i + 1 of a warp hold the gate and the up row of neuron i of unit q4 (q4 + 4) for the 32 tokens of half
                 // ch: the gate lane finishes the first 16 of them, the up lane the last 16
-                const bool isup = lane >= 16;
-                const int nl = lane & 15, tb = ch * 32 + (isup ? 16 : 0);      // neuron of the unit; first token of this lane
+                const bool isup = lane & 1;
+                const int nl = lane >> 1, tb = ch * 32 + (isup ? 16 : 0);      // neuron of the unit; first token of this lane
                 WAIT(d1_full, l & 1);
                 tc_fence_after();
                 float rec[2] = {0.f, 0.f};
@@ -360,7 +376,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     // in stages, so that the exponentials and divisions of different tokens overlap
 #pragma unroll
                     for (int t = 0; t < 16; ++t) {
-                        const float got = __shfl_xor_sync(0xffffffffu, isup ? d[t] : d[16 + t], 16);
+                        const float got = __shfl_xor_sync(0xffffffffu, isup ? d[t] : d[16 + t], 1);
                         g[t] = isup ? got : d[t];
                         d[t] = isup ? d[16 + t] : got;             // up
                     }
@@ -374,6 +390,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     for (int t = 0; t < 16; ++t) {
                         e[t] = real && tb + t < T ? e[t] * d[t] : 0.f;
                         rec[v] += fabsf(e[t]);
+                    }
+                    if (EQ4 && a.h_anchor && real) {
+                        float* ha = a.h_anchor + ((size_t)l * a.I + (u0 + unit) * UN + nl) * a.h_stride + tb;
+#pragma unroll
+                        for (int t = 0; t < 16; t += 4)
+                            if (tb + t < T) *reinterpret_cast<float4*>(ha + t) = make_float4(e[t], e[t + 1], e[t + 2], e[t + 3]);
                     }
                     unsigned char* hp = a.h + (size_t)(u0 + unit) * 4096 + nl * 128;
 #pragma unroll
@@ -393,7 +415,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                         *reinterpret_cast<uint4*>(hp + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     }
                     if (a.record) {
-                        rec[v] += __shfl_xor_sync(0xffffffffu, rec[v], 16);
+                        rec[v] += __shfl_xor_sync(0xffffffffu, rec[v], 1);
                         if (ch == 1 && !isup) sRec[unit * UN + nl] = rec[v];
                     }
                 }
@@ -417,7 +439,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                 WAIT(d2_full, l & 1);
                 tc_fence_after();
                 const int mb = NMB == 2 ? ch : 0, t0 = NMB == 2 ? 0 : ch * 32, t1 = NMB == 2 ? NTOK : t0 + 32;
-                float* rb = a.r + (size_t)js * HS + mb * 128 + q4 * 32 + lane;
+                const size_t col = (size_t)js * HS + mb * 128 + q4 * 32 + lane;
+                float* rb = a.r + col;
+                float* yb = EQ4 && a.y_anchor ? a.y_anchor + (size_t)l * T * H + col : nullptr;
+                const float gt = EQ4 && a.gate ? __ldg(a.gate + (size_t)l * H + col) : 1.f;
                 const uint32_t d2 = tmem + D2_COL + mb * 2 * NTOK + lane_off;
                 if (!gave_up) {
 #pragma unroll 1
@@ -427,7 +452,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                         tmem_ld8(d2 + NTOK + t, lo);
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
-                            if (t + i < T) red_add_f32(rb + (size_t)(t + i) * H, hi[i] + lo[i]);
+                            if (t + i < T) {
+                                const float y = hi[i] + lo[i];
+                                red_add_f32(rb + (size_t)(t + i) * H, EQ4 ? gt * y : y);
+                                if (EQ4 && yb) red_add_f32(yb + (size_t)(t + i) * H, y);
+                            }
                     }
                 }
                 tc_fence_before();
@@ -452,11 +481,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
 // ---- host side
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-template <int HS>
+template <int HS, bool EQ4>
 int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s) {
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, SMEM)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<HS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
+        RM_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<HS, EQ4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
         configured.set(ctx->device, SMEM);
     }
     cudaLaunchConfig_t cfg = {};
@@ -464,7 +493,7 @@ int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = SMEM;
     cfg.stream = s;
-    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<HS>, a, maps));
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<HS, EQ4>, a, maps));
     ctx->launches++;
     return RM_OK;
 }
@@ -484,14 +513,15 @@ size_t rm_sweep_workspace_bytes(const rm_ctx* ctx) {
     return align_up(CTRL_BYTES, 1024) + (size_t)(ctx->g.H / 64) * 8192 + (size_t)units(ctx->g.I) * 4096;
 }
 
-// Dense steps of one episode (no lists, no anchor state)
+// Dense steps of one episode: no lists, no anchor state or the anchor step of Eq. 4
 int rm_launch_step_sweep(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStream_t s) {
     const rm_geom& g = ctx->g;
     WMaps* maps = reinterpret_cast<WMaps*>(ctx->sweep_maps);       // (encoded again only for layers whose address has changed)
     static_assert(sizeof(WMaps) == sizeof(ctx->sweep_maps), "the context holds the tensor maps");
     for (int l = 0; l < sa.L; ++l) {
         if (ctx->sweep_key[l] == sa.packed_layers[l]) continue;
-        const int rc = rm_make_weight_map(&maps->m[l], sa.packed_layers[l], g.I, 3 * g.H, UN);
+        int rc = rm_make_weight_map(&maps->gu[l], sa.packed_layers[l], g.I, 3 * g.H, UN, g.Hs);
+        if (rc == RM_OK) rc = rm_make_weight_map(&maps->dn[l], sa.packed_layers[l], g.I, 3 * g.H, 4 * UN, 0);
         if (rc != RM_OK) return rc;
         ctx->sweep_key[l] = sa.packed_layers[l];
     }
@@ -516,5 +546,13 @@ int rm_launch_step_sweep(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStre
     if (ctx->max_clusters_override > 0 && ctx->max_clusters_override * NSL < G && a.U <= MAXU * ctx->max_clusters_override * NSL)
         G = ctx->max_clusters_override * NSL;
     a.S = G / NSL < a.U ? G / NSL : a.U;
-    return g.H == 1024 ? launch<128>(ctx, a, *maps, G, s) : launch<256>(ctx, a, *maps, G, s);
+    if (sa.anchor_mode == RM_ANCHOR_WRITE) {
+        a.y_anchor = sa.y_anchor;
+        a.h_anchor = sa.h_anchor;
+        a.h_stride = sa.h_stride;
+    }
+    a.gate = sa.gate;
+    const bool eq4 = sa.anchor_mode == RM_ANCHOR_WRITE || sa.gate;
+    if (g.H == 1024) return eq4 ? launch<128, true>(ctx, a, *maps, G, s) : launch<128, false>(ctx, a, *maps, G, s);
+    return eq4 ? launch<256, true>(ctx, a, *maps, G, s) : launch<256, false>(ctx, a, *maps, G, s);
 }

@@ -96,10 +96,9 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tensor_map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tensor_map)), "r"(x), "r"(y), "r"(mbar) : "memory");
 }
-// The same box asked into L2 only
-__device__ __forceinline__ void tma_prefetch_2d(const void* tensor_map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                 ::"l"(reinterpret_cast<uint64_t>(tensor_map)), "r"(x), "r"(y) : "memory");
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tensor_map, int x, int y, int z, uint32_t mbar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tensor_map)), "r"(x), "r"(y), "r"(z), "r"(mbar) : "memory");
 }
 // A contiguous piece of global memory (16-byte aligned, size a multiple of 16) into this CTA's shared memory; its bytes
 // are counted on an mbarrier of this CTA.

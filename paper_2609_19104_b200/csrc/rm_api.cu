@@ -150,6 +150,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->last_variant = 0;
     c->persist_clusters = 0;
     c->slice_clusters = 0;
+    c->stream_clusters[0] = c->stream_clusters[1] = 0;
     c->persist_max_b = 1;
     c->persist_prefetch_kb = 0;
     c->persist_xbuf = nullptr;
@@ -157,7 +158,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->persist_sync_dirty = 0;
     for (int l = 0; l < 64; ++l) c->sweep_key[l] = nullptr;
     for (int b = 0; b < 16; ++b) c->persist_sync_base[b] = c->persist_copy_base[b] = 0;
-    if (major == 10) { rm_fused_init(c); rm_persist_init(c); rm_slice_init(c); }   // failure leaves the portable path in charge
+    if (major == 10) { rm_fused_init(c); rm_persist_init(c); rm_slice_init(c); rm_stream_init(c); }   // failure leaves the portable path in charge
     cudaGetLastError();
     *out = c;
     return RM_OK;
@@ -654,6 +655,8 @@ int rm_get_info(const rm_ctx* ctx, const char* name, int* out) {
     else if (n == "fused_blocks_per_sm") *out = ctx->fused_blocks_per_sm;
     else if (n == "sm_count") *out = ctx->sm_count;
     else if (n == "persist_clusters") *out = ctx->persist_clusters;
+    else if (n == "stream_pairs") *out = ctx->stream_clusters[0];
+    else if (n == "stream_quads") *out = ctx->stream_clusters[1];
     else if (n == "slice_clusters") *out = ctx->slice_clusters;
     else if (n == "last_variant") *out = ctx->last_variant;
     else if (n == "path") *out = ctx->path;

@@ -46,6 +46,7 @@ struct rm_ctx {
     int variant_override;                  // 0 auto, 1 lean kernel, 2 kernel with a dedicated staging buffer
     int last_variant;                      // kernel family of the last layer or step launched (see rm_get_info)
     // whole-step kernel (rm_mlp_persist.cu)
+    int stream_clusters[2];                // co-resident clusters of 2 and of 4 CTAs of the streaming kernel
     int slice_clusters;                    // co-resident 8-CTA clusters of the slice kernel (0: unavailable)
     int persist_clusters;                  // co-resident 8-CTA clusters of the whole-step kernel (0: unavailable)
     int persist_prefetch_kb;               // weight KB a CTA of the whole-step kernel may ask into L2 ahead of its loaders
@@ -152,6 +153,7 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& a, float* zero_buf, 
                           cudaStream_t s);
 int rm_launch_layer_ref(rm_ctx* ctx, const rm_layer_args& a, void* ws, cudaStream_t s);
 // Streaming tensor-core variant (whole tiles per CTA, no clusters): same shapes as the fused path.
+int rm_stream_init(rm_ctx* ctx);
 bool rm_stream_supported(const rm_ctx* ctx, int B, int T);
 int rm_stream_debug_stamps(long long* host_out);
 int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& a, __nv_bfloat16* x_scratch, bool pdl, cudaStream_t s);

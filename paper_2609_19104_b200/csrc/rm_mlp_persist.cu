@@ -194,12 +194,6 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// arrive on the mbarrier at the same shared-memory offset in every CTA of `mask` once all MMAs issued so far by
-// this thread have completed
-__device__ __forceinline__ void mma_commit_mc(uint32_t bar, uint16_t mask) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(bar), "h"(mask) : "memory");
-}
 // OR of a predicate over the threads of a named barrier: one decision for the whole group
 __device__ __forceinline__ bool named_barrier_or(int id, int count, bool pred) {
     uint32_t r;

@@ -32,7 +32,6 @@ namespace {
 
 constexpr int NT = 64;                 // neurons per tile
 constexpr int MAXB = 64;               // episodes per launch
-constexpr int NSTAGE = 6;
 constexpr int W_BYTES = 16384;         // 128 rows (64 gate + 64 up, or 64 neurons x 2 column blocks) x 128 bytes
 constexpr int STAGE = 24576;           // + x block: up to 64 token rows x 128 bytes
 
@@ -110,14 +109,16 @@ __global__ void __launch_bounds__(256) stream_prep_kernel(const PrepArgs a) {
     }
 }
 
-template <int NTOK>
+template <int NTOK, int CL>
 struct SmemST {
+    static constexpr int NSTAGE = CL == 1 ? 6 : 5;
+    static constexpr int NYB = CL == 4 ? 1 : 2;                    // staging buffers of finished blocks
     static constexpr int OFF_RING = 0;
-    static constexpr int OFF_HT = OFF_RING + NSTAGE * STAGE;       // h tile: hi 8 KB, lo 8 KB (64 neurons x 128 bytes)
-    static constexpr int OFF_Y = OFF_HT + 2 * NT * 128;            // 2 x 32 KB: GeLU exchange [2][token][neuron] fp32 (first
+    static constexpr int OFF_HT = OFF_RING + NSTAGE * STAGE;       // h of the group's tiles: hi 8 KB, lo 8 KB each (64 neurons x 128 bytes)
+    static constexpr int OFF_Y = OFF_HT + CL * 2 * NT * 128;       // NYB x 32 KB: GeLU exchange [2][token][neuron] fp32 (first
                                                                    // buffer), then the transposed down blocks [token][128
                                                                    // columns] fp32, alternating between the two buffers
-    static constexpr int OFF_REC = OFF_Y + 65536;                  // record halves of the second token half
+    static constexpr int OFF_REC = OFF_Y + NYB * 32768;                  // record halves of the second token half
     static constexpr int OFF_PREF = OFF_REC + NT * 4;              // tile prefix per episode, counts
     static constexpr int OFF_BAR = ((OFF_PREF + (2 * MAXB + 1) * 4 + 7) / 8) * 8;
     static constexpr int TOTAL = OFF_BAR + 256 + 1024;             // + slack for the 1024-byte alignment
@@ -144,12 +145,17 @@ constexpr int SE = 288;                // threads: 4 epilogue warps (0-3), 4 loa
 // GATHER: the tile's neurons come from an index list, their rows are gathered with 16-byte cp.async (about 16 bytes
 // per clock and SM, the limit of this kernel on lists).  Otherwise the tile is 64 consecutive rows of the layer (dense
 // passes, compact layers) and a whole 64 x 64 block arrives as one tensor-map box.  x always arrives as one box.
-template <int NTOK, bool EQ4, bool GATHER>
+// CL > 1: the tiles of an episode are taken in groups of CL by the CTAs of a cluster.  Each makes the h of its own tile, sends it to
+// the others, and then multiplies the h of all of them with its own share of the output columns: an SM adds 16 bytes per clock
+// to the output whichever way they leave, and a group adds [T x H] once where single tiles add it CL times.
+template <int NTOK, bool EQ4, bool GATHER, int CL>
 __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, const __grid_constant__ CUtensorMap tmW,
                                                             const __grid_constant__ CUtensorMap tmX,
                                                             const __grid_constant__ CUtensorMap tmOut,
                                                             const __grid_constant__ CUtensorMap tmYa) {
-    using S = SmemST<NTOK>;
+    using S = SmemST<NTOK, CL>;
+    constexpr int NSTAGE = S::NSTAGE;
+    static_assert(CL == 1 || !EQ4, "groups of tiles: zero-fill form only");
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
@@ -164,8 +170,10 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
     const uint32_t d1_full = bar0 + 96, d1_free = bar0 + 104, h_full = bar0 + 112, h_free = bar0 + 120;
     auto d2_full = [&](int s) { return bar0 + 128 + 8 * s; };
     auto d2_free = [&](int s) { return bar0 + 144 + 8 * s; };
-    const uint32_t s_tmem = bar0 + 160;
-    volatile uint32_t* g_tmem = reinterpret_cast<volatile uint32_t*>(gbase + S::OFF_BAR + 160);
+    auto h_arr = [&](int t) { return bar0 + 160 + 8 * t; };        // h of the group's tile t has arrived from its CTA
+    const uint32_t s_tmem = bar0 + 192;
+    volatile uint32_t* g_tmem = reinterpret_cast<volatile uint32_t*>(gbase + S::OFF_BAR + 192);
+    const int rk = CL > 1 ? (int)cluster_ctarank() : 0, cid = (int)blockIdx.x / CL, ncl = (int)gridDim.x / CL;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int H = a.H, T = a.T, Hs = H / 8;
@@ -175,31 +183,38 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
 
     if (tid == 0) {
         for (int s = 0; s < NSTAGE; ++s) { mbar_init(full(s), GATHER ? 129 : 1); mbar_init(empty(s), 1); }
-        mbar_init(d1_full, 1); mbar_init(d1_free, 128); mbar_init(h_full, 128); mbar_init(h_free, 1);
+        mbar_init(d1_full, 1); mbar_init(d1_free, 128); mbar_init(h_full, 128); mbar_init(h_free, CL);
+        for (int t = 0; t < CL; ++t) mbar_init(h_arr(t), 1);
         for (int s = 0; s < 2; ++s) { mbar_init(d2_full(s), 1); mbar_init(d2_free(s), 128); }
         fence_mbar_init();
-        int acc = 0;
-        const int cap = (int)(a.list_cap < (int64_t)a.I ? a.list_cap : (int64_t)a.I);
-        for (int b = 0; b < a.B; ++b) {
-            int c = a.I;
-            if (a.count) {
-                c = a.count[(size_t)b * a.count_stride];
-                if (c < 0 || c > cap) { rm_set_status(a.status, RM_ERR_INDEX); c = c < 0 ? 0 : cap; }
-            }
-            gCnt[b] = c;
-            gPref[b] = acc;
-            acc += (c + NT - 1) / NT;
+    }
+    if (tid < a.B) {                       // (a thread per episode: one thread reading them in turn took ~0.4 us each)
+        int c = a.I;
+        if (a.count) {
+            const int cap = (int)(a.list_cap < (int64_t)a.I ? a.list_cap : (int64_t)a.I);
+            c = a.count[(size_t)tid * a.count_stride];
+            if (c < 0 || c > cap) { rm_set_status(a.status, RM_ERR_INDEX); c = c < 0 ? 0 : cap; }
         }
-        gPref[a.B] = acc;
+        gCnt[tid] = c;
     }
     if (warp == 8) tmem_alloc(s_tmem, S::TMEM_COLS);
     tc_fence_before();
     __syncthreads();
+    if (tid == 0) {
+        int acc = 0;
+        for (int b = 0; b < a.B; ++b) {
+            gPref[b] = acc;
+            acc += ((gCnt[b] + NT - 1) / NT + CL - 1) / CL;
+        }
+        gPref[a.B] = acc;
+    }
+    __syncthreads();
+    if (CL > 1) cluster_sync();            // peers' shared memory and barriers are live from here on
     tc_fence_after();
     const uint32_t tmem_d1 = *g_tmem;
     pdl_launch_dependents();
 
-    const int tiles_total = gPref[a.B];
+    const int groups_total = gPref[a.B];
     bool gave_up = false;
     auto wait_bar_at = [&](uint32_t bar, uint32_t parity, int line) {
         if (!mbar_wait(bar, parity)) {
@@ -212,9 +227,11 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
         while (gPref[b + 1] <= g) ++b;
         return b;
     };
-    // neuron of slot q of tile g (-1: past the end of the list, or an index outside the layer)
-    auto neuron_of = [&](int g, int b, int q, bool report) {
-        const int p0 = (g - gPref[b]) * NT;
+    // tiles of group g of episode b; first neuron of its tile t
+    auto tiles_of = [&](int g, int b) { const int left = (gCnt[b] + NT - 1) / NT - (g - gPref[b]) * CL; return left < CL ? left : CL; };
+    auto first_of = [&](int g, int b, int t) { return ((g - gPref[b]) * CL + t) * NT; };
+    // neuron of slot q of the tile at p0 (-1: past the end of the list, or an index outside the layer)
+    auto neuron_of = [&](int b, int p0, int q, bool report) {
         int n = -1;
         if (p0 + q < gCnt[b]) {
             n = a.idx ? __ldg(a.idx + (size_t)b * a.idx_stride + p0 + q) : p0 + q;
@@ -243,16 +260,16 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
             if (bk >= NSTAGE) wait_bar(empty(bk % NSTAGE), ((bk / NSTAGE) - 1) & 1);
         };
         for (int k = 0;; ++k) {
-            const int g = (int)blockIdx.x + k * (int)gridDim.x;
-            if (g >= tiles_total) break;
-            const int b = episode_of(g);
-            const int p0 = (g - gPref[b]) * NT;
+            const int g = cid + k * ncl;
+            if (g >= groups_total) break;
+            const int b = episode_of(g), nt = tiles_of(g, b);
+            const int p0 = first_of(g, b, rk);
             int nq[4];
             const __nv_bfloat16* row[4];
             if (GATHER) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    nq[i] = neuron_of(g, b, r0 + 16 * i, ch == 0);
+                    nq[i] = neuron_of(b, p0, r0 + 16 * i, ch == 0);
                     row[i] = a.packed + (size_t)(nq[i] < 0 ? 0 : nq[i]) * 3 * H + ch * 8;
                 }
             }
@@ -280,8 +297,8 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 if (lt == 0) tma_load_2d(stage_of(bk) + W_BYTES, &tmX, kb * 64, b * T, full(bk % NSTAGE));
                 if (GATHER) cp_async_arrive_noinc(full(bk % NSTAGE));
             };
-            int kb = 0;
-            if (!waited) {
+            int kb = rk < nt ? 0 : KBN;                            // (a CTA without a tile of its own has no gate/up part)
+            if (!waited && kb == 0 && blk == 0) {
                 // the weights do not depend on the previous kernel: fill the ring with them, then wait, then add x
                 const int pre = KBN < NSTAGE ? KBN : NSTAGE;
                 for (int i = 0; i < pre; ++i) issue_w(i, blk + i);
@@ -292,32 +309,51 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 blk += pre;
                 kb = pre;
             }
+            if (!waited && kb < KBN) { pdl_wait(); waited = true; }
             for (; kb < KBN; ++kb, ++blk) {
                 acquire(blk);
                 issue_w(kb, blk);
                 issue_x(kb, blk);
             }
             if (lt == 0) RM_ST(2);                                 // all gate/up blocks issued
-            for (int mb = 0; mb < MBN; ++mb, ++blk) {              // down rows: 64 neurons x 128 output columns
-                acquire(blk);
-                const uint32_t st = stage_of(blk), fb = full(blk % NSTAGE);
-                if (!GATHER && lt == 0) mbar_arrive_expect_tx(fb, DN_TX);
+            // down rows: 64 neurons x 128 output columns per stage, the group's tiles in turn (this CTA's own first, its h is the
+            // first to be there) for each of this CTA's column blocks
+            int dq[CL][4];                                         // lists: neurons of this thread's rows, per tile in that order
+            if (GATHER && CL > 1) {
 #pragma unroll
-                for (int cb = 0; cb < 2; ++cb) {
-                    const int col = mb * 128 + cb * 64, j = col / Hs, x0 = j * 3 * Hs + 2 * Hs + (col - j * Hs);
-                    if (GATHER) {
+                for (int t = 0; t < CL; ++t) {
+                    const int tt = (rk + t) % CL;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const int q = r0 + 16 * i;
-                            cp_async16(st + cb * 8192 + q * 128 + ((ch ^ (q & 7)) << 4), row[i] + x0, nq[i] >= 0);
-                        }
-                    } else if (lt == 0) {
-                        tma_load_2d(st + cb * 8192, &tmW, x0, p0, fb);
-                    }
+                    for (int i = 0; i < 4; ++i) dq[t][i] = tt < nt ? (t == 0 ? nq[i] : neuron_of(b, first_of(g, b, tt), r0 + 16 * i, false)) : -1;
                 }
-                if (GATHER) {
-                    if (lt == 0) mbar_arrive(fb);                  // the arrival that carries the x bytes in gate/up stages
-                    cp_async_arrive_noinc(fb);
+            }
+            for (int mb = rk * (MBN / CL); mb < (rk + 1) * (MBN / CL); ++mb) {
+#pragma unroll
+                for (int t = 0; t < CL; ++t) {
+                    const int tt = (rk + t) % CL;
+                    if (tt >= nt) continue;
+                    acquire(blk);
+                    const uint32_t st = stage_of(blk), fb = full(blk % NSTAGE);
+                    if (!GATHER && lt == 0) mbar_arrive_expect_tx(fb, DN_TX);
+#pragma unroll
+                    for (int cb = 0; cb < 2; ++cb) {
+                        const int col = mb * 128 + cb * 64, j = col / Hs, x0 = j * 3 * Hs + 2 * Hs + (col - j * Hs);
+                        if (GATHER) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int q = r0 + 16 * i, n = CL > 1 ? dq[t][i] : nq[i];
+                                cp_async16(st + cb * 8192 + q * 128 + ((ch ^ (q & 7)) << 4),
+                                           CL > 1 ? a.packed + (size_t)(n < 0 ? 0 : n) * 3 * H + ch * 8 + x0 : row[i] + x0, n >= 0);
+                            }
+                        } else if (lt == 0) {
+                            tma_load_2d(st + cb * 8192, &tmW, x0, first_of(g, b, tt), fb);
+                        }
+                    }
+                    if (GATHER) {
+                        if (lt == 0) mbar_arrive(fb);              // the arrival that carries the x bytes in gate/up stages
+                        cp_async_arrive_noinc(fb);
+                    }
+                    ++blk;
                 }
             }
         }
@@ -328,12 +364,15 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
         const int q = m & 63, half = m >> 6;                       // its neuron slot; token half it finishes
         constexpr int TH = NTOK / 2;                               // tokens per half
         uint32_t mbc = 0;                                          // down blocks consumed so far
+        int own = 0;                                               // tiles of its own this CTA has had
         for (int k = 0;; ++k) {
-            const int g = (int)blockIdx.x + k * (int)gridDim.x;
-            if (g >= tiles_total) break;
-            const int b = episode_of(g);
-            const int n = neuron_of(g, b, q, false);
-            wait_bar(d1_full, k & 1);
+            const int g = cid + k * ncl;
+            if (g >= groups_total) break;
+            const int b = episode_of(g), nt = tiles_of(g, b);
+            if (CL > 1 && m < nt && m != rk) mbar_arrive_expect_tx(h_arr(m), 2 * NT * 128);
+            if (rk < nt) {
+            const int n = neuron_of(b, first_of(g, b, rk), q, false);
+            wait_bar(d1_full, own & 1);
             tc_fence_after();
             if (m == 0) RM_ST(8);
             float v[NTOK];
@@ -405,10 +444,10 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 }
             }
             if (m == 0) RM_ST(42);
-            if (k > 0) wait_bar(h_free, (k - 1) & 1);              // the previous tile's down products are complete
+            if (k > 0) wait_bar(h_free, (k - 1) & 1);              // every CTA's down products of the previous group are complete
             // row q of the h tile: 64 tokens in bf16, 16-byte chunks swizzled by the row; hi at 0, lo at 8 KB
             {
-                unsigned char* rowp = gbase + S::OFF_HT + q * 128;
+                unsigned char* rowp = gbase + S::OFF_HT + rk * (2 * NT * 128) + q * 128;
 #pragma unroll
                 for (int c = 0; c < TH / 8; ++c) {
                     uint32_t hi[4], lo[4];
@@ -428,14 +467,25 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
             }
             fence_proxy_async_smem();
             mbar_arrive(h_full);
+            ++own;
+            if (CL > 1) {
+                named_barrier(1, 128);                             // every row is written and fenced
+                if (m < CL && m != rk) {
+                    const uint32_t src = sHT + rk * (2 * NT * 128);
+                    bulk_copy_to_peer(map_to_rank(src, m), src, 2 * NT * 128, map_to_rank(h_arr(rk), m));
+                }
+            }
             if (m == 0) RM_ST(9);
+            } else if (k > 0) {
+                wait_bar(h_free, (k - 1) & 1);                     // (a waiter follows every phase)
+            }
             // finished down blocks: lane = output column, token columns.  Transposed through shared memory into
             // [token][128 columns]; the copy engine adds the block to the output as one box of the [B, T, H] tensor
             // map (rows past T fall outside the map and are dropped).  The two staging buffers alternate, so one is
             // read while the other fills; the anchor step fills both per block, the ungated block for y_anchor and
             // the gated one for the output.
             const bool ya_b = anchor_mode == RM_ANCHOR_WRITE;
-            for (int mb = 0; mb < MBN; ++mb, ++mbc) {
+            for (int mb = rk * (MBN / CL); mb < (rk + 1) * (MBN / CL); ++mb, ++mbc) {
                 const int slot = mbc & 1;
                 wait_bar(d2_full(slot), (mbc >> 1) & 1);
                 tc_fence_after();
@@ -448,12 +498,12 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 tc_fence_before();
                 mbar_arrive(d2_free(slot));
                 if (m == 0) {                                      // the box(es) sent from the buffer(s) about to be filled have left
-                    if (ya_b) bulk_wait_read_all();
+                    if (ya_b || S::NYB == 1) bulk_wait_read_all();
                     else bulk_wait_read_but_one();
                 }
                 named_barrier(1, 128);                             // the previous block's rows have been read
                 if (!ya_b) {
-                    float* gYb = gY + (mbc & 1) * 8192;            // the copy engine reads one buffer while the other fills
+                    float* gYb = gY + (S::NYB == 1 ? 0 : (mbc & 1) * 8192);            // the copy engine reads one buffer while the other fills
                     const float gm = gate ? gate[(size_t)b * H + mb * 128 + m] : 1.f;
 #pragma unroll
                     for (int t = 0; t < NTOK; ++t)
@@ -498,62 +548,87 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
         auto look_ahead = [&]() {
             next_ok = __all_sync(0xffffffffu, mbar_test_wait(full((blk + 1) % NSTAGE), ((blk + 1) / NSTAGE) & 1));
         };
+        int own = 0;
+        uint32_t arr_par = 0;                                      // parity of the next phase of h_arr, a bit per tile
         for (int k = 0;; ++k) {
-            const int g = (int)blockIdx.x + k * (int)gridDim.x;
-            if (g >= tiles_total) break;
-            if (k > 0) wait_bar(d1_free, (k - 1) & 1);             // the epilogue has read the previous D1
-            tc_fence_after();
-            for (int kb = 0; kb < KBN; ++kb, ++blk) {
-                const uint32_t st = sRing + (blk % NSTAGE) * STAGE;
-                stage_ready();
-                if (lane == 0) {
-                    if (kb == 0) RM_ST(3);
-                    if (kb == KBN - 1) RM_ST(4);
-                }
-                if (GATHER) fence_proxy_async_smem();
+            const int g = cid + k * ncl;
+            if (g >= groups_total) break;
+            const int nt = tiles_of(g, episode_of(g));
+            if (rk < nt) {
+                if (own > 0) wait_bar(d1_free, (own - 1) & 1);     // the epilogue has read the previous D1
                 tc_fence_after();
-                if (elect_one()) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        mma_bf16_ss(tmem_d1, desc_k | desc_addr(st + ks * 32), desc_k | desc_addr(st + W_BYTES + ks * 32),
-                                    IDESC_GU, (kb | ks) != 0);
-                    mma_commit(empty(blk % NSTAGE));
-                }
-                __syncwarp();
-                look_ahead();
-            }
-            if (elect_one()) mma_commit(d1_full);
-            __syncwarp();
-            if (lane == 0) RM_ST(5);
-            wait_bar(h_full, k & 1);
-            if (lane == 0) RM_ST(6);
-            for (int mb = 0; mb < MBN; ++mb, ++blk, ++mbc) {
-                const int slot = mbc & 1;
-                const uint32_t st = sRing + (blk % NSTAGE) * STAGE;
-                if (mbc >= 2) wait_bar(d2_free(slot), ((mbc >> 1) - 1) & 1);
-                stage_ready();
-                if (GATHER) fence_proxy_async_smem();
-                tc_fence_after();
-                if (elect_one()) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t aa = desc_mn | desc_addr(st + ks * 2048);
-                        mma_bf16_ss(tmem_d1 + NTOK * (1 + slot), aa, desc_mn | desc_addr(sHT + ks * 2048), IDESC_DN, ks != 0);
-                        mma_bf16_ss(tmem_d1 + NTOK * (1 + slot), aa, desc_mn | desc_addr(sHT + NT * 128 + ks * 2048), IDESC_DN, true);
+                for (int kb = 0; kb < KBN; ++kb, ++blk) {
+                    const uint32_t st = sRing + (blk % NSTAGE) * STAGE;
+                    stage_ready();
+                    if (lane == 0) {
+                        if (kb == 0) RM_ST(3);
+                        if (kb == KBN - 1) RM_ST(4);
                     }
-                    mma_commit(empty(blk % NSTAGE));
-                    mma_commit(d2_full(slot));
+                    if (GATHER) fence_proxy_async_smem();
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_bf16_ss(tmem_d1, desc_k | desc_addr(st + ks * 32), desc_k | desc_addr(st + W_BYTES + ks * 32),
+                                        IDESC_GU, (kb | ks) != 0);
+                        mma_commit(empty(blk % NSTAGE));
+                    }
+                    __syncwarp();
+                    look_ahead();
                 }
+                if (elect_one()) mma_commit(d1_full);
                 __syncwarp();
-                look_ahead();
+                if (lane == 0) RM_ST(5);
+                wait_bar(h_full, own & 1);
+                ++own;
+                if (lane == 0) RM_ST(6);
             }
-            if (elect_one()) mma_commit(h_free);
+            uint32_t have = 1u << rk;                              // tiles whose h is here
+            for (int mb = 0; mb < MBN / CL; ++mb, ++mbc) {
+                const int slot = mbc & 1;
+                if (mbc >= 2) wait_bar(d2_free(slot), ((mbc >> 1) - 1) & 1);
+                bool first = true;
+#pragma unroll
+                for (int t = 0; t < CL; ++t) {
+                    const int tt = (rk + t) % CL;
+                    if (tt >= nt) continue;
+                    const uint32_t st = sRing + (blk % NSTAGE) * STAGE, ht = sHT + tt * (2 * NT * 128);
+                    if (!((have >> tt) & 1u)) {
+                        wait_bar(h_arr(tt), (arr_par >> tt) & 1u);
+                        arr_par ^= 1u << tt;
+                        have |= 1u << tt;
+                    }
+                    stage_ready();
+                    if (GATHER) fence_proxy_async_smem();
+                    tc_fence_after();
+                    if (elect_one()) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks) {
+                            const uint64_t aa = desc_mn | desc_addr(st + ks * 2048);
+                            mma_bf16_ss(tmem_d1 + NTOK * (1 + slot), aa, desc_mn | desc_addr(ht + ks * 2048), IDESC_DN, !(first && ks == 0));
+                            mma_bf16_ss(tmem_d1 + NTOK * (1 + slot), aa, desc_mn | desc_addr(ht + NT * 128 + ks * 2048), IDESC_DN, true);
+                        }
+                        mma_commit(empty(blk % NSTAGE));
+                    }
+                    __syncwarp();
+                    first = false;
+                    ++blk;
+                    next_ok = __all_sync(0xffffffffu, mbar_test_wait(full(blk % NSTAGE), (blk / NSTAGE) & 1));
+                }
+                if (elect_one()) mma_commit(d2_full(slot));
+                __syncwarp();
+            }
+            if (elect_one()) {
+                if (CL > 1) mma_commit_mc(h_free, (1u << CL) - 1u);
+                else mma_commit(h_free);
+            }
             __syncwarp();
             if (lane == 0) RM_ST(7);
         }
     }
     tc_fence_before();
     if (__syncthreads_or(gave_up)) linger_after_timeout();
+    if (CL > 1) cluster_sync();            // no CTA leaves while a peer's copies or arrivals may be on their way between them
     if (warp == 8) tmem_dealloc(tmem_d1, S::TMEM_COLS);
 }
 
@@ -606,19 +681,24 @@ int make_map_out(CUtensorMap* tm, const float* ptr, uint64_t B, uint64_t T, uint
     return r == CUDA_SUCCESS ? RM_OK : RM_ERR_CUDA;
 }
 
-template <int NTOK>
+template <int NTOK, int CL>
 int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
-    using S = SmemST<NTOK>;
+    using S = SmemST<NTOK, CL>;
     const bool eq4 = a.anchor_mode != RM_ANCHOR_NONE || a.gate != nullptr;
     const bool gather = a.idx != nullptr;
-    auto kern = gather ? (eq4 ? stream_tile_kernel<NTOK, true, true> : stream_tile_kernel<NTOK, false, true>)
-                       : (eq4 ? stream_tile_kernel<NTOK, true, false> : stream_tile_kernel<NTOK, false, false>);
+    auto kern = stream_tile_kernel<NTOK, false, true, CL>;
+    if (CL == 1) {
+        if (gather) kern = eq4 ? stream_tile_kernel<NTOK, true, true, 1> : stream_tile_kernel<NTOK, false, true, 1>;
+        else kern = eq4 ? stream_tile_kernel<NTOK, true, false, 1> : stream_tile_kernel<NTOK, false, false, 1>;
+    }
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, S::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, true, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+        if (CL == 1) {
+            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+        }
         configured.set(ctx->device, S::TOTAL);
     }
     CUtensorMap tmW, tmX, tmOut, tmYa;
@@ -637,17 +717,58 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
     cfg.blockDim = dim3(SE);
     cfg.dynamicSmemBytes = S::TOTAL;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CL;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = CL > 1 ? 2 : 1;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a, tmW, tmX, tmOut, tmYa));
     ctx->launches++;
     return RM_OK;
 }
 
+// co-resident clusters of CL CTAs of the streaming kernel
+template <int CL>
+int query_groups(int* out) {
+    using S = SmemST<64, CL>;
+    auto kern = stream_tile_kernel<64, false, true, CL>;
+    RM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CL * 128);
+    cfg.blockDim = dim3(SE);
+    cfg.dynamicSmemBytes = S::TOTAL;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RM_CUDA_TRY(cudaOccupancyMaxActiveClusters(out, kern, &cfg));
+    return RM_OK;
+}
+
+// Tiles per group: lists of the zero-fill form (see the kernel)
+int pick_group(const rm_ctx* ctx, const rm_layer_args& la, long long per_episode) {
+    if (!la.idx || la.anchor_mode != RM_ANCHOR_NONE || la.gate) return 1;
+    const int force = ctx->l2_prefetch;
+    if (force == 1 || force == 2 || force == 4) return force;
+    return 1;
+}
+
 }  // namespace
+
+int rm_stream_init(rm_ctx* ctx) {
+    int n[2] = {0, 0};
+    int rc = query_groups<2>(&n[0]);
+    if (rc == RM_OK) rc = query_groups<4>(&n[1]);
+    for (int i = 0; i < 2; ++i) ctx->stream_clusters[i] = rc == RM_OK ? n[i] : 0;
+    return rc;
+}
 
 int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int box_rows) {
     return make_map_out(static_cast<CUtensorMap*>(tensor_map), ptr, (uint64_t)B, (uint64_t)T, (uint64_t)H, (uint32_t)box_rows);
@@ -731,9 +852,19 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
     a.h_stride = la.h_stride;
     a.gate = la.gate;
     const int per_episode = la.count ? rm_effective_count_hint(ctx) : g.I;
-    long long tiles = per_episode > 0 ? (long long)((per_episode + NT - 1) / NT) * la.B : 0;
+    const long long per = per_episode > 0 ? (per_episode + NT - 1) / NT : 0, tiles = per * la.B;
     int n_ctas = ctx->sm_count;
     if (tiles > 0 && tiles < n_ctas) n_ctas = (int)tiles;
     if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < n_ctas) n_ctas = ctx->max_clusters_override;
-    return la.T <= 32 ? launch_tiles<32>(ctx, a, n_ctas, s) : launch_tiles<64>(ctx, a, n_ctas, s);
+    const int cl = pick_group(ctx, la, per);
+    if (cl > 1) {
+        const long long groups = (per + cl - 1) / cl * la.B;
+        int clusters = ctx->stream_clusters[cl == 2 ? 0 : 1];
+        if (groups > 0 && groups < clusters) clusters = (int)groups;
+        if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < clusters) clusters = ctx->max_clusters_override;
+        n_ctas = clusters * cl;
+        if (cl == 4) return la.T <= 32 ? launch_tiles<32, 4>(ctx, a, n_ctas, s) : launch_tiles<64, 4>(ctx, a, n_ctas, s);
+        return la.T <= 32 ? launch_tiles<32, 2>(ctx, a, n_ctas, s) : launch_tiles<64, 2>(ctx, a, n_ctas, s);
+    }
+    return la.T <= 32 ? launch_tiles<32, 1>(ctx, a, n_ctas, s) : launch_tiles<64, 1>(ctx, a, n_ctas, s);
 }

@@ -268,7 +268,7 @@ int64_t rm_launch_count(const rm_ctx* ctx);
  *                         itself for widths and chunk lengths that the others do not take), 7 = the sweep kernel (dense
  *                         steps of one episode in one launch)
  *   "stream_min_tiles"    launches with at least this many 64-neuron tiles use variant 4 when the variant is chosen
- *                         per launch (default 48 at H = 1024, 64 at H = 2048)
+ *                         per launch (default 33 at H = 1024, 31 at H = 2048)
  *   "persist_max_batch"   largest B for which the whole-step kernel may be chosen per call (default 1)
  *   "persist_prefetch_kb" whole-step kernel: KB of weight rows a CTA may ask into L2 ahead of its loaders (default 0:
  *                         measured slower than no prefetch)                                                    */
@@ -276,7 +276,7 @@ int rm_set_option(rm_ctx* ctx, const char* name, int value);
 
 /* Read-only facts: "fused_clusters" (co-resident clusters of the tcgen05 kernel, 0 when that path is
  * unavailable for this geometry or device), "fused_blocks_per_sm", "persist_clusters" (co-resident clusters of the
- * whole-step kernel), "slice_clusters" (the same for the slice kernel), "sm_count", "path", "last_variant" (kernel family of the last layer or step launched through this
+ * whole-step kernel), "stream_pairs" (co-resident pairs of CTAs of the streaming kernel), "slice_clusters" (the same for the slice kernel), "sm_count", "path", "last_variant" (kernel family of the last layer or step launched through this
  * context: 0 portable, 1-7 as for the "variant" option), and "status_detail": for
  * the last non-zero status that rm_device_status returned, where the kernel gave up (a bounded wait that ran out:
  * source line of the wait << 12 | CTA index & 0xfff); 0 when that status carried no detail.

@@ -84,10 +84,9 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
     sa.ctrl = reinterpret_cast<int*>(static_cast<char*>(persist_ws(ctx, ws, B, T)) + align_up(rm_persist_workspace_bytes(ctx), 256));
 }
 
-// The streaming variant (whole tiles per CTA) pays off only when a launch has about one 64-neuron tile per SM (one SM
-// gathers at most ~38 GB/s with 16-byte cp.async and adds at most ~20 GB/s with red.global, so a tile costs it
-// ~25 us); below that the cluster kernels, which spread a tile over 8 SMs, win.  H = 1024 only: at H = 2048 the
-// warp-specialised cluster kernel is ahead at every size measured.  `masked` says whether a count is in play.
+// The streaming variant (whole tiles per CTA): a tile costs an SM ~16 us at H = 1024 (its gathers run at ~20 bytes per clock,
+// its adds at 16), however few tiles there are; the cluster kernels, which spread a tile over 8 SMs, win while every cluster
+// has a single tile (stream_min_tiles, see rm_create).  `masked` says whether a count is in play.
 // anchor_write: the anchor step of Eq. 4 adds two boxes per block (y_anchor and the output) and stores h_anchor; measured
 // on the anchor schedule it stays behind the cluster kernels at 64 tiles (352 against 334 us per step), so it keeps
 // the threshold of about a tile per SM
@@ -121,12 +120,11 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->g.Hs = desc->H / RM_NS;
     c->launches = 0;
     c->status_detail = 0;
-    // measured crossover with the cluster kernels.  H = 1024: at 32 tiles the lean kernel is far ahead (270 against
-    // 370 us per step); at 48 the two are level on 3 episodes x 16 tiles (127 against 126) and the streaming variant
-    // is 7 % ahead on one episode of 48 tiles (378 against 350); at 64 it is 10 % ahead, at 80 by 30 %.
-    // H = 2048: the warp-specialised kernel is ahead at 52 tiles (512 against 582), level at 64, behind at 96 (50
-    // against 38 us per layer).
-    c->stream_min_tiles = desc->H == 2048 ? 64 : 48;
+    // Measured crossover with the cluster kernels, us a step of 18 layers and 51 tokens, lean / streaming kernel.  The lean
+    // kernel's time steps up with every round of its 32 (H = 1024) or 15 (H = 2048) co-resident clusters.  H = 1024: 32 tiles 269 / 291,
+    // 36 tiles 363 / 293 (20 tokens: 285 / 251), 46 tiles 408 / 294.  H = 2048: up to 30 tiles 360 to 380 / ~470, 32 tiles
+    // 531 / 475, 52 tiles 658 / 491.
+    c->stream_min_tiles = desc->H == 2048 ? 31 : 33;
     c->d_status = nullptr;
     int major = 0;                         // (two attributes: cudaGetDeviceProperties takes milliseconds)
     if (cudaGetDevice(&c->device) != cudaSuccess ||
@@ -150,7 +148,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->last_variant = 0;
     c->persist_clusters = 0;
     c->slice_clusters = 0;
-    c->stream_clusters[0] = c->stream_clusters[1] = 0;
+    c->stream_pairs = 0;
     c->persist_max_b = 1;
     c->persist_prefetch_kb = 0;
     c->persist_xbuf = nullptr;
@@ -655,8 +653,7 @@ int rm_get_info(const rm_ctx* ctx, const char* name, int* out) {
     else if (n == "fused_blocks_per_sm") *out = ctx->fused_blocks_per_sm;
     else if (n == "sm_count") *out = ctx->sm_count;
     else if (n == "persist_clusters") *out = ctx->persist_clusters;
-    else if (n == "stream_pairs") *out = ctx->stream_clusters[0];
-    else if (n == "stream_quads") *out = ctx->stream_clusters[1];
+    else if (n == "stream_pairs") *out = ctx->stream_pairs;
     else if (n == "slice_clusters") *out = ctx->slice_clusters;
     else if (n == "last_variant") *out = ctx->last_variant;
     else if (n == "path") *out = ctx->path;

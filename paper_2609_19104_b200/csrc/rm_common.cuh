@@ -46,7 +46,7 @@ struct rm_ctx {
     int variant_override;                  // 0 auto, 1 lean kernel, 2 kernel with a dedicated staging buffer
     int last_variant;                      // kernel family of the last layer or step launched (see rm_get_info)
     // whole-step kernel (rm_mlp_persist.cu)
-    int stream_clusters[2];                // co-resident clusters of 2 and of 4 CTAs of the streaming kernel
+    int stream_pairs;                      // co-resident pairs of CTAs of the streaming kernel
     int slice_clusters;                    // co-resident 8-CTA clusters of the slice kernel (0: unavailable)
     int persist_clusters;                  // co-resident 8-CTA clusters of the whole-step kernel (0: unavailable)
     int persist_prefetch_kb;               // weight KB a CTA of the whole-step kernel may ask into L2 ahead of its loaders

@@ -14,7 +14,7 @@
 //                  Four warps load: 16-byte cp.async gathers straight into the swizzled operand layout for index
 //                  lists (they top out near 16 bytes per clock and SM), cp.async.bulk.tensor boxes of 64 neurons x 64
 //                  columns for runs of consecutive neurons (one-row boxes were tried for lists and are far slower);
-//                  four warps read tensor memory and do the arithmetic, one thread issues the tcgen05.mma
+//                  eight warps read tensor memory and do the arithmetic, one thread issues the tcgen05.mma
 //                  instructions.
 //
 // Compared with the cluster kernels this trades the exchange latency (three hops per tile) for re-reading x from L2
@@ -60,66 +60,65 @@ struct PrepArgs {
     float* r_out;
     const float* y_anchor;             // update steps: out starts as r + gate * y_anchor
     const float* gate;
-    int T, H;
+    int T;
 };
 
-// One CTA per token row: x row in bf16, output row = residual (+ gate * y_anchor).
-__global__ void __launch_bounds__(256) stream_prep_kernel(const PrepArgs a) {
-    __shared__ float part[8];
+// One warp per token row: x row in bf16, output row = residual (+ gate * y_anchor).  The CTAs ask for more shared memory than a
+// tile CTA leaves on its SM, so that they, and behind them the next layer's tiles, start when the SMs become free: waiting
+// on the SMs beside the tiles instead they let the next tiles in early, whose first gathers then compete with the last ones
+// of this layer (us a step, 25 %: 8 episodes of 51 tokens 358 -> 338, 12 of 51 581 -> 551, 12 of 20 505 -> 469).
+constexpr int PREP_ROWS = 4;           // rows (warps) per CTA
+constexpr int PREP_SMEM = 40000;
+template <int H>
+__global__ void __launch_bounds__(32 * PREP_ROWS) stream_prep_kernel(const PrepArgs a, int rows) {
+    constexpr int N = H / 128;             // float4 per lane
     pdl_launch_dependents();
+    const int row = blockIdx.x * PREP_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     pdl_wait();                            // the previous layer's adds into r_in are complete
-    const int row = blockIdx.x, b = row / a.T;
-    const float4* src = reinterpret_cast<const float4*>(a.r_in + (size_t)row * a.H);
-    const int n4 = a.H / 4;
-    float4 v[2];
+    if (row >= rows) return;
+    const float4* src = reinterpret_cast<const float4*>(a.r_in + (size_t)row * H) + lane;
+    float4 v[N];
     float ss = 0.f;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int e = threadIdx.x + i * 256;
-        v[i] = e < n4 ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < N; ++i) v[i] = src[32 * i];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
         ss = fmaf(v[i].x, v[i].x, ss); ss = fmaf(v[i].y, v[i].y, ss);
         ss = fmaf(v[i].z, v[i].z, ss); ss = fmaf(v[i].w, v[i].w, ss);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    float tot = 0.f;
+    const float inv = 1.0f / sqrtf(ss / (float)H + 1e-6f);
 #pragma unroll
-    for (int w = 0; w < 8; ++w) tot += part[w];
-    const float inv = 1.0f / sqrtf(tot / (float)a.H + 1e-6f);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int e = threadIdx.x + i * 256;
-        if (e >= n4) continue;
-        __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x * inv, v[i].y * inv);
-        __nv_bfloat162 hi = __floats2bfloat162_rn(v[i].z * inv, v[i].w * inv);
+    for (int i = 0; i < N; ++i) {
+        const int e = lane + 32 * i;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[i].x * inv, v[i].y * inv);
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(v[i].z * inv, v[i].w * inv);
         uint2 u;
-        u.x = *reinterpret_cast<uint32_t*>(&lo);
-        u.y = *reinterpret_cast<uint32_t*>(&hi);
-        reinterpret_cast<uint2*>(a.x + (size_t)row * a.H)[e] = u;
+        u.x = *reinterpret_cast<const uint32_t*>(&lo);
+        u.y = *reinterpret_cast<const uint32_t*>(&hi);
+        reinterpret_cast<uint2*>(a.x + (size_t)row * H)[e] = u;
         float4 o = v[i];
         if (a.y_anchor) {
-            const float4 ya = reinterpret_cast<const float4*>(a.y_anchor + (size_t)row * a.H)[e];
+            const float4 ya = reinterpret_cast<const float4*>(a.y_anchor + (size_t)row * H)[e];
             float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
-            if (a.gate) g = reinterpret_cast<const float4*>(a.gate + (size_t)b * a.H)[e];
+            if (a.gate) g = reinterpret_cast<const float4*>(a.gate + (size_t)(row / a.T) * H)[e];
             o.x = fmaf(g.x, ya.x, o.x); o.y = fmaf(g.y, ya.y, o.y); o.z = fmaf(g.z, ya.z, o.z); o.w = fmaf(g.w, ya.w, o.w);
         }
-        reinterpret_cast<float4*>(a.r_out + (size_t)row * a.H)[e] = o;
+        reinterpret_cast<float4*>(a.r_out + (size_t)row * H)[e] = o;
     }
 }
 
 template <int NTOK, int CL>
 struct SmemST {
     static constexpr int NSTAGE = CL == 1 ? 6 : 5;
-    static constexpr int NYB = CL == 4 ? 1 : 2;                    // staging buffers of finished blocks
     static constexpr int OFF_RING = 0;
     static constexpr int OFF_HT = OFF_RING + NSTAGE * STAGE;       // h of the group's tiles: hi 8 KB, lo 8 KB each (64 neurons x 128 bytes)
-    static constexpr int OFF_Y = OFF_HT + CL * 2 * NT * 128;       // NYB x 32 KB: GeLU exchange [2][token][neuron] fp32 (first
+    static constexpr int OFF_Y = OFF_HT + CL * 2 * NT * 128;       // 2 x 32 KB: GeLU exchange [2][token][neuron] fp32 (first
                                                                    // buffer), then the transposed down blocks [token][128
                                                                    // columns] fp32, alternating between the two buffers
-    static constexpr int OFF_REC = OFF_Y + NYB * 32768;                  // record halves of the second token half
-    static constexpr int OFF_PREF = OFF_REC + NT * 4;              // tile prefix per episode, counts
+    static constexpr int OFF_REC = OFF_Y + 65536;                  // record halves of the second token half
+    static constexpr int OFF_PREF = OFF_REC + 3 * NT * 4;              // tile prefix per episode, counts
     static constexpr int OFF_BAR = ((OFF_PREF + (2 * MAXB + 1) * 4 + 7) / 8) * 8;
     static constexpr int TOTAL = OFF_BAR + 256 + 1024;             // + slack for the 1024-byte alignment
     static_assert(TOTAL <= 232448, "the streaming kernel's buffers exceed the 227 KB a CTA may use");
@@ -140,7 +139,8 @@ __device__ __forceinline__ long long st_now() {
 #define RM_ST(i) do { } while (0)
 #endif
 
-constexpr int SE = 288;                // threads: 4 epilogue warps (0-3), 4 loader warps (4-7), issuer warp (8)
+constexpr int SE = 416;                // threads: 8 epilogue warps (0-7), 4 loader warps (8-11), issuer warp (12)
+constexpr int EP = 256, W_LD = 8, W_IS = 12;
 
 // GATHER: the tile's neurons come from an index list, their rows are gathered with 16-byte cp.async (about 16 bytes
 // per clock and SM, the limit of this kernel on lists).  Otherwise the tile is 64 consecutive rows of the layer (dense
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                                                             const __grid_constant__ CUtensorMap tmYa) {
     using S = SmemST<NTOK, CL>;
     constexpr int NSTAGE = S::NSTAGE;
-    static_assert(CL == 1 || !EQ4, "groups of tiles: zero-fill form only");
+    static_assert(CL == 1 || (CL == 2 && !EQ4), "groups of tiles: zero-fill form only");
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
@@ -183,9 +183,9 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
 
     if (tid == 0) {
         for (int s = 0; s < NSTAGE; ++s) { mbar_init(full(s), GATHER ? 129 : 1); mbar_init(empty(s), 1); }
-        mbar_init(d1_full, 1); mbar_init(d1_free, 128); mbar_init(h_full, 128); mbar_init(h_free, CL);
+        mbar_init(d1_full, 1); mbar_init(d1_free, EP); mbar_init(h_full, EP); mbar_init(h_free, CL);
         for (int t = 0; t < CL; ++t) mbar_init(h_arr(t), 1);
-        for (int s = 0; s < 2; ++s) { mbar_init(d2_full(s), 1); mbar_init(d2_free(s), 128); }
+        for (int s = 0; s < 2; ++s) { mbar_init(d2_full(s), 1); mbar_init(d2_free(s), EP); }
         fence_mbar_init();
     }
     if (tid < a.B) {                       // (a thread per episode: one thread reading them in turn took ~0.4 us each)
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
         }
         gCnt[tid] = c;
     }
-    if (warp == 8) tmem_alloc(s_tmem, S::TMEM_COLS);
+    if (warp == W_IS) tmem_alloc(s_tmem, S::TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     if (tid == 0) {
@@ -212,9 +212,11 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
     if (CL > 1) cluster_sync();            // peers' shared memory and barriers are live from here on
     tc_fence_after();
     const uint32_t tmem_d1 = *g_tmem;
-    pdl_launch_dependents();
 
+    // The next layer's kernels may come in once every CTA has reached its last group: earlier, their first gathers would
+    // compete with those of the CTAs that have another group to do
     const int groups_total = gPref[a.B];
+    pdl_launch_dependents();
     bool gave_up = false;
     auto wait_bar_at = [&](uint32_t bar, uint32_t parity, int line) {
         if (!mbar_wait(bar, parity)) {
@@ -249,9 +251,9 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
     const uint64_t desc_mn = smem_desc_sw128(0, 8192, 1024);
     constexpr uint32_t GU_TX = W_BYTES + NTOK * 128, DN_TX = W_BYTES;
 
-    if (warp >= 4 && warp < 8) {
+    if (warp >= W_LD && warp < W_IS) {
         // ================================================================ loaders
-        const int lt = tid - 128;                                  // loader thread 0..127
+        const int lt = tid - W_LD * 32;                                 // loader thread 0..127
         const int r0 = lt >> 3, ch = lt & 7;                       // gathers: rows r0 + 16 i, 16-byte chunk ch
         uint32_t blk = 0;                                          // stages filled so far
         bool waited = false;                                       // griddepcontrol.wait done (x depends on it)
@@ -358,34 +360,40 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
             }
         }
         if (!waited) pdl_wait();
-    } else if (warp < 4) {
+    } else if (warp < W_LD) {
         // ================================================================ epilogue: tensor memory -> h, output
-        const int m = tid, w4 = warp;                              // accumulator lane of this thread
-        const int q = m & 63, half = m >> 6;                       // its neuron slot; token half it finishes
-        constexpr int TH = NTOK / 2;                               // tokens per half
+        const int w4 = warp & 3, th = warp >> 2, m = w4 * 32 + lane;           // accumulator lane of this thread, its token half
+        const int q = m & 63, half = m >> 6;                       // its neuron slot; which tokens of its half it finishes
+        constexpr int TW = NTOK / 2, TH = TW / 2;                  // tokens it reads, tokens it finishes
+        auto read = [&](uint32_t addr, float (&d)[TW]) {
+            if constexpr (TW == 32) {
+                tmem_ld32(addr, d);
+            } else {
+#pragma unroll
+                for (int c0 = 0; c0 < TW; c0 += 8) tmem_ld8(addr + c0, *reinterpret_cast<float(*)[8]>(d + c0));
+            }
+        };
         uint32_t mbc = 0;                                          // down blocks consumed so far
         int own = 0;                                               // tiles of its own this CTA has had
         for (int k = 0;; ++k) {
             const int g = cid + k * ncl;
             if (g >= groups_total) break;
             const int b = episode_of(g), nt = tiles_of(g, b);
-            if (CL > 1 && m < nt && m != rk) mbar_arrive_expect_tx(h_arr(m), 2 * NT * 128);
+            if (CL > 1 && tid < nt && tid != rk) mbar_arrive_expect_tx(h_arr(tid), 2 * NT * 128);
             if (rk < nt) {
             const int n = neuron_of(b, first_of(g, b, rk), q, false);
             wait_bar(d1_full, own & 1);
             tc_fence_after();
-            if (m == 0) RM_ST(8);
-            float v[NTOK];
-#pragma unroll
-            for (int c0 = 0; c0 < NTOK; c0 += 32)
-                tmem_ld32(tmem_d1 + ((uint32_t)(w4 * 32) << 16) + c0, *reinterpret_cast<float(*)[32]>(v + c0));
+            if (tid == 0) RM_ST(8);
+            float v[TW];
+            read(tmem_d1 + ((uint32_t)(w4 * 32) << 16) + th * TW, v);
             tc_fence_before();
             mbar_arrive(d1_free);
-            if (m == 0) RM_ST(40);
-            // lanes 0..63 hold the gate rows, lanes 64..127 the up rows.  Thread (q, half 0) finishes tokens 0..TH-1
-            // of neuron q, thread (q, half 1) tokens TH..NTOK-1: each passes the other the half it does not need.
-            float* xg = gY;                                        // gate values of the second token half [t][q]
-            float* xu = gY + TH * NT;                              // up values of the first token half   [t][q]
+            if (tid == 0) RM_ST(40);
+            // lanes 0..63 hold the gate rows, lanes 64..127 the up rows.  Of the tokens of its half, thread (q, half 0) finishes the
+            // first TH of neuron q, thread (q, half 1) the others: each passes the other those it does not need.
+            float* xg = gY + th * 2 * TH * NT;                     // gate values of the second part [t][q]
+            float* xu = xg + TH * NT;                              // up values of the first part    [t][q]
             if (half == 0) {
 #pragma unroll
                 for (int t = 0; t < TH; ++t) xg[t * NT + q] = v[TH + t];
@@ -393,9 +401,9 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
 #pragma unroll
                 for (int t = 0; t < TH; ++t) xu[t * NT + q] = v[t];
             }
-            named_barrier(1, 128);
-            if (m == 0) RM_ST(41);
-            const int tb = half * TH;                              // first token of this thread
+            named_barrier(1, EP);
+            if (tid == 0) RM_ST(41);
+            const int tb = th * TW + half * TH;                    // first token of this thread
             float hv[TH];
             float rec = 0.f;
             // in stages over all TH elements, so that the exponentials and divisions of different tokens overlap (one
@@ -436,14 +444,15 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 }
             }
             if (a.record) {
-                if (half == 1) gRec[q] = rec;
-                named_barrier(1, 128);
-                if (half == 0 && n >= 0) {
-                    rec += gRec[q];
+                const int part = th * 2 + half;                    // the four token parts of a neuron
+                if (part != 0) gRec[(part - 1) * NT + q] = rec;
+                named_barrier(1, EP);
+                if (part == 0 && n >= 0) {
+                    rec += gRec[q] + gRec[NT + q] + gRec[2 * NT + q];
                     a.record[(size_t)b * a.record_stride + n] = a.record_scale ? rec * a.record_scale[n] : rec;
                 }
             }
-            if (m == 0) RM_ST(42);
+            if (tid == 0) RM_ST(42);
             if (k > 0) wait_bar(h_free, (k - 1) & 1);              // every CTA's down products of the previous group are complete
             // row q of the h tile: 64 tokens in bf16, 16-byte chunks swizzled by the row; hi at 0, lo at 8 KB
             {
@@ -469,13 +478,13 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
             mbar_arrive(h_full);
             ++own;
             if (CL > 1) {
-                named_barrier(1, 128);                             // every row is written and fenced
-                if (m < CL && m != rk) {
+                named_barrier(1, EP);                             // every row is written and fenced
+                if (tid < CL && tid != rk) {
                     const uint32_t src = sHT + rk * (2 * NT * 128);
-                    bulk_copy_to_peer(map_to_rank(src, m), src, 2 * NT * 128, map_to_rank(h_arr(rk), m));
+                    bulk_copy_to_peer(map_to_rank(src, tid), src, 2 * NT * 128, map_to_rank(h_arr(rk), tid));
                 }
             }
-            if (m == 0) RM_ST(9);
+            if (tid == 0) RM_ST(9);
             } else if (k > 0) {
                 wait_bar(h_free, (k - 1) & 1);                     // (a waiter follows every phase)
             }
@@ -489,53 +498,50 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
                 const int slot = mbc & 1;
                 wait_bar(d2_full(slot), (mbc >> 1) & 1);
                 tc_fence_after();
-                if (m == 0) RM_ST(10 + mb);
-                float y[NTOK];
-#pragma unroll
-                for (int c0 = 0; c0 < NTOK; c0 += 32)
-                    tmem_ld32(tmem_d1 + NTOK * (1 + slot) + ((uint32_t)(w4 * 32) << 16) + c0,
-                              *reinterpret_cast<float(*)[32]>(y + c0));
+                if (tid == 0) RM_ST(10 + mb);
+                float y[TW];
+                read(tmem_d1 + NTOK * (1 + slot) + ((uint32_t)(w4 * 32) << 16) + th * TW, y);
                 tc_fence_before();
                 mbar_arrive(d2_free(slot));
-                if (m == 0) {                                      // the box(es) sent from the buffer(s) about to be filled have left
-                    if (ya_b || S::NYB == 1) bulk_wait_read_all();
+                if (tid == 0) {                                      // the box(es) sent from the buffer(s) about to be filled have left
+                    if (ya_b) bulk_wait_read_all();
                     else bulk_wait_read_but_one();
                 }
-                named_barrier(1, 128);                             // the previous block's rows have been read
+                named_barrier(1, EP);                             // the previous block's rows have been read
                 if (!ya_b) {
-                    float* gYb = gY + (S::NYB == 1 ? 0 : (mbc & 1) * 8192);            // the copy engine reads one buffer while the other fills
+                    float* gYb = gY + (mbc & 1) * 8192;            // the copy engine reads one buffer while the other fills
                     const float gm = gate ? gate[(size_t)b * H + mb * 128 + m] : 1.f;
 #pragma unroll
-                    for (int t = 0; t < NTOK; ++t)
-                        if (t < T) gYb[t * 128 + m] = gm * y[t];
+                    for (int t = 0; t < TW; ++t)
+                        if (th * TW + t < T) gYb[(th * TW + t) * 128 + m] = gm * y[t];
                     fence_proxy_async_smem();
-                    named_barrier(1, 128);
-                    if (m == 0) {
+                    named_barrier(1, EP);
+                    if (tid == 0) {
                         tensor_reduce_add_3d(&tmOut, mb * 128, 0, b, smem_u32(gYb));
                         bulk_commit();
                     }
                 } else {
                     const float gm = gate ? gate[(size_t)b * H + mb * 128 + m] : 1.f;
 #pragma unroll
-                    for (int t = 0; t < NTOK; ++t)
-                        if (t < T) {
-                            gY[t * 128 + m] = y[t];
-                            gY[8192 + t * 128 + m] = gm * y[t];
+                    for (int t = 0; t < TW; ++t)
+                        if (th * TW + t < T) {
+                            gY[(th * TW + t) * 128 + m] = y[t];
+                            gY[8192 + (th * TW + t) * 128 + m] = gm * y[t];
                         }
                     fence_proxy_async_smem();
-                    named_barrier(1, 128);
-                    if (m == 0) {
+                    named_barrier(1, EP);
+                    if (tid == 0) {
                         tensor_reduce_add_3d(&tmYa, mb * 128, 0, b, smem_u32(gY));
                         tensor_reduce_add_3d(&tmOut, mb * 128, 0, b, smem_u32(gY + 8192));
                         bulk_commit();
                     }
                 }
-                if (m == 0) RM_ST(30 + mb);
+                if (tid == 0) RM_ST(30 + mb);
             }
-            if (m == 0) bulk_wait_read_all();
-            named_barrier(1, 128);                                 // the exchange area is free for the next tile
+            if (tid == 0) bulk_wait_read_all();
+            named_barrier(1, EP);                                 // the exchange area is free for the next tile
         }
-    } else if (warp == 8) {
+    } else if (warp == W_IS) {
         // ================================================================ issuer: the whole warp runs the loop and one
         // elected lane issues (a loop that only lane 0 runs costs 100-150 clocks more per stage, and the tensor pipe
         // idles while the issuing thread does anything else).  The test of the next stage's barrier (~200 clocks even
@@ -629,7 +635,7 @@ __global__ void __launch_bounds__(SE, 1) stream_tile_kernel(const StreamArgs a, 
     tc_fence_before();
     if (__syncthreads_or(gave_up)) linger_after_timeout();
     if (CL > 1) cluster_sync();            // no CTA leaves while a peer's copies or arrivals may be on their way between them
-    if (warp == 8) tmem_dealloc(tmem_d1, S::TMEM_COLS);
+    if (warp == W_IS) tmem_dealloc(tmem_d1, S::TMEM_COLS);
 }
 
 // ---- tensor maps (host).  cuTensorMapEncodeTiled is taken from the driver through the runtime, so the library does
@@ -731,43 +737,35 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
     return RM_OK;
 }
 
-// co-resident clusters of CL CTAs of the streaming kernel
-template <int CL>
-int query_groups(int* out) {
-    using S = SmemST<64, CL>;
-    auto kern = stream_tile_kernel<64, false, true, CL>;
-    RM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL * 128);
-    cfg.blockDim = dim3(SE);
-    cfg.dynamicSmemBytes = S::TOTAL;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    RM_CUDA_TRY(cudaOccupancyMaxActiveClusters(out, kern, &cfg));
-    return RM_OK;
-}
-
-// Tiles per group: lists of the zero-fill form (see the kernel)
-int pick_group(const rm_ctx* ctx, const rm_layer_args& la, long long per_episode) {
-    if (!la.idx || la.anchor_mode != RM_ANCHOR_NONE || la.gate) return 1;
-    const int force = ctx->l2_prefetch;
-    if (force == 1 || force == 2 || force == 4) return force;
-    return 1;
+// Tiles per group: pairs for lists of the zero-fill form at H = 2048 and more than 32 tokens, where the adds of a tile (16 blocks
+// of up to 32 KB) outweigh the exchange of h: one episode of 55 % of 16384 629 -> 561 us a step, two of 20 % 540 -> 495; at
+// H = 1024, or 20 tokens, single tiles are level or ahead.
+int pick_group(const rm_ctx* ctx, const rm_layer_args& la) {
+    if (!la.idx || la.anchor_mode != RM_ANCHOR_NONE || la.gate || ctx->stream_pairs <= 0) return 1;
+    return ctx->g.H == 2048 && la.T > 32 ? 2 : 1;
 }
 
 }  // namespace
 
 int rm_stream_init(rm_ctx* ctx) {
-    int n[2] = {0, 0};
-    int rc = query_groups<2>(&n[0]);
-    if (rc == RM_OK) rc = query_groups<4>(&n[1]);
-    for (int i = 0; i < 2; ++i) ctx->stream_clusters[i] = rc == RM_OK ? n[i] : 0;
-    return rc;
+    using S = SmemST<64, 2>;
+    auto kern = stream_tile_kernel<64, false, true, 2>;
+    RM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(256);
+    cfg.blockDim = dim3(SE);
+    cfg.dynamicSmemBytes = S::TOTAL;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    RM_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, kern, &cfg));
+    ctx->stream_pairs = n;
+    return RM_OK;
 }
 
 int rm_make_out_map(void* tensor_map, const float* ptr, int B, int T, int H, int box_rows) {
@@ -815,17 +813,18 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
         p.y_anchor = la.anchor_mode == RM_ANCHOR_UPDATE ? la.y_anchor : nullptr;
         p.gate = la.gate;
         p.T = la.T;
-        p.H = g.H;
+        const int rows = la.B * la.T;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(la.B * la.T);
-        cfg.blockDim = dim3(256);
+        cfg.gridDim = dim3((rows + PREP_ROWS - 1) / PREP_ROWS);
+        cfg.blockDim = dim3(32 * PREP_ROWS);
+        cfg.dynamicSmemBytes = PREP_SMEM;
         cfg.stream = s;
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
         cfg.numAttrs = pdl ? 1 : 0;
-        RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, stream_prep_kernel, p));
+        RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, g.H == 1024 ? stream_prep_kernel<1024> : stream_prep_kernel<2048>, p, rows));
         ctx->launches++;
         x = x_scratch;
     }
@@ -856,15 +855,13 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
     int n_ctas = ctx->sm_count;
     if (tiles > 0 && tiles < n_ctas) n_ctas = (int)tiles;
     if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < n_ctas) n_ctas = ctx->max_clusters_override;
-    const int cl = pick_group(ctx, la, per);
+    const int cl = pick_group(ctx, la);
     if (cl > 1) {
         const long long groups = (per + cl - 1) / cl * la.B;
-        int clusters = ctx->stream_clusters[cl == 2 ? 0 : 1];
+        int clusters = ctx->stream_pairs;
         if (groups > 0 && groups < clusters) clusters = (int)groups;
         if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < clusters) clusters = ctx->max_clusters_override;
-        n_ctas = clusters * cl;
-        if (cl == 4) return la.T <= 32 ? launch_tiles<32, 4>(ctx, a, n_ctas, s) : launch_tiles<64, 4>(ctx, a, n_ctas, s);
-        return la.T <= 32 ? launch_tiles<32, 2>(ctx, a, n_ctas, s) : launch_tiles<64, 2>(ctx, a, n_ctas, s);
+        return la.T <= 32 ? launch_tiles<32, 2>(ctx, a, 2 * clusters, s) : launch_tiles<64, 2>(ctx, a, 2 * clusters, s);
     }
     return la.T <= 32 ? launch_tiles<32, 1>(ctx, a, n_ctas, s) : launch_tiles<64, 1>(ctx, a, n_ctas, s);
 }

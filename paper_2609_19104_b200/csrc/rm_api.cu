@@ -221,8 +221,6 @@ int rm_gather_weights(rm_ctx* ctx, const void* packed_layer, const int32_t* idx,
                                  static_cast<cudaStream_t>(stream));
 }
 
-static int context_pad(int R_max) { return R_max <= 64 ? 64 : (R_max <= 128 ? 128 : 256); }
-
 int rm_context_drift(rm_ctx* ctx, const void* x, const void* x_ref, int P, float* score_out, rm_stream_t stream) {
     if (!ctx || !x || !x_ref || !score_out || P < 0) return RM_ERR_INVALID_ARG;
     if (ctx->g.H % 8 != 0) return RM_ERR_UNSUPPORTED;
@@ -235,7 +233,7 @@ constexpr int RM_CONTEXT_MAX_ROWS = 1024;      // four passes of 256 rows over t
 
 size_t rm_context_workspace_bytes(const rm_ctx* ctx, int R_max) {
     if (!ctx || R_max < 1 || R_max > RM_CONTEXT_MAX_ROWS || !rm_context_supported(ctx)) return 0;
-    return rm_context_workspace_bytes_impl(ctx, context_pad(R_max));
+    return rm_context_workspace_bytes_impl(ctx, R_max);
 }
 
 int rm_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, const void* x, const int32_t* rows,
@@ -246,9 +244,9 @@ int rm_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, 
     if (R_max < 1 || R_max > RM_CONTEXT_MAX_ROWS || S > R_max) return RM_ERR_SHAPE;
     if (!all_aligned({Wg, Wu, Wd, x, rows, y_ref, y_out, ws})) return RM_ERR_ALIGN;
     if (!ws || ws_bytes < rm_context_workspace_bytes(ctx, R_max)) return RM_ERR_WORKSPACE;
-    // rows beyond 256 take further passes; a single pass rounds its capacity up to the tile it runs in
-    return rm_launch_context_ffn(ctx, Wg, Wu, Wd, x, rows, count_dev, P, S, R_max <= 256 ? context_pad(R_max) : R_max, y_ref,
-                                 y_out, ws, static_cast<cudaStream_t>(stream));
+    // rows beyond 256 take further passes; the capacity is rounded up to what the passes hold (the rows that this adds are zero)
+    return rm_launch_context_ffn(ctx, Wg, Wu, Wd, x, rows, count_dev, P, S, R_max, y_ref, y_out, ws,
+                                 static_cast<cudaStream_t>(stream));
 }
 
 int rm_mask_compact(rm_ctx* ctx, const rm_mask_src* src, int32_t* idx_out, int32_t* count_out, int64_t stride,

@@ -8,9 +8,11 @@
 //   phase A : H1[r, n] = bf16(gelu_tanh(<Xc_r, Wg_n>) * <Xc_r, Wu_n>)  one CTA per 128 neurons, K = H
 //   phase B : Yp[s][r, c] = sum over the s-th slice of n of H1[r, n] Wd[c, n]   one CTA per (128 columns, K slice)
 //   scatter : y_out = y_ref, then y_out[rows[r], :] = sum_s Yp[s][r, :]
-// Both products are D[128 x NR] (+)= A[128 x 64] B[NR x 64]^T per stage: A = weight rows (K contiguous, as the model
-// stores them), B = activation rows, fp32 accumulators in tensor memory (phase A holds two, gate and up: all 512 columns
-// at NR = 256).
+// Both products are D[256 x N] (+)= A[256 x 64] B[N x 64]^T per stage, by pairs of CTAs (cta_group::2): A = weight rows (K
+// contiguous, as the model stores them), 128 per CTA; B = activation rows, half of them in each CTA; fp32 accumulators in tensor
+// memory (phase A holds two, gate and up: all 512 columns at N = 256).  What bounds a product is what an SM can take in, ~30
+// bytes per clock: a pair halves the activations each CTA loads (48 instead of 64 KB a stage in phase A, 32 instead of 48 in
+// phase B).  Activation rows are padded to a multiple of 32.  @MEASURED@
 #include <cuda.h>
 
 #include <mutex>
@@ -23,11 +25,6 @@ using namespace sm100;
 namespace {
 
 constexpr int CT = 192;                // threads: epilogue warps 0-3, loader warp 4 (one lane), issuer warp 5 (one lane)
-
-__device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t mbar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(mbar) : "memory");
-}
 
 // ---------------------------------------------------------------- Eq. 2: one warp per row
 __global__ void __launch_bounds__(256) drift_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ xr,
@@ -136,121 +133,132 @@ __global__ void __launch_bounds__(256) ctx_scatter_kernel(const float* __restric
 // ---------------------------------------------------------------- the two products
 // DUAL (phase A): A0 = Wg rows, A1 = Wu rows of this CTA's 128 neurons over all K = H; epilogue GeLU*u -> bf16 H1.
 // !DUAL (phase B): A0 = Wd rows of this CTA's 128 output columns over its K slice; epilogue fp32 partial -> Yp.
-template <int NR, bool DUAL>
+template <bool DUAL>
 struct SmemCtx {
     static constexpr int A_BYTES = 128 * 128;                      // 128 rows x 64 bf16
-    static constexpr int B_BYTES = NR * 128;
-    static constexpr int STAGE = (DUAL ? 2 : 1) * A_BYTES + B_BYTES;
-    static constexpr int NSTAGE = (200 * 1024) / STAGE > 6 ? 6 : (200 * 1024) / STAGE;
+    static constexpr int STAGE = (DUAL ? 3 : 2) * A_BYTES;         // the last part: up to 128 activation rows x 64 bf16
+    static constexpr int NSTAGE = DUAL ? 4 : 6;
     static constexpr int OFF_STG = NSTAGE * STAGE;                 // epilogue staging: 32 rows x 256 bytes
     static constexpr int OFF_BAR = OFF_STG + 8192;
     static constexpr int TOTAL = OFF_BAR + 256 + 1024;
-    static constexpr int TMEM_COLS = (DUAL ? 2 : 1) * NR < 32 ? 32 : (DUAL ? 2 : 1) * NR;
 };
 
 struct CtxGemmArgs {
-    int kblocks;                       // 64-wide K blocks per CTA
-    int I, H, r_pad;
-    __nv_bfloat16* h1;                 // phase A output [r_pad, I]
-    float* yp;                         // phase B output [ksplit, r_pad, H]
+    int kblocks;                       // 64-wide K blocks of the whole product (phase B: cut evenly over gridDim.y)
+    int n;                             // activation rows: a multiple of 32, at most 256
+    int rows;                          // weight rows (neurons or output columns)
+    int I, H;
+    __nv_bfloat16* h1;                 // phase A output [n, I]
+    float* yp;                         // phase B output [gridDim.y, n, H]
     int* status;
 };
 
 #define wait_bar(bar, parity) wait_bar_at((bar), (parity), __LINE__)
 
-template <int NR, bool DUAL>
+template <bool DUAL>
 __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, const __grid_constant__ CUtensorMap tmA0,
                                                          const __grid_constant__ CUtensorMap tmA1,
                                                          const __grid_constant__ CUtensorMap tmB) {
-    using S = SmemCtx<NR, DUAL>;
-    constexpr int NSTAGE = S::NSTAGE;
+    using S = SmemCtx<DUAL>;
+    constexpr int NSTAGE = S::NSTAGE, OFF_B = (DUAL ? 2 : 1) * S::A_BYTES, TMEM_COLS = DUAL ? 512 : 256;
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
     const uint32_t bar0 = base + S::OFF_BAR;
-    auto full = [&](int s) { return bar0 + 8 * s; };
-    auto empty = [&](int s) { return bar0 + 64 + 8 * s; };
+    auto full = [&](int s) { return bar0 + 8 * s; };               // (rank 0: the boxes of both CTAs have landed)
+    auto empty = [&](int s) { return bar0 + 64 + 8 * s; };         // the products reading a stage are complete
     const uint32_t d_full = bar0 + 128, s_tmem = bar0 + 136;
     volatile uint32_t* g_tmem = reinterpret_cast<volatile uint32_t*>(gbase + S::OFF_BAR + 136);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_ctarank(), n = a.n;
 
     if (tid == 0) {
         for (int s = 0; s < NSTAGE; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
         mbar_init(d_full, 1);
         fence_mbar_init();
     }
-    if (warp == 5) tmem_alloc(s_tmem, S::TMEM_COLS);
+    if (warp == 5) tmem_alloc_pair(s_tmem, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
+    cluster_sync();                        // the other CTA's barriers and tensor memory are there
     tc_fence_after();
     const uint32_t tmem = *g_tmem;
     pdl_launch_dependents();
 
     bool gave_up = false;
     auto wait_bar_at = [&](uint32_t bar, uint32_t parity, int line) {
-        if (!mbar_wait(bar, parity)) {
+        if (!gave_up && !mbar_wait(bar, parity)) {
             rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
             gave_up = true;
         }
     };
     // this CTA's block of A rows and its K range
-    const int m0 = DUAL ? (int)blockIdx.x * 128 : (int)blockIdx.x * 128;       // neurons (A) or output columns (B)
-    const int kb0 = DUAL ? 0 : (int)blockIdx.y * a.kblocks;
-    constexpr uint32_t IDESC = idesc_bf16_f32(128, NR, false, false);
-    const uint64_t desc_k = smem_desc_sw128(0, 16, 1024);
+    const int m0 = (int)blockIdx.x * 128;
+    const int kb0 = DUAL ? 0 : a.kblocks * (int)blockIdx.y / (int)gridDim.y;
+    const int kbn = (DUAL ? a.kblocks : a.kblocks * ((int)blockIdx.y + 1) / (int)gridDim.y) - kb0;
 
     if (warp == 4 && lane == 0) {
         // ---- loader: the weights do not depend on the previous kernel, the activations do
-        bool waited = false;
-        const int pre = a.kblocks < NSTAGE ? a.kblocks : NSTAGE;
-        for (int kb = 0; kb < pre; ++kb) {
-            const uint32_t st = base + kb * S::STAGE;
-            mbar_arrive_expect_tx(full(kb), S::STAGE);
-            tma_box(st, &tmA0, (kb0 + kb) * 64, m0, full(kb));
-            if (DUAL) tma_box(st + S::A_BYTES, &tmA1, (kb0 + kb) * 64, m0, full(kb));
-        }
+        const int half = n / 2;
+        const uint32_t bytes = 2u * ((DUAL ? 2u : 1u) * S::A_BYTES + (uint32_t)half * 128u);
+        auto weights = [&](int kb, int s) {
+            const uint32_t st = base + s * S::STAGE, fb = map_to_rank(full(s), 0);
+            if (rank == 0) mbar_arrive_expect_tx(full(s), bytes);
+            tma_load_2d_pair(st, &tmA0, (kb0 + kb) * 64, m0, fb);
+            if (DUAL) tma_load_2d_pair(st + S::A_BYTES, &tmA1, (kb0 + kb) * 64, m0, fb);
+        };
+        auto rows = [&](int kb, int s) {
+            tma_load_2d_pair(base + s * S::STAGE + OFF_B, &tmB, (kb0 + kb) * 64, rank * half, map_to_rank(full(s), 0));
+        };
+        const int pre = kbn < NSTAGE ? kbn : NSTAGE;
+        for (int kb = 0; kb < pre; ++kb) weights(kb, kb);
         pdl_wait();
-        waited = true;
-        for (int kb = 0; kb < pre; ++kb)
-            tma_box(base + kb * S::STAGE + (DUAL ? 2 : 1) * S::A_BYTES, &tmB, (kb0 + kb) * 64, 0, full(kb));
-        for (int kb = pre; kb < a.kblocks; ++kb) {
+        for (int kb = 0; kb < pre; ++kb) rows(kb, kb);
+        for (int kb = pre; kb < kbn && !gave_up; ++kb) {
             const int s = kb % NSTAGE;
             wait_bar(empty(s), ((kb / NSTAGE) - 1) & 1);
-            const uint32_t st = base + s * S::STAGE;
-            mbar_arrive_expect_tx(full(s), S::STAGE);
-            tma_box(st, &tmA0, (kb0 + kb) * 64, m0, full(s));
-            if (DUAL) tma_box(st + S::A_BYTES, &tmA1, (kb0 + kb) * 64, m0, full(s));
-            tma_box(st + (DUAL ? 2 : 1) * S::A_BYTES, &tmB, (kb0 + kb) * 64, 0, full(s));
+            if (gave_up) break;
+            weights(kb, s);
+            rows(kb, s);
         }
-        (void)waited;
-    } else if (warp == 5 && lane == 0) {
-        // ---- issuer
-        for (int kb = 0; kb < a.kblocks; ++kb) {
+    } else if (warp == 5 && rank == 0) {
+        // ---- issuer: the whole warp runs the loop, one elected lane issues; the next stage's barrier is tested behind the
+        // current stage's products
+        const uint32_t idesc = idesc_bf16_f32(256, n, false, false);
+        const uint64_t desc_k = smem_desc_sw128(0, 16, 1024);
+        bool ok = false;
+        for (int kb = 0; kb < kbn && !gave_up; ++kb) {
             const int s = kb % NSTAGE;
             const uint32_t st = base + s * S::STAGE;
-            wait_bar(full(s), (kb / NSTAGE) & 1);
+            if (!ok) wait_bar(full(s), (kb / NSTAGE) & 1);
+            gave_up = __any_sync(0xffffffffu, gave_up);
+            if (gave_up) break;
             tc_fence_after();
+            if (elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t bd = desc_k | desc_addr(st + (DUAL ? 2 : 1) * S::A_BYTES + ks * 32);
-                mma_bf16_ss(tmem, desc_k | desc_addr(st + ks * 32), bd, IDESC, (kb | ks) != 0);
-                if (DUAL) mma_bf16_ss(tmem + NR, desc_k | desc_addr(st + S::A_BYTES + ks * 32), bd, IDESC, (kb | ks) != 0);
+                for (int ks = 0; ks < 4; ++ks) {
+                    const uint64_t bd = desc_k | desc_addr(st + OFF_B + ks * 32);
+                    mma_bf16_ss_pair(tmem, desc_k | desc_addr(st + ks * 32), bd, idesc, (kb | ks) != 0);
+                    if (DUAL) mma_bf16_ss_pair(tmem + 256, desc_k | desc_addr(st + S::A_BYTES + ks * 32), bd, idesc, (kb | ks) != 0);
+                }
+                mma_commit_pair(empty(s));
+                if (kb == kbn - 1) mma_commit_pair(d_full);
             }
-            mma_commit(empty(s));
+            __syncwarp();
+            ok = __all_sync(0xffffffffu, mbar_test_wait(full((kb + 1) % NSTAGE), ((kb + 1) / NSTAGE) & 1));
         }
-        mma_commit(d_full);
     } else if (warp < 4) {
         // ---- epilogue: lane = A row (neuron or output column), registers = activation rows
         const int m = tid;
         wait_bar(d_full, 0);
         tc_fence_after();
         unsigned char* stg = gbase + S::OFF_STG;
-        for (int c0 = 0; c0 < NR; c0 += 32) {
+        for (int c0 = 0; c0 < n && m0 < a.rows && !gave_up; c0 += 32) {
             float v[32];
             tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
             if (DUAL) {
                 float u[32];
-                tmem_ld32(tmem + NR + ((uint32_t)(warp * 32) << 16) + c0, u);
+                tmem_ld32(tmem + 256 + ((uint32_t)(warp * 32) << 16) + c0, u);
                 // h for 32 activation rows x this neuron -> staging [row][128 neurons] bf16, then 16-byte stores
                 named_barrier(1, 128);
                 // in stages over the 32 values, so that the exponentials and divisions of different rows overlap
@@ -265,13 +273,13 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
                 named_barrier(1, 128);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int e = m + 128 * i;                     // 512 chunks of 16 bytes: row e / 16, chunk e % 16
-                    const int t = e >> 4, ch = e & 15;
-                    const uint4 q = reinterpret_cast<const uint4*>(stg)[e];
+                    const int e2 = m + 128 * i;                    // 512 chunks of 16 bytes: row e2 / 16, chunk e2 % 16
+                    const int t = e2 >> 4, ch = e2 & 15;
+                    const uint4 q = reinterpret_cast<const uint4*>(stg)[e2];
                     *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = q;
                 }
             } else {
-                float* dst = a.yp + ((size_t)blockIdx.y * a.r_pad + c0) * a.H + m0 + m;
+                float* dst = a.yp + ((size_t)blockIdx.y * n + c0) * a.H + m0 + m;
 #pragma unroll
                 for (int t = 0; t < 32; ++t) dst[(size_t)t * a.H] = v[t];
             }
@@ -280,7 +288,8 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
     }
     tc_fence_before();
     if (__syncthreads_or(gave_up)) linger_after_timeout();
-    if (warp == 5) tmem_dealloc(tmem, S::TMEM_COLS);
+    cluster_sync();                        // neither CTA leaves while the other may signal it or read its shared memory
+    if (warp == 5) tmem_dealloc_pair(tmem, TMEM_COLS);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -314,71 +323,71 @@ int make_map(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uin
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-template <int NR>
-int run_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, const __nv_bfloat16* xc, __nv_bfloat16* h1,
-            float* yp, int ksplit, cudaStream_t s) {
-    const int H = ctx->g.H, I = ctx->g.I;
-    using SA = SmemCtx<NR, true>;
-    using SB = SmemCtx<NR, false>;
+template <bool DUAL>
+int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap& t0, const CUtensorMap& t1, const CUtensorMap& tb, cudaStream_t s) {
+    using S = SmemCtx<DUAL>;
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, SA::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<NR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SA::TOTAL));
-        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<NR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SB::TOTAL));
-        configured.set(ctx->device, SA::TOTAL);
+    if (!configured.covers(ctx->device, S::TOTAL)) {
+        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+        configured.set(ctx->device, S::TOTAL);
     }
-    CUtensorMap tg, tu, tx, td, th;
-    int rc;
-    if ((rc = make_map(&tg, Wg, I, H, 128)) != RM_OK) return rc;
-    if ((rc = make_map(&tu, Wu, I, H, 128)) != RM_OK) return rc;
-    if ((rc = make_map(&tx, xc, NR, H, NR)) != RM_OK) return rc;
-    if ((rc = make_map(&td, Wd, H, I, 128)) != RM_OK) return rc;
-    if ((rc = make_map(&th, h1, NR, I, NR)) != RM_OK) return rc;
-    cudaLaunchAttribute at[1];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(CT);
+    cfg.dynamicSmemBytes = S::TOTAL;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    CtxGemmArgs a{};
-    a.I = I; a.H = H; a.r_pad = NR; a.h1 = h1; a.yp = yp; a.status = ctx->d_status;
-    {
-        a.kblocks = H / 64;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(I / 128);
-        cfg.blockDim = dim3(CT);
-        cfg.dynamicSmemBytes = SA::TOTAL;
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_gemm_kernel<NR, true>, a, tg, tu, tx));
-        ctx->launches++;
-    }
-    {
-        a.kblocks = I / 64 / ksplit;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(H / 128, ksplit);
-        cfg.blockDim = dim3(CT);
-        cfg.dynamicSmemBytes = SB::TOTAL;
-        cfg.stream = s;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_gemm_kernel<NR, false>, a, td, td, th));
-        ctx->launches++;
-    }
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 2;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_gemm_kernel<DUAL>, a, t0, t1, tb));
+    ctx->launches++;
     return RM_OK;
 }
 
-// K slices of the second product: as many as keep about one CTA per SM, dividing the 64-wide K blocks evenly
+// weight maps: one set per call, whatever the number of passes
+struct FfnMaps { CUtensorMap g, u, d; };
+
+int run_ffn(rm_ctx* ctx, const FfnMaps& w, const __nv_bfloat16* xc, __nv_bfloat16* h1, float* yp, int n, int ksplit, cudaStream_t s) {
+    const int H = ctx->g.H, I = ctx->g.I;
+    CUtensorMap tx, th;
+    int rc;
+    if ((rc = make_map(&tx, xc, n, H, n / 2)) != RM_OK) return rc;
+    if ((rc = make_map(&th, h1, n, I, n / 2)) != RM_OK) return rc;
+    CtxGemmArgs a{};
+    a.n = n; a.I = I; a.H = H; a.h1 = h1; a.yp = yp; a.status = ctx->d_status;
+    a.kblocks = H / 64;
+    a.rows = I;
+    if ((rc = launch_gemm<true>(ctx, a, dim3((I / 128 + 1) / 2 * 2), w.g, w.u, tx, s)) != RM_OK) return rc;
+    a.kblocks = I / 64;
+    a.rows = H;
+    return launch_gemm<false>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s);
+}
+
+// K slices of the second product: as many as keep about one CTA per SM (at least two K blocks each)
 int pick_ksplit(const rm_ctx* ctx) {
-    const int col_blocks = ctx->g.H / 128, kblocks = ctx->g.I / 64;
-    int best = 1;
-    for (int ks = 1; ks <= 32; ++ks)
-        if (kblocks % ks == 0 && col_blocks * ks <= (ctx->sm_count > 0 ? ctx->sm_count : 148)) best = ks;
-    return best;
+    const int cols = (ctx->g.H / 128 + 1) / 2 * 2, kblocks = ctx->g.I / 64;
+    int ks = (ctx->sm_count > 0 ? ctx->sm_count : 148) / cols;
+    if (ks > kblocks / 2) ks = kblocks / 2;
+    return ks < 1 ? 1 : (ks > 32 ? 32 : ks);
+}
+// A capacity of more than 256 rows takes several passes over the weights, of equal size (multiples of 32)
+int pass_rows(int cap) {
+    const int passes = (cap + 255) / 256;
+    return ((cap + passes - 1) / passes + 31) / 32 * 32;
 }
 
 }  // namespace
 
 bool rm_context_supported(const rm_ctx* ctx) { return ctx->g.H % 128 == 0 && ctx->g.I % 128 == 0; }
 
-size_t rm_context_workspace_bytes_impl(const rm_ctx* ctx, int r_pad) {
+size_t rm_context_workspace_bytes_impl(const rm_ctx* ctx, int cap) {
+    const int r_pad = pass_rows(cap);
     const size_t xc = align_up((size_t)r_pad * ctx->g.H * sizeof(__nv_bfloat16), 1024);
     const size_t h1 = align_up((size_t)r_pad * ctx->g.I * sizeof(__nv_bfloat16), 1024);
     const size_t yp = align_up((size_t)pick_ksplit(ctx) * r_pad * ctx->g.H * sizeof(float), 1024);
@@ -401,11 +410,14 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    // Up to 256 rows go through the products at once; a longer sequence takes further passes over the weights (the
-    // paper's own setting, 40 % of 768 visual rows plus 48 others = 356 rows, takes two).
-    for (int q_lo = 0; q_lo < cap; q_lo += 256) {
-        const int left = cap - q_lo;
-        const int r_pad = left <= 64 ? 64 : (left <= 128 ? 128 : 256);
+    const int r_pad = pass_rows(cap);
+    if (cap <= 256) cap = r_pad;           // (one pass: whatever it holds)
+    FfnMaps maps;
+    int rc;
+    if ((rc = make_map(&maps.g, Wg, I, H, 128)) != RM_OK) return rc;
+    if ((rc = make_map(&maps.u, Wu, I, H, 128)) != RM_OK) return rc;
+    if ((rc = make_map(&maps.d, Wd, H, I, 128)) != RM_OK) return rc;
+    for (int q_lo = 0; q_lo < cap; q_lo += r_pad) {
         char* w = static_cast<char*>(ws);
         __nv_bfloat16* xc = reinterpret_cast<__nv_bfloat16*>(w);
         w += align_up((size_t)r_pad * H * sizeof(__nv_bfloat16), 1024);
@@ -423,11 +435,7 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
                                            q_lo, cap, xc, ctx->d_status));
             ctx->launches++;
         }
-        int rc = RM_ERR_SHAPE;
-        if (r_pad == 64) rc = run_ffn<64>(ctx, Wg, Wu, Wd, xc, h1, yp, ksplit, s);
-        else if (r_pad == 128) rc = run_ffn<128>(ctx, Wg, Wu, Wd, xc, h1, yp, ksplit, s);
-        else if (r_pad == 256) rc = run_ffn<256>(ctx, Wg, Wu, Wd, xc, h1, yp, ksplit, s);
-        if (rc != RM_OK) return rc;
+        if ((rc = run_ffn(ctx, maps, xc, h1, yp, r_pad, ksplit, s)) != RM_OK) return rc;
         {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(r_pad + (q_lo == 0 ? P : 0));      // the first pass also copies the kept reference rows

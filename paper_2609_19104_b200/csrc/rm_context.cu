@@ -5,14 +5,19 @@
 // is a pair of dense contractions at the ridge of the roofline, so it runs on the tensor cores with every operand
 // block arriving as one cp.async.bulk.tensor box:
 //   gather  : Xc[r,:] = x[rows[r],:]                                   (R_pad rows, zero beyond the list)
-//   phase A : H1[r, n] = bf16(gelu_tanh(<Xc_r, Wg_n>) * <Xc_r, Wu_n>)  one CTA per 128 neurons, K = H
-//   phase B : Yp[s][r, c] = sum over the s-th slice of n of H1[r, n] Wd[c, n]   one CTA per (128 columns, K slice)
-//   scatter : y_out = y_ref, then y_out[rows[r], :] = sum_s Yp[s][r, :]
+//   phase A : H1[r, n] = bf16(gelu_tanh(<Xc_r, Wg_n>) * <Xc_r, Wu_n>)  one CTA per <= 128 neurons, K = H
+//   phase B : y_out[rows[r], c] += sum over the s-th slice of n of H1[r, n] Wd[c, n]   one CTA per (128 columns, K slice)
+// (phase A's idle warps clear the output rows of the list and copy the kept reference rows)
 // Both products are D[256 x N] (+)= A[256 x 64] B[N x 64]^T per stage, by pairs of CTAs (cta_group::2): A = weight rows (K
 // contiguous, as the model stores them), 128 per CTA; B = activation rows, half of them in each CTA; fp32 accumulators in tensor
 // memory (phase A holds two, gate and up: all 512 columns at N = 256).  What bounds a product is what an SM can take in, ~30
 // bytes per clock: a pair halves the activations each CTA loads (48 instead of 64 KB a stage in phase A, 32 instead of 48 in
-// phase B).  Activation rows are padded to a multiple of 32.  @MEASURED@
+// phase B).  Activation rows are padded to a multiple of 32; a CTA of phase A has as many neurons as spread
+// them over all SMs (112 instead of 128 at H = 2048, I = 16384); phase B adds its K slices to the output through the copy
+// engine.  Drift, selection and recomputation of 240 of 816 rows at H = 2048, I = 16384 (us a pass): single CTAs and a kernel
+// summing the slices 78.9, pairs 71.9, without that kernel and on all SMs 67.7 (96 rows 60.5, 366 rows 114).  Of that the
+// products take 31 + ~8 for filling and draining the pipelines; fetching further weight blocks into L2 ahead of time (while phase
+// A waits for its rows, or for phase B) made it 0.4 - 2 us slower.
 #include <cuda.h>
 
 #include <mutex>
@@ -26,25 +31,37 @@ namespace {
 
 constexpr int CT = 192;                // threads: epilogue warps 0-3, loader warp 4 (one lane), issuer warp 5 (one lane)
 
+constexpr int ROW_CHUNK = 8;           // 16-byte loads of a row that a lane has in flight (drift, gather: latency is all they cost)
+
 // ---------------------------------------------------------------- Eq. 2: one warp per row
 __global__ void __launch_bounds__(256) drift_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ xr,
                                                     int P, int H, float* __restrict__ score) {
     pdl_launch_dependents();               // the selection kernel behind this one may set up
+    pdl_wait();
     const int p = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (p >= P) return;
     const uint4* a = reinterpret_cast<const uint4*>(x + (size_t)p * H);
     const uint4* b = reinterpret_cast<const uint4*>(xr + (size_t)p * H);
     float sd = 0.f, sx = 0.f;
-    for (int e = lane; e < H / 8; e += 32) {
-        const uint4 ua = a[e], ub = b[e];
-        const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&ua);
-        const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&ub);
+    for (int e0 = lane; e0 < H / 8; e0 += 32 * ROW_CHUNK) {
+        uint4 ua[ROW_CHUNK], ub[ROW_CHUNK];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 fa = __bfloat1622float2(pa[i]), fb = __bfloat1622float2(pb[i]);
-            const float d0 = fa.x - fb.x, d1 = fa.y - fb.y;
-            sd = fmaf(d0, d0, sd); sd = fmaf(d1, d1, sd);
-            sx = fmaf(fa.x, fa.x, sx); sx = fmaf(fa.y, fa.y, sx);
+        for (int c = 0; c < ROW_CHUNK; ++c) {
+            const int e = e0 + 32 * c;
+            ua[c] = ub[c] = make_uint4(0, 0, 0, 0);
+            if (e < H / 8) { ua[c] = a[e]; ub[c] = b[e]; }
+        }
+#pragma unroll
+        for (int c = 0; c < ROW_CHUNK; ++c) {
+            const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&ua[c]);
+            const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&ub[c]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 fa = __bfloat1622float2(pa[i]), fb = __bfloat1622float2(pb[i]);
+                const float d0 = fa.x - fb.x, d1 = fa.y - fb.y;
+                sd = fmaf(d0, d0, sd); sd = fmaf(d1, d1, sd);
+                sx = fmaf(fa.x, fa.x, sx); sx = fmaf(fa.y, fa.y, sx);
+            }
         }
     }
 #pragma unroll
@@ -86,53 +103,30 @@ __global__ void __launch_bounds__(256) ctx_gather_kernel(const __nv_bfloat16* __
     }
     uint4* d = reinterpret_cast<uint4*>(xc + (size_t)r * H);
     const uint4* s = src >= 0 ? reinterpret_cast<const uint4*>(x + (size_t)src * H) : nullptr;
-    for (int e = lane; e < H / 8; e += 32) d[e] = s ? s[e] : make_uint4(0, 0, 0, 0);
+    for (int e0 = lane; e0 < H / 8; e0 += 32 * ROW_CHUNK) {
+        uint4 v[ROW_CHUNK];
+#pragma unroll
+        for (int c = 0; c < ROW_CHUNK; ++c) v[c] = s && e0 + 32 * c < H / 8 ? s[e0 + 32 * c] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int c = 0; c < ROW_CHUNK; ++c)
+            if (e0 + 32 * c < H / 8) d[e0 + 32 * c] = v[c];
+    }
 }
 
-// ---------------------------------------------------------------- scatter: recomputed rows and kept reference rows
-// CTAs 0 .. r_pad-1: output row of recomputed row r = sum of the K slices.  CTAs r_pad .. r_pad+P-1: visual row p keeps
-// its reference output unless it is in the (ascending) list.
-__global__ void __launch_bounds__(256) ctx_scatter_kernel(const float* __restrict__ yp, int ksplit, int r_pad,
-                                                          const int32_t* __restrict__ rows, const int32_t* __restrict__ count,
-                                                          int P, int S, int H, int q_lo, int cap, const float* __restrict__ y_ref,
-                                                          float* __restrict__ y_out) {
-    pdl_wait();                            // the partial products come from the kernel in front
-    bool bad;
-    const int c = ctx_count(count, P, S, cap, &bad);
-    if ((int)blockIdx.x >= r_pad) {       // (the first pass of a call only: its grid alone has these CTAs)
-        const int p = (int)blockIdx.x - r_pad;
-        if (y_out == y_ref) return;
-        int lo = 0, hi = c;                // is p in rows[0 .. c)?
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (rows[mid] < p) lo = mid + 1; else hi = mid;
-        }
-        if (lo < c && rows[lo] == p) return;
-        for (int e = threadIdx.x; e < H / 4; e += blockDim.x)
-            reinterpret_cast<float4*>(y_out + (size_t)p * H)[e] = reinterpret_cast<const float4*>(y_ref + (size_t)p * H)[e];
-        return;
-    }
-    const int r = blockIdx.x, q = q_lo + r;
-    int dst = -1;
+// The output row of recomputed row q of the sequence (-1: none).  A listed row must be a visual row: the gather zeroed another
+// and recorded the error; adding to it would spoil the always-recomputed row of the same number.
+__device__ __forceinline__ int out_row(const int32_t* rows, int q, int c, int P, int S) {
     if (q < c) {
-        dst = rows[q];
-        if (dst >= P) dst = -1;            // a listed row must be a visual row: the gather zeroed it and recorded the error;
-                                           // writing it would race with the always-recomputed row of the same number
-    } else if (q < c + S) dst = P + (q - c);
-    if (dst < 0 || dst >= P + S) return;
-    for (int e = threadIdx.x; e < H / 4; e += blockDim.x) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s = 0; s < ksplit; ++s) {
-            const float4 v = reinterpret_cast<const float4*>(yp + ((size_t)s * r_pad + r) * H)[e];
-            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-        }
-        reinterpret_cast<float4*>(y_out + (size_t)dst * H)[e] = acc;
+        const int d = rows[q];
+        return d >= 0 && d < P ? d : -1;
     }
+    return q < c + S ? P + (q - c) : -1;
 }
 
 // ---------------------------------------------------------------- the two products
 // DUAL (phase A): A0 = Wg rows, A1 = Wu rows of this CTA's 128 neurons over all K = H; epilogue GeLU*u -> bf16 H1.
-// !DUAL (phase B): A0 = Wd rows of this CTA's 128 output columns over its K slice; epilogue fp32 partial -> Yp.
+// !DUAL (phase B): A0 = Wd rows of this CTA's 128 output columns over its K slice; the fp32 sums are added to the output rows
+// by the copy engine (512 bytes per row), which phase A's idle warps have cleared; they copy the kept reference rows as well.
 template <bool DUAL>
 struct SmemCtx {
     static constexpr int A_BYTES = 128 * 128;                      // 128 rows x 64 bf16
@@ -147,9 +141,14 @@ struct CtxGemmArgs {
     int kblocks;                       // 64-wide K blocks of the whole product (phase B: cut evenly over gridDim.y)
     int n;                             // activation rows: a multiple of 32, at most 256
     int rows;                          // weight rows (neurons or output columns)
+    int mr;                            // weight rows per CTA: a multiple of 8, at most 128
     int I, H;
     __nv_bfloat16* h1;                 // phase A output [n, I]
-    float* yp;                         // phase B output [gridDim.y, n, H]
+    const int32_t* list;               // visual rows to recompute, their number
+    const int32_t* count;
+    int P, S, q_lo, cap;               // this pass has the rows q_lo <= q < q_lo + n of the sequence
+    const float* y_ref;
+    float* y_out;
     int* status;
 };
 
@@ -193,14 +192,14 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
         }
     };
     // this CTA's block of A rows and its K range
-    const int m0 = (int)blockIdx.x * 128;
+    const int m0 = (int)blockIdx.x * a.mr;
     const int kb0 = DUAL ? 0 : a.kblocks * (int)blockIdx.y / (int)gridDim.y;
     const int kbn = (DUAL ? a.kblocks : a.kblocks * ((int)blockIdx.y + 1) / (int)gridDim.y) - kb0;
 
     if (warp == 4 && lane == 0) {
         // ---- loader: the weights do not depend on the previous kernel, the activations do
         const int half = n / 2;
-        const uint32_t bytes = 2u * ((DUAL ? 2u : 1u) * S::A_BYTES + (uint32_t)half * 128u);
+        const uint32_t bytes = 2u * ((DUAL ? 2u : 1u) * (uint32_t)a.mr + (uint32_t)half) * 128u;
         auto weights = [&](int kb, int s) {
             const uint32_t st = base + s * S::STAGE, fb = map_to_rank(full(s), 0);
             if (rank == 0) mbar_arrive_expect_tx(full(s), bytes);
@@ -250,6 +249,33 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
     } else if (warp < 4) {
         // ---- epilogue: lane = A row (neuron or output column), registers = activation rows
         const int m = tid;
+        pdl_wait();
+        bool bad;
+        const int c = ctx_count(a.count, a.P, a.S, a.cap, &bad);
+        if (DUAL) {
+            // output rows of this pass start from zero; in the first pass the visual rows that are not in the (ascending) list
+            // keep their reference output
+            const int n_copy = a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0;
+            for (int i = blockIdx.x; i < n + n_copy; i += gridDim.x) {
+                int dst = -1;
+                const float4* from = nullptr;
+                if (i < n) {
+                    dst = out_row(a.list, a.q_lo + i, c, a.P, a.S);
+                } else {
+                    const int p = i - n;
+                    int lo = 0, hi = c;                            // is p in list[0 .. c)?
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (a.list[mid] < p) lo = mid + 1; else hi = mid;
+                    }
+                    if (!(lo < c && a.list[lo] == p)) { dst = p; from = reinterpret_cast<const float4*>(a.y_ref + (size_t)p * a.H); }
+                }
+                if (dst < 0) continue;
+                float4* to = reinterpret_cast<float4*>(a.y_out + (size_t)dst * a.H);
+#pragma unroll 4
+                for (int e = m; e < a.H / 4; e += 128) to[e] = from ? from[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
         wait_bar(d_full, 0);
         tc_fence_after();
         unsigned char* stg = gbase + S::OFF_STG;
@@ -275,16 +301,27 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
                 for (int i = 0; i < 4; ++i) {
                     const int e2 = m + 128 * i;                    // 512 chunks of 16 bytes: row e2 / 16, chunk e2 % 16
                     const int t = e2 >> 4, ch = e2 & 15;
-                    const uint4 q = reinterpret_cast<const uint4*>(stg)[e2];
-                    *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = q;
+                    if (ch * 8 >= a.mr || m0 + ch * 8 >= a.rows) continue;
+                    *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = reinterpret_cast<const uint4*>(stg)[e2];
                 }
             } else {
-                float* dst = a.yp + ((size_t)blockIdx.y * n + c0) * a.H + m0 + m;
+                // the ring is free (every product has completed): [row][128 columns]
+                float* out = reinterpret_cast<float*>(gbase) + c0 * 128 + m;
 #pragma unroll
-                for (int t = 0; t < 32; ++t) dst[(size_t)t * a.H] = v[t];
+                for (int t = 0; t < 32; ++t) out[t * 128] = v[t];
             }
         }
         tc_fence_before();
+        if (!DUAL) {
+            fence_proxy_async_smem();
+            named_barrier(1, 128);
+            for (int r = m; r < n && m0 < a.rows && !gave_up; r += 128) {
+                const int dst = out_row(a.list, a.q_lo + r, c, a.P, a.S);
+                if (dst >= 0) bulk_reduce_add_f32(a.y_out + (size_t)dst * a.H + m0, base + r * 512, 512);
+            }
+            bulk_commit();
+            bulk_wait_read_all();
+        }
     }
     tc_fence_before();
     if (__syncthreads_or(gave_up)) linger_after_timeout();
@@ -353,19 +390,28 @@ int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap&
 // weight maps: one set per call, whatever the number of passes
 struct FfnMaps { CUtensorMap g, u, d; };
 
-int run_ffn(rm_ctx* ctx, const FfnMaps& w, const __nv_bfloat16* xc, __nv_bfloat16* h1, float* yp, int n, int ksplit, cudaStream_t s) {
+// Neurons per CTA of the first product: as few as spread them over all SMs (2048/16384: 112 on 148 SMs instead of 128 on 128)
+int neurons_per_cta(const rm_ctx* ctx) {
+    const int ctas = ctx->sm_count >= 2 ? ctx->sm_count / 2 * 2 : 148;
+    const int mr = ((ctx->g.I + ctas - 1) / ctas + 7) / 8 * 8;
+    return mr > 128 ? 128 : mr;
+}
+
+// `a`: the list and the output
+int run_ffn(rm_ctx* ctx, const FfnMaps& w, const __nv_bfloat16* xc, __nv_bfloat16* h1, int n, int ksplit, CtxGemmArgs a, cudaStream_t s) {
     const int H = ctx->g.H, I = ctx->g.I;
     CUtensorMap tx, th;
     int rc;
     if ((rc = make_map(&tx, xc, n, H, n / 2)) != RM_OK) return rc;
     if ((rc = make_map(&th, h1, n, I, n / 2)) != RM_OK) return rc;
-    CtxGemmArgs a{};
-    a.n = n; a.I = I; a.H = H; a.h1 = h1; a.yp = yp; a.status = ctx->d_status;
+    a.n = n; a.I = I; a.H = H; a.h1 = h1; a.status = ctx->d_status;
     a.kblocks = H / 64;
     a.rows = I;
-    if ((rc = launch_gemm<true>(ctx, a, dim3((I / 128 + 1) / 2 * 2), w.g, w.u, tx, s)) != RM_OK) return rc;
+    a.mr = neurons_per_cta(ctx);
+    if ((rc = launch_gemm<true>(ctx, a, dim3(((I + a.mr - 1) / a.mr + 1) / 2 * 2), w.g, w.u, tx, s)) != RM_OK) return rc;
     a.kblocks = I / 64;
     a.rows = H;
+    a.mr = 128;
     return launch_gemm<false>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s);
 }
 
@@ -390,15 +436,22 @@ size_t rm_context_workspace_bytes_impl(const rm_ctx* ctx, int cap) {
     const int r_pad = pass_rows(cap);
     const size_t xc = align_up((size_t)r_pad * ctx->g.H * sizeof(__nv_bfloat16), 1024);
     const size_t h1 = align_up((size_t)r_pad * ctx->g.I * sizeof(__nv_bfloat16), 1024);
-    const size_t yp = align_up((size_t)pick_ksplit(ctx) * r_pad * ctx->g.H * sizeof(float), 1024);
-    return xc + h1 + yp;
+    return xc + h1;
 }
 
 int rm_launch_context_drift(rm_ctx* ctx, const void* x, const void* x_ref, int P, float* score, cudaStream_t s) {
-    drift_kernel<<<(P + 7) / 8, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x_ref), P,
-                                            ctx->g.H, score);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((P + 7) / 8);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, drift_kernel, static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x_ref),
+                                   P, ctx->g.H, score));
     ctx->launches++;
-    RM_CUDA_TRY(cudaGetLastError());
     return RM_OK;
 }
 
@@ -414,16 +467,14 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
     if (cap <= 256) cap = r_pad;           // (one pass: whatever it holds)
     FfnMaps maps;
     int rc;
-    if ((rc = make_map(&maps.g, Wg, I, H, 128)) != RM_OK) return rc;
-    if ((rc = make_map(&maps.u, Wu, I, H, 128)) != RM_OK) return rc;
+    if ((rc = make_map(&maps.g, Wg, I, H, neurons_per_cta(ctx))) != RM_OK) return rc;
+    if ((rc = make_map(&maps.u, Wu, I, H, neurons_per_cta(ctx))) != RM_OK) return rc;
     if ((rc = make_map(&maps.d, Wd, H, I, 128)) != RM_OK) return rc;
     for (int q_lo = 0; q_lo < cap; q_lo += r_pad) {
         char* w = static_cast<char*>(ws);
         __nv_bfloat16* xc = reinterpret_cast<__nv_bfloat16*>(w);
         w += align_up((size_t)r_pad * H * sizeof(__nv_bfloat16), 1024);
         __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(w);
-        w += align_up((size_t)r_pad * I * sizeof(__nv_bfloat16), 1024);
-        float* yp = reinterpret_cast<float*>(w);
         {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((r_pad + 7) / 8);
@@ -435,18 +486,13 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
                                            q_lo, cap, xc, ctx->d_status));
             ctx->launches++;
         }
-        if ((rc = run_ffn(ctx, maps, xc, h1, yp, r_pad, ksplit, s)) != RM_OK) return rc;
-        {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(r_pad + (q_lo == 0 ? P : 0));      // the first pass also copies the kept reference rows
-            cfg.blockDim = dim3(256);
-            cfg.stream = s;
-            cfg.attrs = at;
-            cfg.numAttrs = 1;
-            RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_scatter_kernel, static_cast<const float*>(yp), ksplit, r_pad, rows, count, P, S, H,
-                                           q_lo, cap, y_ref, y_out));
-            ctx->launches++;
-        }
+        CtxGemmArgs a{};
+        a.list = rows;
+        a.count = count;
+        a.P = P; a.S = S; a.q_lo = q_lo; a.cap = cap;
+        a.y_ref = y_ref;
+        a.y_out = y_out;
+        if ((rc = run_ffn(ctx, maps, xc, h1, r_pad, ksplit, a, s)) != RM_OK) return rc;
     }
     return RM_OK;
 }

@@ -29,7 +29,7 @@ using namespace sm100;
 
 namespace {
 
-constexpr int CT = 192;                // threads: epilogue warps 0-3, loader warp 4 (one lane), issuer warp 5 (one lane)
+constexpr int EPI = 256, CT = EPI + 64;  // threads: epilogue warps 0-7, loader warp 8 (one lane), issuer warp 9 (one lane)
 
 constexpr int ROW_CHUNK = 8;           // 16-byte loads of a row that a lane has in flight (drift, gather: latency is all they cost)
 
@@ -123,6 +123,19 @@ __device__ __forceinline__ int out_row(const int32_t* rows, int q, int c, int P,
     return q < c + S ? P + (q - c) : -1;
 }
 
+// Is p in the ascending list?  By a whole warp: lane j looks at the last entry of the j-th of 32 parts, then the lanes share the
+// part that can hold p (two dependent loads for up to 1024 entries; a binary search by one lane takes ten).
+__device__ __forceinline__ bool listed(const int32_t* list, int c, int p, int lane) {
+    const int per = (c + 31) / 32;
+    int last = lane * per + per - 1;
+    if (last >= c) last = c - 1;
+    const unsigned below = __ballot_sync(0xffffffffu, c > 0 && list[last] < p);       // parts wholly below p: the first few
+    const int lo = __popc(below) * per;
+    bool hit = false;
+    for (int e = lo + lane; e < lo + per && e < c; e += 32) hit |= list[e] == p;
+    return __any_sync(0xffffffffu, hit);
+}
+
 // ---------------------------------------------------------------- the two products
 // DUAL (phase A): A0 = Wg rows, A1 = Wu rows of this CTA's 128 neurons over all K = H; epilogue GeLU*u -> bf16 H1.
 // !DUAL (phase B): A0 = Wd rows of this CTA's 128 output columns over its K slice; the fp32 sums are added to the output rows
@@ -132,8 +145,7 @@ struct SmemCtx {
     static constexpr int A_BYTES = 128 * 128;                      // 128 rows x 64 bf16
     static constexpr int STAGE = (DUAL ? 3 : 2) * A_BYTES;         // the last part: up to 128 activation rows x 64 bf16
     static constexpr int NSTAGE = DUAL ? 4 : 6;
-    static constexpr int OFF_STG = NSTAGE * STAGE;                 // epilogue staging: 32 rows x 256 bytes
-    static constexpr int OFF_BAR = OFF_STG + 8192;
+    static constexpr int OFF_BAR = NSTAGE * STAGE;                 // (the epilogue stages its results in the ring)
     static constexpr int TOTAL = OFF_BAR + 256 + 1024;
 };
 
@@ -155,7 +167,8 @@ struct CtxGemmArgs {
 #define wait_bar(bar, parity) wait_bar_at((bar), (parity), __LINE__)
 
 template <bool DUAL>
-__global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, const __grid_constant__ CUtensorMap tmA0,
+// (at most 96 registers: a CTA of phase A starts beside one of the selection kernel)
+__global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, const __grid_constant__ CUtensorMap tmA0,
                                                          const __grid_constant__ CUtensorMap tmA1,
                                                          const __grid_constant__ CUtensorMap tmB) {
     using S = SmemCtx<DUAL>;
@@ -176,7 +189,7 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
         mbar_init(d_full, 1);
         fence_mbar_init();
     }
-    if (warp == 5) tmem_alloc_pair(s_tmem, TMEM_COLS);
+    if (warp == EPI / 32 + 1) tmem_alloc_pair(s_tmem, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     cluster_sync();                        // the other CTA's barriers and tensor memory are there
@@ -196,7 +209,7 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
     const int kb0 = DUAL ? 0 : a.kblocks * (int)blockIdx.y / (int)gridDim.y;
     const int kbn = (DUAL ? a.kblocks : a.kblocks * ((int)blockIdx.y + 1) / (int)gridDim.y) - kb0;
 
-    if (warp == 4 && lane == 0) {
+    if (warp == EPI / 32 && lane == 0) {
         // ---- loader: the weights do not depend on the previous kernel, the activations do
         const int half = n / 2;
         const uint32_t bytes = 2u * ((DUAL ? 2u : 1u) * (uint32_t)a.mr + (uint32_t)half) * 128u;
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
             weights(kb, s);
             rows(kb, s);
         }
-    } else if (warp == 5 && rank == 0) {
+    } else if (warp == EPI / 32 + 1 && rank == 0) {
         // ---- issuer: the whole warp runs the loop, one elected lane issues; the next stage's barrier is tested behind the
         // current stage's products
         const uint32_t idesc = idesc_bf16_f32(256, n, false, false);
@@ -246,57 +259,61 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
             __syncwarp();
             ok = __all_sync(0xffffffffu, mbar_test_wait(full((kb + 1) % NSTAGE), ((kb + 1) / NSTAGE) & 1));
         }
-    } else if (warp < 4) {
-        // ---- epilogue: lane = A row (neuron or output column), registers = activation rows
-        const int m = tid;
+    } else if (warp < EPI / 32) {
+        // ---- epilogue: lane = A row (neuron or output column), registers = 32 activation rows; warps 0-3 and 4-7 take turns
+        const int m = tid & 127, group = tid >> 7;
         pdl_wait();
         bool bad;
         const int c = ctx_count(a.count, a.P, a.S, a.cap, &bad);
+        int dst = -1;                      // phase B: the output row that this thread adds
         if (DUAL) {
-            // output rows of this pass start from zero; in the first pass the visual rows that are not in the (ascending) list
-            // keep their reference output
-            const int n_copy = a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0;
-            for (int i = blockIdx.x; i < n + n_copy; i += gridDim.x) {
-                int dst = -1;
+            // a warp per row: output rows of this pass start from zero; in the first pass the visual rows that are not in the
+            // (ascending) list keep their reference output
+            const int rows = n + (a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0);
+            for (int i = blockIdx.x + warp * (int)gridDim.x; i < rows; i += (EPI / 32) * (int)gridDim.x) {
                 const float4* from = nullptr;
+                int to_row = -1;
                 if (i < n) {
-                    dst = out_row(a.list, a.q_lo + i, c, a.P, a.S);
-                } else {
-                    const int p = i - n;
-                    int lo = 0, hi = c;                            // is p in list[0 .. c)?
-                    while (lo < hi) {
-                        const int mid = (lo + hi) >> 1;
-                        if (a.list[mid] < p) lo = mid + 1; else hi = mid;
-                    }
-                    if (!(lo < c && a.list[lo] == p)) { dst = p; from = reinterpret_cast<const float4*>(a.y_ref + (size_t)p * a.H); }
+                    to_row = out_row(a.list, a.q_lo + i, c, a.P, a.S);
+                } else if (!listed(a.list, c, i - n, lane)) {
+                    to_row = i - n;
+                    from = reinterpret_cast<const float4*>(a.y_ref + (size_t)to_row * a.H);
                 }
-                if (dst < 0) continue;
-                float4* to = reinterpret_cast<float4*>(a.y_out + (size_t)dst * a.H);
+                if (to_row < 0) continue;
+                float4* to = reinterpret_cast<float4*>(a.y_out + (size_t)to_row * a.H);
 #pragma unroll 4
-                for (int e = m; e < a.H / 4; e += 128) to[e] = from ? from[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = lane; e < a.H / 4; e += 32) to[e] = from ? from[e] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
+        } else if (tid < n) {
+            dst = out_row(a.list, a.q_lo + tid, c, a.P, a.S);
         }
         wait_bar(d_full, 0);
         tc_fence_after();
-        unsigned char* stg = gbase + S::OFF_STG;
-        for (int c0 = 0; c0 < n && m0 < a.rows && !gave_up; c0 += 32) {
+        // the ring is free: every product that reads it, the other CTA's included, is complete
+        for (int c0 = group * 32; c0 < n && m0 < a.rows && !gave_up; c0 += 64) {
             float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + c0, v);
+            tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0, v);
             if (DUAL) {
                 float u[32];
-                tmem_ld32(tmem + 256 + ((uint32_t)(warp * 32) << 16) + c0, u);
+                tmem_ld32(tmem + 256 + ((uint32_t)((warp & 3) * 32) << 16) + c0, u);
                 // h for 32 activation rows x this neuron -> staging [row][128 neurons] bf16, then 16-byte stores
-                named_barrier(1, 128);
-                // in stages over the 32 values, so that the exponentials and divisions of different rows overlap
-                // (one warp per scheduler runs this; a value-by-value chain costs ~140 clocks per value)
-                float e[32];
+                // in stages over 16 values, so that the exponentials and divisions of different rows overlap
+                // (a value-by-value chain costs ~140 clocks per value)
+                unsigned char* stg = gbase + c0 * 256;
 #pragma unroll
-                for (int t = 0; t < 32; ++t) e[t] = __expf(-1.5957691216057308f * (v[t] + 0.044715f * v[t] * v[t] * v[t]));
+                for (int t0 = 0; t0 < 32; t0 += 16) {
+                    float e[16];
 #pragma unroll
-                for (int t = 0; t < 32; ++t) e[t] = __fdividef(v[t], 1.0f + e[t]) * u[t];
+                    for (int t = 0; t < 16; ++t) {
+                        const float g = v[t0 + t];
+                        e[t] = __expf(-1.5957691216057308f * (g + 0.044715f * g * g * g));
+                    }
 #pragma unroll
-                for (int t = 0; t < 32; ++t) reinterpret_cast<__nv_bfloat16*>(stg)[t * 128 + m] = __float2bfloat16_rn(e[t]);
-                named_barrier(1, 128);
+                    for (int t = 0; t < 16; ++t) e[t] = __fdividef(v[t0 + t], 1.0f + e[t]) * u[t0 + t];
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) reinterpret_cast<__nv_bfloat16*>(stg)[(t0 + t) * 128 + m] = __float2bfloat16_rn(e[t]);
+                }
+                if (group) named_barrier(2, 128); else named_barrier(1, 128);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int e2 = m + 128 * i;                    // 512 chunks of 16 bytes: row e2 / 16, chunk e2 % 16
@@ -305,8 +322,7 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
                     *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = reinterpret_cast<const uint4*>(stg)[e2];
                 }
             } else {
-                // the ring is free (every product has completed): [row][128 columns]
-                float* out = reinterpret_cast<float*>(gbase) + c0 * 128 + m;
+                float* out = reinterpret_cast<float*>(gbase) + c0 * 128 + m;       // [row][128 columns]
 #pragma unroll
                 for (int t = 0; t < 32; ++t) out[t * 128] = v[t];
             }
@@ -314,11 +330,8 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
         tc_fence_before();
         if (!DUAL) {
             fence_proxy_async_smem();
-            named_barrier(1, 128);
-            for (int r = m; r < n && m0 < a.rows && !gave_up; r += 128) {
-                const int dst = out_row(a.list, a.q_lo + r, c, a.P, a.S);
-                if (dst >= 0) bulk_reduce_add_f32(a.y_out + (size_t)dst * a.H + m0, base + r * 512, 512);
-            }
+            named_barrier(1, EPI);
+            if (dst >= 0 && m0 < a.rows && !gave_up) bulk_reduce_add_f32(a.y_out + (size_t)dst * a.H + m0, base + tid * 512, 512);
             bulk_commit();
             bulk_wait_read_all();
         }
@@ -326,7 +339,7 @@ __global__ void __launch_bounds__(CT, 1) ctx_gemm_kernel(const CtxGemmArgs a, co
     tc_fence_before();
     if (__syncthreads_or(gave_up)) linger_after_timeout();
     cluster_sync();                        // neither CTA leaves while the other may signal it or read its shared memory
-    if (warp == 5) tmem_dealloc_pair(tmem, TMEM_COLS);
+    if (warp == EPI / 32 + 1) tmem_dealloc_pair(tmem, TMEM_COLS);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,

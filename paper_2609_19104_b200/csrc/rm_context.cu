@@ -14,10 +14,16 @@
 // bytes per clock: a pair halves the activations each CTA loads (48 instead of 64 KB a stage in phase A, 32 instead of 48 in
 // phase B).  Activation rows are padded to a multiple of 32; a CTA of phase A has as many neurons as spread
 // them over all SMs (112 instead of 128 at H = 2048, I = 16384); phase B adds its K slices to the output through the copy
-// engine.  Drift, selection and recomputation of 240 of 816 rows at H = 2048, I = 16384 (us a pass): single CTAs and a kernel
-// summing the slices 78.9, pairs 71.9, without that kernel and on all SMs 67.7 (96 rows 60.5, 366 rows 114).  Of that the
-// products take 31 + ~8 for filling and draining the pipelines; fetching further weight blocks into L2 ahead of time (while phase
-// A waits for its rows, or for phase B) made it 0.4 - 2 us slower.
+// engine.
+//
+// Drift, selection and recomputation of 240 of 816 rows at H = 2048, I = 16384 (us a pass): single CTAs and a kernel summing the
+// slices 78.9, pairs 71.9, without that kernel and on all SMs 67.7, eight epilogue warps and a warp per copied row 63.9 (96 rows
+// 61.5 -> 56, 366 rows 122 -> 110).  In time: drift 4 - 6, selection 6, gather 3, phase A 22 and its epilogue 4 (two
+// MUFU operations per value), 3 to the next kernel, phase B 10, its additions 4 (an SM's copy engine adds ~16 bytes per clock;
+// red.global.add.v4 from the threads instead: +5).  The products take in 30 bytes per clock and SM and run at the rate of HBM,
+// so that fetching further weights into L2 ahead of time (while phase A waits for its rows, or for phase B) does not help
+// (0.4 - 2 us slower).  Both phases in one kernel would save the 3 us between them, but its CTAs would wait on one another, and
+// a call has to run beside whatever else is on the device.
 #include <cuda.h>
 
 #include <mutex>
@@ -137,11 +143,17 @@ __device__ __forceinline__ bool listed(const int32_t* list, int c, int p, int la
 }
 
 // ---------------------------------------------------------------- the two products
-// DUAL (phase A): A0 = Wg rows, A1 = Wu rows of this CTA's 128 neurons over all K = H; epilogue GeLU*u -> bf16 H1.
-// !DUAL (phase B): A0 = Wd rows of this CTA's 128 output columns over its K slice; the fp32 sums are added to the output rows
+// Phase A: Wg rows and Wu rows of this CTA's neurons over all K = H; epilogue GeLU*u -> bf16 H1.
+//   WIDE     up to 128 neurons: one tile of Wg rows, one of Wu rows, an accumulator for each
+//   PACKED   up to 64 neurons: Wg rows in the upper half of one tile, Wu rows in the lower one, one accumulator; half the
+//            products of WIDE, whose tiles would be half empty (H = 1024, I = 4096, 32 neurons per CTA, 240 rows: the products
+//            alone took 8 us of phase A's 11)
+// Phase B (DOWN): Wd rows of this CTA's 128 output columns over its K slice; the fp32 sums are added to the output rows
 // by the copy engine (512 bytes per row), which phase A's idle warps have cleared; they copy the kept reference rows as well.
-template <bool DUAL>
+enum { DOWN = 0, WIDE = 1, PACKED = 2 };
+template <int MODE>
 struct SmemCtx {
+    static constexpr bool DUAL = MODE == WIDE;
     static constexpr int A_BYTES = 128 * 128;                      // 128 rows x 64 bf16
     static constexpr int STAGE = (DUAL ? 3 : 2) * A_BYTES;         // the last part: up to 128 activation rows x 64 bf16
     static constexpr int NSTAGE = DUAL ? 4 : 6;
@@ -166,12 +178,13 @@ struct CtxGemmArgs {
 
 #define wait_bar(bar, parity) wait_bar_at((bar), (parity), __LINE__)
 
-template <bool DUAL>
+template <int MODE>
 // (at most 96 registers: a CTA of phase A starts beside one of the selection kernel)
 __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, const __grid_constant__ CUtensorMap tmA0,
                                                          const __grid_constant__ CUtensorMap tmA1,
                                                          const __grid_constant__ CUtensorMap tmB) {
-    using S = SmemCtx<DUAL>;
+    using S = SmemCtx<MODE>;
+    constexpr bool DUAL = S::DUAL, GATED = MODE != DOWN;
     constexpr int NSTAGE = S::NSTAGE, OFF_B = (DUAL ? 2 : 1) * S::A_BYTES, TMEM_COLS = DUAL ? 512 : 256;
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
@@ -206,18 +219,18 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
     };
     // this CTA's block of A rows and its K range
     const int m0 = (int)blockIdx.x * a.mr;
-    const int kb0 = DUAL ? 0 : a.kblocks * (int)blockIdx.y / (int)gridDim.y;
-    const int kbn = (DUAL ? a.kblocks : a.kblocks * ((int)blockIdx.y + 1) / (int)gridDim.y) - kb0;
+    const int kb0 = GATED ? 0 : a.kblocks * (int)blockIdx.y / (int)gridDim.y;
+    const int kbn = (GATED ? a.kblocks : a.kblocks * ((int)blockIdx.y + 1) / (int)gridDim.y) - kb0;
 
     if (warp == EPI / 32 && lane == 0) {
         // ---- loader: the weights do not depend on the previous kernel, the activations do
         const int half = n / 2;
-        const uint32_t bytes = 2u * ((DUAL ? 2u : 1u) * (uint32_t)a.mr + (uint32_t)half) * 128u;
+        const uint32_t bytes = 2u * ((GATED ? 2u : 1u) * (uint32_t)a.mr + (uint32_t)half) * 128u;
         auto weights = [&](int kb, int s) {
             const uint32_t st = base + s * S::STAGE, fb = map_to_rank(full(s), 0);
             if (rank == 0) mbar_arrive_expect_tx(full(s), bytes);
             tma_load_2d_pair(st, &tmA0, (kb0 + kb) * 64, m0, fb);
-            if (DUAL) tma_load_2d_pair(st + S::A_BYTES, &tmA1, (kb0 + kb) * 64, m0, fb);
+            if (GATED) tma_load_2d_pair(st + (DUAL ? S::A_BYTES : S::A_BYTES / 2), &tmA1, (kb0 + kb) * 64, m0, fb);
         };
         auto rows = [&](int kb, int s) {
             tma_load_2d_pair(base + s * S::STAGE + OFF_B, &tmB, (kb0 + kb) * 64, rank * half, map_to_rank(full(s), 0));
@@ -266,7 +279,7 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
         bool bad;
         const int c = ctx_count(a.count, a.P, a.S, a.cap, &bad);
         int dst = -1;                      // phase B: the output row that this thread adds
-        if (DUAL) {
+        if (GATED) {
             // a warp per row: output rows of this pass start from zero; in the first pass the visual rows that are not in the
             // (ascending) list keep their reference output
             const int rows = n + (a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0);
@@ -293,7 +306,7 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
         for (int c0 = group * 32; c0 < n && m0 < a.rows && !gave_up; c0 += 64) {
             float v[32];
             tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0, v);
-            if (DUAL) {
+            if constexpr (DUAL) {
                 float u[32];
                 tmem_ld32(tmem + 256 + ((uint32_t)((warp & 3) * 32) << 16) + c0, u);
                 // h for 32 activation rows x this neuron -> staging [row][128 neurons] bf16, then 16-byte stores
@@ -321,6 +334,35 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
                     if (ch * 8 >= a.mr || m0 + ch * 8 >= a.rows) continue;
                     *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = reinterpret_cast<const uint4*>(stg)[e2];
                 }
+            } else if constexpr (MODE == PACKED) {
+                // the gate's lanes compute the first 16 rows, the up product's lanes the others: each hands over its half
+                float* xch = reinterpret_cast<float*>(gbase + (c0 >> 5) * 12288);              // [32][64]
+                __nv_bfloat16* stg = reinterpret_cast<__nv_bfloat16*>(xch + 32 * 64);          // [32][64]
+                const int mine = (warp & 2) * 8, nu = m & 63;
+#pragma unroll
+                for (int t = 0; t < 16; ++t) xch[((mine ^ 16) + t) * 64 + nu] = mine ? v[t] : v[16 + t];
+                if (group) named_barrier(2, 128); else named_barrier(1, 128);
+                if (nu < a.mr) {
+                    float e[16], g[16], u[16];
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) {
+                        const float other = xch[(mine + t) * 64 + nu];
+                        g[t] = mine ? other : v[t];
+                        u[t] = mine ? v[16 + t] : other;
+                    }
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) e[t] = __expf(-1.5957691216057308f * (g[t] + 0.044715f * g[t] * g[t] * g[t]));
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) stg[(mine + t) * 64 + nu] = __float2bfloat16_rn(__fdividef(g[t], 1.0f + e[t]) * u[t]);
+                }
+                if (group) named_barrier(2, 128); else named_barrier(1, 128);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int e2 = m + 128 * i;                    // 256 chunks of 16 bytes: row e2 / 8, chunk e2 % 8
+                    const int t = e2 >> 3, ch = e2 & 7;
+                    if (ch * 8 >= a.mr || m0 + ch * 8 >= a.rows) continue;
+                    *reinterpret_cast<uint4*>(a.h1 + (size_t)(c0 + t) * a.I + m0 + ch * 8) = reinterpret_cast<const uint4*>(stg)[e2];
+                }
             } else {
                 float* out = reinterpret_cast<float*>(gbase) + c0 * 128 + m;       // [row][128 columns]
 #pragma unroll
@@ -328,7 +370,7 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
             }
         }
         tc_fence_before();
-        if (!DUAL) {
+        if (!GATED) {
             fence_proxy_async_smem();
             named_barrier(1, EPI);
             if (dst >= 0 && m0 < a.rows && !gave_up) bulk_reduce_add_f32(a.y_out + (size_t)dst * a.H + m0, base + tid * 512, 512);
@@ -373,12 +415,12 @@ int make_map(CUtensorMap* tm, const void* ptr, uint64_t rows, uint64_t cols, uin
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-template <bool DUAL>
+template <int MODE>
 int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap& t0, const CUtensorMap& t1, const CUtensorMap& tb, cudaStream_t s) {
-    using S = SmemCtx<DUAL>;
+    using S = SmemCtx<MODE>;
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, S::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
         configured.set(ctx->device, S::TOTAL);
     }
     cudaLaunchConfig_t cfg = {};
@@ -395,7 +437,7 @@ int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap&
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_gemm_kernel<DUAL>, a, t0, t1, tb));
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_gemm_kernel<MODE>, a, t0, t1, tb));
     ctx->launches++;
     return RM_OK;
 }
@@ -421,11 +463,13 @@ int run_ffn(rm_ctx* ctx, const FfnMaps& w, const __nv_bfloat16* xc, __nv_bfloat1
     a.kblocks = H / 64;
     a.rows = I;
     a.mr = neurons_per_cta(ctx);
-    if ((rc = launch_gemm<true>(ctx, a, dim3(((I + a.mr - 1) / a.mr + 1) / 2 * 2), w.g, w.u, tx, s)) != RM_OK) return rc;
+    const dim3 grid_a(((I + a.mr - 1) / a.mr + 1) / 2 * 2);
+    rc = a.mr <= 64 ? launch_gemm<PACKED>(ctx, a, grid_a, w.g, w.u, tx, s) : launch_gemm<WIDE>(ctx, a, grid_a, w.g, w.u, tx, s);
+    if (rc != RM_OK) return rc;
     a.kblocks = I / 64;
     a.rows = H;
     a.mr = 128;
-    return launch_gemm<false>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s);
+    return launch_gemm<DOWN>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s);
 }
 
 // K slices of the second product: as many as keep about one CTA per SM (at least two K blocks each)

@@ -54,6 +54,18 @@ def test_context_cache_matches_the_oracle(lib, H, I, P, S, rho, R_max):
     run_case(lib, H, I, P, S, rho, R_max)
 
 
+@pytest.mark.parametrize("I", [
+    128,                                  # 8 neurons per CTA
+    9472,                                 # 64 per CTA: the most whose gate and up rows share one tile
+    9600,                                 # 72: a tile each, the last CTA's ragged
+    18944,                                # 128: full tiles on all SMs
+    19072,                                # more CTAs than SMs
+])
+@pytest.mark.parametrize("H,P,S,rho,R_max", [(128, 70, 7, 0.4, 36), (384, 310, 20, 0.9, 320)])
+def test_neurons_per_cta(lib, I, H, P, S, rho, R_max):
+    run_case(lib, H, I, P, S, rho, R_max)
+
+
 def test_context_cache_paper_shape(lib):
     # the VLM's FFN: H = 2048, I = 16384, 768 visual rows + 48 others, a quarter of the visual rows recomputed
     run_case(lib, 2048, 16384, 768, 48, 0.25, 256)

@@ -180,11 +180,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
     volatile int* sAbort = &sAbortW;
 
     // ---- set-up
-    if (blockIdx.x == 0) {                 // the launch's counters, then (below) its epoch
-        for (int e = tid; e < a.B * CS * 2; e += NTHREADS) a.ctrl[CTRL_LINE * (1 + e)] = 0;
-        if (tid == 0) { a.ctrl[2] = 0; a.ctrl[3] = 0; }
-        __threadfence();
-    }
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) { mbar_init(g_full(s), 1); mbar_init(g_empty(s), 2); mbar_init(d_full(s), 1); mbar_init(d_empty(s), 8); }
         mbar_init(p_full(0), 1); mbar_init(p_full(1), 1); mbar_init(h_full, 1); mbar_init(h_free, CS * 8);
@@ -192,6 +187,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         fence_mbar_init();
         *sAbort = 0;
         sSeen = 0;
+    }
+    // x rows past T, columns past Hs, and weight slots that no copy has filled yet have to hold finite numbers: zeros
+    for (int e = tid; e < 64 * LY(xp) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_x))[e] = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = tid; e < (LY(off_item) - LY(off_g)) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_g))[e] = make_uint4(0u, 0u, 0u, 0u);
+    pdl_wait();                            // (a dependent launch: nothing above depends on the kernel in front)
+    if (blockIdx.x == 0) {                 // the launch's counters, then (below) its epoch
+        for (int e = tid; e < a.B * CS * 2; e += NTHREADS) a.ctrl[CTRL_LINE * (1 + e)] = 0;
+        if (tid == 0) { a.ctrl[2] = 0; a.ctrl[3] = 0; }
+        __threadfence();
     }
     {
         // counts, then this cluster's part of every item.  The lists of a layer's episodes, laid end to end, are cut evenly
@@ -243,9 +247,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
             }
         }
     }
-    // x rows past T, columns past Hs, and weight slots that no copy has filled yet have to hold finite numbers: zeros
-    for (int e = tid; e < 64 * LY(xp) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_x))[e] = make_uint4(0u, 0u, 0u, 0u);
-    for (int e = tid; e < (LY(off_item) - LY(off_g)) / 16; e += NTHREADS) reinterpret_cast<uint4*>(gbase + LY(off_g))[e] = make_uint4(0u, 0u, 0u, 0u);
     fence_proxy_async_smem();
     __syncthreads();
     cluster_sync();                        // peers' shared memory and barriers are live from here on
@@ -745,8 +746,11 @@ int query(int* out) {
 template <int HS, int NG, int TS, bool EQ4>
 int launch(rm_ctx* ctx, const SArgs& a, int clusters, int smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cluster_config(cfg, at, clusters, smem, s);
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, slice_kernel<HS, NG, TS, EQ4>, a));
     ctx->launches++;
     return RM_OK;

@@ -106,11 +106,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
     const int rot = c % (KB / kps);
     const int n_add = a.S * NSL;                                   // CTAs that add (S <= U: every split has units)
 
-    if (c == 0) {
-        for (int e = tid; e < C_H + 8 * G; e += NTHREADS)
-            if (e >= 2) a.ctrl[e] = 0;
-        __threadfence();
-    }
     if (tid == 0) {
         for (int s = 0; s < NWS; ++s) { mbar_init(w_full(s), 1); mbar_init(w_empty(s), 1); }
         for (int s = 0; s < NAS; ++s) { mbar_init(a_full(s), 1); mbar_init(a_empty(s), 1); }
@@ -124,7 +119,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
     tc_fence_after();
     const uint32_t tmem = *g_tmem;
     pdl_launch_dependents();               // (a dependent waits for this grid's end)
-    if (c == 0 && tid == 0) epoch_publish(a.ctrl, a.epoch);
+    if (warp != 8) pdl_wait();             // (a dependent launch itself: the first weights need nothing from the kernel in front)
+    if (c == 0 && warp < 8) {
+        for (int e = tid; e < C_H + 8 * G; e += 256)
+            if (e >= 2) a.ctrl[e] = 0;
+        __threadfence();
+        named_barrier(1, 256);
+        if (tid == 0) epoch_publish(a.ctrl, a.epoch);
+    }
 
     bool gave_up = false;
     auto wait_at = [&](uint32_t bar, uint32_t parity, int line) {
@@ -159,6 +161,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     dst = lane * 8192;
                     bytes = 8192u * NCB;
                 }
+                if (pass == 1 && ws == 0) pdl_wait();
                 if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
                 gave_up = __any_sync(0xffffffffu, gave_up);
                 if (gave_up) break;
@@ -493,6 +496,11 @@ int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s
     cfg.blockDim = dim3(NTHREADS);
     cfg.dynamicSmemBytes = SMEM;
     cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<HS, EQ4>, a, maps));
     ctx->launches++;
     return RM_OK;

@@ -326,7 +326,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
         // y accumulates the CTAs' partial sums with atomics: start it from the residual (or zero)
         // (a kernel of its own, so that the layer's CTAs can set up and gather their first weights while it runs)
         if (y != residual) {
-            const int rc = rm_launch_copy(ctx, y, residual, (size_t)T * ctx->g.H, false, s);
+            const int rc = rm_launch_copy(ctx, y, residual, nullptr, (size_t)T * ctx->g.H, s);
             if (rc != RM_OK) return rc;
         }
         if (use_persist(ctx, 1, T, count_dev != nullptr, false)) {
@@ -353,7 +353,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
         }
         if (use_stream(ctx, count_dev != nullptr, 1, T)) {
             ctx->last_variant = 4;
-            return rm_launch_layer_stream(ctx, a, nullptr, false, s);
+            return rm_launch_layer_stream(ctx, a, nullptr, y == residual, s);
         }
         return rm_launch_layer_fused(ctx, a, nullptr, false, ctx->use_pdl && y != residual, s);
     }
@@ -428,8 +428,9 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     const bool stream = fused && use_stream(ctx, count_dev != nullptr, B, T, an.mode == RM_ANCHOR_WRITE);
     const bool direct_out = fused && r_out != r_in;
     if (fused && !stream) {
-        RM_CUDA_TRY(cudaMemsetAsync(g.L == 1 && direct_out ? r_out : rot[1], 0, n_bytes, s));
-        if (direct_out && g.L > 1) RM_CUDA_TRY(cudaMemsetAsync(r_out, 0, n_bytes, s));
+        const int rc = rm_launch_copy(ctx, g.L == 1 && direct_out ? r_out : rot[1], nullptr, direct_out && g.L > 1 ? r_out : nullptr,
+                                      n_bytes / sizeof(float), s);
+        if (rc != RM_OK) return rc;
     }
     // the anchor step's outputs are accumulated by the CTAs' atomics: start them from zero
     if (fused && an.mode == RM_ANCHOR_WRITE)
@@ -461,7 +462,7 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
             const bool last = l == g.L - 1;
             a.r_out = (last && direct_out) ? r_out : rot[l & 1];
             ctx->last_variant = 4;
-            rc = rm_launch_layer_stream(ctx, a, reinterpret_cast<__nv_bfloat16*>(layer_ws), ctx->use_pdl && l > 0, s);
+            rc = rm_launch_layer_stream(ctx, a, reinterpret_cast<__nv_bfloat16*>(layer_ws), l == 0, s);
             cur = a.r_out;
         } else if (fused) {
             const bool last = l == g.L - 1;
@@ -469,7 +470,7 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
             // the buffer cleared here is the output of layer l+1 (unless that layer writes to r_out directly); it
             // was the input of layer l-1, which has completed by the time this layer passes its dependency wait
             float* zero = (l + 1 < g.L && !(l + 1 == g.L - 1 && direct_out)) ? rot[(l + 2) % 3] : nullptr;
-            rc = rm_launch_layer_fused(ctx, a, zero, true, ctx->use_pdl && l > 0, s);
+            rc = rm_launch_layer_fused(ctx, a, zero, true, ctx->use_pdl && (l > 0 || an.mode != RM_ANCHOR_WRITE), s);
             cur = a.r_out;
         } else {
             a.r_out = r_out;                               // in place after the first layer
@@ -571,7 +572,7 @@ int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, co
     const float* in_dev = static_cast<const float*>(pinned_device_pointer(r_in_host, n_bytes));
     float* out_dev = static_cast<float*>(pinned_device_pointer(r_out_host, n_bytes));
     if (in_dev) {
-        const int rc = rm_launch_copy(ctx, stage, in_dev, n_bytes / sizeof(float), false, s);
+        const int rc = rm_launch_copy(ctx, stage, in_dev, nullptr, n_bytes / sizeof(float), s);
         if (rc != RM_OK) return rc;
     } else {
         RM_CUDA_TRY(cudaMemcpyAsync(stage, r_in_host, n_bytes, cudaMemcpyHostToDevice, s));
@@ -579,7 +580,7 @@ int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, co
     int rc = step_device(ctx, packed_layers, stage, idx, count_dev, stride, stage, nullptr, nullptr, B, T, ws, s);
     if (rc != RM_OK) return rc;
     if (out_dev) {
-        rc = rm_launch_copy(ctx, out_dev, stage, n_bytes / sizeof(float), ctx->use_pdl != 0, s);
+        rc = rm_launch_copy(ctx, out_dev, stage, nullptr, n_bytes / sizeof(float), s);
         if (rc != RM_OK) return rc;
     } else {
         RM_CUDA_TRY(cudaMemcpyAsync(r_out_host, stage, n_bytes, cudaMemcpyDeviceToHost, s));

@@ -104,7 +104,7 @@ __device__ __forceinline__ float rm_gelu_tanh(float g) {
 // ---- kernels implemented in the other translation units (host launchers)
 int rm_launch_pack(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, void* packed, float* colnorm,
                    cudaStream_t s);
-int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, size_t n, bool pdl, cudaStream_t s);
+int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, float* clear, size_t n, cudaStream_t s);
 int rm_launch_gather_rows(rm_ctx* ctx, const void* packed, const int32_t* idx, const int32_t* count, int64_t cap,
                           void* out, cudaStream_t s);
 // Context Cache (row-sparse dense FFN on the tensor cores)
@@ -156,7 +156,7 @@ int rm_launch_layer_ref(rm_ctx* ctx, const rm_layer_args& a, void* ws, cudaStrea
 int rm_stream_init(rm_ctx* ctx);
 bool rm_stream_supported(const rm_ctx* ctx, int B, int T);
 int rm_stream_debug_stamps(long long* host_out);
-int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& a, __nv_bfloat16* x_scratch, bool pdl, cudaStream_t s);
+int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& a, __nv_bfloat16* x_scratch, bool first, cudaStream_t s);
 // Whole-step kernel: every layer of a step in one launch.  H in {1024, 2048}, T <= 64, B <= 16, L <= 64, zero-fill form.
 struct rm_step_args {
     const void* const* packed_layers;      // host array of L device pointers

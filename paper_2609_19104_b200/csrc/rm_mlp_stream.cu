@@ -688,7 +688,7 @@ int make_map_out(CUtensorMap* tm, const float* ptr, uint64_t B, uint64_t T, uint
 }
 
 template <int NTOK, int CL>
-int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
+int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, bool dependent, cudaStream_t s) {
     using S = SmemST<NTOK, CL>;
     const bool eq4 = a.anchor_mode != RM_ANCHOR_NONE || a.gate != nullptr;
     const bool gather = a.idx != nullptr;
@@ -725,7 +725,7 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, cudaStream_t s) {
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = CL;
     at[1].val.clusterDim.y = 1;
@@ -801,8 +801,9 @@ bool rm_stream_supported(const rm_ctx* ctx, int B, int T) {
 }
 
 // One layer.  Without la.x: la.r_in is normalised into x_scratch and la.r_out (a different buffer) is set to the
-// residual (+ gate * y_anchor in update steps) before the tiles are added.  With la.x the caller has prepared la.r_out.
-int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* x_scratch, bool pdl, cudaStream_t s) {
+// residual (+ gate * y_anchor in update steps) before the tiles are added.  With la.x the caller has prepared la.r_out.  `first`:
+// no kernel of the same call stands in front (one that let this one in early would also have to wait for what writes the list).
+int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* x_scratch, bool first, cudaStream_t s) {
     const rm_geom& g = ctx->g;
     const __nv_bfloat16* x = la.x;
     if (!x) {
@@ -823,7 +824,7 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = pdl ? 1 : 0;
+        cfg.numAttrs = ctx->use_pdl && !first ? 1 : 0;             // (the tiles read the list before they wait for this grid)
         RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, g.H == 1024 ? stream_prep_kernel<1024> : stream_prep_kernel<2048>, p, rows));
         ctx->launches++;
         x = x_scratch;
@@ -850,6 +851,7 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
     a.h_anchor = la.h_anchor;
     a.h_stride = la.h_stride;
     a.gate = la.gate;
+    const bool dependent = !la.x || !first;                        // a kernel of this call stands in front
     const int per_episode = la.count ? rm_effective_count_hint(ctx) : g.I;
     const long long per = per_episode > 0 ? (per_episode + NT - 1) / NT : 0, tiles = per * la.B;
     int n_ctas = ctx->sm_count;
@@ -861,7 +863,7 @@ int rm_launch_layer_stream(rm_ctx* ctx, const rm_layer_args& la, __nv_bfloat16* 
         int clusters = ctx->stream_pairs;
         if (groups > 0 && groups < clusters) clusters = (int)groups;
         if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < clusters) clusters = ctx->max_clusters_override;
-        return la.T <= 32 ? launch_tiles<32, 2>(ctx, a, 2 * clusters, s) : launch_tiles<64, 2>(ctx, a, 2 * clusters, s);
+        return la.T <= 32 ? launch_tiles<32, 2>(ctx, a, 2 * clusters, dependent, s) : launch_tiles<64, 2>(ctx, a, 2 * clusters, dependent, s);
     }
-    return la.T <= 32 ? launch_tiles<32, 1>(ctx, a, n_ctas, s) : launch_tiles<64, 1>(ctx, a, n_ctas, s);
+    return la.T <= 32 ? launch_tiles<32, 1>(ctx, a, n_ctas, dependent, s) : launch_tiles<64, 1>(ctx, a, n_ctas, dependent, s);
 }

@@ -83,18 +83,23 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4* __restric
 
 // dst = src (src NULL: zeros), n4 float4.  Either side may be pinned host memory: a step's 209 KB (51 x 1024 fp32) cross
 // PCIe in one kernel with every load in flight at once, where the copy engine's start-up and its hand-over to and from
-// the kernel in the same stream cost about 7 us per direction.
-__global__ void __launch_bounds__(256) copy_kernel(float4* dst, const float4* src, size_t n4) {
-    sm100::pdl_launch_dependents();        // a kernel behind this one may set up
-    sm100::pdl_wait();                     // (launched as a dependent: the kernel in front writes src)
-    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256)
+// the kernel in the same stream cost about 7 us per direction.  `clear` (or NULL): a second buffer that starts from zero.
+// A layer kernel behind this one reads its index list and first weights before it waits for this grid.  Those may come from the
+// kernel in front, so the layer kernel is let in only when that one is complete.  (A dependent launch in place of a plain one, or
+// of two memsets: a layer of 1024/4096 14.4 -> 13.2 us, a step of 18 layers of 32 tokens 136 -> 130.)
+__global__ void __launch_bounds__(256) copy_kernel(float4* dst, const float4* src, float4* clear, size_t n4) {
+    sm100::pdl_wait();
+    sm100::pdl_launch_dependents();
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (size_t)gridDim.x * 256) {
         dst[i] = src ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (clear) clear[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 }
 
 }  // namespace
 
 // A multiple of 4 floats, 16-byte aligned on both sides
-int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, size_t n, bool pdl, cudaStream_t s) {
+int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, float* clear, size_t n, cudaStream_t s) {
     const size_t n4 = n / 4, ctas = (n4 + 255) / 256;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(ctas < 592 ? ctas : 592));
@@ -104,8 +109,9 @@ int rm_launch_copy(rm_ctx* ctx, float* dst, const float* src, size_t n, bool pdl
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, copy_kernel, reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n4));
+    cfg.numAttrs = ctx->use_pdl ? 1 : 0;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, copy_kernel, reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src),
+                                   reinterpret_cast<float4*>(clear), n4));
     ctx->launches++;
     return RM_OK;
 }

@@ -39,7 +39,9 @@ KERNEL_FAMILY = {0: "portable CUDA-core kernels (norm, gate/up, down)",
                  2: "fused_layer_kernel, two tiles in flight",
                  3: "fused_layer_ws_kernel (warp-specialised per-layer cluster kernel)",
                  4: "stream_prep_kernel + stream_tile_kernel (per-layer streaming kernel)",
-                 5: "step_kernel (whole step in one launch)"}
+                 5: "step_kernel (whole step in one launch)",
+                 6: "slice_kernel (whole step in one launch, any width, long chunks)",
+                 7: "sweep_kernel (whole dense step in one launch)"}
 
 
 def measured_hbm_peak():

@@ -22,33 +22,48 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
     return ctx->path != 1 && rm_fused_supported(ctx, B, T);
 }
 
-// The whole-step kernel (variant 5).  Chosen by itself where it is measured ahead of the per-layer kernels (single
-// episodes; us per step, cold L2: lean per-layer kernel / streaming kernel / whole-step kernel):
-//   H = 2048, I = 16384:  K =  492: 236 / 572 / 262    820: 265 / 571 / 262    1147: 360 / 571 / 266
-//                         1639: 377 / 577 / 273    3277: 605 / 577 / 308    4916: 829 / 554 / 462
-//                         6882: 1058 / 584 / 532    7373: 1066 / 605 / 544    8192: 1183 / 624 / 652
-//                         9012: 1279 / 665 / 687    9503: 1301 / 1039 / 701    12288: 1632 / 1139 / 871
-//                         14746: 1962 / 1114 / 960    16384 (every neuron listed): 2158 / 1130 / 1081
-//   H = 1024, I = 4096:   K =  820: 176 / 344 / 188    902: 178 / 345 / 190    984: 200 / 343 / 193
-//                         1024: 199 / 345 / 193    1229: 231 / 345 / 195    2048: 270 / 346 / 203    4096: 404 / 337 / 291
-// The streaming kernel's time steps up with every wave of 64-neuron tiles over the SMs (148 tiles per wave), the lean
-// kernel's with every 64-neuron tile beyond 15; the whole-step kernel grows evenly with K and has a fixed cost of
-// ~10-15 us per layer.  So, with K the caller's count hint (the whole layer for a dense pass): at H = 1024 from 23.5 %
-// of the neurons upwards; at H = 2048 from 5 % upwards, except where the streaming kernel's single wave is nearly full
-// (7700 neurons up to 148 tiles).  Without a hint at H = 2048 it is chosen as well (it adapts to the counts on
-// the device), at H = 1024 the lean kernel.  Batches stay with the streaming kernel.  `steps`: a whole stack (false:
-// the one-layer entry, which would pay the kernel's set-up for a single layer).
-inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool steps) {
+// The whole-step kernel (variant 5).  Chosen by itself where it is measured ahead of the per-layer kernels (single episodes).
+// Its time per layer is ~10 us at H = 1024 and ~14 us at H = 2048, with little growth in K or T (chains between CTAs); the
+// lean per-layer kernel's grows with T (tiles of 32 or 64 token columns; T > 55: one CTA per SM) and by a step at every
+// 64-neuron tile that makes a cluster's run longer; the streaming kernel's by a step at every wave of tiles over the SMs.
+// us per step of 6 layers, whole-step / per-layer kernels (s: streaming), by T:
+//   H = 1024  K =  500: 8: 61/42    32: 63/45    52: 65/56    56: 65/63    64: 66/67
+//                  900: 8: 61/44    32: 64/47    52: 65/59    56: 65/71    64: 66/76
+//                 1024: 8: 63/47    32: 66/54    48: 68/68    52: 68/68    64: 69/103
+//                 1280: 8: 64/54    32: 67/59    33: 67/69    52: 69/77    64: 70/109
+//                 1900: 8: 66/64    32: 69/69    33: 69/78    52: 71/86
+//                 2048: 8: 67/66    32: 70/72    33: 71/81    52: 72/90
+//   H = 2048  K =  500: 8: 82/54    32: 88/62    48: 91/77    64: 93/84
+//                  960: 8: 83/65    32: 88/74    48: 91/88    56: 92/93    64: 94/97
+//                 1024: 8: 85/86    32: 90/95    48: 93/110   64: 95/126
+//                 4600: 8: 142/144s 32: 148/152s 51: 153/167s
+//                 4900: 8: 147/143s 32: 154/152s 51: 158/167s
+//                 6100: 8: 158/146s 32: 166/157s 40: 167/168s 64: 171/171s
+//                 6500: 8: 161/146s 32: 170/159s 40: 172/170s 64: 175/173s
+//                 9400: 8: 223/167s 32: 233/198s 64: 238/216s   (10000, beyond a wave of 148 tiles: 225/272s, 239/329s)
+// with the anchor update (Eq. 4), whose sums the streaming kernel is slow at (4600: 148/224s):
+//   H = 1024  K =  600: 8: 66/46    32: 72/50    51: 75/63    60: 76/72    64: 78/76
+//                  900: 8: 68/47    32: 74/52    51: 78/65    60: 79/78    64: 81/83
+//                 1400: 8: 73/59    32: 80/66    40: 82/81    51: 83/86    64: 86/125
+//                 2048: 8: 76/70    32: 83/77    33: 83/90
+//   H = 2048  K =  960: 8: 92/71    32: 104/82   64: 117/112       1100: 8: 93/93   33: 107/112
+// So, in tiles of 64 neurons, with K the caller's count hint (the whole layer for a dense pass): up to the bounds below the
+// layer kernels; from the bounds of H = 2048 up to one wave the streaming kernel.  Without a hint the whole-step kernel at
+// H = 2048 (it adapts to the counts on the device), the lean kernel at H = 1024.  Batches stay with the streaming kernel.
+// `steps`: a whole stack (false: the one-layer entry, which would pay the kernel's set-up for a single layer).
+inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool eq4, bool steps) {
     if (ctx->path == 1 || !rm_persist_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 5) return true;
     if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b || !steps) return false;
-    const long long I = ctx->g.I, K = masked ? rm_effective_count_hint(ctx) : I;
+    const long long K = masked ? rm_effective_count_hint(ctx) : ctx->g.I, tiles = (K + 63) / 64;
+    if (K <= 0) return ctx->g.H == 2048;
     if (ctx->g.H == 2048) {
-        if (K <= 0) return true;
-        if (K * 100 < I * 5) return false;
-        return !(K > 7700 && (K + 63) / 64 <= ctx->sm_count);
+        if (tiles <= (eq4 || T <= 55 ? 15 : 13)) return false;
+        return eq4 || tiles < (T <= 32 ? 77 : 101) || tiles > ctx->sm_count;
     }
-    return K > 0 && K * 1000 >= I * 235;
+    if (T <= 32) return tiles > (eq4 ? 32 : 29);
+    if (rm_fused_two_per_sm(ctx, T)) return tiles > (eq4 ? 20 : T <= 48 ? 16 : 15);
+    return tiles > (eq4 ? 13 : 8);
 }
 
 inline void* persist_ws(const rm_ctx* ctx, void* ws, int B, int T) {
@@ -329,7 +344,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
             const int rc = rm_launch_copy(ctx, y, residual, nullptr, (size_t)T * ctx->g.H, s);
             if (rc != RM_OK) return rc;
         }
-        if (use_persist(ctx, 1, T, count_dev != nullptr, false)) {
+        if (use_persist(ctx, 1, T, count_dev != nullptr, false, false)) {
             // the whole-step kernel on a stack of one layer whose input is the caller's x
             const void* one[1] = {packed_layer};
             rm_step_args sa{};
@@ -375,14 +390,16 @@ struct AnchorIO {                      // whole-stack anchor state (Eq. 4); mode
 static int step_device(rm_ctx* ctx, const void* const* packed_layers, const float* r_in, const int32_t* idx,
                        const int32_t* count_dev, int64_t stride, float* r_out, float* records_out,
                        const float* record_scale, int B, int T, void* ws, cudaStream_t s,
-                       const AnchorIO& an = AnchorIO()) {
+                       const AnchorIO& an = AnchorIO(), const float** result = nullptr) {
+    // `result` (or NULL): where the output is, instead of a copy into r_out when the step runs in place
     const rm_geom& g = ctx->g;
     const size_t n_bytes = (size_t)B * T * g.H * sizeof(float);
     const size_t r_bytes = align_up(n_bytes, 256);
+    if (result) *result = r_out;
     char* layer_ws = static_cast<char*>(ws) + 4 * r_bytes;
     const bool slice = use_slice(ctx, B, T, records_out != nullptr);
     const bool sweep = !slice && use_sweep(ctx, B, T, !idx && !count_dev && an.mode != RM_ANCHOR_UPDATE);
-    if (slice || sweep || use_persist(ctx, B, T, count_dev != nullptr, true)) {
+    if (slice || sweep || use_persist(ctx, B, T, count_dev != nullptr, an.mode != RM_ANCHOR_NONE || an.gate, true)) {
         // the whole step in one launch: the layers add into r_out in place (the kernel starts it as a copy of r_in)
         rm_step_args sa{};
         sa.packed_layers = packed_layers;
@@ -480,7 +497,8 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
         }
         if (rc != RM_OK) return rc;
     }
-    if (fused && !direct_out) RM_CUDA_TRY(cudaMemcpyAsync(r_out, cur, n_bytes, cudaMemcpyDeviceToDevice, s));
+    if (result) *result = cur;
+    else if (fused && !direct_out) return rm_launch_copy(ctx, r_out, cur, nullptr, n_bytes / sizeof(float), s);
     return RM_OK;
 }
 
@@ -577,13 +595,14 @@ int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, co
     } else {
         RM_CUDA_TRY(cudaMemcpyAsync(stage, r_in_host, n_bytes, cudaMemcpyHostToDevice, s));
     }
-    int rc = step_device(ctx, packed_layers, stage, idx, count_dev, stride, stage, nullptr, nullptr, B, T, ws, s);
+    const float* out = nullptr;
+    int rc = step_device(ctx, packed_layers, stage, idx, count_dev, stride, stage, nullptr, nullptr, B, T, ws, s, AnchorIO(), &out);
     if (rc != RM_OK) return rc;
     if (out_dev) {
-        rc = rm_launch_copy(ctx, out_dev, stage, nullptr, n_bytes / sizeof(float), s);
+        rc = rm_launch_copy(ctx, out_dev, out, nullptr, n_bytes / sizeof(float), s);
         if (rc != RM_OK) return rc;
     } else {
-        RM_CUDA_TRY(cudaMemcpyAsync(r_out_host, stage, n_bytes, cudaMemcpyDeviceToHost, s));
+        RM_CUDA_TRY(cudaMemcpyAsync(r_out_host, out, n_bytes, cudaMemcpyDeviceToHost, s));
     }
     RM_CUDA_TRY(cudaStreamSynchronize(s));
     return RM_OK;

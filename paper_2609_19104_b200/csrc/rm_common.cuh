@@ -149,6 +149,7 @@ size_t rm_ref_workspace_bytes(const rm_ctx* ctx, int B, int T);
 int rm_fused_init(rm_ctx* ctx);
 int rm_fused_debug_stamps(long long* host_out, int n);
 bool rm_fused_supported(const rm_ctx* ctx, int B, int T);
+bool rm_fused_two_per_sm(const rm_ctx* ctx, int T);
 int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& a, float* zero_buf, bool add_residual, bool pdl,
                           cudaStream_t s);
 int rm_launch_layer_ref(rm_ctx* ctx, const rm_layer_args& a, void* ws, cudaStream_t s);

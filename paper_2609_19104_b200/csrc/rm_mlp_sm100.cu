@@ -1597,6 +1597,12 @@ bool rm_fused_supported(const rm_ctx* ctx, int B, int T) {
     return (H == 1024 || H == 2048) && T >= 1 && T <= 64 && B >= 1 && B <= MAXB && ctx->fused_clusters > 0;
 }
 
+// H = 1024: the lean kernel fits an SM twice (228 KB of shared memory, of which every resident CTA also takes 1 KB of system space)
+bool rm_fused_two_per_sm(const rm_ctx* ctx, int T) {
+    const int bytes = T <= 32 ? Smem<32, 128, false>::total_bytes(T) : Smem<64, 128, false>::total_bytes(T);
+    return ctx->g.H == 1024 && 2 * (bytes + 1024) <= 228 * 1024;
+}
+
 int rm_fused_init(rm_ctx* ctx) {
     // The occupancy query counts one CTA per SM for kernels that allocate tensor memory; clusters beyond that
     // number simply queue, so it is a sizing hint, not a limit.
@@ -1650,12 +1656,10 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     // co-resident, two more than twice the number the occupancy query reports for one CTA per SM.  H = 2048 (one CTA
     // per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
     // which runs the phases of consecutive tiles concurrently.
-    // (an SM has 228 KB of shared memory, of which every resident CTA also takes 1 KB of system space)
-    const int lean_bytes = la.T <= 32 ? Smem<32, 128, false>::total_bytes(la.T) : Smem<64, 128, false>::total_bytes(la.T);
-    const bool two_per_sm = ctx->g.H == 1024 && 2 * (lean_bytes + 1024) <= 228 * 1024;
+    const bool two_per_sm = rm_fused_two_per_sm(ctx, la.T);
     int cap = two_per_sm ? 2 * ctx->fused_clusters + 2 : ctx->fused_clusters;
     if (ctx->max_clusters_override > 0) cap = ctx->max_clusters_override;
-    int variant = ctx->variant_override >= 5 ? 0 : ctx->variant_override;    // 5: a call the whole-step kernel does not cover
+    int variant = ctx->variant_override >= 5 ? 0 : ctx->variant_override;    // 5 and above: a call that the named kernel does not cover
     if (variant == 0) variant = (ctx->g.H == 1024 || (tiles > 0 && tiles <= cap)) ? 1 : 3;
     if (variant == 3) {
         const int fits_t = ctx->g.H == 1024 ? SmemWS<64, 128>::total_bytes(la.T) : SmemWS<64, 256>::total_bytes(la.T);

@@ -24,7 +24,7 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 
 // The whole-step kernel (variant 5).  Chosen by itself where it is measured ahead of the per-layer kernels (single episodes).
 // Its time per layer is ~10 us at H = 1024 and ~14 us at H = 2048, with little growth in K or T (chains between CTAs); the
-// lean per-layer kernel's grows with T (tiles of 32 or 64 token columns; T > 55: one CTA per SM) and by a step at every
+// lean per-layer kernel's grows with T (tiles of 32 or 64 token columns; T > 52: one CTA per SM) and by a step at every
 // 64-neuron tile that makes a cluster's run longer; the streaming kernel's by a step at every wave of tiles over the SMs.
 // us per step of 6 layers, whole-step / per-layer kernels (s: streaming), by T:
 //   H = 1024  K =  500: 8: 61/42    32: 63/45    52: 65/56    56: 65/63    64: 66/67
@@ -105,14 +105,17 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 // anchor_write: the anchor step of Eq. 4 adds two boxes per block (y_anchor and the output) and stores h_anchor; measured
 // on the anchor schedule it stays behind the cluster kernels at 64 tiles (352 against 334 us per step), so it keeps
 // the threshold of about a tile per SM
-inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, bool anchor_write = false) {
+// Where the lean kernel fits an SM only once (H = 1024, T > 52), its clusters walk two tiles from 17 tiles on: half the threshold
+// (2 episodes of 60 tokens, 3600 neurons, us per 6 layers, lean / streaming: 10 tiles 68 / 101, 18 tiles 114 / 102)
+inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, bool anchor_write = false, bool eq4 = false) {
     if (ctx->path == 1 || !rm_stream_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 4) return true;
     if (ctx->variant_override != 0 && ctx->variant_override != 5 && ctx->variant_override != 7) return false;   // 5, 7: a call the whole-step kernel does not cover
     const int per_episode = masked ? rm_effective_count_hint(ctx) : ctx->g.I;
     if (per_episode <= 0) return false;
     const long long tiles = (long long)((per_episode + 63) / 64) * B;
-    return tiles >= (anchor_write && ctx->stream_min_tiles < 112 ? 112 : ctx->stream_min_tiles);
+    const int least = !eq4 && ctx->g.H == 1024 && !rm_fused_two_per_sm(ctx, T) ? (ctx->stream_min_tiles + 1) / 2 : ctx->stream_min_tiles;
+    return tiles >= (anchor_write && least < 112 ? 112 : least);
 }
 
 }  // namespace
@@ -442,7 +445,8 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     // Fused path: layer l reads rot[l%3] (the caller's r_in for l = 0), accumulates into rot[(l+1)%3] and clears
     // rot[(l+2)%3] for the layer after next; the last layer accumulates straight into r_out when that is a
     // different buffer from r_in.
-    const bool stream = fused && use_stream(ctx, count_dev != nullptr, B, T, an.mode == RM_ANCHOR_WRITE);
+    const bool stream = fused && use_stream(ctx, count_dev != nullptr, B, T, an.mode == RM_ANCHOR_WRITE,
+                                             an.mode != RM_ANCHOR_NONE || an.gate);
     const bool direct_out = fused && r_out != r_in;
     if (fused && !stream) {
         const int rc = rm_launch_copy(ctx, g.L == 1 && direct_out ? r_out : rot[1], nullptr, direct_out && g.L > 1 ? r_out : nullptr,

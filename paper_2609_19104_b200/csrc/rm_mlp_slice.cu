@@ -13,7 +13,7 @@
 //   down    : [tokens] x [the slice's columns], accumulated in registers over the rounds of the item, then added to the
 //             fp32 residual stream with red.global.add
 // A layer's adds go into a buffer of their own (three in turn, cleared one layer ahead); the residual itself is added by
-// the clusters in equal shares of token rows, from the registers in which the row was normalised.  A CTA waits for the
+// the clusters in equal shares of token rows.  A CTA waits for the
 // layer before only on its own slice: counter (episode, slice) counts the clusters that have added their part.
 //
 // Why mma.sync and not tcgen05: with at most 64 token rows the products of a step are small (config of 1024/4096, 25 % of the

@@ -82,6 +82,7 @@ inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
 // The sweep kernel (variant 7): dense steps of one episode, where a cluster of the whole-step kernel would walk more than one
 // tile of 256 neurons per layer.  us per step of 18 layers, 51 tokens, whole-step / sweep: H = 1024, I = 3000: 213 / 248,
 // 3500: 220 / 263, 4096: 282 / 255, 6000: 309 / 279; H = 2048, I = 8000: 540 / 430, 16384: 1085 / 750.
+// The line lies at the same place from 8 to 64 tokens (6 layers, 8 tokens: 3840 72 / 85, 3900 93 / 86).
 inline bool use_sweep(const rm_ctx* ctx, int B, int T, bool dense) {
     if (ctx->path == 1 || !dense || !rm_sweep_supported(ctx, B, T)) return false;
     if (ctx->variant_override != 0) return ctx->variant_override == 7;

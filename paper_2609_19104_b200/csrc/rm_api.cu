@@ -73,7 +73,7 @@ inline void* persist_ws(const rm_ctx* ctx, void* ws, int B, int T) {
 
 // The slice kernel (variant 6): where the tcgen05 kernels do not reach (widths other than 1024 and 2048, chunks of more than
 // 64 tokens), instead of the CUDA-core kernels.  One step of 12 layers of 1536/6144 with 25 % of the neurons and 51 tokens:
-// 244 us against 9360.
+// 272 us against 9335.
 inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
     if (ctx->path == 1 || !rm_slice_supported(ctx, B, T, record)) return false;
     return ctx->variant_override == 6 || (ctx->path == 0 && !rm_fused_supported(ctx, B, T));
@@ -93,10 +93,8 @@ inline void* sweep_ws(const rm_ctx* ctx, void* ws, int B, int T) {
     return reinterpret_cast<void*>(align_up(reinterpret_cast<size_t>(p), 1024));
 }
 
-// the slice kernel's buffers in a workspace of (B, T)
+// the slice kernel's control block and partial sums in a workspace of (B, T)
 inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, int T) {
-    const size_t r_bytes = align_up((size_t)B * T * ctx->g.H * sizeof(float), 256);
-    for (int i = 0; i < 3; ++i) sa.rot[i] = reinterpret_cast<float*>(static_cast<char*>(ws) + i * r_bytes);
     sa.ctrl = reinterpret_cast<int*>(static_cast<char*>(persist_ws(ctx, ws, B, T)) + align_up(rm_persist_workspace_bytes(ctx), 256));
 }
 

@@ -177,8 +177,7 @@ struct rm_step_args {
     float* h_anchor;                       // [L,B,I,h_stride]
     int64_t h_stride;
     const float* gate;                     // [L,B,H] output gate, or NULL
-    float* rot[3];                         // slice kernel: [B,T,H] buffers of the layers in between
-    int* ctrl;                             // slice kernel: control block
+    int* ctrl;                             // slice kernel: control block, then its partial sums
 };
 // Slice kernel: every layer of a step in one launch, any H up to 2048, any T (rm_mlp_slice.cu)
 int rm_slice_init(rm_ctx* ctx);

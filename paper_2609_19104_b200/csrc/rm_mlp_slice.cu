@@ -8,13 +8,20 @@
 //             accumulators in registers)
 //   owner   : tile i of the round belongs to CTA i mod 8.  The partial sums travel to it as bulk copies between the
 //             CTAs' shared memories (laid out in the weight stage that the products have just read), counted on its
-//             mbarrier; it adds the 8 slices' sums, applies gelu_tanh(g) * u, splits h into a bf16 pair hi + lo (relative error
-//             2^-17) and copies its rows to the other CTAs' h tiles
-//   down    : [tokens] x [the slice's columns], accumulated in registers over the rounds of the item, then added to the
-//             fp32 residual stream with red.global.add
-// A layer's adds go into a buffer of their own (three in turn, cleared one layer ahead); the residual itself is added by
-// the clusters in equal shares of token rows.  A CTA waits for the
-// layer before only on its own slice: counter (episode, slice) counts the clusters that have added their part.
+//             mbarrier; it adds the 8 slices' sums, applies gelu_tanh(g) * u, splits h into three bf16 terms (together its 24
+//             bits) and copies its rows to the other CTAs' h tiles
+//   down    : [tokens] x [the slice's columns], accumulated in registers over the rounds of the item, then stored as this
+//             cluster's partial sums
+//   sum     : once every cluster of an item has stored its part, each takes an equal share of the token rows, adds the parts in
+//             the clusters' order and the residual, and writes the rows
+// Nothing is added in the order of arrival, so that a step gives the same bits every time.  A CTA waits for other clusters
+// only on its own slice: counters (episode, slice) count the clusters that have stored their part and those that have
+// written their rows.
+//
+// The sums are as close to 64 bits as those of the CUDA-core kernels, which take the same shapes (fp32 throughout, one order):
+// one layer of 1536/6144, 25 %, 51 tokens, relative error 4.1e-7 against 7.2e-7; 2048/8192, 90 tokens 5.2e-7 against 7.4e-7.  With
+// h in two terms, exponentials and divisions of reduced precision and a chain of products over the whole list it is 2.5e-6.
+// Order and precision cost 13 %: 12 layers of 1536/6144 take 272 us, adding h of 17 bits in the order of arrival 241.
 //
 // Why mma.sync and not tcgen05: with at most 64 token rows the products of a step are small (config of 1024/4096, 25 % of the
 // neurons: 0.4 us of tensor time per layer and product at the 1024 multiply-adds per clock and SM that mma.sync was
@@ -40,19 +47,20 @@ constexpr int CS = 8;                  // CTAs per cluster = column slices of th
 constexpr int TN = 8;                  // neurons of a tile: 8 gate rows and 8 up rows make one 16-row operand
 constexpr int SN = 2 * TN;             // neurons of a weight stage
 constexpr int MAX_ITEMS = 512;         // layers x episodes of one launch
-constexpr int MAXL = 64, MAXB = 64;
+constexpr int MAXL = 64;
 constexpr int NTHREADS = 640;          // warps 0-7: normalisation and gate/up (group A); 8-15: owner, down, adds (group B);
 constexpr int W_B = 8, W_G = 16;       // 16 / 17: loaders of the gate/up and of the down pieces
-constexpr int HPITCH = 272;            // bytes of an h row: 64 tokens hi, 64 tokens lo, 16 to spread the banks
+constexpr int HPITCH = 400;            // bytes of an h row: three terms of 64 tokens, 16 to spread the banks
 constexpr int P_SRC = 4096;            // partial sums of a tile from one CTA: [8-token tile][neuron][token pair] (gate, gate, up, up)
 constexpr int P_SLOT = CS * P_SRC;
 constexpr int SSB = 4;                 // buffers of the row sums of squares: a CTA can be two items ahead of another
 constexpr int MAX_STAGES = 16;
-constexpr int EXACT_STAGES = 7;        // of the 128-column slice
+constexpr int EXACT_STAGES = 6;        // of the 128-column slice
+constexpr int GROUP = 8;               // episodes (chunks) of one launch: a part of every cluster for each is kept in the workspace
 
-// the control block's counters, lines of 32 ints: per (episode, slice) the CTAs that have set up the first output buffer, and the
-// CTAs that have added their part
-__host__ __device__ constexpr int ctrl_init(int e, int j) { return CTRL_LINE * (1 + (e * CS + j) * 2); }
+// the control block's counters, lines of 32 ints: per (episode, slice) the CTAs that have stored their part, and the CTAs that have
+// written their rows (both cumulative over the layers)
+__host__ __device__ constexpr int ctrl_part(int e, int j) { return CTRL_LINE * (1 + (e * CS + j) * 2); }
 __host__ __device__ constexpr int ctrl_done(int e, int j) { return CTRL_LINE * (2 + (e * CS + j) * 2); }
 __host__ __device__ constexpr size_t ctrl_bytes(int B) { return (size_t)CTRL_LINE * (1 + 2 * CS * B) * sizeof(int); }
 
@@ -80,7 +88,7 @@ __host__ __device__ constexpr Lay make_layout(int Hs, int ts, int stages) {
     y.off_g = y.off_h + ts * CS * TN * HPITCH;
     y.off_d = y.off_g + stages * y.g_stage;
     y.off_item = y.off_d + stages * y.d_stage;
-    y.total = y.off_item + MAX_ITEMS * 16 + 128;
+    y.total = y.off_item + MAX_ITEMS * 12 + 128;
     return y;
 }
 
@@ -88,7 +96,7 @@ struct SArgs {
     const __nv_bfloat16* packed[MAXL];
     const float* r_in;                 // [B,T,H] r_0
     float* r_out;                      // [B,T,H] r_L
-    float* rot[3];                     // [B,T,H] outputs of the layers in between, in turn
+    float* part;                       // [B][clusters][T][H]: a layer's partial sums, by episode and share
     const __nv_bfloat16* x_ext;        // [T,H]: the only layer takes this as its input (no normalisation), or NULL
     const int32_t* idx;                // list (b, l) at idx + b * idx_b_stride + l * idx_l_stride; NULL: positions
     const int32_t* count;              // count (b, l) at count[b * count_b_stride + l]; NULL: every neuron
@@ -101,7 +109,8 @@ struct SArgs {
     int* status;
     int L, B, T, I, Hs;
     int nb;                            // episodes of the caller
-    int n_sub;                         // token chunks per episode: "episode" e of the kernel is chunk e % n_sub of e / n_sub
+    int n_sub;                         // token chunks per episode: "episode" e of the kernel is chunk (e0 + e) % n_sub of (e0 + e) / n_sub
+    int e0;                            // first chunk of this launch
     int T_all;                         // tokens per episode of the caller (T: tokens per chunk; the last one may hold fewer)
     int anchor_mode;                   // Eq. 4 (EQ4 instantiation): RM_ANCHOR_*
     float* y_anchor;                   // [L,B,T,H]
@@ -125,18 +134,22 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], 
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void red_add_v2(float* p, float a, float b) {
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
-}
 // (relaxed: it only says that this CTA's reads of a buffer are over; the values have been used by then.  A release at cluster
 // scope waits for every earlier store and add, an acquire at cluster scope empties the L1 cache)
 __device__ __forceinline__ void arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // What a cluster does for one (layer, episode): n neurons of the list from position `start` (0: another cluster's, or an
-// empty list whose residual this cluster passes on), `share` of `parts` of the item's token rows.
-struct Item { int start, n, parts_share, target; };                // parts | share << 8 | takes part << 16; target: arrivals
-                                                                   // on the episode's counter that complete the layer before
+// empty list whose rows this cluster passes on), `share` of `parts` of the item's token rows; `target`: arrivals on the episode's
+// counters that complete the layer before.
+struct Item {
+    int start, n;
+    unsigned bits;                     // parts | share << 8 | takes part << 16 | target << 17
+    __device__ int parts() const { return (int)(bits & 0xffu); }
+    __device__ int share() const { return (int)((bits >> 8) & 0xffu); }
+    __device__ bool mine() const { return (bits >> 16) & 1u; }
+    __device__ int target() const { return (int)(bits >> 17); }
+};
 
 // A cluster's run of n neurons is tiles of 8, cut into rounds of at most `most` tiles, as even as they come: round r of nrd
 // starts at neuron pos and has nr.
@@ -206,13 +219,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         if (it < n_items) {
             int k = a.I;
             if (a.count) {
-                k = a.count[(size_t)(e / a.n_sub) * a.count_b_stride + l];
+                k = a.count[(size_t)((a.e0 + e) / a.n_sub) * a.count_b_stride + l];
                 if (k < 0 || k > cap) { rm_set_status(a.status, RM_ERR_INDEX); k = k < 0 ? 0 : cap; }
             }
             items[it].n = k;
         }
         __syncthreads();
-        Item r{0, 0, 0, 0};
+        Item r{0, 0, 0};
         if (it < n_items) {
             const unsigned K = (unsigned)items[it].n;
             unsigned S = 0, P = 0;
@@ -222,7 +235,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                 P += b2 < e ? K2 : 0u;
             }
             if (K == 0) {
-                r.parts_share = 1 | (e % NC == c ? 1 << 16 : 0);
+                r.bits = 1u | (e % NC == c ? 1u << 16 : 0u);
             } else {
                 int parts = 0, share = 0;
                 for (int k = 0; k < NC; ++k) {
@@ -233,17 +246,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                         ++parts;
                     }
                 }
-                r.parts_share = parts | share << 8 | (r.n > 0 ? 1 << 16 : 0);
+                r.bits = (unsigned)(parts | share << 8 | (r.n > 0 ? 1 << 16 : 0));
             }
         }
         __syncthreads();
         if (it < n_items) items[it] = r;
         __syncthreads();
         if (tid < B) {
-            int t = 0;
+            unsigned t = 0;
             for (int l2 = 0; l2 < a.L; ++l2) {
-                items[l2 * B + tid].target = t;
-                t += items[l2 * B + tid].parts_share & 0xff;
+                Item& q = items[l2 * B + tid];
+                q.bits |= t << 17;
+                t += (unsigned)q.parts();
             }
         }
     }
@@ -268,18 +282,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         gave_up = __any_sync(0xffffffffu, gave_up);
     };
     // first token row (of the caller's [B, T_all]) and tokens of episode e
+    auto episode_of = [&](int e) { return a.n_sub == 1 ? a.e0 + e : (a.e0 + e) / a.n_sub; };
     auto row0_of = [&](int e) {
-        if (a.n_sub == 1) return (size_t)e * a.T;
-        const int b = e / a.n_sub, s = e - b * a.n_sub;
-        return (size_t)b * a.T_all + (size_t)s * a.T;
+        const int b = episode_of(e);
+        return (size_t)b * a.T_all + (size_t)(a.e0 + e - b * a.n_sub) * a.T;
     };
     auto tokens_of = [&](int e) {
         if (a.n_sub == 1) return a.T;
-        const int s = e % a.n_sub, left = a.T_all - s * a.T;
+        const int s = (a.e0 + e) % a.n_sub, left = a.T_all - s * a.T;
         return left < a.T ? left : a.T;
     };
-    auto list_of = [&](int l, int e) { return a.idx ? a.idx + (size_t)(a.n_sub == 1 ? e : e / a.n_sub) * a.idx_b_stride + (size_t)l * a.idx_l_stride : nullptr; };
-    auto out_of = [&](int l) { return l == a.L - 1 ? a.r_out : a.rot[l % 3]; };
+    auto list_of = [&](int l, int e) { return a.idx ? a.idx + (size_t)episode_of(e) * a.idx_b_stride + (size_t)l * a.idx_l_stride : nullptr; };
     const int most = 8 * TS < 2 * NST ? 8 * TS : 2 * NST;          // tiles per round: every one of its stages fits the ring
 
     if (warp >= W_G) {
@@ -341,13 +354,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         uint32_t g_pass = 0;
         for (int it = 0, l = 0, e = 0; it < n_items; ++it, (++e == a.B ? (e = 0, ++l) : 0)) {
             const Item w = items[it];
-            if (!(w.parts_share >> 16)) continue;
+            if (!w.mine()) continue;
             const int Te = tokens_of(e);
-            const float4* src = reinterpret_cast<const float4*>((l == 0 ? a.r_in : out_of(l - 1)) + (row0_of(e) + t) * H + (size_t)j * Hs) + q;
-            // ---- every cluster has added its part of the layer before to this slice (one thread looks)
+            const float4* src = reinterpret_cast<const float4*>((l == 0 ? a.r_in : a.r_out) + (row0_of(e) + t) * H + (size_t)j * Hs) + q;
+            // ---- every row of the layer before has been written in this slice (one thread looks)
             if (tid == 0 && !gave_up) {
                 if (pi == 0) gave_up = epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
-                if (l > 0 && !gave_up) gave_up = counter_wait(a.ctrl + ctrl_done(e, j), w.target, __LINE__, a, sAbort);
+                if (l > 0 && !gave_up) gave_up = counter_wait(a.ctrl + ctrl_done(e, j), w.target(), __LINE__, a, sAbort);
                 asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(&sSeen)), "r"(pi + 1) : "memory");
             }
             ++pi;
@@ -489,18 +502,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
         const int np = (a.T + 7) / 8 * 4;                          // token pairs
         const uint32_t h_lane = base + LY(off_h) + ((lane & 7) + ((lane >> 4) & 1) * 8) * HPITCH + (m0 * 16 + ((lane >> 3) & 1) * 8) * 2;
         const uint32_t d_lane = base + LY(off_d) + ((lane & 7) + ((lane >> 3) & 1) * 8) * LY(dp) + (cp0 * 16 + (lane >> 4) * 8) * 2;
+        const int parts_max = (int)cluster_count_x();
         uint32_t R = 0, p_par = 0, d_pass = 0;
         int d_slot = 0, pi = 0;
         bool stop = false;
-        for (int it = 0, l = 0, e = 0; it < n_items && !stop; ++it, (++e == a.B ? (e = 0, ++l) : 0)) {
-            const Item w = items[it];
-            if (!(w.parts_share >> 16)) continue;
-            const int Te = tokens_of(e), b = a.n_sub == 1 ? e : e / a.n_sub, nb = a.nb;
-            const size_t tok0 = (size_t)(e - b * a.n_sub) * a.T;   // first token of the chunk inside its episode
+        for (int l = 0; l < a.L && !stop; ++l) {
+        for (int e = 0; e < a.B && !stop; ++e) {
+            const Item w = items[l * a.B + e];
+            if (!w.mine()) continue;
+            const int Te = tokens_of(e), b = episode_of(e);
+            const size_t tok0 = (size_t)(a.e0 + e - b * a.n_sub) * a.T;        // first token of the chunk inside its episode
             const int32_t* list = list_of(l, e);
-            // ---- while group A prepares x: this cluster's share of the layer's residual (+ gate * y_a in an update step) and
-            // of the clearing of the next layer's output buffer.  Both need the layer before to be complete, which group A's
-            // first thread has seen.
+            // the layer before is complete (group A's first thread has seen it): what this CTA reads of it and writes over it below
             if (bt == 0 && !gave_up) {
                 int seen = 0;
                 for (uint32_t i = 0; i < (1u << 24); ++i) {
@@ -512,36 +525,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
             ++pi;
             stop = barrier_or(2, 256, gave_up || *sAbort);
             if (stop) break;
-            {
-                const int parts = w.parts_share & 0xff, share = (w.parts_share >> 8) & 0xff, n4 = Hs / 4;
-                const size_t lb = (size_t)l * nb + b, layer = (size_t)nb * a.T_all * H;
-                const float* in = l == 0 ? a.r_in : out_of(l - 1);
-                for (int z = bt; z < (Te - share + parts - 1) / parts * n4; z += 256) {
-                    const int ri = z / n4, k = z - ri * n4;
-                    const size_t o = (row0_of(e) + share + ri * parts) * H + (size_t)j * Hs + 4 * k;
-                    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (in) r = __ldcg(reinterpret_cast<const float4*>(in + o));
-                    if (EQ4 && anchor_mode == RM_ANCHOR_UPDATE) {
-                        const float4 ya = __ldcg(reinterpret_cast<const float4*>(a.y_anchor + l * layer + o));
-                        float4 g = make_float4(1.f, 1.f, 1.f, 1.f);
-                        if (a.gate) g = __ldg(reinterpret_cast<const float4*>(a.gate + lb * H + (size_t)j * Hs) + k);
-                        r.x = fmaf(g.x, ya.x, r.x); r.y = fmaf(g.y, ya.y, r.y); r.z = fmaf(g.z, ya.z, r.z); r.w = fmaf(g.w, ya.w, r.w);
-                    }
-                    float* out = out_of(l) + o;
-                    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (l > 0) red_add_v4(out, r.x, r.y, r.z, r.w);
-                    else if (out != in + o || !a.x_ext) *reinterpret_cast<float4*>(out) = r;
-                    if (l + 1 < a.L) *reinterpret_cast<float4*>(out_of(l + 1) + o) = zero;
-                    if (EQ4 && anchor_mode == RM_ANCHOR_WRITE) {
-                        if (l == 0) *reinterpret_cast<float4*>(a.y_anchor + o) = zero;
-                        if (l + 1 < a.L) *reinterpret_cast<float4*>(a.y_anchor + (l + 1) * layer + o) = zero;
-                    }
-                }
-            }
-            if (l == 0) {                                          // the first layer's output buffer is set up (this CTA's share)
-                stop = barrier_or(2, 256, gave_up || *sAbort);
-                if (bt == 0 && !stop) red_release_gpu(a.ctrl + ctrl_init(e, j), 1);
-            }
             float acc[2][NG][4];
 #pragma unroll
             for (int m = 0; m < 2; ++m)
@@ -570,7 +553,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                         float2 ha = make_float2(0.f, 0.f);
                         float2* hap = nullptr;
                         if (EQ4 && anchor_mode != RM_ANCHOR_NONE && n >= 0 && 2 * lane < Te) {
-                            hap = reinterpret_cast<float2*>(a.h_anchor + (((size_t)l * nb + b) * a.I + n) * a.h_stride + tok0) + lane;
+                            hap = reinterpret_cast<float2*>(a.h_anchor + (((size_t)l * a.nb + b) * a.I + n) * a.h_stride + tok0) + lane;
                             if (anchor_mode == RM_ANCHOR_UPDATE) ha = __ldcg(hap);
                         }
                         WAIT(p_full(s), (p_par >> s) & 1u);
@@ -584,10 +567,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                                 v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
                             }
                             // GeLU-tanh(g) = g / (1 + exp(-2 z)), z = sqrt(2/pi) (g + 0.044715 g^3)
-                            const float e0 = __expf(-1.5957691216057308f * (v.x + 0.044715f * v.x * v.x * v.x));
-                            const float e1 = __expf(-1.5957691216057308f * (v.y + 0.044715f * v.y * v.y * v.y));
-                            if (n >= 0 && 2 * lane < Te) h0 = __fdividef(v.x, 1.0f + e0) * v.z;
-                            if (n >= 0 && 2 * lane + 1 < Te) h1 = __fdividef(v.y, 1.0f + e1) * v.w;
+                            const float e0 = expf(-1.5957691216057308f * (v.x + 0.044715f * v.x * v.x * v.x));
+                            const float e1 = expf(-1.5957691216057308f * (v.y + 0.044715f * v.y * v.y * v.y));
+                            if (n >= 0 && 2 * lane < Te) h0 = v.x / (1.0f + e0) * v.z;
+                            if (n >= 0 && 2 * lane + 1 < Te) h1 = v.y / (1.0f + e1) * v.w;
                         }
                         if (a.record) {
                             float rec = fabsf(h0) + fabsf(h1);
@@ -607,15 +590,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                     // every CTA of the cluster is done with the h tile of the round before
                     if (s == 0 && R >= 1) WAIT(h_free, (R - 1) & 1);
                     if (s < own) {
-                        const __nv_bfloat162 hi = __floats2bfloat162_rn(h0, h1);
-                        const float2 hf = __bfloat1622float2(hi);
-                        const __nv_bfloat162 lo = __floats2bfloat162_rn(h0 - hf.x, h1 - hf.y);
+                        // 24 bits in three terms of 8: the first cut off (it must not round up to infinity), the others rounded
+                        const float c0 = __uint_as_float(__float_as_uint(h0) & 0xffff0000u), c1 = __uint_as_float(__float_as_uint(h1) & 0xffff0000u);
+                        const float f0 = isinf(h0) ? 0.f : h0 - c0, f1 = isinf(h1) ? 0.f : h1 - c1;
+                        const __nv_bfloat162 mid = __floats2bfloat162_rn(f0, f1);
+                        const float2 mf = __bfloat1622float2(mid);
                         unsigned char* hr = hb + ((j + 8 * s) * TN + bw) * HPITCH + lane * 4;
-                        *reinterpret_cast<__nv_bfloat162*>(hr) = hi;
-                        *reinterpret_cast<__nv_bfloat162*>(hr + 128) = lo;
+                        *reinterpret_cast<uint32_t*>(hr) = __float_as_uint(c0) >> 16 | __float_as_uint(c1);
+                        *reinterpret_cast<__nv_bfloat162*>(hr + 128) = mid;
+                        *reinterpret_cast<__nv_bfloat162*>(hr + 256) = __floats2bfloat162_rn(f0 - mf.x, f1 - mf.y);
                     }
-                    if (s == 0 && (tiles & 1) && bt < TN * 16)     // the last stage's second half, which nobody owns
-                        *reinterpret_cast<uint4*>(hb + (tiles * TN + (bt >> 4)) * HPITCH + (bt & 15) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    if (s == 0 && (tiles & 1) && bt < TN * 24)     // the last stage's second half, which nobody owns
+                        *reinterpret_cast<uint4*>(hb + (tiles * TN + bt / 24) * HPITCH + bt % 24 * 16) = make_uint4(0u, 0u, 0u, 0u);
                     fence_proxy_async_smem();
                     stop = barrier_or(2, 256, gave_up || *sAbort);
                     if (bt == 32 && (s + 1 == own || own == 0)) mbar_arrive_expect_tx(h_full, (uint32_t)(tiles - own) * (TN * HPITCH));
@@ -636,25 +622,35 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
 #pragma unroll 1
                 for (int s = 0; s < ns; ++s) {
                     const uint32_t ha = h_lane + s * SN * HPITCH, wd = d_lane + d_slot * LY(d_stage);
-                    uint32_t Ah[2][4], Al[2][4], Bw[NG / 2][4];
+                    // (a stage's products start from zero and are added in fp32: the tensor core cuts off what does not fit its
+                    // accumulator, and over a list of hundreds of neurons that would add up)
+                    uint32_t Bw[NG / 2][4];
 #pragma unroll
                     for (int n = 0; n < NG / 2; ++n)
                         if (HS || n < cpn) ldm4t(wd + n * 32, Bw[n]);
 #pragma unroll
                     for (int m = 0; m < 2; ++m)
-                        if (m < mcnt) { ldm4t(ha + m * 32, Ah[m]); ldm4t(ha + 128 + m * 32, Al[m]); }
+                        if (m < mcnt) {
+                            uint32_t A[3][4];
 #pragma unroll
-                    for (int hl = 0; hl < 2; ++hl)
+                            for (int k = 0; k < 3; ++k) ldm4t(ha + k * 128 + m * 32, A[k]);
 #pragma unroll
-                        for (int m = 0; m < 2; ++m)
-                            if (m < mcnt) {
+                            for (int n = 0; n < NG / 2; ++n)
+                                if (HS || n < cpn) {
+                                    float p[2][4];
 #pragma unroll
-                                for (int n = 0; n < NG / 2; ++n)
-                                    if (HS || n < cpn) {
-                                        mma16816(acc[m][2 * n], hl ? Al[m] : Ah[m], Bw[n][0], Bw[n][1]);
-                                        mma16816(acc[m][2 * n + 1], hl ? Al[m] : Ah[m], Bw[n][2], Bw[n][3]);
+                                    for (int i = 0; i < 2; ++i) p[i][0] = p[i][1] = p[i][2] = p[i][3] = 0.f;
+#pragma unroll
+                                    for (int k = 2; k >= 0; --k) {
+                                        mma16816(p[0], A[k], Bw[n][0], Bw[n][1]);
+                                        mma16816(p[1], A[k], Bw[n][2], Bw[n][3]);
                                     }
-                            }
+#pragma unroll
+                                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                                        for (int q = 0; q < 4; ++q) acc[m][2 * n + i][q] += p[i][q];
+                                }
+                        }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(d_empty(d_slot));
                     if (++d_slot == NST) { d_slot = 0; ++d_pass; }
@@ -662,39 +658,69 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
                 if (lane < CS) arrive_remote(map_to_rank(h_free, lane));
             }
             if (stop) break;
-            // ---- the item's sums are complete: into the output buffer of the layer (the first layer's has to be set up by
-            // every cluster before)
-            if (l == 0) {
-                if (bt == 0 && !gave_up) gave_up = counter_wait(a.ctrl + ctrl_init(e, j), w.parts_share & 0xff, __LINE__, a, sAbort);
-                stop = barrier_or(2, 256, gave_up || *sAbort);
-                if (stop) break;
-            }
+            // ---- the item's sums are complete: this cluster's part of them
             if (w.n > 0) {
-                const size_t row0 = row0_of(e);
-                float* ob = out_of(l) + row0 * H + (size_t)j * Hs;
-                const float* gp = EQ4 && a.gate ? a.gate + ((size_t)l * nb + b) * H + (size_t)j * Hs : nullptr;
-                float* yb = EQ4 && anchor_mode == RM_ANCHOR_WRITE ? a.y_anchor + ((size_t)l * nb * a.T_all + row0) * H + (size_t)j * Hs : nullptr;
+                float* pb = a.part + (size_t)(e * parts_max + w.share()) * a.T * H + (size_t)j * Hs;
 #pragma unroll
                 for (int n = 0; n < NG; ++n) {
                     const int col = (cp0 * 2 + n) * 8 + (lane & 3) * 2;
                     if ((n >> 1) >= cpn || col >= Hs) continue;
-                    float2 g = make_float2(1.f, 1.f);
-                    if (EQ4 && gp) g = __ldg(reinterpret_cast<const float2*>(gp + col));
 #pragma unroll
                     for (int m = 0; m < 2; ++m)
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int t = (m0 + m) * 16 + h * 8 + (lane >> 2);
-                            if (m >= mcnt || t >= Te) continue;
-                            const float y0 = acc[m][n][2 * h], y1 = acc[m][n][2 * h + 1];
-                            red_add_v2(ob + (size_t)t * H + col, EQ4 ? g.x * y0 : y0, EQ4 ? g.y * y1 : y1);
-                            if (EQ4 && yb) red_add_v2(yb + (size_t)t * H + col, y0, y1);
+                            if (m < mcnt && t < Te) *reinterpret_cast<float2*>(pb + (size_t)t * H + col) = make_float2(acc[m][n][2 * h], acc[m][n][2 * h + 1]);
                         }
                 }
             }
-            // (the barrier orders every thread's adds before thread 0's release, which is cumulative)
+            // (the barrier orders every thread's stores before thread 0's release, which is cumulative)
+            stop = barrier_or(2, 256, gave_up || *sAbort);
+            if (bt == 0 && !stop) red_release_gpu(a.ctrl + ctrl_part(e, j), 1);
+        }
+        // ---- the rows of the layer: this cluster's share of every item that it takes part in.  (Behind all of the layer's items:
+        // a cluster that has finished its part of one waits for the others' with its other products done.)
+        for (int e = 0; e < a.B && !stop; ++e) {
+            const Item w = items[l * a.B + e];
+            if (!w.mine()) continue;
+            const int parts = w.parts(), share = w.share(), n4 = Hs / 4, b = episode_of(e), Te = tokens_of(e);
+            const size_t lb = (size_t)l * a.nb + b, layer = (size_t)a.nb * a.T_all * H;
+            const float* in = l == 0 ? a.r_in : a.r_out;
+            if (parts > 1) {
+                // (every warp looks for itself: a barrier behind one thread's look is 3 us a step of 12 layers)
+                if (lane == 0 && !gave_up) gave_up = counter_wait(a.ctrl + ctrl_part(e, j), w.target() + parts, __LINE__, a, sAbort);
+                __syncwarp();
+            }
+            const float* pe = a.part + (size_t)e * parts_max * a.T * H + (size_t)j * Hs;
+            for (int z = bt; z < (Te - share + parts - 1) / parts * n4; z += 256) {
+                const int ri = z / n4, k = z - ri * n4, t = share + ri * parts;
+                const size_t o = (row0_of(e) + t) * H + (size_t)j * Hs + 4 * k;
+                float4 r = make_float4(0.f, 0.f, 0.f, 0.f), y = r, g = make_float4(1.f, 1.f, 1.f, 1.f);
+                if (in) r = __ldcg(reinterpret_cast<const float4*>(in + o));
+                if (w.n > 0) {
+                    const float4* p = reinterpret_cast<const float4*>(pe + (size_t)t * H) + k;
+#pragma unroll 1
+                    for (int i0 = 0; i0 < parts; i0 += 16) {
+                        float4 v[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) v[i] = i0 + i < parts ? __ldcg(p + (size_t)(i0 + i) * a.T * H / 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) { y.x += v[i].x; y.y += v[i].y; y.z += v[i].z; y.w += v[i].w; }
+                    }
+                }
+                if (EQ4) {
+                    if (anchor_mode == RM_ANCHOR_WRITE) *reinterpret_cast<float4*>(a.y_anchor + l * layer + o) = y;
+                    if (anchor_mode == RM_ANCHOR_UPDATE) {
+                        const float4 ya = __ldcg(reinterpret_cast<const float4*>(a.y_anchor + l * layer + o));
+                        y.x += ya.x; y.y += ya.y; y.z += ya.z; y.w += ya.w;
+                    }
+                    if (a.gate) g = __ldg(reinterpret_cast<const float4*>(a.gate + lb * H + (size_t)j * Hs) + k);
+                }
+                *reinterpret_cast<float4*>(a.r_out + o) = make_float4(fmaf(g.x, y.x, r.x), fmaf(g.y, y.y, r.y), fmaf(g.z, y.z, r.z), fmaf(g.w, y.w, r.w));
+            }
             stop = barrier_or(2, 256, gave_up || *sAbort);
             if (bt == 0 && !stop) red_release_gpu(a.ctrl + ctrl_done(e, j), 1);
+        }
         }
     }
 #undef WAIT
@@ -713,7 +739,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
 }
 
 // ---- host side
-constexpr int SMEM_MAX = 232448 - 1024;                            // (1 KB for the static part)
+constexpr int SMEM_MAX = 232448 - 256;                             // (the rest for the static part)
 
 template <int HS, int NG, int TS, bool EQ4>
 int configure(int smem) {
@@ -793,14 +819,15 @@ bool rm_slice_supported(const rm_ctx* ctx, int B, int T, bool record) {
     if (ctx->slice_clusters <= 0 || T < 1 || B < 1) return false;
     int n_sub, part;
     cut_tokens(T, n_sub, part);
-    return B * n_sub <= MAXB && ctx->g.L <= MAXL && ctx->g.L * B * n_sub <= MAX_ITEMS && !(record && n_sub > 1);
+    return ctx->g.L <= MAXL && !(record && n_sub > 1);
 }
 
 size_t rm_slice_workspace_bytes(const rm_ctx* ctx, int B, int T) {
     if (ctx->slice_clusters <= 0) return 0;
     int n_sub, part;
     cut_tokens(T, n_sub, part);
-    return B * n_sub <= MAXB ? ctrl_bytes(B * n_sub) : 0;
+    const int e = B * n_sub < GROUP ? B * n_sub : GROUP;
+    return ctrl_bytes(GROUP) + (size_t)e * ctx->slice_clusters * part * ctx->g.H * sizeof(float);
 }
 
 int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
@@ -811,15 +838,8 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     for (int l = 0; l < sa.L; ++l) a.packed[l] = static_cast<const __nv_bfloat16*>(sa.packed_layers[l]);
     a.r_in = sa.r_in ? sa.r_in : sa.r;
     a.r_out = sa.r;
-    for (int i = 0; i < 3; ++i) a.rot[i] = sa.rot[i];
     a.x_ext = static_cast<const __nv_bfloat16*>(sa.x_ext);
-    if (sa.x_ext) {
-        a.r_in = sa.r_in;
-    } else if (a.r_in == a.r_out && sa.L < 3) {
-        // in place, and the last layer's buffer would be cleared while the first layer still reads it
-        RM_CUDA_TRY(cudaMemcpyAsync(sa.rot[2], sa.r, (size_t)sa.B * sa.T * g.H * sizeof(float), cudaMemcpyDeviceToDevice, s));
-        a.r_in = sa.rot[2];
-    }
+    if (sa.x_ext) a.r_in = sa.r_in;
     a.idx = sa.idx;
     a.count = sa.count;
     a.idx_b_stride = sa.idx_b_stride;
@@ -830,10 +850,9 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     a.rec_b_stride = sa.rec_b_stride;
     a.record_scale = sa.record_scale;
     a.ctrl = sa.ctrl;
-    a.epoch = rm_next_epoch();
+    a.part = reinterpret_cast<float*>(reinterpret_cast<char*>(sa.ctrl) + ctrl_bytes(GROUP));
     a.status = ctx->d_status;
     a.L = sa.L;
-    a.B = sa.B * n_sub;
     a.T = part;
     a.I = g.I;
     a.Hs = g.Hs;
@@ -850,7 +869,14 @@ int rm_launch_step_slice(rm_ctx* ctx, const rm_step_args& sa, cudaStream_t s) {
     const bool eq4 = sa.anchor_mode != RM_ANCHOR_NONE || sa.gate != nullptr;
     a.lay = layout_of(g.Hs);
     const int smem = a.lay.total;
-    if (g.Hs == 128) return eq4 ? launch<128, 4, 2, true>(ctx, a, nc, smem, s) : launch<128, 4, 2, false>(ctx, a, nc, smem, s);
-    if (g.Hs < 128) return eq4 ? launch<0, 4, 2, true>(ctx, a, nc, smem, s) : launch<0, 4, 2, false>(ctx, a, nc, smem, s);
-    return eq4 ? launch<0, 8, 1, true>(ctx, a, nc, smem, s) : launch<0, 8, 1, false>(ctx, a, nc, smem, s);
+    for (a.e0 = 0; a.e0 < sa.B * n_sub; a.e0 += GROUP) {
+        a.B = sa.B * n_sub - a.e0 < GROUP ? sa.B * n_sub - a.e0 : GROUP;
+        a.epoch = rm_next_epoch();
+        int rc;
+        if (g.Hs == 128) rc = eq4 ? launch<128, 4, 2, true>(ctx, a, nc, smem, s) : launch<128, 4, 2, false>(ctx, a, nc, smem, s);
+        else if (g.Hs < 128) rc = eq4 ? launch<0, 4, 2, true>(ctx, a, nc, smem, s) : launch<0, 4, 2, false>(ctx, a, nc, smem, s);
+        else rc = eq4 ? launch<0, 8, 1, true>(ctx, a, nc, smem, s) : launch<0, 8, 1, false>(ctx, a, nc, smem, s);
+        if (rc != RM_OK) return rc;
+    }
+    return RM_OK;
 }

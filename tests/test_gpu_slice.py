@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from harness import assert_close, dev, lists_to_padded
+from harness import REL_L2_TOL, assert_close, dev, lists_to_padded
 from test_gpu_anchor import make_case, run_write
 from test_gpu_edges import step_case
 
@@ -72,3 +72,53 @@ def test_slice_kernel_in_a_replayed_graph(lib):
     assert ctx.rm_device_status() == 0
     del g
     model.close()
+
+
+@pytest.mark.parametrize("H,I,T,L,B,density", [
+    (384, 1300, 51, 1, 1, 0.25), (512, 2048, 51, 1, 1, 0.06), (1536, 6144, 51, 1, 1, 0.25), (1792, 3000, 33, 1, 1, 1.0), (2048, 4096, 90, 1, 1, 0.3),
+    (1024, 3500, 70, 1, 1, 0.6), (1536, 6144, 51, 6, 1, 0.25), (1088, 900, 20, 3, 9, 0.5)])
+def test_other_widths_lose_nothing_against_the_cuda_core_kernels(lib, H, I, T, L, B, density):
+    """The CUDA-core kernels, which take the same shapes, sum in fp32 in one order: the same bits every time, and an error against
+    64 bits that the slice kernel must not exceed.  (25 % for where the roundings that both share are the larger part.  Behind one
+    layer single roundings of x to bf16 differ and hide the sums.)  Nine episodes: two launches."""
+    import math
+
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(H + I + T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    ctx = lib.Context(L, H, I, T, B)
+    W = [[(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))] for _ in range(L)]
+    layers = [ctx.rm_pack_weights(*w) for w in W]
+    k, stride = max(1, int(density * I)), (I + 3) // 4 * 4
+    idx = torch.zeros(B, L, stride, dtype=torch.int32, device="cuda")
+    for b in range(B):
+        for l in range(L):
+            idx[b, l, :k] = torch.randperm(I, generator=g, device="cuda")[:k].sort().values.int()
+    cnt = torch.full((B, L), k, dtype=torch.int32, device="cuda")
+    r = rnd(B, T, H).bfloat16().float()
+
+    def run(path):
+        ctx.rm_set_option("path", path)
+        out = torch.full_like(r, 7.0)
+        ctx.rm_action_expert_step(layers, r, idx, cnt, stride, out, B=B)
+        assert ctx.rm_get_info("last_variant") == (0 if path else 6)
+        return out
+
+    first, portable = run(0), run(1)
+    for _ in range(3):
+        assert torch.equal(first, run(0))
+    in_place = r.clone()
+    ctx.rm_action_expert_step(layers, in_place, idx, cnt, stride, in_place, B=B)
+    assert torch.equal(first, in_place)
+    assert ctx.rm_device_status() == 0
+    if L == 1:
+        gate, up, down = (w.double() for w in W[0])
+        i = idx[0, 0, :k].long()
+        x = (r[0].double() / torch.sqrt((r[0].double() ** 2).mean(-1, keepdim=True) + 1e-6)).float().bfloat16().double()
+        z = x @ gate[i].T
+        y = (0.5 * z * (1 + torch.tanh(math.sqrt(2 / math.pi) * (z + 0.044715 * z ** 3))) * (x @ up[i].T)) @ down[:, i].T
+        err = [float((o[0].double() - r[0].double() - y).norm() / y.norm()) for o in (first, portable)]
+        assert err[0] <= 1.25 * err[1], err
+    else:
+        assert float((first - portable).norm() / portable.norm()) <= REL_L2_TOL
+    ctx.close()

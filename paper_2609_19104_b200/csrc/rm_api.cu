@@ -168,11 +168,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->stream_pairs = 0;
     c->persist_max_b = 1;
     c->persist_prefetch_kb = 0;
-    c->persist_xbuf = nullptr;
-    c->persist_sync = nullptr;
-    c->persist_sync_dirty = 0;
     for (int l = 0; l < 64; ++l) c->sweep_key[l] = nullptr;
-    for (int b = 0; b < 16; ++b) c->persist_sync_base[b] = c->persist_copy_base[b] = 0;
     if (major == 10) { rm_fused_init(c); rm_persist_init(c); rm_slice_init(c); rm_stream_init(c); }   // failure leaves the portable path in charge
     cudaGetLastError();
     *out = c;
@@ -619,7 +615,6 @@ int rm_device_status(rm_ctx* ctx, int* host_out, rm_stream_t stream) {
     RM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(v), s));
     RM_CUDA_TRY(cudaStreamSynchronize(s));
     *host_out = v[0];
-    if (v[0] != 0) ctx->persist_sync_dirty = 1;                 // a whole-step launch may have stopped half way
     ctx->status_detail = v[0] ? v[1] : 0;
     std::memcpy(ctx->status_log, v, sizeof(v));
     return RM_OK;

@@ -51,14 +51,8 @@ struct rm_ctx {
     int persist_clusters;                  // co-resident 8-CTA clusters of the whole-step kernel (0: unavailable)
     int persist_prefetch_kb;               // weight KB a CTA of the whole-step kernel may ask into L2 ahead of its loaders
     int persist_max_b;                     // largest batch the whole-step kernel is chosen for when the variant is automatic
-    const void* persist_xbuf;              // buffer the cached tensor map below describes
-    const int* persist_sync;               // the workspace's arrival counters this context has been counting on
-    int persist_sync_base[16];             // their values after the launches so far
-    int persist_copy_base[16];             // the same for the counters of the r_in -> r copies
-    int persist_sync_dirty;                // a launch may have left them at an unknown count: clear before the next one
     const void* sweep_key[64];             // layers whose tensor maps the sweep kernel has (NULL: none yet)
     alignas(64) unsigned char sweep_maps[2 * 64 * 128];
-    alignas(64) unsigned char persist_tm[128];   // CUtensorMap of the clusters' x copies in the workspace
 };
 
 // The count the kernel selection works with: the caller's hint, else what the last compaction through this context

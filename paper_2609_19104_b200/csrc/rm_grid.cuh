@@ -1,8 +1,10 @@
 // What the kernels that hold a whole step share: the control block of a launch, counters between CTAs, bounded waits.
 //
-// Control block (workspace, ints): [0,1] epoch of the running launch, [2] CTAs that have left, [3] abort flag, then the kernel's
-// own counters from CTRL_LINE on.  CTA 0 clears the counters and then publishes the launch's epoch; a CTA touches a counter
-// only once it has seen the epoch; the last CTA to leave takes it back, so that a captured launch can be replayed.
+// Control block (workspace, ints): [0,1] epoch of the running launch, [2] CTAs that have left, [3] abort flag (the low half of the
+// epoch of the launch that gives up), then the kernel's own counters from CTRL_LINE on.  CTA 0 clears the counters and then
+// publishes the launch's epoch; a CTA touches a counter only once it has seen the epoch; the last CTA to leave takes it
+// back, so that a captured launch can be replayed.  Nothing is expected of what the block holds before: between two launches
+// other calls, of other sizes, use the same workspace.
 //
 // Every wait is bounded and returns true when the waiter has to give up: the wait ran out (status RM_ERR_TIMEOUT with the
 // wait's source line and the CTA), or this CTA or the grid is aborting.
@@ -26,19 +28,21 @@ __device__ __forceinline__ void st_release_gpu(int* p, int v) {
     asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// (A: the kernel's arguments, with `status` and `ctrl`)
+// (A: the kernel's arguments, with `status`, `ctrl` and `epoch`)
+template <class A>
+__device__ __forceinline__ bool aborting(const A& a) { return ld_acquire_gpu(a.ctrl + 3) == (int)(unsigned)a.epoch; }
 template <class A>
 __device__ __forceinline__ void report_timeout(const A& a, volatile int* abort_cta, int line) {
     rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
     *abort_cta = 1;
-    atomicExch(a.ctrl + 3, 1);
+    atomicExch(a.ctrl + 3, (int)(unsigned)a.epoch);
 }
 template <class A>
 __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, const A& a, volatile int* abort_cta) {
     for (uint32_t i = 0; i < (1u << 22); ++i) {
         if (sm100::mbar_try_wait(bar, parity)) return false;
         if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && (*abort_cta || ((i & 16383u) == 16383u && ld_acquire_gpu(a.ctrl + 3) == 1))) {
+        if ((i & 1023u) == 1023u && (*abort_cta || ((i & 16383u) == 16383u && aborting(a)))) {
             *abort_cta = 1;
             return true;
         }
@@ -50,7 +54,7 @@ template <class A>
 __device__ __forceinline__ bool counter_wait(const int* counter, int target, int line, const A& a, volatile int* abort_cta) {
     for (uint32_t i = 0; i < (1u << 21); ++i) {
         if (ld_acquire_gpu(counter) >= target) return false;
-        if ((i & 255u) == 255u && (*abort_cta || ld_acquire_gpu(a.ctrl + 3) == 1)) { *abort_cta = 1; return true; }
+        if ((i & 255u) == 255u && (*abort_cta || aborting(a))) { *abort_cta = 1; return true; }
     }
     report_timeout(a, abort_cta, line);
     return true;
@@ -73,8 +77,10 @@ __device__ __forceinline__ void epoch_publish(int* ctrl, unsigned long long epoc
 }
 // by one thread of every CTA on its way out (it has seen the epoch)
 __device__ __forceinline__ void epoch_leave(int* ctrl) {
-    if (atomicAdd(ctrl + 2, 1) == (int)gridDim.x - 1)
+    if (atomicAdd(ctrl + 2, 1) == (int)gridDim.x - 1) {
+        ctrl[3] = 0;
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(ctrl), "l"(0ull) : "memory");
+    }
 }
 // OR of a predicate over the threads of a named barrier
 __device__ __forceinline__ bool barrier_or(int id, int count, bool pred) {

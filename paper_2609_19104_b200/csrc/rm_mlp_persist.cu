@@ -34,6 +34,7 @@
 #include <mutex>
 
 #include "rm_common.cuh"
+#include "rm_grid.cuh"
 #include "rm_sm100.cuh"
 
 using namespace sm100;
@@ -54,12 +55,13 @@ constexpr int NXW = 4;                 // warps that issue the x copies (copies 
 constexpr int NTHREADS = 608;          // warps: 0-7 epilogue and normalisation, 8-11 loaders, 12 issuer, 13-16 x copies, 17 L2 prefetch,
                                        // 18 stage watcher
 constexpr int W_LOAD0 = 8, W_MMA = 12, W_X0 = 13, W_PF = 17, W_WATCH = 18;
-constexpr int SYNC_ABORT = MAXB;       // sync[0..MAXB): per-episode arrival counters; sync[MAXB]: abort flag
+// The launch's counters, behind the control block's first line (rm_grid.cuh): sync[0..MAXB) per-episode arrivals
 constexpr int SYNC_COPY = 32;          // sync[32..32+MAXB): per-episode counters of the CTAs that have copied r_in into r
 constexpr int SYNC_READ = 48;          // sync[48..48+MAXB): per-episode counters of the CTAs that have read r for a layer's normalisation
 constexpr int SYNC_ITEM = 64;          // sync[64..64+MAX_ITEMS): batches count the arrivals of every (layer, episode) by itself
 constexpr int SYNC_RITEM = SYNC_ITEM + MAX_ITEMS;      // ... and the CTAs that have read the item's input rows
-constexpr int SYNC_BYTES = (SYNC_RITEM + MAX_ITEMS) * 4;
+constexpr int SYNC_INTS = SYNC_RITEM + MAX_ITEMS;
+constexpr int CTRL_BYTES = ((grid::CTRL_LINE + SYNC_INTS) * 4 + 255) / 256 * 256;
 
 struct PArgs {
     const __nv_bfloat16* packed[MAXL];
@@ -73,14 +75,14 @@ struct PArgs {
     float* record;                     // record (b, l, n) at record[b * rec_b_stride + l * I + n]; NULL: none
     int64_t rec_b_stride;
     const float* record_scale;         // [L, I] or NULL
-    int* sync;                         // [0..MAXB): per-episode arrival counters, never reset between launches; [MAXB]: abort flag
-    int sync_base[MAXB];               // value of each counter when this launch starts (the host keeps count)
-    int copy_base[MAXB];               // the same for the copy counters
+    int* ctrl;                         // control block
+    unsigned long long epoch;          // of this launch
+    int* sync;                         // its counters, cleared by the launch itself
     int* status;
     int L, B, T, I;
-    int per_item;                      // arrivals are counted per (layer, episode) on counters cleared before the launch (batches:
-                                       // a cluster that takes no part in an episode runs ahead of those that do, so one
-                                       // counter per episode could not tell the layers apart); else per episode, never cleared
+    int per_item;                      // arrivals are counted per (layer, episode) (batches: a cluster that takes no part in an
+                                       // episode runs ahead of those that do, so one counter per episode could not tell the
+                                       // layers apart); else per episode, over all layers
     int x_ext;                         // layer 0 takes x from the caller's buffer (single-layer entry): no normalisation
     int pf_bytes;                      // weight bytes a CTA may have asked into L2 ahead of its loaders (0: no prefetch)
     // Anchor-relative update (Eq. 4) and output gate; read by the EQ4 instantiation only
@@ -146,34 +148,36 @@ __device__ __noinline__ uint32_t landed_stages(const int* count, uint32_t stage,
     }
     return ready;
 }
-__device__ __noinline__ void report_timeout(int* status, volatile int* abort_flag, int* sync, int line) {
+// (tag: the abort flag of this launch, the low half of its epoch)
+__device__ __forceinline__ bool aborting(volatile int* abort_flag, const int* ctrl, int tag) { return *abort_flag || ld_acquire_gpu(ctrl + 3) == tag; }
+__device__ __noinline__ void report_timeout(int* status, volatile int* abort_flag, int* ctrl, int tag, int line) {
     rm_set_status_at(status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
     *abort_flag = 1;
-    atomicExch(sync + SYNC_ABORT, 1);
+    atomicExch(ctrl + 3, tag);
 }
 // The part of a bounded wait that runs when the phase was not complete at the first look.  Returns true when the waiter
 // has to give up: the wait ran out (status RM_ERR_TIMEOUT with the wait's source line and the CTA), or this CTA or the
 // grid is aborting.
-__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, volatile int* abort_flag, int* sync, int* status) {
+__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, volatile int* abort_flag, int* ctrl, int tag, int* status) {
     for (uint32_t i = 0; i < (1u << 22); ++i) {
         if (mbar_try_wait(bar, parity)) return false;
         if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && (*abort_flag || ((i & 16383u) == 16383u && ld_acquire_gpu(sync + SYNC_ABORT)))) {
+        if ((i & 1023u) == 1023u && (*abort_flag || ((i & 16383u) == 16383u && ld_acquire_gpu(ctrl + 3) == tag))) {
             *abort_flag = 1;
             return true;
         }
     }
-    report_timeout(status, abort_flag, sync, line);
+    report_timeout(status, abort_flag, ctrl, tag, line);
     return true;
 }
 // A bounded wait for a counter in global memory, out of line (for the path that is rarely taken).  Returns true when
 // the waiter has to give up.
-__device__ __noinline__ bool counter_wait_slow(const int* counter, int target, int line, volatile int* abort_flag, int* sync, int* status) {
+__device__ __noinline__ bool counter_wait_slow(const int* counter, int target, int line, volatile int* abort_flag, int* ctrl, int tag, int* status) {
     for (uint32_t i = 0; i < (1u << 21); ++i) {
         if (ld_acquire_gpu(counter) >= target) return false;
-        if ((i & 255u) == 255u && (*abort_flag || ld_acquire_gpu(sync + SYNC_ABORT))) { *abort_flag = 1; return true; }
+        if ((i & 255u) == 255u && aborting(abort_flag, ctrl, tag)) { *abort_flag = 1; return true; }
     }
-    report_timeout(status, abort_flag, sync, line);
+    report_timeout(status, abort_flag, ctrl, tag, line);
     return true;
 }
 __device__ __forceinline__ void st_release_cta(int* p, int v) {         // shared memory
@@ -430,6 +434,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     // a dependent launch: everything up to here needs nothing from the kernel in front (a step of 18 layers of 1024/4096, 25 %,
     // behind another one: 193.4 -> 189.6 us)
     pdl_wait();
+    if (blockIdx.x == 0) {                 // the launch's counters, then (below) its epoch
+        for (int e = tid; e < SYNC_INTS; e += NTHREADS) a.sync[e] = 0;
+        if (tid == 0) { a.ctrl[2] = 0; a.ctrl[3] = 0; }
+        __threadfence();
+    }
     {
         const int cap = (int)(a.list_cap < (int64_t)I ? a.list_cap : (int64_t)I);
         for (int it = tid; it < n_items; it += NTHREADS) {
@@ -443,6 +452,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
         }
     }
     __syncthreads();
+    if (blockIdx.x == 0 && tid == W_PF * 32) grid::epoch_publish(a.ctrl, a.epoch);
     {
         // This cluster's run in every item's list: one thread per item (sK holds the counts; afterwards sP the run starts
         // and sK the run lengths).  One thread doing all of them took ~3 us of every launch.
@@ -481,6 +491,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     tc_fence_after();
     const uint32_t tmem = *g_tmem;
     pdl_launch_dependents();                                       // (a dependent waits for this grid's end: its CTAs are resident by then)
+    // (the warps that use the launch's counters)
+    const int tag = (int)(unsigned)a.epoch;
+    if (warp < 8) {
+        if (tid == 0) grid::epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
+        named_barrier(1, 256);
+    }
     // r starts as a copy of r_in: cluster 0's CTA j copies column slice j of every episode and counts itself on the
     // episode's copy counter; nobody adds into r before the 8 copies are counted
     const int pre = a.r_in != a.r ? CS : 0;
@@ -513,13 +529,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     // loops that run all the time stay compact.
     bool gave_up = false;
     auto timed_out = [&](int line) {
-        report_timeout(a.status, sAbort, a.sync, line);
+        report_timeout(a.status, sAbort, a.ctrl, tag, line);
         gave_up = true;
     };
     auto wait_at = [&](uint32_t bar, uint32_t parity, int line) {
         if (gave_up) return;
         if (mbar_test_wait(bar, parity)) return;
-        gave_up = wait_slow(bar, parity, line, sAbort, a.sync, a.status);
+        gave_up = wait_slow(bar, parity, line, sAbort, a.ctrl, tag, a.status);
     };
 #define WAIT(bar, parity) wait_at((bar), (parity), __LINE__)
 
@@ -889,7 +905,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
             const bool xf_ok = nu >= 1 ? mbar_test_wait(x_free(slot), (nu - 1) & 1) : true;     // looked at before the stores
             if (l > 0) {
                 // every CTA has added its part of layer l-1 to this episode's rows
-                const int target = a.per_item ? n_ctas : a.sync_base[b] + n_ctas * l;
+                const int target = a.per_item ? n_ctas : n_ctas * l;
                 const int* counter = a.per_item ? a.sync + SYNC_ITEM + (l - 1) * B + b : a.sync + b;
                 // one thread per CTA watches the counter (with every warp's lane 0 polling, ~1000 threads read the line
                 // that the last arrivals have to get through); the barrier passes its acquire on to the others
@@ -897,9 +913,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                     bool ok = false;
                     for (uint32_t i = 0; i < (1u << 21); ++i) {
                         if (ld_acquire_gpu(counter) >= target) { ok = true; break; }
-                        if ((i & 255u) == 255u && (*sAbort || ld_acquire_gpu(a.sync + SYNC_ABORT))) break;
+                        if ((i & 255u) == 255u && aborting(sAbort, a.ctrl, tag)) break;
                     }
-                    if (!ok) { if (!*sAbort && !ld_acquire_gpu(a.sync + SYNC_ABORT)) timed_out(__LINE__); gave_up = true; *sAbort = 1; }
+                    if (!ok) { if (!aborting(sAbort, a.ctrl, tag)) timed_out(__LINE__); gave_up = true; *sAbort = 1; }
                 }
                 named_barrier(1, 256);
             }
@@ -1131,16 +1147,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
             const bool upd = EQ4 && anchor_mode == RM_ANCHOR_UPDATE;
             const bool ext = item_ext(env, l);
             const int* rctr = a.per_item ? a.sync + SYNC_RITEM + item : a.sync + SYNC_READ + b;
-            const int rtarget = a.per_item ? n_ctas : a.sync_base[b] + n_ctas * (l + 1);
+            const int rtarget = a.per_item ? n_ctas : n_ctas * (l + 1);
             if (run.ntiles == 0 && upd) {
                 // no tiles, yet rows to add to: the same order of events as for a CTA with tiles (see the arrival below)
                 if (et == 0 && !gave_up) {
                     if (!a.per_item && l > 0)
-                        gave_up = counter_wait_slow(a.sync + b, a.sync_base[b] + n_ctas * l, __LINE__, sAbort, a.sync, a.status);
+                        gave_up = counter_wait_slow(a.sync + b, n_ctas * l, __LINE__, sAbort, a.ctrl, tag, a.status);
                     red_release_gpu(const_cast<int*>(rctr), 1);
-                    if (!gave_up) gave_up = counter_wait_slow(rctr, rtarget, __LINE__, sAbort, a.sync, a.status);
+                    if (!gave_up) gave_up = counter_wait_slow(rctr, rtarget, __LINE__, sAbort, a.ctrl, tag, a.status);
                     if (l == 0 && pre && !gave_up)                 // r holds its copy of r_in
-                        gave_up = counter_wait_slow(a.sync + SYNC_COPY + b, a.copy_base[b] + pre, __LINE__, sAbort, a.sync, a.status);
+                        gave_up = counter_wait_slow(a.sync + SYNC_COPY + b, pre, __LINE__, sAbort, a.ctrl, tag, a.status);
                 }
                 stop = named_barrier_or(1, 256, gave_up || *sAbort);
             }
@@ -1155,17 +1171,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                 WAIT(d2_full(d2b), nu & 1);
                 tc_fence_after();
                 if (et == 0) RM_PS(item, 5);
-                if (rseen < rtarget && !gave_up) gave_up = counter_wait_slow(rctr, rtarget, __LINE__, sAbort, a.sync, a.status);
+                if (rseen < rtarget && !gave_up) gave_up = counter_wait_slow(rctr, rtarget, __LINE__, sAbort, a.ctrl, tag, a.status);
                 __syncwarp();
                 if (l == 0 && pre) {
                     // r has to hold its copy of r_in before anything is added to it
                     if (lane == 0 && !gave_up) {
                         bool ok = false;
                         for (uint32_t w8 = 0; w8 < (1u << 21); ++w8) {
-                            if (ld_acquire_gpu(a.sync + SYNC_COPY + b) >= a.copy_base[b] + pre) { ok = true; break; }
-                            if ((w8 & 255u) == 255u && (*sAbort || ld_acquire_gpu(a.sync + SYNC_ABORT))) break;
+                            if (ld_acquire_gpu(a.sync + SYNC_COPY + b) >= pre) { ok = true; break; }
+                            if ((w8 & 255u) == 255u && aborting(sAbort, a.ctrl, tag)) break;
                         }
-                        if (!ok) { if (!*sAbort && !ld_acquire_gpu(a.sync + SYNC_ABORT)) timed_out(__LINE__); gave_up = true; *sAbort = 1; }
+                        if (!ok) { if (!aborting(sAbort, a.ctrl, tag)) timed_out(__LINE__); gave_up = true; *sAbort = 1; }
                     }
                     __syncwarp();
                 }
@@ -1225,13 +1241,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                 // early arrivals would stand in for a slower CTA's.
                 const bool empty = run.ntiles == 0 && !upd;
                 if (empty && !a.per_item && l > 0 && !gave_up)
-                    gave_up = counter_wait_slow(a.sync + b, a.sync_base[b] + n_ctas * l, __LINE__, sAbort, a.sync, a.status);
+                    gave_up = counter_wait_slow(a.sync + b, n_ctas * l, __LINE__, sAbort, a.ctrl, tag, a.status);
                 // (CTAs that have not normalised this item -- no tiles, or x from the caller -- count as readers here)
                 if (empty || (ext && run.ntiles > 0)) red_release_gpu(const_cast<int*>(rctr), 1);
                 red_release_gpu(a.per_item ? a.sync + SYNC_ITEM + item : a.sync + b, 1);
                 RM_PS(item, 7);
             }
         }
+        // (this CTA's last counter: the round trip of the leave runs beside the end of the other warps)
+        if (et == 0 && !grid::epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort)) grid::epoch_leave(a.ctrl);
     }
 #undef WAIT
     tc_fence_before();
@@ -1329,7 +1347,6 @@ inline size_t align_up(size_t v, size_t al) { return (v + al - 1) / al * al; }
 
 int rm_persist_init(rm_ctx* ctx) {
     ctx->persist_clusters = 0;
-    ctx->persist_xbuf = nullptr;
     int n = 0, rc = RM_OK;
     if (ctx->g.H == 1024) rc = query_clusters<128>(&n);
     else if (ctx->g.H == 2048) rc = query_clusters<256>(&n);
@@ -1347,7 +1364,7 @@ bool rm_persist_supported(const rm_ctx* ctx, int B, int T) {
 
 size_t rm_persist_workspace_bytes(const rm_ctx* ctx) {
     if (ctx->persist_clusters <= 0) return 0;
-    return SYNC_BYTES + (size_t)ctx->persist_clusters * 2 * NTOK * ctx->g.H * sizeof(__nv_bfloat16);
+    return CTRL_BYTES + (size_t)ctx->persist_clusters * 2 * NTOK * ctx->g.H * sizeof(__nv_bfloat16);
 }
 
 int rm_persist_debug_stamps(long long* host_out, int n) {
@@ -1366,8 +1383,10 @@ int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaSt
     for (int l = 0; l < sa.L; ++l) a.packed[l] = static_cast<const __nv_bfloat16*>(sa.packed_layers[l]);
     a.r = sa.r;
     a.r_in = sa.r_in ? sa.r_in : sa.r;
-    a.sync = reinterpret_cast<int*>(ws);
-    a.xbuf = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + SYNC_BYTES);
+    a.ctrl = reinterpret_cast<int*>(ws);
+    a.epoch = rm_next_epoch();
+    a.sync = a.ctrl + grid::CTRL_LINE;
+    a.xbuf = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + CTRL_BYTES);
     a.per_item = sa.B > 1 ? 1 : 0;
     a.idx = sa.idx;
     a.count = sa.count;
@@ -1387,35 +1406,12 @@ int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaSt
     a.pf_bytes = ctx->persist_prefetch_kb * 1024;
     int nc = ctx->persist_clusters;
     if (ctx->max_clusters_override > 0 && ctx->max_clusters_override < nc) nc = ctx->max_clusters_override;
-    // the caller's x (single-layer entry) as a tensor map; otherwise any valid map (the kernel does not use it): one over
-    // the workspace, made once per workspace
-    if (!sa.x_ext && ctx->persist_xbuf != a.xbuf) {
-        const int rc = make_x_map(reinterpret_cast<CUtensorMap*>(ctx->persist_tm), a.xbuf, (uint64_t)NTOK, (uint64_t)g.H);
-        if (rc != RM_OK) return rc;
-        ctx->persist_xbuf = a.xbuf;
-    }
-    alignas(64) CUtensorMap tm_ext;
+    // the caller's x (single-layer entry) as a tensor map; the kernel does not look at it otherwise
+    alignas(64) CUtensorMap tm_ext{};
     if (sa.x_ext) {
         const int rc = make_x_map(&tm_ext, sa.x_ext, (uint64_t)sa.T, (uint64_t)g.H);
         if (rc != RM_OK) return rc;
-    } else {
-        tm_ext = *reinterpret_cast<const CUtensorMap*>(ctx->persist_tm);
     }
-    int nc_ctas = nc * CS;
-    const int pre = a.r_in != a.r ? CS : 0;
-    // The arrival counters live in the workspace and only ever count up; the host keeps their values.  They are cleared
-    // when the workspace is new to this context, after a launch whose status was not clean (its count is unknown), and
-    // long before they could wrap.
-    bool reset = ctx->persist_sync != a.sync || ctx->persist_sync_dirty || a.per_item;
-    for (int b = 0; b < MAXB; ++b) reset = reset || ctx->persist_sync_base[b] > (1 << 30);
-    if (reset) {
-        RM_CUDA_TRY(cudaMemsetAsync(a.sync, 0, a.per_item ? SYNC_BYTES : 256, s));
-        for (int b = 0; b < MAXB; ++b) ctx->persist_sync_base[b] = ctx->persist_copy_base[b] = 0;
-        ctx->persist_sync = a.sync;
-        ctx->persist_sync_dirty = 0;
-    }
-    for (int b = 0; b < MAXB; ++b) { a.sync_base[b] = ctx->persist_sync_base[b]; a.copy_base[b] = ctx->persist_copy_base[b]; }
-    for (int b = 0; b < sa.B; ++b) { ctx->persist_sync_base[b] += nc_ctas * sa.L; ctx->persist_copy_base[b] += pre; }
     // (the instantiation without Eq. 4 and gate is the one the plain steps run: it carries none of their code)
     const bool eq4 = sa.anchor_mode != RM_ANCHOR_NONE || sa.gate != nullptr;
     a.anchor_mode = sa.anchor_mode;
@@ -1426,8 +1422,6 @@ int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaSt
     // the anchor step's sums are accumulated by the CTAs' atomics: start them from zero
     if (sa.anchor_mode == RM_ANCHOR_WRITE)
         RM_CUDA_TRY(cudaMemsetAsync(sa.y_anchor, 0, (size_t)sa.L * sa.B * sa.T * g.H * sizeof(float), s));
-    const int rc = g.H == 1024 ? (eq4 ? launch<128, true>(ctx, a, tm_ext, nc, s) : launch<128, false>(ctx, a, tm_ext, nc, s))
-                               : (eq4 ? launch<256, true>(ctx, a, tm_ext, nc, s) : launch<256, false>(ctx, a, tm_ext, nc, s));
-    if (rc != RM_OK) ctx->persist_sync_dirty = 1;               // nothing ran: the counters are behind the host's count
-    return rc;
+    return g.H == 1024 ? (eq4 ? launch<128, true>(ctx, a, tm_ext, nc, s) : launch<128, false>(ctx, a, tm_ext, nc, s))
+                       : (eq4 ? launch<256, true>(ctx, a, tm_ext, nc, s) : launch<256, false>(ctx, a, tm_ext, nc, s));
 }

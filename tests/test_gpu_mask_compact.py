@@ -155,6 +155,37 @@ def test_lists_and_records_spread_over_ctas(lib, I, n_lists, W):
         check_lists(out_idx, out_cnt, [np.flatnonzero(m[i]) for i in range(n_lists)])
 
 
+# Between what a CTA may have without asking and the next larger amount: 48 KB with the kernel's own 17168 bytes, so 31985 to 32768
+# bytes of words.  (I, lists, records, reduction, bytes): 128 bytes per 1024 neurons, times 2 + planes * CTAs of the cluster
+SHARED_MEMORY_EDGE = [(14000, 2, 9, "TOPK", 14 * 128 * 18), (65536, 2, 2, "TOPK", 64 * 128 * 4), (42900, 1, 8, "THRESHOLD", 42 * 128 * 6),
+                      (14000, 2, 16, "GROUP", 14 * 128 * 18), (15300, 2, 9, "TOPK", 15 * 128 * 18)]
+
+
+@pytest.mark.parametrize("case", SHARED_MEMORY_EDGE)
+def test_first_call_at_the_edge_of_the_default_shared_memory(lib, case):
+    """In a process of its own: an earlier, larger call raises the limit for the smaller ones behind it."""
+    import os
+    import subprocess
+    import sys
+    code = f"""
+import sys
+sys.path[:0] = [{os.path.dirname(os.path.dirname(os.path.abspath(__file__)))!r}, {os.path.dirname(os.path.abspath(__file__))!r}]
+import numpy as np, oracle, paper_2609_19104_b200 as lib
+from test_gpu_mask_compact import adversarial_records, check_lists, run_compact
+I, n_lists, W, reduce, _ = {case!r}
+recs = [adversarial_records(I, n_lists, 90 + w) for w in range(W)]
+k, votes = I // 3, (W + 1) // 2
+idx, cnt, status = run_compact(lib, I, recs, lib.RM_SRC_SCORE_F32, getattr(lib, 'RM_REDUCE_' + reduce), n_lists, k=k, min_votes=votes, threshold=0.5)
+assert status == 0
+per = [[r[i] for r in recs] for i in range(n_lists)]
+want = ([oracle.compact_group(r, k) for r in per] if reduce == 'GROUP' else
+        [oracle.compact_scores(r, getattr(oracle, 'RULE_' + reduce), k=k, threshold=0.5, min_votes=votes) for r in per])
+check_lists(idx, cnt, want)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
 def test_truncation_is_reported_not_fatal(lib):
     I = 512
     m = np.ones((1, I), dtype=np.uint8)

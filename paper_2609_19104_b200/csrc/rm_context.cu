@@ -92,8 +92,9 @@ __device__ __forceinline__ int ctx_count(const int32_t* count, int P, int S, int
 __global__ void __launch_bounds__(256) ctx_gather_kernel(const __nv_bfloat16* __restrict__ x, const int32_t* __restrict__ rows,
                                                          const int32_t* __restrict__ count, int P, int S, int H, int r_pad,
                                                          int q_lo, int cap, __nv_bfloat16* __restrict__ xc, int* status) {
-    pdl_launch_dependents();               // the first product may start now: its weight loads need nothing from here
     pdl_wait();                            // the row list comes from the kernel in front
+    pdl_launch_dependents();               // the first product may start now: its weight loads need nothing from here (and the kernel
+                                           // in front, which may have written the weights, is complete)
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= r_pad) return;
     bool bad;

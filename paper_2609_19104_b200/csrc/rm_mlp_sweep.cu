@@ -118,8 +118,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *g_tmem;
+    // A dependent launch itself, whatever is in front: the weights may be what that kernel writes, so nothing is read before
+    // this wait; and what this kernel lets in may count on everything in front of it being complete
+    pdl_wait();
     pdl_launch_dependents();               // (a dependent waits for this grid's end)
-    if (warp != 8) pdl_wait();             // (a dependent launch itself: the first weights need nothing from the kernel in front)
     if (c == 0 && warp < 8) {
         for (int e = tid; e < C_H + 8 * G; e += 256)
             if (e >= 2) a.ctrl[e] = 0;
@@ -161,7 +163,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     dst = lane * 8192;
                     bytes = 8192u * NCB;
                 }
-                if (pass == 1 && ws == 0) pdl_wait();
                 if (pass > 0) WAIT(w_empty(ws), (pass - 1) & 1);
                 gave_up = __any_sync(0xffffffffu, gave_up);
                 if (gave_up) break;

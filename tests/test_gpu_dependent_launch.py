@@ -65,3 +65,134 @@ def test_chain_without_host_waits(lib, H, I, L, T, B, in_place):
         # the step bound covers for 18
         assert float((a - b).norm() / b.norm()) <= REL_L2_TOL, f"output {i}"
     ctx.close()
+
+
+def both_ways(body):
+    """What body(sync) returns with the device idle between the calls and without any wait: every output within the step bound."""
+    import torch
+    outs = []
+    for sync in (torch.cuda.synchronize, lambda: None):
+        torch.cuda.synchronize()
+        outs.append(body(sync))
+        torch.cuda.synchronize()
+    for i, (want, got) in enumerate(zip(*outs)):
+        assert torch.isfinite(got).all() and float((got - want).norm() / want.norm()) <= REL_L2_TOL, f"output {i}"
+
+
+def weights(g, H, I, n):
+    import torch
+    return [[(0.64 / H ** 0.5 * torch.randn(*s, generator=g, device="cuda")).bfloat16() for s in ((I, H), (I, H), (H, I))] for _ in range(n)]
+
+
+@pytest.mark.parametrize("H,I,T,L,variant", [(1024, 4096, 51, 1, 0), (2048, 4096, 20, 2, 0), (1024, 4096, 51, 1, 5), (1024, 4096, 51, 1, 4), (1024, 1000, 51, 1, 1)])
+@pytest.mark.parametrize("front", ["pack", "copy", "drift"])
+def test_dense_steps_behind_the_kernel_that_writes_their_weights(lib, H, I, T, L, variant, front):
+    """Layer 0 is written by the kernel in front of the step, or by the one in front of that (a drift kernel, which lets the step in
+    before it has waited itself)."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(H + T)
+    ctx = lib.Context(L, H, I, T)
+    ctx.rm_set_option("variant", variant)
+    sets = weights(g, H, I, 3 + L - 1)
+    ready = [ctx.rm_pack_weights(*w) for w in sets]
+    layer0 = torch.empty_like(ready[0])
+    layers = [layer0] + ready[3:]
+    r = torch.randn(1, T, H, generator=g, device="cuda").bfloat16().float()
+    out, rec, score = torch.empty_like(r), torch.zeros(1, L, I, device="cuda"), torch.zeros(8, device="cuda")
+    small = torch.randn(8, H, generator=g, device="cuda").bfloat16()
+
+    def body(sync):
+        keep = []
+        for i in range(ROUNDS):
+            if front == "pack":
+                ctx.rm_pack_weights(*sets[i % 3], packed_out=layer0)
+            else:
+                layer0.copy_(ready[i % 3])
+            sync()
+            if front == "drift":
+                ctx.rm_context_drift(small, small, 8, score)
+                sync()
+            ctx.rm_action_expert_step(layers, r, None, None, I, out, records_out=rec)
+            sync()
+            keep += [out.clone(), rec.clone()]
+        return keep
+
+    both_ways(body)
+    assert ctx.rm_get_info("last_variant") == (variant or 7) and ctx.rm_device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("H,I,T,host", [(1024, 4096, 51, False), (2048, 4096, 20, False), (1024, 2048, 51, True)])
+def test_chain_of_the_anchor_schedule_and_of_host_steps(lib, H, I, T, host):
+    """A group: anchor step, a mask of its records, updates with it.  With activations on the device, or host to host."""
+    import torch
+    L, hs = 3, (T + 3) // 4 * 4
+    g = torch.Generator(device="cuda").manual_seed(H + I)
+    ctx = lib.Context(L, H, I, T)
+    layers = [ctx.rm_pack_weights(*w) for w in weights(g, H, I, L)]
+    rs = [torch.randn(1, T, H, generator=g, device="cuda").bfloat16().float() for _ in range(3)]
+    gate = 1.0 + 0.25 * torch.randn(L, 1, H, generator=g, device="cuda")
+    pinned = [r.cpu().pin_memory() for r in rs]
+    host_out = torch.empty(1, T, H).pin_memory()
+
+    def body(sync):
+        ya, ha, rec = torch.zeros(L, 1, T, H, device="cuda"), torch.zeros(L, 1, I, hs, device="cuda"), torch.zeros(1, L, I, device="cuda")
+        idx, cnt = torch.zeros(L, I, dtype=torch.int32, device="cuda"), torch.zeros(L, dtype=torch.int32, device="cuda")
+        out, keep = torch.empty_like(rs[0]), []
+        for i in range(ROUNDS):
+            ctx.rm_action_expert_step_ex(layers, rs[i % 3], None, None, I, out, lib.RM_ANCHOR_WRITE, ya, ha, hs, out_gate=gate, records_out=rec)
+            sync()
+            keep += [out.clone(), ya.clone()]
+            # (the mask comes from other records than the step's: their last bits could move a tie)
+            ctx.rm_mask_compact([ha[:, 0, :, :T].abs().sum(-1).bfloat16().float()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_THRESHOLD, idx, cnt, I,
+                                n_lists=L, threshold=-1.0)
+            sync()
+            if host:
+                keep.append(ctx.rm_action_expert_step_host(layers, pinned[(i + 1) % 3], idx, cnt, I, host_out).clone())
+            else:
+                ctx.rm_action_expert_step_ex(layers, rs[(i + 1) % 3], idx, cnt, I, out, lib.RM_ANCHOR_UPDATE, ya, ha, hs, out_gate=gate)
+                sync()
+                keep.append(out.clone())
+        return keep
+
+    both_ways(body)
+    assert ctx.rm_device_status() == 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("H,I,P,S,R", [(1024, 2048, 300, 16, 96), (2048, 4096, 700, 40, 400)])
+@pytest.mark.parametrize("with_drift", [True, False])
+def test_context_cache_behind_the_kernels_that_write_its_weights(lib, H, I, P, S, R, with_drift):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(H + P)
+    ctx = lib.Context(1, H, I, 64)
+    sets = weights(g, H, I, 3)
+    w = [torch.empty_like(t) for t in sets[0]]
+    xs = [torch.randn(P + S, H, generator=g, device="cuda").bfloat16() for _ in range(3)]
+    ref, y_ref = torch.randn(P, H, generator=g, device="cuda").bfloat16(), torch.randn(P, H, generator=g, device="cuda")
+    fixed = torch.arange(0, 2 * (R - S), 2, dtype=torch.int32, device="cuda")[:R - S].clamp(max=P - 1)
+    fixed = torch.unique(fixed).int()
+    n_fixed = torch.tensor([fixed.numel()], dtype=torch.int32, device="cuda")
+
+    def body(sync):
+        x, score = torch.empty_like(xs[0]), torch.zeros(P, device="cuda")
+        rows, cnt = torch.zeros((P + 3) // 4 * 4, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        y, keep = torch.empty(P + S, H, device="cuda"), []
+        for i in range(ROUNDS):
+            x.copy_(xs[i % 3])
+            for t, new in zip(w, sets[(i + 1) % 3]):
+                t.copy_(new)
+            sync()
+            if with_drift:
+                ctx.rm_context_drift(x, ref, P, score)
+                sync()
+                ctx.rm_mask_compact([score], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, rows, cnt, rows.numel(), n_lists=1, k=R - S, I=P)
+                sync()
+            ctx.rm_context_ffn(*w, x, rows if with_drift else fixed, cnt if with_drift else n_fixed, P, S, R, y_ref, y)
+            sync()
+            keep.append(y.clone())
+        return keep
+
+    both_ways(body)
+    assert ctx.rm_device_status() == 0
+    ctx.close()

@@ -249,7 +249,8 @@ int64_t rm_launch_count(const rm_ctx* ctx);
 /* Tuning knobs (host-side, take effect on later calls).  Names:
  *   "path"                0 = choose per shape (default), 1 = portable CUDA-core kernels only, 2 = the tcgen05
  *                         cluster kernel or RM_ERR_UNSUPPORTED
- *   "pdl"                 1 = chain the layers of a step with programmatic dependent launch (default)
+ *   "pdl"                 1 = launch the kernels as programmatic dependents of the ones in front of them (default); 0 = every
+ *                         kernel of every call starts when the stream's earlier work is complete
  *   "neurons_per_cluster" active neurons a cluster should get before another cluster is used (default 64)
  *   "count_hint"          expected active neurons per layer and episode: the kernel family is chosen by it, and a
  *                         per-layer launch uses only as many clusters as it needs, so that the next layer's CTAs can

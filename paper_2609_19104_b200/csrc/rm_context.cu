@@ -431,7 +431,7 @@ int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap&
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = 2;
     at[1].val.clusterDim.y = 1;
@@ -500,7 +500,7 @@ size_t rm_context_workspace_bytes_impl(const rm_ctx* ctx, int cap) {
 int rm_launch_context_drift(rm_ctx* ctx, const void* x, const void* x_ref, int P, float* score, cudaStream_t s) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((P + 7) / 8);
     cfg.blockDim = dim3(256);
@@ -520,7 +520,7 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
     const int ksplit = pick_ksplit(ctx);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl;
     const int r_pad = pass_rows(cap);
     if (cap <= 256) cap = r_pad;           // (one pass: whatever it holds)
     FfnMaps maps;

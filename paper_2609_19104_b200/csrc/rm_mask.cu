@@ -400,7 +400,7 @@ int launch_mask(rm_ctx* ctx, const MaskParams& p, int n_lists, size_t smem, cuda
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = p.cluster;
     at[1].val.clusterDim.y = 1;

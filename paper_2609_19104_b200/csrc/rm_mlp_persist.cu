@@ -1335,7 +1335,7 @@ int launch(rm_ctx* ctx, const PArgs& a, const CUtensorMap& tmXext, int n_cluster
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = ctx->use_pdl ? 2 : 1;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, step_kernel<HS8, EQ4>, a, tmXext));
     ctx->launches++;
     return RM_OK;

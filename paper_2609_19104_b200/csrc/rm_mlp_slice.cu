@@ -776,7 +776,7 @@ int launch(rm_ctx* ctx, const SArgs& a, int clusters, int smem, cudaStream_t s) 
     cluster_config(cfg, at, clusters, smem, s);
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = ctx->use_pdl ? 2 : 1;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, slice_kernel<HS, NG, TS, EQ4>, a));
     ctx->launches++;
     return RM_OK;

@@ -725,7 +725,7 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, bool dependent, c
     cfg.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    at[0].val.programmaticStreamSerializationAllowed = dependent && ctx->use_pdl ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = CL;
     at[1].val.clusterDim.y = 1;

@@ -501,7 +501,7 @@ int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = ctx->use_pdl ? 1 : 0;
     RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_kernel<HS, EQ4>, a, maps));
     ctx->launches++;
     return RM_OK;

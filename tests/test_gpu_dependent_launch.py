@@ -196,3 +196,57 @@ def test_context_cache_behind_the_kernels_that_write_its_weights(lib, H, I, P, S
     both_ways(body)
     assert ctx.rm_device_status() == 0
     ctx.close()
+
+
+def captured_edges(calls):
+    """(programmatic, other) dependency edges of the calls, captured into a graph that is not run."""
+    import ctypes
+
+    import torch
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        calls()
+    get = ctypes.CDLL("libcuda.so.1").cuGraphGetEdges_v2
+    h, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert get(h, None, None, None, ctypes.byref(n)) == 0
+    ends, data = [(ctypes.c_void_p * n.value)() for _ in range(2)], (ctypes.c_ubyte * 8 * n.value)()
+    assert get(h, ends[0], ends[1], data, ctypes.byref(n)) == 0
+    programmatic = sum(d[2] == 1 for d in data)                      # CUgraphEdgeData: from_port, to_port, type, 5 reserved bytes
+    return programmatic, n.value - programmatic
+
+
+@pytest.mark.parametrize("H,T,B,variant", [(1024, 51, 1, 5), (1024, 51, 1, 7), (1024, 51, 1, 6), (768, 51, 1, 6), (1024, 20, 1, 1), (1024, 51, 4, 4), (2048, 51, 2, 4)])
+def test_option_pdl_governs_every_launch(lib, H, T, B, variant):
+    import torch
+    L, I, P, S = 2, 2048, 96, 8
+    g = torch.Generator(device="cuda").manual_seed(H + T + B)
+    ctx = lib.Context(L, H, I, T, B)
+    ctx.rm_set_option("variant", variant)
+    w = weights(g, H, I, 1)[0]
+    layers = [ctx.rm_pack_weights(*w) for _ in range(L)]
+    r = torch.randn(B, T, H, generator=g, device="cuda").bfloat16().float()
+    out, y = torch.empty_like(r), torch.empty(T, H, device="cuda")
+    rec = torch.rand(B * L, I, generator=g, device="cuda")
+    idx, cnt = torch.zeros(B * L, I, dtype=torch.int32, device="cuda"), torch.zeros(B * L, dtype=torch.int32, device="cuda")
+    x, x_ref = torch.randn(P + S, H, generator=g, device="cuda").bfloat16(), torch.randn(P, H, generator=g, device="cuda").bfloat16()
+    score, rows, n = torch.zeros(P, device="cuda"), torch.zeros(P, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    y_ref, y_ctx = torch.zeros(P, H, device="cuda"), torch.zeros(P + S, H, device="cuda")
+
+    def calls():
+        for _ in range(2):
+            ctx.rm_mask_compact([rec], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, idx, cnt, I, n_lists=B * L, k=I // 4)
+            dense = variant == 7
+            ctx.rm_action_expert_step(layers, r, None if dense else idx, None if dense else cnt, I, out, B=B)
+            assert ctx.rm_get_info("last_variant") == variant
+            ctx.rm_sparse_mlp(layers[0], x[:min(T, P)], None, idx, cnt, y)
+            ctx.rm_context_drift(x, x_ref, P, score)
+            ctx.rm_mask_compact([score], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, rows, n, P, n_lists=1, k=P // 4, I=P)
+            ctx.rm_context_ffn(*w, x, rows, n, P, S, 64, y_ref, y_ctx)
+
+    calls()                                                          # (workspaces, kernel attributes)
+    torch.cuda.synchronize()
+    on = captured_edges(calls)
+    ctx.rm_set_option("pdl", 0)
+    off = captured_edges(calls)
+    assert on[0] >= 10 and off[0] == 0 and off[1] > 0, (on, off)
+    ctx.close()

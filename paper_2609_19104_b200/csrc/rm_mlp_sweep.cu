@@ -40,6 +40,7 @@ constexpr int ASTAGE = 16384, NAS = 4; // activation ring: two 64-column blocks 
 constexpr int NTHREADS = 352;          // warps 0-7 epilogue and normalisation, 8 weights, 9 activations, 10 issuer
 constexpr int OFF_A = NWS * WSTAGE, OFF_MISC = OFF_A + NAS * ASTAGE;
 constexpr int SMEM = OFF_MISC + 2048 + 1024;
+static_assert(512 + 2 * MAXU * UN * 4 <= 2048, "the record sums exceed the miscellaneous area");
 constexpr int TMEM_COLS = 512, D2_COL = 128;                       // D1 at 0 and 64, D2 from 128 (128 columns per 128-column block)
 
 // control block: [CTRL_LINE] token rows normalised, [2 CTRL_LINE] CTAs that have added their part (both cumulative over the
@@ -88,7 +89,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
     volatile uint32_t* g_tmem = reinterpret_cast<volatile uint32_t*>(gbase + OFF_MISC + 272);
     volatile int* sAbort = reinterpret_cast<volatile int*>(gbase + OFF_MISC + 276);
     float* sPart = reinterpret_cast<float*>(gbase + OFF_MISC + 288);       // 8 partial sums of a row
-    float* sRec = reinterpret_cast<float*>(gbase + OFF_MISC + 512);        // record sums of the second token half
+    // record sums of the second token half, layers in turn: a CTA without a split and without a row of x has no barrier between the
+    // reads of one layer and the writes of the next
+    float* sRec = reinterpret_cast<float*>(gbase + OFF_MISC + 512);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c = (int)blockIdx.x, G = (int)gridDim.x;
     const int T = a.T, L = a.L, U = a.U;
@@ -420,7 +423,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     }
                     if (a.record) {
                         rec[v] += __shfl_xor_sync(0xffffffffu, rec[v], 1);
-                        if (ch == 1 && !isup) sRec[unit * UN + nl] = rec[v];
+                        if (ch == 1 && !isup) sRec[(l & 1) * MAXU * UN + unit * UN + nl] = rec[v];
                     }
                 }
                 tc_fence_before();
@@ -433,7 +436,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) sweep_kernel(const __grid_constan
                     for (int v = 0; v < 2; ++v) {
                         const int unit = 4 * v + q4, n = (u0 + unit) * UN + nl;
                         if (unit >= nu || n >= a.I) continue;
-                        const float r = rec[v] + sRec[unit * UN + nl];
+                        const float r = rec[v] + sRec[(l & 1) * MAXU * UN + unit * UN + nl];
                         a.record[(size_t)l * a.I + n] = a.record_scale ? r * a.record_scale[(size_t)l * a.I + n] : r;
                     }
                 }

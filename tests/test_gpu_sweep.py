@@ -56,3 +56,32 @@ def test_anchor_step_matches_the_oracle(lib, H, I, T, L):
         assert np.all(np.abs(h_an.cpu().numpy()[l, 0, :, :T].T - want_h[l]) <= 2e-2 + 1e-2 * np.abs(want_h[l]))
     assert ctx.rm_device_status() == 0
     model.close()
+
+
+@pytest.mark.parametrize("H,I,T,L", [(1024, 4096, 51, 18), (2048, 4000, 64, 12), (1024, 18944, 64, 4)])
+def test_records_of_every_layer_are_that_layers(lib, H, I, T, L):
+    """All CTAs at work, the last of them (of 148: 144 to 147) with neurons but neither a split of the down sweep nor a row of x: nothing
+    but the layers in turn keeps one layer's record sums from the next's."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(H + I)
+    ctx = lib.Context(L, H, I, T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    # Every layer has gate and up weights of its own, but adds next to nothing (columns of 1e-4), so that x differs between the two
+    # kernels in single roundings to bf16 only.  One moves a hidden value by at most 2^-8 |x| |w| |u| = 2^-8 * 4 * 4.5 * 0.64 / sqrt(H) * 3
+    # = 4e-3 at H = 1024; the fp32 sums add sqrt(H T) 2^-24 of a record.  Another layer's sum over the second token half is off by
+    # about its size, 5 to 10.
+    scale = lambda i: 1e-4 if i == 2 else 0.64 / H ** 0.5
+    layers = [ctx.rm_pack_weights(*[(scale(i) * rnd(*s)).bfloat16() for i, s in enumerate(((I, H), (I, H), (H, I)))]) for _ in range(L)]
+    r = rnd(1, T, H).bfloat16().float()
+    out, rec, want = torch.empty_like(r), torch.zeros(1, L, I, device="cuda"), torch.zeros(1, L, I, device="cuda")
+    ctx.rm_set_option("path", 1)
+    ctx.rm_action_expert_step(layers, r, None, None, I, out, records_out=want)
+    ctx.rm_set_option("path", 0)
+    ctx.rm_set_option("variant", 7)
+    for _ in range(5):
+        rec.fill_(-1.0)
+        ctx.rm_action_expert_step(layers, r, None, None, I, out, records_out=rec)
+        assert ctx.rm_get_info("last_variant") == 7
+        assert torch.all((rec - want).abs() <= 1e-3 * want + 5e-3)
+    assert ctx.rm_device_status() == 0
+    ctx.close()

@@ -297,13 +297,15 @@ class Context:
         return y
 
     def _layer_ptrs(self, packed_layers):
+        if len(packed_layers) < self.L:
+            raise ValueError(f"{len(packed_layers)} packed layers for a model of {self.L}")
         return (ctypes.c_void_p * len(packed_layers))(*[_ptr(p) for p in packed_layers])
 
     def rm_action_expert_step(self, packed_layers, r_in, idx, count_dev, stride: int, r_out, records_out=None,
                               record_scale=None, B: int = 1, T: Optional[int] = None, ws=None):
         T = int(r_in.shape[-2]) if T is None else T
         ws, ws_bytes = self._scratch(B, T, ws)
-        _check(_native.step(self._hv, packed_layers, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T, ws,
+        _check(_native.step(self._hv, packed_layers, self.L, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T, ws,
                             ws_bytes), "rm_action_expert_step")
         return r_out
 
@@ -313,7 +315,7 @@ class Context:
         """The step with the anchor-relative update (Eq. 4): y_anchor [L,B,T,H], h_anchor [L,B,I,h_stride] fp32."""
         T = int(r_in.shape[-2]) if T is None else T
         ws, ws_bytes = self._scratch(B, T, ws)
-        _check(_native.step_ex(self._hv, packed_layers, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T,
+        _check(_native.step_ex(self._hv, packed_layers, self.L, r_in, idx, count_dev, stride, r_out, records_out, record_scale, B, T,
                                anchor_mode, y_anchor, h_anchor, h_stride, out_gate, ws, ws_bytes), "rm_action_expert_step_ex")
         return r_out
 
@@ -322,7 +324,7 @@ class Context:
         """r_in_host / r_out_host are CPU tensors (pinned for asynchronous copies); returns after the result landed."""
         T = int(r_in_host.shape[-2]) if T is None else T
         ws, ws_bytes = self._scratch(B, T, ws)
-        _check(_native.step_host(self._hv, packed_layers, r_in_host, idx, count_dev, stride, r_out_host, B, T, ws, ws_bytes),
+        _check(_native.step_host(self._hv, packed_layers, self.L, r_in_host, idx, count_dev, stride, r_out_host, B, T, ws, ws_bytes),
                "rm_action_expert_step_host")
         return r_out_host
 

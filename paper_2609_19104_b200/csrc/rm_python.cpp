@@ -3,10 +3,12 @@
 // A call of this library can be shorter on the GPU than its marshalling through ctypes was on the host (a mask compaction:
 // 8 us of Python and ctypes for ~5 us of kernel; 18 layer pointers alone: 7 us).  These functions take the tensors
 // themselves, read their data pointers, and release the interpreter lock around the call.  Integer arguments may be
-// anything int() accepts; a tensor argument may be None (NULL).
+// anything int() accepts, within the range of the C argument; a tensor argument may be None (NULL).
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <climits>
+#include <new>
 #include <vector>
 
 #include "rmuscle.h"
@@ -44,11 +46,27 @@ struct Args {                              // positional arguments, converted on
         if (v == -1 && PyErr_Occurred()) bad = true;
         return v;
     }
+    int i32() {
+        const long long v = integer();
+        if (!bad && (v < INT_MIN || v > INT_MAX)) {
+            PyErr_Format(PyExc_OverflowError, "argument %zd is outside the range of a 32-bit integer", i - 1);
+            bad = true;
+        }
+        return bad ? 0 : (int)v;
+    }
+    bool truth() {
+        PyObject* o = next();
+        const int v = bad ? 0 : PyObject_IsTrue(o);
+        if (v < 0) bad = true;
+        return v > 0;
+    }
     double real() {
         PyObject* o = next();
         if (bad) return 0.0;
-        const double v = PyFloat_AsDouble(o);
-        if (v == -1.0 && PyErr_Occurred()) bad = true;
+        PyObject* f = PyNumber_Float(o);
+        if (!f) { bad = true; return 0.0; }
+        const double v = PyFloat_AS_DOUBLE(f);
+        Py_DECREF(f);
         return v;
     }
     static void* pointer_of(PyObject* o, bool& bad) {
@@ -71,9 +89,29 @@ struct Args {                              // positional arguments, converted on
         PyObject* s = PySequence_Fast(o, "a sequence of tensors is expected");
         if (!s) { bad = true; return; }
         const Py_ssize_t m = PySequence_Fast_GET_SIZE(s);
-        out.resize((size_t)m);
+        try {
+            out.resize((size_t)m);
+        } catch (const std::bad_alloc&) {
+            PyErr_NoMemory();
+            bad = true;
+        }
         for (Py_ssize_t k = 0; k < m && !bad; ++k) out[(size_t)k] = pointer_of(PySequence_Fast_GET_ITEM(s, k), bad);
         Py_DECREF(s);
+    }
+    void layers(std::vector<void*>& out) { // a sequence of a step's packed layers, then their number: the call reads that many
+        pointers(out);
+        const int L = i32();
+        if (!bad && (long long)out.size() < L) {
+            PyErr_Format(PyExc_ValueError, "%zd packed layers for a model of %d", (Py_ssize_t)out.size(), L);
+            bad = true;
+        }
+    }
+    bool done() {                          // every argument has been read
+        if (!bad && i != n) {
+            PyErr_Format(PyExc_TypeError, "%zd arguments where %zd are expected", n, i);
+            bad = true;
+        }
+        return !bad;
     }
     rm_ctx* context() { return reinterpret_cast<rm_ctx*>((uintptr_t)integer()); }
 };
@@ -110,19 +148,19 @@ RM_FN(mask_compact) {
     std::vector<void*> rec;
     in.pointers(rec);
     rm_mask_src s{};
-    s.kind = (int32_t)in.integer();
-    s.reduce = (int32_t)in.integer();
+    s.kind = in.i32();
+    s.reduce = in.i32();
     s.threshold = (float)in.real();
-    s.k = (int32_t)in.integer();
-    s.min_votes = (int32_t)in.integer();
+    s.k = in.i32();
+    s.min_votes = in.i32();
     s.scale = in.pointer<const float>();
-    s.scale_per_list = in.integer() != 0;
-    s.n_lists = (int32_t)in.integer();
-    s.I = (int32_t)in.integer();
+    s.scale_per_list = in.truth();
+    s.n_lists = in.i32();
+    s.I = in.i32();
     int32_t* idx = in.pointer<int32_t>();
     int32_t* cnt = in.pointer<int32_t>();
     const int64_t stride = in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     s.n_records = (int32_t)rec.size();
     if (rec.empty()) rec.push_back(nullptr);
     s.records = rec.data();
@@ -137,10 +175,10 @@ RM_FN(sparse_mlp) {
     float* r = in.pointer<float>();
     int32_t *idx = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
     float *y = in.pointer<float>(), *rec = in.pointer<float>(), *sc = in.pointer<float>();
-    const int T = (int)in.integer();
+    const int T = in.i32();
     void* ws = in.pointer();
     const size_t nws = (size_t)in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_sparse_mlp(ctx, packed, x, r, idx, cnt, y, rec, sc, T, ws, nws, st); });
 }
 
@@ -151,66 +189,66 @@ RM_FN(sparse_mlp_static) {
     float* r = in.pointer<float>();
     int32_t *idx = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
     float* y = in.pointer<float>();
-    const int T = (int)in.integer(), H = (int)in.integer(), I = (int)in.integer();
-    void* st = current_stream(in.bad);
+    const int T = in.i32(), H = in.i32(), I = in.i32();
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_sparse_mlp_static(packed, x, r, idx, cnt, y, T, H, I, st); });
 }
 
-// (ctx, layers, r_in, idx, count, stride, r_out, records_out, record_scale, B, T, ws, ws_bytes)
+// (ctx, layers, L, r_in, idx, count, stride, r_out, records_out, record_scale, B, T, ws, ws_bytes)
 RM_FN(step) {
     Args in{args, n_args};
     rm_ctx* ctx = in.context();
     std::vector<void*> layers;
-    in.pointers(layers);
+    in.layers(layers);
     float* r_in = in.pointer<float>();
     int32_t *idx = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
     const int64_t stride = in.integer();
     float *r_out = in.pointer<float>(), *rec = in.pointer<float>(), *sc = in.pointer<float>();
-    const int B = (int)in.integer(), T = (int)in.integer();
+    const int B = in.i32(), T = in.i32();
     void* ws = in.pointer();
     const size_t nws = (size_t)in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_action_expert_step(ctx, layers.data(), r_in, idx, cnt, stride, r_out, rec, sc, B, T, ws, nws, st); });
 }
 
-// (ctx, layers, r_in, idx, count, stride, r_out, records_out, record_scale, B, T, anchor_mode, y_anchor, h_anchor, h_stride,
+// (ctx, layers, L, r_in, idx, count, stride, r_out, records_out, record_scale, B, T, anchor_mode, y_anchor, h_anchor, h_stride,
 //  out_gate, ws, ws_bytes)
 RM_FN(step_ex) {
     Args in{args, n_args};
     rm_ctx* ctx = in.context();
     std::vector<void*> layers;
-    in.pointers(layers);
+    in.layers(layers);
     float* r_in = in.pointer<float>();
     int32_t *idx = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
     const int64_t stride = in.integer();
     float *r_out = in.pointer<float>(), *rec = in.pointer<float>(), *sc = in.pointer<float>();
-    const int B = (int)in.integer(), T = (int)in.integer(), mode = (int)in.integer();
+    const int B = in.i32(), T = in.i32(), mode = in.i32();
     float *ya = in.pointer<float>(), *ha = in.pointer<float>();
     const int64_t hs = in.integer();
     float* gate = in.pointer<float>();
     void* ws = in.pointer();
     const size_t nws = (size_t)in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] {
         return rm_action_expert_step_ex(ctx, layers.data(), r_in, idx, cnt, stride, r_out, rec, sc, B, T, mode, ya, ha, hs, gate,
                                         ws, nws, st);
     });
 }
 
-// (ctx, layers, r_in_host, idx, count, stride, r_out_host, B, T, ws, ws_bytes)
+// (ctx, layers, L, r_in_host, idx, count, stride, r_out_host, B, T, ws, ws_bytes)
 RM_FN(step_host) {
     Args in{args, n_args};
     rm_ctx* ctx = in.context();
     std::vector<void*> layers;
-    in.pointers(layers);
+    in.layers(layers);
     float* r_in = in.pointer<float>();
     int32_t *idx = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
     const int64_t stride = in.integer();
     float* r_out = in.pointer<float>();
-    const int B = (int)in.integer(), T = (int)in.integer();
+    const int B = in.i32(), T = in.i32();
     void* ws = in.pointer();
     const size_t nws = (size_t)in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_action_expert_step_host(ctx, layers.data(), r_in, idx, cnt, stride, r_out, B, T, ws, nws, st); });
 }
 
@@ -219,9 +257,9 @@ RM_FN(context_drift) {
     Args in{args, n_args};
     rm_ctx* ctx = in.context();
     void *x = in.pointer(), *xr = in.pointer();
-    const int P = (int)in.integer();
+    const int P = in.i32();
     float* score = in.pointer<float>();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_context_drift(ctx, x, xr, P, score, st); });
 }
 
@@ -231,11 +269,11 @@ RM_FN(context_ffn) {
     rm_ctx* ctx = in.context();
     void *wg = in.pointer(), *wu = in.pointer(), *wd = in.pointer(), *x = in.pointer();
     int32_t *rows = in.pointer<int32_t>(), *cnt = in.pointer<int32_t>();
-    const int P = (int)in.integer(), S = (int)in.integer(), R = (int)in.integer();
+    const int P = in.i32(), S = in.i32(), R = in.i32();
     float *yr = in.pointer<float>(), *yo = in.pointer<float>();
     void* ws = in.pointer();
     const size_t nws = (size_t)in.integer();
-    void* st = current_stream(in.bad);
+    void* st = in.done() ? current_stream(in.bad) : nullptr;
     return call(in, [&] { return rm_context_ffn(ctx, wg, wu, wd, x, rows, cnt, P, S, R, yr, yo, ws, nws, st); });
 }
 

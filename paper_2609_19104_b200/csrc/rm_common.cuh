@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "rmuscle.h"
 
 // Packed layer layout (private to the library).  Neuron n owns 3*H bf16 stored contiguously.  The chunk is cut
@@ -51,6 +53,7 @@ struct rm_ctx {
     int persist_clusters;                  // co-resident 8-CTA clusters of the whole-step kernel (0: unavailable)
     int persist_prefetch_kb;               // weight KB a CTA of the whole-step kernel may ask into L2 ahead of its loaders
     int persist_max_b;                     // largest batch the whole-step kernel is chosen for when the variant is automatic
+    std::mutex sweep_mutex;
     const void* sweep_key[64];             // layers whose tensor maps the sweep kernel has (NULL: none yet)
     alignas(64) unsigned char sweep_maps[2 * 64 * 128];
 };

@@ -528,10 +528,14 @@ size_t rm_sweep_workspace_bytes(const rm_ctx* ctx) {
 // Dense steps of one episode: no lists, no anchor state or the anchor step of Eq. 4
 int rm_launch_step_sweep(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStream_t s) {
     const rm_geom& g = ctx->g;
-    WMaps* maps = reinterpret_cast<WMaps*>(ctx->sweep_maps);       // (encoded again only for layers whose address has changed)
+    // The maps are encoded again only for layers whose address has changed.  The context may serve several threads with models of
+    // their own: they take turns from here to the launch, which copies the maps.
+    std::lock_guard<std::mutex> lock(ctx->sweep_mutex);
+    WMaps* maps = reinterpret_cast<WMaps*>(ctx->sweep_maps);
     static_assert(sizeof(WMaps) == sizeof(ctx->sweep_maps), "the context holds the tensor maps");
     for (int l = 0; l < sa.L; ++l) {
         if (ctx->sweep_key[l] == sa.packed_layers[l]) continue;
+        ctx->sweep_key[l] = nullptr;
         int rc = rm_make_weight_map(&maps->gu[l], sa.packed_layers[l], g.I, 3 * g.H, UN, g.Hs);
         if (rc == RM_OK) rc = rm_make_weight_map(&maps->dn[l], sa.packed_layers[l], g.I, 3 * g.H, 4 * UN, 0);
         if (rc != RM_OK) return rc;

@@ -1,0 +1,118 @@
+"""Several host threads and streams at once: every call has its own stream, workspace and buffers, as the header asks, and gives what it
+gives alone.  Steps whose CTAs wait for one another share the device with others of their kind and with ordinary kernels."""
+import threading
+
+import pytest
+
+from harness import REL_L2_TOL
+
+pytestmark = pytest.mark.gpu
+
+ROUNDS = 40
+
+
+class Job:
+    """A model, and steps with it on a stream of its own.  `ctx`: shared with other jobs of the same geometry, or its own."""
+
+    def __init__(self, lib, H, I, L, T, K, B=1, seed=0, ctx=None, priority=0):
+        import torch
+        g = torch.Generator(device="cuda").manual_seed(H + I + T + seed)
+        rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+        self.ctx = ctx or lib.Context(L, H, I, T, B)
+        self.layers = [self.ctx.rm_pack_weights(*[(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))]) for _ in range(L)]
+        self.B, self.stride = B, (I + 3) // 4 * 4
+        self.idx = self.cnt = None
+        if K:
+            self.idx = torch.zeros(B * L, self.stride, dtype=torch.int32, device="cuda")
+            self.cnt = torch.zeros(B * L, dtype=torch.int32, device="cuda")
+            self.ctx.rm_mask_compact([rnd(B * L, I).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, self.idx, self.cnt, self.stride,
+                                     n_lists=B * L, k=K)
+        self.r = rnd(B, T, H).bfloat16().float()
+        self.ws = torch.empty(self.ctx.workspace_bytes(B, T), dtype=torch.uint8, device="cuda")
+        self.out = torch.empty_like(self.r)
+        self.K = K
+        self.step()
+        self.want = self.out.clone()
+        self.variant = self.ctx.rm_get_info("last_variant")
+        torch.cuda.synchronize()
+        assert self.ctx.rm_device_status() == 0
+        self.stream, self.worst, self.error = torch.cuda.Stream(priority=priority), None, None
+
+    def step(self):
+        self.ctx.rm_action_expert_step(self.layers, self.r, self.idx, self.cnt, self.stride, self.out, B=self.B, ws=self.ws)
+
+    def loop(self):
+        import torch
+        try:
+            with torch.cuda.stream(self.stream):
+                errors = []
+                for _ in range(ROUNDS):
+                    self.out.fill_(7.0)
+                    self.step()
+                    errors.append((self.out - self.want).norm() / self.want.norm())
+                self.worst = float(torch.stack(errors).max())
+        except Exception as e:                                       # (a thread's exception would be lost)
+            self.error = e
+
+
+def run(jobs):
+    import torch
+    threads = [threading.Thread(target=j.loop) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for i, j in enumerate(jobs):
+        assert j.error is None, j.error
+        assert j.ctx.rm_device_status() == 0 and j.worst <= REL_L2_TOL, (i, j.worst)
+    for j in jobs:
+        j.ctx.close()
+
+
+@pytest.mark.parametrize("a,b", [
+    ((1536, 4096, 4, 51, 1000), (768, 2048, 6, 20, 500)),             # slice kernels
+    ((1536, 4096, 4, 51, 1000), (1024, 4096, 4, 51, 1400)),           # slice and whole-step kernel
+    ((1024, 4096, 4, 51, 1400), (2048, 4096, 3, 40, 2000)),           # whole-step kernels
+    ((1024, 4096, 4, 51, 0), (2048, 5000, 3, 64, 0)),                 # sweep kernels
+    ((1024, 4096, 4, 51, 0), (1536, 4096, 4, 100, 700)),              # sweep and slice kernel
+    ((1024, 4096, 4, 51, 1400), (1024, 4096, 4, 51, 900, 6)),         # whole-step and streaming kernel
+])
+def test_two_models_on_two_streams(lib, a, b):
+    run([Job(lib, *a), Job(lib, *b)])
+
+
+def test_four_streams(lib):
+    run([Job(lib, 1536, 4096, 3, 51, 1000), Job(lib, 1024, 4096, 3, 51, 1400), Job(lib, 1024, 4096, 3, 51, 0), Job(lib, 1024, 4096, 3, 20, 300)])
+
+
+def test_threads_that_share_a_context(lib):
+    """Two models of one geometry through one context: dense steps, whose tensor maps the context keeps by layer."""
+    ctx = lib.Context(3, 1024, 4096, 51)
+    run([Job(lib, 1024, 4096, 3, 51, 0, seed=s, ctx=ctx) for s in range(3)])
+
+
+@pytest.mark.parametrize("job", [(1536, 4096, 4, 51, 1000), (1024, 4096, 4, 51, 1400), (1024, 4096, 4, 51, 0)])
+def test_beside_ordinary_kernels(lib, job):
+    """A step with matrix products of another stream on the device."""
+    import torch
+    j = Job(lib, *job)
+    a = torch.randn(4096, 4096, device="cuda").bfloat16()
+    other, go = torch.cuda.Stream(), threading.Event()
+
+    def products():
+        with torch.cuda.stream(other):
+            b = a
+            while not go.is_set():
+                for _ in range(8):
+                    b = a @ a
+                other.synchronize()
+
+    t = threading.Thread(target=products)
+    t.start()
+    j.loop()
+    go.set()
+    t.join()
+    torch.cuda.synchronize()
+    assert j.error is None and j.ctx.rm_device_status() == 0 and j.worst <= REL_L2_TOL, (j.error, j.worst)
+    j.ctx.close()

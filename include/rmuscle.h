@@ -14,6 +14,11 @@
  *     unless its comment says so.  Argument validation is synchronous and returns a negative rm_status.
  *   - Conditions detected on the device (index >= I, count > stride) never trap: the kernel clamps or skips,
  *     records the code in the context's status word, and rm_device_status reports it.
+ *   - Steps (and one-layer calls of widths other than 1024 and 2048 or of more than 64 tokens) may run as one kernel with a
+ *     CTA on most of the SMs, whose CTAs wait for one another ("last_variant" 5, 6, 7).  Other streams' kernels may hold SMs meanwhile:
+ *     the resident CTAs wait at least 10 s for the others, then give up (RM_ERR_TIMEOUT).  Such calls of several streams of equal
+ *     priority take their turns; on streams of different priority each could hold SMs that the other needs, so order those by
+ *     events, or use rm_set_option("path", 1), whose kernels never wait for one another.
  *   - Index lists are strictly ascending int32.  The number of valid entries is read from DEVICE memory, so a
  *     list built by rm_mask_compact can be consumed without a host round trip.  A count of 0 is legal.
  */
@@ -60,7 +65,8 @@ int rm_destroy(rm_ctx* ctx);
  * up row and down column stored next to one another so that one active neuron is one contiguous read). */
 size_t rm_packed_layer_bytes(const rm_ctx* ctx);
 
-/* Bytes of scratch that rm_sparse_mlp / rm_action_expert_step need for B episodes of T tokens. */
+/* Bytes of scratch that rm_sparse_mlp / rm_action_expert_step need for B episodes of T tokens.  The contents do not matter and are not
+ * kept: calls of any size may follow one another on one workspace.  Calls that overlap on the device need one each. */
 size_t rm_workspace_bytes(const rm_ctx* ctx, int B, int T);
 
 /* One-off repacking of a layer (not on the timed path).

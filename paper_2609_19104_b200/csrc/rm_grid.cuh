@@ -7,7 +7,10 @@
 // other calls, of other sizes, use the same workspace.
 //
 // Every wait is bounded and returns true when the waiter has to give up: the wait ran out (status RM_ERR_TIMEOUT with the
-// wait's source line and the CTA), or this CTA or the grid is aborting.
+// wait's source line and the CTA), or this CTA or the grid is aborting.  The bounds are 10 s and more: a CTA that is resident
+// waits for those that are not yet, which is as long as another stream's kernel holds their SMs.  (A look at a counter takes 0.16
+// us when nobody else looks, one at a word in shared memory 20 ns; mbarrier.try_wait takes 0.1 to 4 us, so those waits go by the
+// clock as well.)
 #pragma once
 #include "rm_common.cuh"
 #include "rm_sm100.cuh"
@@ -15,6 +18,17 @@
 namespace grid {
 
 constexpr int CTRL_LINE = 32;
+constexpr uint32_t COUNTER_POLLS = 1u << 26, SHARED_POLLS = 1u << 29, BARRIER_POLLS = 1u << 27;
+// Time limit of a wait, looked at now and then (first look: the wait begins)
+struct Limit {
+    unsigned long long begin = 0;
+    __device__ __forceinline__ bool over() {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (!begin) begin = t;
+        return t - begin > 12000000000ull;
+    }
+};
 
 __device__ __forceinline__ int ld_acquire_gpu(const int* p) {
     int v;
@@ -39,12 +53,16 @@ __device__ __forceinline__ void report_timeout(const A& a, volatile int* abort_c
 }
 template <class A>
 __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, const A& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 22); ++i) {
+    Limit limit;
+    for (uint32_t i = 0; i < BARRIER_POLLS; ++i) {
         if (sm100::mbar_try_wait(bar, parity)) return false;
         if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && (*abort_cta || ((i & 16383u) == 16383u && aborting(a)))) {
-            *abort_cta = 1;
-            return true;
+        if ((i & 1023u) == 1023u) {
+            if (*abort_cta || ((i & 16383u) == 16383u && aborting(a))) {
+                *abort_cta = 1;
+                return true;
+            }
+            if (limit.over()) break;
         }
     }
     report_timeout(a, abort_cta, line);
@@ -52,7 +70,7 @@ __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, int lin
 }
 template <class A>
 __device__ __forceinline__ bool counter_wait(const int* counter, int target, int line, const A& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 21); ++i) {
+    for (uint32_t i = 0; i < COUNTER_POLLS; ++i) {
         if (ld_acquire_gpu(counter) >= target) return false;
         if ((i & 255u) == 255u && (*abort_cta || aborting(a))) { *abort_cta = 1; return true; }
     }
@@ -61,7 +79,7 @@ __device__ __forceinline__ bool counter_wait(const int* counter, int target, int
 }
 template <class A>
 __device__ __forceinline__ bool epoch_wait(const int* ctrl, unsigned long long epoch, int line, const A& a, volatile int* abort_cta) {
-    for (uint32_t i = 0; i < (1u << 21); ++i) {
+    for (uint32_t i = 0; i < COUNTER_POLLS; ++i) {
         unsigned long long v;
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(ctrl) : "memory");
         if (v == epoch) return false;

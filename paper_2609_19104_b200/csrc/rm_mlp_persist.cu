@@ -141,7 +141,7 @@ __device__ __forceinline__ int ld_relaxed_cta(const int* p) {          // shared
 // loop: returns the count once it exceeds `stage`, or what it last read when the bounded wait ran out or the CTA aborts.
 __device__ __noinline__ uint32_t landed_stages(const int* count, uint32_t stage, const int* abort_flag) {
     uint32_t ready = 0;
-    for (uint32_t i = 0; i < (1u << 24); ++i) {
+    for (uint32_t i = 0; i < grid::SHARED_POLLS; ++i) {
         ready = (uint32_t)ld_relaxed_cta(count);
         if (stage < ready) break;
         if ((i & 4095u) == 4095u && *reinterpret_cast<const volatile int*>(abort_flag)) break;
@@ -159,12 +159,16 @@ __device__ __noinline__ void report_timeout(int* status, volatile int* abort_fla
 // has to give up: the wait ran out (status RM_ERR_TIMEOUT with the wait's source line and the CTA), or this CTA or the
 // grid is aborting.
 __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, volatile int* abort_flag, int* ctrl, int tag, int* status) {
-    for (uint32_t i = 0; i < (1u << 22); ++i) {
+    grid::Limit limit;
+    for (uint32_t i = 0; i < grid::BARRIER_POLLS; ++i) {
         if (mbar_try_wait(bar, parity)) return false;
         if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && (*abort_flag || ((i & 16383u) == 16383u && ld_acquire_gpu(ctrl + 3) == tag))) {
-            *abort_flag = 1;
-            return true;
+        if ((i & 1023u) == 1023u) {
+            if (*abort_flag || ((i & 16383u) == 16383u && ld_acquire_gpu(ctrl + 3) == tag)) {
+                *abort_flag = 1;
+                return true;
+            }
+            if (limit.over()) break;
         }
     }
     report_timeout(status, abort_flag, ctrl, tag, line);
@@ -173,7 +177,7 @@ __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, 
 // A bounded wait for a counter in global memory, out of line (for the path that is rarely taken).  Returns true when
 // the waiter has to give up.
 __device__ __noinline__ bool counter_wait_slow(const int* counter, int target, int line, volatile int* abort_flag, int* ctrl, int tag, int* status) {
-    for (uint32_t i = 0; i < (1u << 21); ++i) {
+    for (uint32_t i = 0; i < grid::COUNTER_POLLS; ++i) {
         if (ld_acquire_gpu(counter) >= target) return false;
         if ((i & 255u) == 255u && aborting(abort_flag, ctrl, tag)) { *abort_flag = 1; return true; }
     }
@@ -688,10 +692,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                     if (!ext) {
                         const uint32_t rph = (k.use >> 1) & 1;
                         bool ok = false;
-                        for (uint32_t i = 0; i < (1u << 22) && !ok; ++i) {
+                        grid::Limit limit;
+                        for (uint32_t i = 0; i < grid::BARRIER_POLLS && !ok; ++i) {
                             ok = mbar_try_wait_cluster(x_ready(slot), rph);
                             if (!ok && i > 64) __nanosleep(32);
-                            if ((i & 1023u) == 1023u && *sAbort) break;
+                            if ((i & 1023u) == 1023u && (*sAbort || limit.over())) break;
                         }
                         if (!ok) { if (!*sAbort) timed_out(__LINE__); gave_up = true; break; }
                         if (xq == 0) RM_PS(k.item, 0);
@@ -911,7 +916,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                 // that the last arrivals have to get through); the barrier passes its acquire on to the others
                 if (et == 0 && !gave_up) {
                     bool ok = false;
-                    for (uint32_t i = 0; i < (1u << 21); ++i) {
+                    for (uint32_t i = 0; i < grid::COUNTER_POLLS; ++i) {
                         if (ld_acquire_gpu(counter) >= target) { ok = true; break; }
                         if ((i & 255u) == 255u && aborting(sAbort, a.ctrl, tag)) break;
                     }
@@ -1177,7 +1182,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
                     // r has to hold its copy of r_in before anything is added to it
                     if (lane == 0 && !gave_up) {
                         bool ok = false;
-                        for (uint32_t w8 = 0; w8 < (1u << 21); ++w8) {
+                        for (uint32_t w8 = 0; w8 < grid::COUNTER_POLLS; ++w8) {
                             if (ld_acquire_gpu(a.sync + SYNC_COPY + b) >= pre) { ok = true; break; }
                             if ((w8 & 255u) == 255u && aborting(sAbort, a.ctrl, tag)) break;
                         }

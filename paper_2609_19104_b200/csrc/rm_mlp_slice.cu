@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) slice_kernel(const __grid_constan
             // the layer before is complete (group A's first thread has seen it): what this CTA reads of it and writes over it below
             if (bt == 0 && !gave_up) {
                 int seen = 0;
-                for (uint32_t i = 0; i < (1u << 24); ++i) {
+                for (uint32_t i = 0; i < SHARED_POLLS; ++i) {
                     asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(seen) : "r"(smem_u32(&sSeen)) : "memory");
                     if (seen > pi || *sAbort) break;
                 }

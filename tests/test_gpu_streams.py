@@ -116,3 +116,44 @@ def test_beside_ordinary_kernels(lib, job):
     torch.cuda.synchronize()
     assert j.error is None and j.ctx.rm_device_status() == 0 and j.worst <= REL_L2_TOL, (j.error, j.worst)
     j.ctx.close()
+
+
+HOLD = r"""
+extern "C" __global__ void hold(int ms) {
+    extern __shared__ char room[];
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+    for (int i = 0; i < 8000; ++i) {                   /* (4 s at most, whatever the timer says) */
+        __nanosleep(500000);
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        if (t - t0 > (unsigned long long)ms * 1000000ull) break;
+    }
+}
+"""
+
+
+@pytest.mark.parametrize("job", [(1536, 4096, 4, 51, 1000), (1024, 4096, 4, 51, 1400), (1024, 4096, 4, 51, 0)])
+def test_device_shared_with_a_kernel_that_holds_sms_for_long(lib, job):
+    """100 of the SMs belong to another stream's kernel for 2 s.  Some of the step's CTAs are resident meanwhile and wait for the others:
+    the step is late, not wrong."""
+    import torch
+    j = Job(lib, *job)
+    hold = torch.cuda._compile_kernel(HOLD, "hold")
+    room = 200 * 1024
+    hold.set_shared_memory_config(room)
+    other, start, end = torch.cuda.Stream(), torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    hold(grid=(1, 1, 1), block=(32, 1, 1), args=[1], shared_mem=room, stream=other)
+    torch.cuda.synchronize()
+    start.record(j.stream)
+    hold(grid=(100, 1, 1), block=(32, 1, 1), args=[2000], shared_mem=room, stream=other)
+    with torch.cuda.stream(j.stream):
+        torch.cuda._sleep(2_000_000)                                   # (the other kernel is on the device first)
+        j.out.fill_(7.0)
+        j.step()
+    end.record(j.stream)
+    torch.cuda.synchronize()
+    status = j.ctx.rm_device_status()
+    assert status == 0, f"wait at line {j.ctx.rm_get_info('status_detail') >> 12} after {start.elapsed_time(end):.0f} ms"
+    assert start.elapsed_time(end) > 1500, "the step was not held up: the test shows nothing"
+    assert float((j.out - j.want).norm() / j.want.norm()) <= REL_L2_TOL
+    j.ctx.close()

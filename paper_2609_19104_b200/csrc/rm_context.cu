@@ -6,24 +6,24 @@
 // block arriving as one cp.async.bulk.tensor box:
 //   gather  : Xc[r,:] = x[rows[r],:]                                   (R_pad rows, zero beyond the list)
 //   phase A : H1[r, n] = bf16(gelu_tanh(<Xc_r, Wg_n>) * <Xc_r, Wu_n>)  one CTA per <= 128 neurons, K = H
-//   phase B : y_out[rows[r], c] += sum over the s-th slice of n of H1[r, n] Wd[c, n]   one CTA per (128 columns, K slice)
-// (phase A's idle warps clear the output rows of the list and copy the kept reference rows)
+//   phase B : yp[s, r, c] = sum over the s-th slice of n of H1[r, n] Wd[c, n]           one CTA per (128 columns, K slice)
+//   sum     : y_out[rows[r], c] = sum over s of yp[s, r, c], in the order of s: the same bits every time
+// (phase A's idle warps copy the kept reference rows)
 // Both products are D[256 x N] (+)= A[256 x 64] B[N x 64]^T per stage, by pairs of CTAs (cta_group::2): A = weight rows (K
 // contiguous, as the model stores them), 128 per CTA; B = activation rows, half of them in each CTA; fp32 accumulators in tensor
 // memory (phase A holds two, gate and up: all 512 columns at N = 256).  What bounds a product is what an SM can take in, ~30
 // bytes per clock: a pair halves the activations each CTA loads (48 instead of 64 KB a stage in phase A, 32 instead of 48 in
 // phase B).  Activation rows are padded to a multiple of 32; a CTA of phase A has as many neurons as spread
-// them over all SMs (112 instead of 128 at H = 2048, I = 16384); phase B adds its K slices to the output through the copy
-// engine.
+// them over all SMs (112 instead of 128 at H = 2048, I = 16384); phase B's K slices are stored by the copy engine and summed by
+// a kernel of its own.
 //
-// Drift, selection and recomputation of 240 of 816 rows at H = 2048, I = 16384 (us a pass): single CTAs and a kernel summing the
-// slices 78.9, pairs 71.9, without that kernel and on all SMs 67.7, eight epilogue warps and a warp per copied row 63.9 (96 rows
-// 61.5 -> 56, 366 rows 122 -> 110).  In time: drift 4 - 6, selection 6, gather 3, phase A 22 and its epilogue 4 (two
-// MUFU operations per value), 3 to the next kernel, phase B 10, its additions 4 (an SM's copy engine adds ~16 bytes per clock;
-// red.global.add.v4 from the threads instead: +5).  The products take in 30 bytes per clock and SM and run at the rate of HBM,
-// so that fetching further weights into L2 ahead of time (while phase A waits for its rows, or for phase B) does not help
-// (0.4 - 2 us slower).  Both phases in one kernel would save the 3 us between them, but its CTAs would wait on one another, and
-// a call has to run beside whatever else is on the device.
+// Drift, selection and recomputation of 240 of 816 rows at H = 2048, I = 16384, calls back to back (the power limit holds the clock
+// at ~1.67 GHz): 75.5 us, of which the sums' kernel is 4.5 (adding the slices to the output in the order of arrival by the copy
+// engine: 71.0, but no two runs agree); single CTAs instead of pairs +7, products not on all SMs +2.  In time, at 1.97 GHz: drift
+// 4 - 6, selection 6, gather 3, phase A 22 and its epilogue 4 (two MUFU operations per value), 3 to the next kernel, phase B 10.
+// The products take in 30 bytes per clock and SM and run at the rate of HBM, so that fetching further weights into L2 ahead of
+// time (while phase A waits for its rows, or for phase B) does not help (0.4 - 2 us slower).  Both phases in one kernel would save
+// the 3 us between them, but its CTAs would wait on one another, and a call has to run beside whatever else is on the device.
 #include <cuda.h>
 
 #include <mutex>
@@ -149,8 +149,7 @@ __device__ __forceinline__ bool listed(const int32_t* list, int c, int p, int la
 //   PACKED   up to 64 neurons: Wg rows in the upper half of one tile, Wu rows in the lower one, one accumulator; half the
 //            products of WIDE, whose tiles would be half empty (H = 1024, I = 4096, 32 neurons per CTA, 240 rows: the products
 //            alone took 8 us of phase A's 11)
-// Phase B (DOWN): Wd rows of this CTA's 128 output columns over its K slice; the fp32 sums are added to the output rows
-// by the copy engine (512 bytes per row), which phase A's idle warps have cleared; they copy the kept reference rows as well.
+// Phase B (DOWN): Wd rows of this CTA's 128 output columns over its K slice; the copy engine stores the fp32 sums (512 bytes per row).
 enum { DOWN = 0, WIDE = 1, PACKED = 2 };
 template <int MODE>
 struct SmemCtx {
@@ -174,6 +173,7 @@ struct CtxGemmArgs {
     int P, S, q_lo, cap;               // this pass has the rows q_lo <= q < q_lo + n of the sequence
     const float* y_ref;
     float* y_out;
+    float* yp;                         // phase B output [K slices, n, H]
     int* status;
 };
 
@@ -279,24 +279,16 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
         pdl_wait();
         bool bad;
         const int c = ctx_count(a.count, a.P, a.S, a.cap, &bad);
-        int dst = -1;                      // phase B: the output row that this thread adds
+        int dst = -1;                      // phase B: the output row of the sums that this thread stores (-1: none, they are not wanted)
         if (GATED) {
-            // a warp per row: output rows of this pass start from zero; in the first pass the visual rows that are not in the
-            // (ascending) list keep their reference output
-            const int rows = n + (a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0);
+            // in the first pass the visual rows that are not in the (ascending) list keep their reference output: a warp per row
+            const int rows = a.q_lo == 0 && a.y_out != a.y_ref ? a.P : 0;
             for (int i = blockIdx.x + warp * (int)gridDim.x; i < rows; i += (EPI / 32) * (int)gridDim.x) {
-                const float4* from = nullptr;
-                int to_row = -1;
-                if (i < n) {
-                    to_row = out_row(a.list, a.q_lo + i, c, a.P, a.S);
-                } else if (!listed(a.list, c, i - n, lane)) {
-                    to_row = i - n;
-                    from = reinterpret_cast<const float4*>(a.y_ref + (size_t)to_row * a.H);
-                }
-                if (to_row < 0) continue;
-                float4* to = reinterpret_cast<float4*>(a.y_out + (size_t)to_row * a.H);
+                if (listed(a.list, c, i, lane)) continue;
+                const float4* from = reinterpret_cast<const float4*>(a.y_ref + (size_t)i * a.H);
+                float4* to = reinterpret_cast<float4*>(a.y_out + (size_t)i * a.H);
 #pragma unroll 4
-                for (int e = lane; e < a.H / 4; e += 32) to[e] = from ? from[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = lane; e < a.H / 4; e += 32) to[e] = from[e];
             }
         } else if (tid < n) {
             dst = out_row(a.list, a.q_lo + tid, c, a.P, a.S);
@@ -374,7 +366,7 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
         if (!GATED) {
             fence_proxy_async_smem();
             named_barrier(1, EPI);
-            if (dst >= 0 && m0 < a.rows && !gave_up) bulk_reduce_add_f32(a.y_out + (size_t)dst * a.H + m0, base + tid * 512, 512);
+            if (dst >= 0 && m0 < a.rows && !gave_up) bulk_store(a.yp + ((size_t)blockIdx.y * n + tid) * a.H + m0, base + tid * 512, 512);
             bulk_commit();
             bulk_wait_read_all();
         }
@@ -383,6 +375,28 @@ __global__ void __launch_bounds__(CT, 2) ctx_gemm_kernel(const CtxGemmArgs a, co
     if (__syncthreads_or(gave_up)) linger_after_timeout();
     cluster_sync();                        // neither CTA leaves while the other may signal it or read its shared memory
     if (warp == EPI / 32 + 1) tmem_dealloc_pair(tmem, TMEM_COLS);
+}
+
+// ---------------------------------------------------------------- output rows: the K slices' sums in their order
+constexpr int SUM_CHUNK = 8;           // slices that a thread has in flight
+__global__ void __launch_bounds__(256) ctx_sum_kernel(const CtxGemmArgs a, int ksplit) {
+    pdl_wait();
+    pdl_launch_dependents();
+    bool bad;
+    const int r = (int)blockIdx.x, c = ctx_count(a.count, a.P, a.S, a.cap, &bad), dst = out_row(a.list, a.q_lo + r, c, a.P, a.S);
+    if (dst < 0) return;
+    for (int e = (int)threadIdx.x; e < a.H / 4; e += 256) {
+        const float4* p = reinterpret_cast<const float4*>(a.yp + (size_t)r * a.H) + e;
+        float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s0 = 0; s0 < ksplit; s0 += SUM_CHUNK) {
+            float4 v[SUM_CHUNK];
+#pragma unroll
+            for (int i = 0; i < SUM_CHUNK; ++i) v[i] = s0 + i < ksplit ? __ldcg(p + (size_t)(s0 + i) * a.n * (a.H / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < SUM_CHUNK; ++i) { y.x += v[i].x; y.y += v[i].y; y.z += v[i].z; y.w += v[i].w; }
+        }
+        reinterpret_cast<float4*>(a.y_out + (size_t)dst * a.H)[e] = y;
+    }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -470,7 +484,19 @@ int run_ffn(rm_ctx* ctx, const FfnMaps& w, const __nv_bfloat16* xc, __nv_bfloat1
     a.kblocks = I / 64;
     a.rows = H;
     a.mr = 128;
-    return launch_gemm<DOWN>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s);
+    if ((rc = launch_gemm<DOWN>(ctx, a, dim3((H / 128 + 1) / 2 * 2, ksplit), w.d, w.d, th, s)) != RM_OK) return rc;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = ctx->use_pdl;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    RM_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctx_sum_kernel, a, ksplit));
+    ctx->launches++;
+    return RM_OK;
 }
 
 // K slices of the second product: as many as keep about one CTA per SM (at least two K blocks each)
@@ -494,7 +520,8 @@ size_t rm_context_workspace_bytes_impl(const rm_ctx* ctx, int cap) {
     const int r_pad = pass_rows(cap);
     const size_t xc = align_up((size_t)r_pad * ctx->g.H * sizeof(__nv_bfloat16), 1024);
     const size_t h1 = align_up((size_t)r_pad * ctx->g.I * sizeof(__nv_bfloat16), 1024);
-    return xc + h1;
+    const size_t yp = (size_t)pick_ksplit(ctx) * r_pad * ctx->g.H * sizeof(float);
+    return xc + h1 + yp;
 }
 
 int rm_launch_context_drift(rm_ctx* ctx, const void* x, const void* x_ref, int P, float* score, cudaStream_t s) {
@@ -533,6 +560,7 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
         __nv_bfloat16* xc = reinterpret_cast<__nv_bfloat16*>(w);
         w += align_up((size_t)r_pad * H * sizeof(__nv_bfloat16), 1024);
         __nv_bfloat16* h1 = reinterpret_cast<__nv_bfloat16*>(w);
+        w += align_up((size_t)r_pad * I * sizeof(__nv_bfloat16), 1024);
         {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((r_pad + 7) / 8);
@@ -550,6 +578,7 @@ int rm_launch_context_ffn(rm_ctx* ctx, const void* Wg, const void* Wu, const voi
         a.P = P; a.S = S; a.q_lo = q_lo; a.cap = cap;
         a.y_ref = y_ref;
         a.y_out = y_out;
+        a.yp = reinterpret_cast<float*>(w);
         if ((rc = run_ffn(ctx, maps, xc, h1, r_pad, ksplit, a, s)) != RM_OK) return rc;
     }
     return RM_OK;

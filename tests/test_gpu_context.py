@@ -123,3 +123,29 @@ def test_context_argument_checks(lib):
     with pytest.raises(lib.RmError):
         ctx.rm_context_ffn(t, t, t, t, i32, i32, 8, 2, 32, t, t)
     ctx.close()
+
+
+@pytest.mark.parametrize("H,I,P,S,R_max", [(2048, 16384, 768, 48, 240), (1024, 4096, 500, 30, 400), (384, 1152, 90, 7, 41), (128, 19072, 64, 0, 64)])
+def test_the_same_bits_every_time(lib, H, I, P, S, R_max):
+    """The K slices' sums are added in their order, as they were by the kernels that went by one CTA per tile."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(H + P)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    ctx = lib.Context(1, H, I, 64)
+    W = [(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))]
+    x, y_ref = rnd(P + S, H).bfloat16(), rnd(P, H)
+    k = R_max - S
+    rows = torch.zeros((P + 3) // 4 * 4, dtype=torch.int32, device="cuda")
+    rows[:k] = torch.randperm(P, generator=g, device="cuda")[:k].sort().values.int()
+    cnt = torch.tensor([k], dtype=torch.int32, device="cuda")
+    first = None
+    for _ in range(6):
+        y = torch.full((P + S, H), 7.0, device="cuda")
+        ctx.rm_context_ffn(*W, x, rows, cnt, P, S, R_max, y_ref, y)
+        first = y if first is None else first
+        assert torch.equal(y, first)
+    in_place = torch.cat([y_ref, torch.full((S, H), 7.0, device="cuda")])
+    ctx.rm_context_ffn(*W, x, rows, cnt, P, S, R_max, in_place, in_place)
+    assert torch.equal(in_place, first)
+    assert ctx.rm_device_status() == 0
+    ctx.close()

@@ -82,7 +82,8 @@ inline bool use_slice(const rm_ctx* ctx, int B, int T, bool record) {
 // The sweep kernel (variant 7): dense steps of one episode, where a cluster of the whole-step kernel would walk more than one
 // tile of 256 neurons per layer.  us per step of 18 layers, 51 tokens, whole-step / sweep: H = 1024, I = 3000: 213 / 248,
 // 3500: 220 / 263, 4096: 282 / 255, 6000: 309 / 279; H = 2048, I = 8000: 540 / 430, 16384: 1085 / 750.
-// The line lies at the same place from 8 to 64 tokens (6 layers, 8 tokens: 3840 72 / 85, 3900 93 / 86).
+// The line lies at the same place from 8 to 64 tokens (6 layers, 8 tokens: 3840 72 / 85, 3900 93 / 86) and at H = 2048 (51 tokens:
+// 3840 110 / 124, 3900 150 / 124, 4500 152 / 125, 6000 165 / 133).
 inline bool use_sweep(const rm_ctx* ctx, int B, int T, bool dense) {
     if (ctx->path == 1 || !dense || !rm_sweep_supported(ctx, B, T)) return false;
     if (ctx->variant_override != 0) return ctx->variant_override == 7;
@@ -101,20 +102,26 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 // The streaming variant (whole tiles per CTA): a tile costs an SM ~16 us at H = 1024 (its gathers run at ~20 bytes per clock,
 // its adds at 16), however few tiles there are; the cluster kernels, which spread a tile over 8 SMs, win while every cluster
 // has a single tile (stream_min_tiles, see rm_create).  `masked` says whether a count is in play.
-// anchor_write: the anchor step of Eq. 4 adds two boxes per block (y_anchor and the output) and stores h_anchor; measured
-// on the anchor schedule it stays behind the cluster kernels at 64 tiles (352 against 334 us per step), so it keeps
-// the threshold of about a tile per SM
+// With the anchor state of Eq. 4 the tiles do more (the anchor step adds two boxes per block and stores h_anchor, an update step reads
+// it), in the layer kernels beside other tiles.  us per 6 layers, 4 episodes, streaming / layer kernels:
+//   anchor step, H = 1024, T = 20: 40 tiles 111 / 106, 44 112 / 125     T = 51: 56 158 / 150, 60 159 / 171     T = 60: 32 169 / 186
+//                H = 2048, T = 20: 32 tiles 190 / 212     T = 51: 32 278 / 287     T = 56: 48 288 / 248, 56 289 / 289, 64 290 / 330
+//   update step, H = 1024, T = 20: 36 tiles 96 / 104      T = 51: 36 116 / 147
+//                H = 2048, T = 8: 32 tiles 189 / 171, 52 195 / 185     T = 20: 32 193 / 179, 52 196 / 193     T = 51: 32 219 / 245
 // Where the lean kernel fits an SM only once (H = 1024, T > 52), its clusters walk two tiles from 17 tiles on: half the threshold
 // (2 episodes of 60 tokens, 3600 neurons, us per 6 layers, lean / streaming: 10 tiles 68 / 101, 18 tiles 114 / 102)
-inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, bool anchor_write = false, bool eq4 = false) {
+inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_mode = RM_ANCHOR_NONE, bool eq4 = false) {
     if (ctx->path == 1 || !rm_stream_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 4) return true;
     if (ctx->variant_override != 0 && ctx->variant_override != 5 && ctx->variant_override != 7) return false;   // 5, 7: a call the whole-step kernel does not cover
     const int per_episode = masked ? rm_effective_count_hint(ctx) : ctx->g.I;
     if (per_episode <= 0) return false;
     const long long tiles = (long long)((per_episode + 63) / 64) * B;
-    const int least = !eq4 && ctx->g.H == 1024 && !rm_fused_two_per_sm(ctx, T) ? (ctx->stream_min_tiles + 1) / 2 : ctx->stream_min_tiles;
-    return tiles >= (anchor_write && least < 112 ? 112 : least);
+    const bool wide = ctx->g.H == 2048, once = !wide && !rm_fused_two_per_sm(ctx, T);
+    int least = !eq4 && once ? (ctx->stream_min_tiles + 1) / 2 : ctx->stream_min_tiles, eq4_least = 0;
+    if (anchor_mode == RM_ANCHOR_WRITE) eq4_least = wide ? (T > 52 ? 53 : 0) : T <= 32 ? 41 : once ? 0 : 57;
+    if (anchor_mode == RM_ANCHOR_UPDATE && wide && T <= 32) eq4_least = 64;
+    return tiles >= (least > eq4_least ? least : eq4_least);
 }
 
 }  // namespace
@@ -440,7 +447,7 @@ static int step_device(rm_ctx* ctx, const void* const* packed_layers, const floa
     // Fused path: layer l reads rot[l%3] (the caller's r_in for l = 0), accumulates into rot[(l+1)%3] and clears
     // rot[(l+2)%3] for the layer after next; the last layer accumulates straight into r_out when that is a
     // different buffer from r_in.
-    const bool stream = fused && use_stream(ctx, count_dev != nullptr, B, T, an.mode == RM_ANCHOR_WRITE,
+    const bool stream = fused && use_stream(ctx, count_dev != nullptr, B, T, an.mode,
                                              an.mode != RM_ANCHOR_NONE || an.gate);
     const bool direct_out = fused && r_out != r_in;
     if (fused && !stream) {

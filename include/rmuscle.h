@@ -271,8 +271,9 @@ int64_t rm_launch_count(const rm_ctx* ctx);
  *                         of consecutive tiles run concurrently; for clusters that walk many tiles), 4 = streaming
  *                         (no clusters: every CTA owns whole tiles; for launches with many tiles), 5 = the whole-step
  *                         kernel (every layer of a step in one launch; B <= 16; calls it does not cover are chosen per
- *                         launch), 6 = the slice kernel (every layer of a step in one launch, H up to 2048, any T; chosen by
- *                         itself for widths and chunk lengths that the others do not take), 7 = the sweep kernel (dense
+ *                         launch), 6 = the slice kernel (every layer of a step in one launch, H up to 2048, any T, but
+ *                         no records of more than 64 tokens; chosen by itself for widths and chunk lengths that the others
+ *                         do not take), 7 = the sweep kernel (dense
  *                         steps of one episode in one launch)
  *   "stream_min_tiles"    launches with at least this many 64-neuron tiles use variant 4 when the variant is chosen
  *                         per launch (default 33 at H = 1024, 31 at H = 2048)

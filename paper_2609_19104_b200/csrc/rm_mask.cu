@@ -18,7 +18,7 @@
 //     which send their flag words to the first CTA through distributed shared memory;
 //   - one scan per ordered ranking, over the (chunk, warp) counts, instead of one per chunk.
 //   - one long record is divided over the CTAs of a cluster, which add up their bins.
-// Measured, 18 lists, us per call back to back: 3-of-4 vote of top-615 sets of 4096: 29.9 -> 7.7; top-3277 of 16384: 26.8 -> 9.7
+// Measured, 18 lists, us per call back to back: 3-of-4 vote of top-615 sets of 4096: 29.9 -> 7.7; top-3277 of 16384: 26.8 -> 9.7 to 10.7
 // (14.6 with one CTA per list).
 #include "rm_common.cuh"
 #include "rm_sm100.cuh"

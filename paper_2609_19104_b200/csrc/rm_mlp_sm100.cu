@@ -178,11 +178,11 @@ __device__ __noinline__ void stage_partial(float* __restrict__ stage, const floa
     }
 }
 
-template <int NTOK, int HS, bool PIPE>
+template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1>
 struct Smem {
     static constexpr int KB = HS / 64;                       // 64-column (128-byte) blocks per slice
     static constexpr int NB = PIPE ? 2 : 1;                  // buffers of the exchange state (tiles in flight)
-    static constexpr bool STAGED = PIPE && HS == 128;        // dedicated staging area for the outgoing partial sums
+    static constexpr bool STAGED = OCC == 1 && HS == 128;    // dedicated staging area for the outgoing partial sums
     static constexpr int X_BYTES = KB * NTOK * 128;
     static constexpr int GU_STAGE = KB * 128 * 128;
     static constexpr int DN_STAGE = KB * NT * 128;
@@ -220,13 +220,14 @@ struct TileRef {
 };
 
 // EQ4 = false compiles the anchor-relative update and the output gate out (the zero-fill step pays nothing for them)
-template <int NTOK, int HS, bool PIPE, bool EQ4>
-__global__ void __launch_bounds__(FT, (HS == 128 && !PIPE ? 2 : 1)) fused_layer_kernel(const FusedArgs a,
+// OCC: CTAs per SM that the registers allow
+template <int NTOK, int HS, bool PIPE, bool EQ4, int OCC>
+__global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
                                                                                                const __grid_constant__ CUtensorMap tmOut) {
     const int anchor_mode = EQ4 ? a.anchor_mode : (int)RM_ANCHOR_NONE;
     const float* const gate = EQ4 ? a.gate : nullptr;
     const float* const ya_update = anchor_mode == RM_ANCHOR_UPDATE ? a.y_anchor : nullptr;
-    using S = Smem<NTOK, HS, PIPE>;
+    using S = Smem<NTOK, HS, PIPE, OCC>;
     constexpr int NB = S::NB;
     constexpr int KB = S::KB;
     extern __shared__ unsigned char smem_dyn[];
@@ -1518,16 +1519,20 @@ int launch_fused_ws(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, c
     return RM_OK;
 }
 
-template <int NTOK, int HS, bool PIPE>
+// Shared memory that keeps a second CTA off the SM (of the 228 KB)
+constexpr int ALONE_BYTES = 116 * 1024;
+
+template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1>
 int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cudaStream_t s) {
-    using S = Smem<NTOK, HS, PIPE>;
+    using S = Smem<NTOK, HS, PIPE, OCC>;
     const bool eq4 = a.anchor_mode != RM_ANCHOR_NONE || a.gate != nullptr;
-    auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true> : fused_layer_kernel<NTOK, HS, PIPE, false>;
-    const int smem = S::total_bytes(a.T);
+    auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true, OCC> : fused_layer_kernel<NTOK, HS, PIPE, false, OCC>;
+    int smem = S::total_bytes(a.T);
+    if (OCC == 1 && smem < ALONE_BYTES) smem = ALONE_BYTES;
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, smem)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, false, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         configured.set(ctx->device, smem);
     }
     cudaLaunchConfig_t cfg = {};
@@ -1555,7 +1560,7 @@ int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cuda
 template <int NTOK, int HS, bool PIPE>
 int max_clusters(int T, int* out) {
     using S = Smem<NTOK, HS, PIPE>;
-    auto kern = fused_layer_kernel<NTOK, HS, PIPE, false>;
+    auto kern = fused_layer_kernel<NTOK, HS, PIPE, false, HS == 128 && !PIPE ? 2 : 1>;
     const int smem = S::total_bytes(T);
     RM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};
@@ -1651,16 +1656,26 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     // caller's hint); 0 = unknown.
     const int per_episode = la.count ? rm_effective_count_hint(ctx) : ctx->g.I;
     const long long tiles = per_episode > 0 ? (long long)((per_episode + NT - 1) / NT) * la.B : 0;
-    // Variant.  H = 1024: the lean kernel for every launch (112 KB and 107 registers: two CTAs per SM, so a cluster's
-    // exchange waits are covered by its SM-mate and consecutive layers overlap); measured, 33 of its clusters are
-    // co-resident, two more than twice the number the occupancy query reports for one CTA per SM.  H = 2048 (one CTA
-    // per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
+    // Variant.  H = 1024: the lean kernel (112 KB and at most 128 registers: two CTAs per SM, so a cluster's exchange waits are
+    // covered by its SM-mate and consecutive layers overlap); measured, 33 of its clusters are co-resident, two more than
+    // twice the number the occupancy query reports for one CTA per SM.  Where no second CTA would fit the SM (more than 52 tokens), and
+    // where all clusters of a launch, in a stack those of the layer behind it too, find SMs of their own, it is built for one
+    // CTA per SM: nothing shares an SM by chance, values stay in registers, and outgoing sums have an area of their own.  us, two per
+    // SM / one, 6 layers: T = 8, 7 tiles 41.7 / 39.3; T = 32, 7 tiles 45.5 / 43.3; T = 51, 7 tiles 55.9 / 53.9, 12 tiles 57.8 / 63.7
+    // (two layers no longer fit side by side); T = 60, 12 tiles 69.0 / 67.0; T = 64, 7 tiles 62.6 / 58.3, 12 tiles 72.6 / 68.4;
+    // with Eq. 4 T = 20, 7 tiles 46.6 / 44.2; one layer alone, T = 51, 12 tiles 11.9 / 11.6.
+    // Its clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers 88.0 / 80.5.
+    // H = 2048 (one CTA per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
     // which runs the phases of consecutive tiles concurrently.
     const bool two_per_sm = rm_fused_two_per_sm(ctx, la.T);
     int cap = two_per_sm ? 2 * ctx->fused_clusters + 2 : ctx->fused_clusters;
     if (ctx->max_clusters_override > 0) cap = ctx->max_clusters_override;
     int variant = ctx->variant_override >= 5 ? 0 : ctx->variant_override;    // 5 and above: a call that the named kernel does not cover
-    if (variant == 0) variant = (ctx->g.H == 1024 || (tiles > 0 && tiles <= cap)) ? 1 : 3;
+    if (variant == 0) {
+        if (ctx->g.H == 1024) variant = !two_per_sm && tiles > ctx->fused_clusters ? 2 : 1;
+        else variant = tiles > 0 && tiles <= cap ? 1 : 3;
+    }
+    const bool alone = !two_per_sm || (tiles > 0 && tiles <= (la.x ? ctx->fused_clusters : ctx->fused_clusters / 2));
     if (variant == 3) {
         const int fits_t = ctx->g.H == 1024 ? SmemWS<64, 128>::total_bytes(la.T) : SmemWS<64, 256>::total_bytes(la.T);
         if (fits_t > 232448) variant = 2;
@@ -1686,6 +1701,8 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     if (ctx->g.H == 1024) {
         if (pipe)
             return small_t ? launch_fused<32, 128, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, true>(ctx, a, nc, pdl, s);
+        if (alone)
+            return small_t ? launch_fused<32, 128, false, 1>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 1>(ctx, a, nc, pdl, s);
         return small_t ? launch_fused<32, 128, false>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false>(ctx, a, nc, pdl, s);
     }
     // H = 2048: the two-tile variant when its buffers fit the 227 KB of an SM (they do up to T = 60), else serial

@@ -159,6 +159,13 @@ __device__ __noinline__ void flush_partial(float* __restrict__ r_out, float* __r
     }
 }
 
+// The slow part of a wait, once in the kernel
+__device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, int* status) {
+    if (mbar_wait(bar, parity)) return true;
+    rm_set_status_at(status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
+    return false;
+}
+
 // The same accumulator, scaled by the gate, laid out in shared memory as [128-column block][token][128 columns] for
 // the copy engine's bulk add (one box of the [B, T, H] tensor map per block).  Out of line for the same reason.
 template <int NTOK, int HS>
@@ -220,8 +227,12 @@ struct TileRef {
 };
 
 // EQ4 = false compiles the anchor-relative update and the output gate out (the zero-fill step pays nothing for them)
-// OCC: CTAs per SM that the registers allow
-template <int NTOK, int HS, bool PIPE, bool EQ4, int OCC>
+// OCC: CTAs per SM that the registers allow.  LATE: a tile's outgoing partial sums always lie in the gate/up stage, which is refilled
+// only once they have been read -- for launches whose clusters have one tile each as far as the host knows.  (The code that sends
+// rows from registers otherwise costs registers where it is not used.)  A layer is a chain of latencies, and instructions on it
+// count: with this, the integer division of the residual's share and the first tile's bounds before the dependency wait, and one
+// rsqrt for a root and a division, 6 layers of 10 tiles take, T = 20 / 32 / 51, 40.4 / 43.0 / 55.6 us instead of 43.7 / 46.1 / 57.0.
+template <int NTOK, int HS, bool PIPE, bool EQ4, int OCC, bool LATE>
 __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
                                                                                                const __grid_constant__ CUtensorMap tmOut) {
     const int anchor_mode = EQ4 ? a.anchor_mode : (int)RM_ANCHOR_NONE;
@@ -380,10 +391,18 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
         n_share = last_c - first_c + 1;
         my_share = cid - first_c;
     };
-    int share_b = -1, share_n = 1, share_my = 0;
-    if (a.add_residual && g_lo < g_hi) {
-        share_b = tile_ref(g_lo).b;
-        residual_share(share_b, share_n, share_my);
+    constexpr int PARTS = FT / NTOK;                       // x preparation: threads per token row
+    int share_b = -1;
+    bool share_row = false;                                // this thread's row is added here
+    TileRef tr0{};
+    if (g_lo < g_hi) {
+        tr0 = tile_ref(g_lo);
+        if (a.add_residual) {
+            int n_share, my_share;
+            share_b = tr0.b;
+            residual_share(share_b, n_share, my_share);
+            share_row = tid / PARTS % n_share == my_share;
+        }
     }
 
     RM_WALL(1);
@@ -406,7 +425,10 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     auto phase_of = [&](int i) { return (uint32_t)(PIPE ? ((i >> 1) & 1) : (i & 1)); };
     bool gave_up = false;
     auto wait_bar_at = [&](uint32_t bar, uint32_t parity, int line) {
-        if (!mbar_wait(bar, parity)) {
+        if (NTOK == 32 && !EQ4) {
+            // (the loop out of line: 2 to 3 % of a step with short chunks; with the registers of the others it costs 1 %)
+            if (!mbar_test_wait(bar, parity) && !wait_slow(bar, parity, line, a.status)) gave_up = true;
+        } else if (!mbar_wait(bar, parity)) {
             rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));
             gave_up = true;
         }
@@ -415,14 +437,14 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     // ---- phase: x slice of episode b -> bf16, 128-byte-swizzled K-major operand tile (cluster-collective)
     auto xprep = [&](int b) {
         cur_b = b;
-        constexpr int PARTS = FT / NTOK;                   // threads per token row
         constexpr int CPP = HS / PARTS;                    // columns per thread
         const int t = tid / PARTS, part = tid % PARTS;
         // clusters whose runs contain tiles of this episode share the addition of its residual rows
-        int n_share = 1, my_share = 0;
-        if (a.add_residual) {
-            if (b == share_b) { n_share = share_n; my_share = share_my; }
-            else residual_share(b, n_share, my_share);
+        bool add_row = share_row;
+        if (a.add_residual && b != share_b) {
+            int n_share, my_share;
+            residual_share(b, n_share, my_share);
+            add_row = t % n_share == my_share;
         }
         if (a.x) {
             const uint4* src = reinterpret_cast<const uint4*>(a.x + ((size_t)b * T + t) * H + (size_t)j * HS + part * CPP);
@@ -459,7 +481,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
                 st_async_f32(map_to_rank(sSS + (j * 64 + t) * 4, dst), ss, map_to_rank(bar_s, dst));
             // residual: token row t of this episode is added by exactly one of the clusters that work on the
             // episode, from the values already in registers, while the exchange is in flight
-            if (a.add_residual && t < T && (t % n_share) == my_share) {
+            if (a.add_residual && t < T && add_row) {
                 const size_t row = ((size_t)b * T + t) * H;
                 const int col = j * HS + part * CPP;
 #pragma unroll
@@ -471,7 +493,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             float tot = 0.f;
 #pragma unroll
             for (int src = 0; src < CS; ++src) tot += gSS[src * 64 + t];
-            const float inv = 1.0f / sqrtf(tot / (float)H + 1e-6f);
+            const float inv = __frsqrt_rn(fmaf(tot, 1.0f / (CS * HS), 1e-6f));    // (one rounding instead of two; the division is exact)
 #pragma unroll
             for (int i = 0; i < CPP / 8; ++i) {
                 const int k = part * CPP + i * 8;
@@ -487,15 +509,14 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     // per-thread stores send only the columns that exist in tensor memory (the row pad can exceed the token tile).
     const int p_cols = PR < NTOK ? PR : NTOK;
     auto p_tx_bytes = [&](int i) {
-        const bool bulk = S::STAGED || (!(i + 1 < n_tiles) && p_bytes <= S::GU_STAGE);
+        const bool bulk = S::STAGED || LATE || (!(i + 1 < n_tiles) && p_bytes <= S::GU_STAGE);
         return bulk ? p_bytes : CS * 16 * p_cols * 4;
     };
-    auto open_tile = [&](int i) {
+    auto open_tile = [&](int i, const TileRef& tr) {
         if (tid == 0) {
             mbar_arrive_expect_tx(bar_p(buf_of(i)), p_tx_bytes(i));
             mbar_arrive_expect_tx(bar_h(buf_of(i)), CS * 2048);
         }
-        const TileRef tr = tile_ref(g_lo + i);
         if (tr.b != cur_b) xprep(tr.b);
     };
 
@@ -522,7 +543,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
         const int pb = buf_of(i);
         const uint32_t d1 = tmem_d1 + pb * NTOK;
         const bool stage_in_gu = !refill && p_bytes <= S::GU_STAGE;
-        if (S::STAGED || stage_in_gu) {
+        if (S::STAGED || LATE || stage_in_gu) {
             unsigned char* stg = S::STAGED ? gbase + S::OFF_P + NB * p_bytes : gbase + S::OFF_GU;
             for (int c0 = (warp >> 2) * 32; c0 < NTOK; c0 += 64) {
                 float v[32];
@@ -732,8 +753,8 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
         // ---- one tile at a time: open, gate/up, scatter, owner work, down.  Loads of the next tile are issued as
         // soon as the stage they go to is free, so they travel during the exchanges.
         for (int i = 0; i < n_tiles; ++i) {
-            const TileRef tr = tile_ref(g_lo + i);
-            open_tile(i);
+            const TileRef tr = i == 0 ? tr0 : tile_ref(g_lo + i);
+            open_tile(i, tr);
             cp_async_wait<0>();            // this tile's gate/up and down rows have landed
             fence_proxy_async_smem();
             __syncthreads();
@@ -745,7 +766,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             tc_fence_after();
             RM_STAMP(7);
             const bool refill = i + 1 < n_tiles;
-            if (refill) issue_gu(g_lo + i + 1);
+            if (refill && !LATE) issue_gu(g_lo + i + 1);
             cp_async_commit();
             scatter(i, refill);
             if (i == 0) shared_duties();
@@ -755,6 +776,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             wait_bar(bar_h(0), phase_of(i));           // h of the whole tile (all 8 owners' atoms) is here
             RM_STAMP(11);
             mma_dn(i, tr);
+            if (refill && LATE) issue_gu(g_lo + i + 1);            // (h is complete: every owner has read the staged sums)
             wait_bar(bar_dn, par_dn);                  // the down stage and the h tiles may be reused
             par_dn ^= 1;
             tc_fence_after();
@@ -769,7 +791,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     } else if (n_tiles > 0) {
         // ---- two tiles in flight: the gate/up product and the scatter of tile i+1 are issued before the owner work
         // and the down projection of tile i, so each exchange travels while the other tile's work runs.
-        open_tile(0);
+        open_tile(0, tr0);
         cp_async_wait<0>();
         fence_proxy_async_smem();
         __syncthreads();
@@ -785,7 +807,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             const TileRef tr = tile_ref(g_lo + i);
             const bool more = i + 1 < n_tiles;
             if (more) {
-                open_tile(i + 1);
+                open_tile(i + 1, tile_ref(g_lo + i + 1));
                 if (i == 0) cp_async_wait<0>(); else cp_async_wait<1>();      // gate/up rows of tile i+1 have landed
                 fence_proxy_async_smem();
                 __syncthreads();
@@ -1522,17 +1544,17 @@ int launch_fused_ws(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, c
 // Shared memory that keeps a second CTA off the SM (of the 228 KB)
 constexpr int ALONE_BYTES = 116 * 1024;
 
-template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1>
+template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1, bool LATE = false>
 int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cudaStream_t s) {
     using S = Smem<NTOK, HS, PIPE, OCC>;
     const bool eq4 = a.anchor_mode != RM_ANCHOR_NONE || a.gate != nullptr;
-    auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true, OCC> : fused_layer_kernel<NTOK, HS, PIPE, false, OCC>;
+    auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE> : fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>;
     int smem = S::total_bytes(a.T);
     if (OCC == 1 && smem < ALONE_BYTES) smem = ALONE_BYTES;
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, smem)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, false, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         configured.set(ctx->device, smem);
     }
     cudaLaunchConfig_t cfg = {};
@@ -1560,7 +1582,7 @@ int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cuda
 template <int NTOK, int HS, bool PIPE>
 int max_clusters(int T, int* out) {
     using S = Smem<NTOK, HS, PIPE>;
-    auto kern = fused_layer_kernel<NTOK, HS, PIPE, false, HS == 128 && !PIPE ? 2 : 1>;
+    auto kern = fused_layer_kernel<NTOK, HS, PIPE, false, HS == 128 && !PIPE ? 2 : 1, false>;
     const int smem = S::total_bytes(T);
     RM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};
@@ -1703,6 +1725,8 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
             return small_t ? launch_fused<32, 128, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, true>(ctx, a, nc, pdl, s);
         if (alone)
             return small_t ? launch_fused<32, 128, false, 1>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 1>(ctx, a, nc, pdl, s);
+        if (tiles > 0 && tiles <= nc)
+            return small_t ? launch_fused<32, 128, false, 2, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 2, true>(ctx, a, nc, pdl, s);
         return small_t ? launch_fused<32, 128, false>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false>(ctx, a, nc, pdl, s);
     }
     // H = 2048: the two-tile variant when its buffers fit the 227 KB of an SM (they do up to T = 60), else serial

@@ -167,9 +167,10 @@ __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, 
 }
 
 // The same accumulator, scaled by the gate, laid out in shared memory as [128-column block][token][128 columns] for
-// the copy engine's bulk add (one box of the [B, T, H] tensor map per block).  Out of line for the same reason.
+// the copy engine's bulk add (one box of the [B, T, H] tensor map per block).  In line in the layer kernel, where it is on every
+// layer's chain (out of line: 10 tiles, 6 layers, T = 20 / 32 / 51 39.1 -> 40.2, 41.8 -> 42.9, 54.1 -> 54.8 us), out of line in the other.
 template <int NTOK, int HS>
-__device__ __noinline__ void stage_partial(float* __restrict__ stage, const float* __restrict__ gate, uint32_t tmem_d2,
+__device__ __forceinline__ void stage_partial(float* __restrict__ stage, const float* __restrict__ gate, uint32_t tmem_d2,
                                            int wrow, int lane, int c0_first, int c0_step, int T, int col_base) {
 #pragma unroll
     for (int mm = 0; mm < HS / 128; ++mm) {
@@ -183,6 +184,12 @@ __device__ __noinline__ void stage_partial(float* __restrict__ stage, const floa
                 if (c0 + k < T) stage[(mm * NTOK + c0 + k) * 128 + cl] = gc * v[k];
         }
     }
+}
+
+template <int NTOK, int HS>
+__device__ __noinline__ void stage_partial_call(float* __restrict__ stage, const float* __restrict__ gate, uint32_t tmem_d2, int wrow, int lane,
+                                                int c0_first, int c0_step, int T, int col_base) {
+    stage_partial<NTOK, HS>(stage, gate, tmem_d2, wrow, lane, c0_first, c0_step, T, col_base);
 }
 
 template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1>
@@ -700,8 +707,11 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     auto flush = [&](const TileRef& tr, bool final_tile) {
         if (final_tile && anchor_mode != RM_ANCHOR_WRITE) {
             float* stage = reinterpret_cast<float*>(gbase + S::OFF_GU);
-            stage_partial<NTOK, HS>(stage, gate ? gate + (size_t)tr.b * H : nullptr, tmem_d2, warp & 3, lane, (warp >> 2) * 32,
-                                    64, T, j * HS);
+            const float* g = gate ? gate + (size_t)tr.b * H : nullptr;
+            if constexpr (EQ4 && NTOK == 64 && HS == 256)          // (in line its registers cost more there: 15 tiles of 51 tokens 97 -> 100)
+                stage_partial_call<NTOK, HS>(stage, g, tmem_d2, warp & 3, lane, (warp >> 2) * 32, 64, T, j * HS);
+            else
+                stage_partial<NTOK, HS>(stage, g, tmem_d2, warp & 3, lane, (warp >> 2) * 32, 64, T, j * HS);
             tc_fence_before();
             fence_proxy_async_smem();
             __syncthreads();
@@ -1171,7 +1181,7 @@ __global__ void __launch_bounds__(WT, 1) fused_layer_ws_kernel(const FusedArgs a
                 float tot = 0.f;
 #pragma unroll
                 for (int src = 0; src < CS; ++src) tot += gSS[src * 64 + t];
-                const float inv = 1.0f / sqrtf(tot / (float)H + 1e-6f);
+                const float inv = __frsqrt_rn(fmaf(tot, 1.0f / (CS * HS), 1e-6f));
 #pragma unroll
                 for (int i = 0; i < CPP / 8; ++i) {
                     const int k = part * CPP + i * 8;
@@ -1250,7 +1260,7 @@ __global__ void __launch_bounds__(WT, 1) fused_layer_ws_kernel(const FusedArgs a
                     // goes there as [token][128 columns] per 128-column block, scaled by the gate, and the copy
                     // engine adds each block to the output as one box of the [B, T, H] tensor map.
                     float* stage = reinterpret_cast<float*>(gbase + S::OFF_GU);
-                    stage_partial<NTOK, HS>(stage, gate ? gate + (size_t)b * H : nullptr, tmem_d2, warp, lane, 0, 32, T, j * HS);
+                    stage_partial_call<NTOK, HS>(stage, gate ? gate + (size_t)b * H : nullptr, tmem_d2, warp, lane, 0, 32, T, j * HS);
                     tc_fence_before();
                     fence_proxy_async_smem();
                     named_barrier(2, 128);
@@ -1731,7 +1741,11 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     }
     // H = 2048: the two-tile variant when its buffers fit the 227 KB of an SM (they do up to T = 60), else serial
     const bool fits = Smem<64, 256, true>::total_bytes(la.T) <= 232448;
-    if (small_t)
-        return pipe ? launch_fused<32, 256, true>(ctx, a, nc, pdl, s) : launch_fused<32, 256, false>(ctx, a, nc, pdl, s);
-    return (pipe && fits) ? launch_fused<64, 256, true>(ctx, a, nc, pdl, s) : launch_fused<64, 256, false>(ctx, a, nc, pdl, s);
+    const bool late = tiles > 0 && tiles <= nc;
+    if (small_t) {
+        if (pipe) return launch_fused<32, 256, true>(ctx, a, nc, pdl, s);
+        return late ? launch_fused<32, 256, false, 1, true>(ctx, a, nc, pdl, s) : launch_fused<32, 256, false>(ctx, a, nc, pdl, s);
+    }
+    if (pipe && fits) return launch_fused<64, 256, true>(ctx, a, nc, pdl, s);
+    return late ? launch_fused<64, 256, false, 1, true>(ctx, a, nc, pdl, s) : launch_fused<64, 256, false>(ctx, a, nc, pdl, s);
 }

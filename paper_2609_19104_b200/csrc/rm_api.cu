@@ -50,12 +50,16 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 // So, in tiles of 64 neurons, with K the caller's count hint (the whole layer for a dense pass): up to the bounds below the
 // layer kernels; from the bounds of H = 2048 up to one wave the streaming kernel.  Without a hint the whole-step kernel at
 // H = 2048 (it adapts to the counts on the device), the lean kernel at H = 1024.  Batches stay with the streaming kernel.
-// `steps`: a whole stack (false: the one-layer entry, which would pay the kernel's set-up for a single layer).
+// `steps`: a whole stack (false: the one-layer entry, which pays the kernel's set-up for a single layer, and only where a streaming
+// tile takes longer still; H = 2048, us, whole-step / streaming / two-tile kernel:
+//   T =  8: 36 tiles 24.4/23.6/18.7   45: 25.1/23.6/22.2     T = 32: 36: 22.6/24.5/20.0   48: 23.0/24.7/23.8   57: 24.1/24.7/24.1
+//   T = 48: 30 tiles 20.9/27.0/20.5   33: 21.0/27.0/22.2   57: 22.4/27.2/26.9   63: 29.7/27.4/30.0     T = 64: 33: 21.3/27.5/26.8   57: 22.4/27.5/33.0).
 inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool eq4, bool steps) {
     if (ctx->path == 1 || !rm_persist_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 5) return true;
-    if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b || !steps) return false;
+    if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b) return false;
     const long long K = masked ? rm_effective_count_hint(ctx) : ctx->g.I, tiles = (K + 63) / 64;
+    if (!steps) return ctx->g.H == 2048 && T > 16 && tiles >= (T > 32 ? 31 : 46) && tiles < 60;
     if (K <= 0) return ctx->g.H == 2048;
     if (ctx->g.H == 2048) {
         if (tiles <= (eq4 || T <= 55 ? 15 : 13)) return false;
@@ -109,8 +113,9 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 //   update step, H = 1024, T = 20: 36 tiles 96 / 104      T = 51: 36 116 / 147
 //                H = 2048, T = 8: 32 tiles 189 / 171, 52 195 / 185     T = 20: 32 193 / 179, 52 196 / 193     T = 51: 32 219 / 245
 // Where the lean kernel fits an SM only once (H = 1024, T > 52), its clusters walk two tiles from 17 tiles on: half the threshold
-// (2 episodes of 60 tokens, 3600 neurons, us per 6 layers, lean / streaming: 10 tiles 68 / 101, 18 tiles 114 / 102)
-inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_mode = RM_ANCHOR_NONE, bool eq4 = false) {
+// (2 episodes of 60 tokens, 3600 neurons, us per 6 layers, lean / streaming: 10 tiles 68 / 101, 18 tiles 114 / 102).  One layer
+// alone has the two-tile variant there (T = 56, 18 tiles 15.0 / 17.8 us, 30 16.3 / 17.9), at H = 2048 up to 59 tiles with short chunks.
+inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_mode = RM_ANCHOR_NONE, bool eq4 = false, bool steps = true) {
     if (ctx->path == 1 || !rm_stream_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 4) return true;
     if (ctx->variant_override != 0 && ctx->variant_override != 5 && ctx->variant_override != 7) return false;   // 5, 7: a call the whole-step kernel does not cover
@@ -119,6 +124,7 @@ inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_
     const long long tiles = (long long)((per_episode + 63) / 64) * B;
     const bool wide = ctx->g.H == 2048, once = !wide && !rm_fused_two_per_sm(ctx, T);
     int least = !eq4 && once ? (ctx->stream_min_tiles + 1) / 2 : ctx->stream_min_tiles, eq4_least = 0;
+    if (!steps) least = once ? ctx->stream_min_tiles - 2 : wide && T <= 32 ? ctx->stream_min_tiles + 29 : ctx->stream_min_tiles;
     if (anchor_mode == RM_ANCHOR_WRITE) eq4_least = wide ? (T > 52 ? 53 : 0) : T <= 32 ? 41 : once ? 0 : 57;
     if (anchor_mode == RM_ANCHOR_UPDATE && wide && T <= 32) eq4_least = 64;
     return tiles >= (least > eq4_least ? least : eq4_least);
@@ -371,7 +377,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
             ctx->last_variant = 5;
             return rm_launch_step_persist(ctx, sa, persist_ws(ctx, ws, 1, T), s);
         }
-        if (use_stream(ctx, count_dev != nullptr, 1, T)) {
+        if (use_stream(ctx, count_dev != nullptr, 1, T, RM_ANCHOR_NONE, false, false)) {
             ctx->last_variant = 4;
             return rm_launch_layer_stream(ctx, a, nullptr, y == residual, s);
         }

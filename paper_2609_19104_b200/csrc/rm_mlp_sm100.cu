@@ -1698,14 +1698,15 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     // with Eq. 4 T = 20, 7 tiles 46.6 / 44.2; one layer alone, T = 51, 12 tiles 11.9 / 11.6.
     // Its clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers 88.0 / 80.5.
     // H = 2048 (one CTA per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
-    // which runs the phases of consecutive tiles concurrently.
+    // which runs the phases of consecutive tiles concurrently.  One layer alone of up to 52 tokens: the two-tile variant (us, warp-
+    // specialised / two-tile, T = 40: 18 tiles 18.0 / 17.8, 27 18.8 / 18.2; T = 16: 36 tiles 19.9 / 19.0).
     const bool two_per_sm = rm_fused_two_per_sm(ctx, la.T);
     int cap = two_per_sm ? 2 * ctx->fused_clusters + 2 : ctx->fused_clusters;
     if (ctx->max_clusters_override > 0) cap = ctx->max_clusters_override;
     int variant = ctx->variant_override >= 5 ? 0 : ctx->variant_override;    // 5 and above: a call that the named kernel does not cover
     if (variant == 0) {
         if (ctx->g.H == 1024) variant = !two_per_sm && tiles > ctx->fused_clusters ? 2 : 1;
-        else variant = tiles > 0 && tiles <= cap ? 1 : 3;
+        else variant = tiles > 0 && tiles <= cap ? 1 : tiles > 0 && la.x && la.T <= 52 ? 2 : 3;
     }
     const bool alone = !two_per_sm || (tiles > 0 && tiles <= (la.x ? ctx->fused_clusters : ctx->fused_clusters / 2));
     if (variant == 3) {

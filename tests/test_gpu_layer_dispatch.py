@@ -1,0 +1,32 @@
+"""Which kernel the one-layer entry takes follows width, chunk length and list length; at the borders both sides agree."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,T,borders", [
+    (1024, 60, [(15, 1), (16, 2), (30, 2), (31, 4)]), (2048, 16, [(15, 1), (16, 2), (59, 2), (60, 4)]),
+    (2048, 32, [(45, 2), (46, 5), (59, 5), (60, 4)]), (2048, 33, [(30, 2), (31, 5), (59, 5), (60, 4)]), (2048, 61, [(30, 2), (31, 5)])])
+def test_borders_of_one_layer(lib, H, T, borders):
+    import torch
+    I = 3968
+    g = torch.Generator(device="cuda").manual_seed(H + T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    ctx = lib.Context(1, H, I, T)
+    layer = ctx.rm_pack_weights(*[(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))])
+    x, r = rnd(T, H).bfloat16(), rnd(T, H)
+    for tiles, kernel in borders:
+        idx, cnt = torch.zeros(I, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        ctx.rm_mask_compact([rnd(1, I).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, idx, cnt, I, n_lists=1, k=64 * tiles - 5)
+        outs = []
+        for variant in (0, 1, 0):
+            ctx.rm_set_option("variant", variant)
+            y = r.clone() if len(outs) == 2 else torch.empty_like(r)           # (the last one in place)
+            outs.append(ctx.rm_sparse_mlp(layer, x, y if len(outs) == 2 else r, idx, cnt, y))
+            if variant == 0:
+                assert ctx.rm_get_info("last_variant") == kernel, (tiles, ctx.rm_get_info("last_variant"))
+        for out in outs:
+            # (one layer on the same bf16 input: only the order of fp32 sums of hidden values to 17 bits differs)
+            assert torch.isfinite(out).all() and float((out - outs[1]).norm() / (outs[1] - r).norm()) <= 1e-4, tiles
+    assert ctx.rm_device_status() == 0
+    ctx.close()

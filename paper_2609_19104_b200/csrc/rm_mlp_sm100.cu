@@ -432,8 +432,9 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     auto phase_of = [&](int i) { return (uint32_t)(PIPE ? ((i >> 1) & 1) : (i & 1)); };
     bool gave_up = false;
     auto wait_bar_at = [&](uint32_t bar, uint32_t parity, int line) {
-        if (NTOK == 32 && !EQ4) {
-            // (the loop out of line: 2 to 3 % of a step with short chunks; with the registers of the others it costs 1 %)
+        if (!EQ4 && (NTOK == 32 || (HS == 128 && !PIPE && OCC == 1))) {
+            // (the loop out of line: 2 to 3 % of a step with short chunks, 1 to 2 % of one of more than 52 tokens (15 tiles of 64 tokens:
+            // 71.5 -> 70.1 us); with the registers of the others it costs 1 %)
             if (!mbar_test_wait(bar, parity) && !wait_slow(bar, parity, line, a.status)) gave_up = true;
         } else if (!mbar_wait(bar, parity)) {
             rm_set_status_at(a.status, RM_ERR_TIMEOUT, (line << 12) | (int)(blockIdx.x & 0xfffu));

@@ -818,7 +818,11 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             const TileRef tr = tile_ref(g_lo + i);
             const bool more = i + 1 < n_tiles;
             if (more) {
-                open_tile(i + 1, tile_ref(g_lo + i + 1));
+                const TileRef nx = tile_ref(g_lo + i + 1);
+                // The x of a second tile of another episode: its sums of squares go where the first one's still lie, and nothing so far has
+                // made this CTA wait for its peers to have read those.  (From the third tile on h of the tile before the last one has.)
+                if (i == 0 && nx.b != tr.b) cluster_sync();
+                open_tile(i + 1, nx);
                 if (i == 0) cp_async_wait<0>(); else cp_async_wait<1>();      // gate/up rows of tile i+1 have landed
                 fence_proxy_async_smem();
                 __syncthreads();

@@ -64,6 +64,12 @@ def test_streaming_variant_with_few_ctas(lib):
     step_case(lib, H=1024, I=1024, T=40, L=2, B=2, density=0.6, variant=4, max_clusters=3)
 
 
+@pytest.mark.parametrize("H,T,B,variant,max_clusters", [(1024, 60, 16, 0, 0), (1024, 33, 16, 2, 0), (1024, 20, 3, 2, 1), (2048, 40, 16, 2, 0), (2048, 8, 5, 2, 2)])
+def test_two_tile_kernel_whose_tiles_are_of_different_episodes(lib, H, T, B, variant, max_clusters):
+    """One tile an episode, several to a cluster's run: x is prepared anew while the first tile's products are on their way."""
+    step_case(lib, H=H, I=64, T=T, L=4, B=B, density=0.9, variant=variant, hint=64, max_clusters=max_clusters, config=94)
+
+
 def test_gather_read_microbenchmark_runs_and_reports_bad_counts(lib):
     import torch
     H, I, T = 1024, 512, 8

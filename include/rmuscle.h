@@ -15,7 +15,8 @@
  *   - Conditions detected on the device (index >= I, count > stride) never trap: the kernel clamps or skips,
  *     records the code in the context's status word, and rm_device_status reports it.
  *   - Steps (and one-layer calls of widths other than 1024 and 2048 or of more than 64 tokens) may run as one kernel with a
- *     CTA on most of the SMs, whose CTAs wait for one another ("last_variant" 5, 6, 7).  Other streams' kernels may hold SMs meanwhile:
+ *     CTA on most of the SMs, whose CTAs wait for one another ("last_variant" 5, 6, 7; a one-layer call that reports 5 waits only
+ *     within its clusters of 8 CTAs, which the device starts together).  Other streams' kernels may hold SMs meanwhile:
  *     the resident CTAs wait at least 10 s for the others, then give up (RM_ERR_TIMEOUT).  Such calls of several streams of equal
  *     priority take their turns; on streams of different priority each could hold SMs that the other needs, so order those by
  *     events, or use rm_set_option("path", 1), whose kernels never wait for one another.

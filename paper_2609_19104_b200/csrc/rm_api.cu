@@ -160,7 +160,8 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     if (cudaGetDevice(&c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device) != cudaSuccess ||
-        cudaMalloc(&c->d_status, 256) != cudaSuccess || cudaMemset(c->d_status, 0, 256) != cudaSuccess) {
+        cudaMalloc(&c->d_status, (RM_STATUS_INTS + RM_ALONE_INTS) * sizeof(int)) != cudaSuccess ||
+        cudaMemset(c->d_status, 0, (RM_STATUS_INTS + RM_ALONE_INTS) * sizeof(int)) != cudaSuccess) {
         if (c->d_status) cudaFree(c->d_status);
         delete c;
         return RM_ERR_CUDA;
@@ -375,7 +376,7 @@ int rm_sparse_mlp(rm_ctx* ctx, const void* packed_layer, const void* x, const fl
             sa.T = T;
             sa.x_ext = x;
             ctx->last_variant = 5;
-            return rm_launch_step_persist(ctx, sa, persist_ws(ctx, ws, 1, T), s);
+            return rm_launch_step_persist(ctx, sa, nullptr, s);      // (the workspace stays untouched, as by the layer kernels)
         }
         if (use_stream(ctx, count_dev != nullptr, 1, T, RM_ANCHOR_NONE, false, false)) {
             ctx->last_variant = 4;
@@ -623,7 +624,7 @@ int rm_action_expert_step_host(rm_ctx* ctx, const void* const* packed_layers, co
 int rm_device_status(rm_ctx* ctx, int* host_out, rm_stream_t stream) {
     if (!ctx || !host_out) return RM_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int v[64] = {0};
+    int v[RM_STATUS_INTS] = {0};
     RM_CUDA_TRY(cudaMemcpyAsync(v, ctx->d_status, sizeof(v), cudaMemcpyDeviceToHost, s));
     RM_CUDA_TRY(cudaMemsetAsync(ctx->d_status, 0, sizeof(v), s));
     RM_CUDA_TRY(cudaStreamSynchronize(s));

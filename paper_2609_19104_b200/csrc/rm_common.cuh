@@ -25,14 +25,18 @@ struct rm_geom {
     }
 };
 
+constexpr int RM_STATUS_INTS = 64;         // the status block
+constexpr int RM_ALONE_INTS = 128;
+
 struct rm_ctx {
     rm_model_desc desc;
     rm_geom g;
     int device;
     int sm_count;
-    int* d_status;                         // device status word, then the detail word of the first error
+    int* d_status;                         // device status word, then the detail word of the first error (RM_STATUS_INTS); then the
+                                           // control block of one-layer launches of the whole-step kernel (RM_ALONE_INTS)
     int status_detail;                     // detail word seen by the last rm_device_status call
-    int status_log[64];                    // the whole status block of that call
+    int status_log[RM_STATUS_INTS];                  // the whole status block of that call
     int64_t launches;                      // host-side launch counter
     // tensor-core path (rm_mlp_sm100.cu)
     int fused_clusters;                    // co-resident 8-CTA clusters of the fused layer kernel (0: unavailable)
@@ -83,7 +87,7 @@ static inline bool rm_aligned16(const void* p) { return (reinterpret_cast<uintpt
 __device__ __forceinline__ void rm_set_status(int* status, int code) {
     if (status) atomicCAS(status, 0, code);
 }
-constexpr int RM_STATUS_LOG = 60;        // detail words kept per status read (the status block is 64 ints)
+constexpr int RM_STATUS_LOG = RM_STATUS_INTS - 4;        // detail words kept per status read
 // The first error of a launch also leaves a detail word (where a wait gave up) next to the status word.
 __device__ __forceinline__ void rm_set_status_at(int* status, int code, int detail) {
     if (!status) return;

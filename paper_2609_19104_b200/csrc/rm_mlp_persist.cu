@@ -62,6 +62,7 @@ constexpr int SYNC_ITEM = 64;          // sync[64..64+MAX_ITEMS): batches count 
 constexpr int SYNC_RITEM = SYNC_ITEM + MAX_ITEMS;      // ... and the CTAs that have read the item's input rows
 constexpr int SYNC_INTS = SYNC_RITEM + MAX_ITEMS;
 constexpr int CTRL_BYTES = ((grid::CTRL_LINE + SYNC_INTS) * 4 + 255) / 256 * 256;
+static_assert(grid::CTRL_LINE + SYNC_ITEM <= RM_ALONE_INTS, "the counters of one layer and one episode");
 
 struct PArgs {
     const __nv_bfloat16* packed[MAXL];
@@ -83,7 +84,10 @@ struct PArgs {
     int per_item;                      // arrivals are counted per (layer, episode) (batches: a cluster that takes no part in an
                                        // episode runs ahead of those that do, so one counter per episode could not tell the
                                        // layers apart); else per episode, over all layers
-    int x_ext;                         // layer 0 takes x from the caller's buffer (single-layer entry): no normalisation
+    int x_ext;                         // one layer alone, whose x is the caller's buffer: no normalisation, and no CTA waits for one of
+                                       // another cluster.  No epoch then, and the control block is the context's own, not one in the
+                                       // workspace: the abort flag counts, nobody looks at what the arrivals leave in its counters.
+                                       // (A branch around the arrivals cost a step of 18 layers 0.9 %.)
     int pf_bytes;                      // weight bytes a CTA may have asked into L2 ahead of its loaders (0: no prefetch)
     // Anchor-relative update (Eq. 4) and output gate; read by the EQ4 instantiation only
     int anchor_mode;                   // RM_ANCHOR_NONE / _WRITE / _UPDATE
@@ -439,7 +443,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     // behind another one: 193.4 -> 189.6 us)
     pdl_wait();
     if (blockIdx.x == 0) {                 // the launch's counters, then (below) its epoch
-        for (int e = tid; e < SYNC_INTS; e += NTHREADS) a.sync[e] = 0;
+        if (!a.x_ext)
+            for (int e = tid; e < SYNC_INTS; e += NTHREADS) a.sync[e] = 0;
         if (tid == 0) { a.ctrl[2] = 0; a.ctrl[3] = 0; }
         __threadfence();
     }
@@ -456,7 +461,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
         }
     }
     __syncthreads();
-    if (blockIdx.x == 0 && tid == W_PF * 32) grid::epoch_publish(a.ctrl, a.epoch);
+    if (blockIdx.x == 0 && tid == W_PF * 32 && !a.x_ext) grid::epoch_publish(a.ctrl, a.epoch);
     {
         // This cluster's run in every item's list: one thread per item (sK holds the counts; afterwards sP the run starts
         // and sK the run lengths).  One thread doing all of them took ~3 us of every launch.
@@ -497,7 +502,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
     pdl_launch_dependents();                                       // (a dependent waits for this grid's end: its CTAs are resident by then)
     // (the warps that use the launch's counters)
     const int tag = (int)(unsigned)a.epoch;
-    if (warp < 8) {
+    if (warp < 8 && !a.x_ext) {
         if (tid == 0) grid::epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort);
         named_barrier(1, 256);
     }
@@ -1254,7 +1259,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) step_kernel(const __grid_constant
             }
         }
         // (this CTA's last counter: the round trip of the leave runs beside the end of the other warps)
-        if (et == 0 && !grid::epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort)) grid::epoch_leave(a.ctrl);
+        if (et == 0 && !a.x_ext && !grid::epoch_wait(a.ctrl, a.epoch, __LINE__, a, sAbort)) grid::epoch_leave(a.ctrl);
     }
 #undef WAIT
     tc_fence_before();
@@ -1384,14 +1389,15 @@ int rm_persist_debug_stamps(long long* host_out, int n) {
 
 int rm_launch_step_persist(rm_ctx* ctx, const rm_step_args& sa, void* ws, cudaStream_t s) {
     const rm_geom& g = ctx->g;
+    if (sa.x_ext && (sa.L != 1 || sa.B != 1 || sa.r_in || sa.anchor_mode == RM_ANCHOR_UPDATE)) return RM_ERR_UNSUPPORTED;
     PArgs a{};
     for (int l = 0; l < sa.L; ++l) a.packed[l] = static_cast<const __nv_bfloat16*>(sa.packed_layers[l]);
     a.r = sa.r;
     a.r_in = sa.r_in ? sa.r_in : sa.r;
-    a.ctrl = reinterpret_cast<int*>(ws);
+    a.ctrl = sa.x_ext ? ctx->d_status + RM_STATUS_INTS : reinterpret_cast<int*>(ws);
     a.epoch = rm_next_epoch();
     a.sync = a.ctrl + grid::CTRL_LINE;
-    a.xbuf = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + CTRL_BYTES);
+    a.xbuf = sa.x_ext ? nullptr : reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(ws) + CTRL_BYTES);
     a.per_item = sa.B > 1 ? 1 : 0;
     a.idx = sa.idx;
     a.count = sa.count;

@@ -55,6 +55,29 @@ class Job:
             self.error = e
 
 
+class LayerJob(Job):
+    """One layer alone instead of a step."""
+
+    def __init__(self, lib, H, I, T, K, ctx=None, ws=None, priority=0, seed=0):
+        import torch
+        g = torch.Generator(device="cuda").manual_seed(H + T + K + seed)
+        rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+        self.ctx = ctx or lib.Context(1, H, I, T)
+        self.layer = self.ctx.rm_pack_weights(*[(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))])
+        self.idx, self.cnt = torch.zeros(1, I, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        self.ctx.rm_mask_compact([rnd(1, I).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, self.idx, self.cnt, I, n_lists=1, k=K)
+        self.x, self.r = rnd(T, H).bfloat16(), rnd(T, H)
+        self.ws = torch.empty(self.ctx.workspace_bytes(1, T), dtype=torch.uint8, device="cuda") if ws is None else ws
+        self.out = torch.empty_like(self.r)
+        self.step()
+        self.want, self.variant = self.out.clone(), self.ctx.rm_get_info("last_variant")
+        torch.cuda.synchronize()
+        self.stream, self.worst, self.error = torch.cuda.Stream(priority=priority), None, None
+
+    def step(self):
+        self.ctx.rm_sparse_mlp(self.layer, self.x, self.r, self.idx, self.cnt, self.out, ws=self.ws)
+
+
 def run(jobs):
     import torch
     threads = [threading.Thread(target=j.loop) for j in jobs]
@@ -90,6 +113,17 @@ def test_threads_that_share_a_context(lib):
     """Two models of one geometry through one context: dense steps, whose tensor maps the context keeps by layer."""
     ctx = lib.Context(3, 1024, 4096, 51)
     run([Job(lib, 1024, 4096, 3, 51, 0, seed=s, ctx=ctx) for s in range(3)])
+
+
+@pytest.mark.parametrize("priority", [0, -1])
+def test_single_layers_on_streams_that_share_a_context_and_its_workspace(lib, priority):
+    """The whole-step kernel on one layer, four times at once, beside a step on a stream of its own (of equal or lower priority)."""
+    import torch
+    ctx = lib.Context(1, 2048, 4096, 48)
+    ws = torch.empty(ctx.workspace_bytes(1, 48), dtype=torch.uint8, device="cuda")
+    jobs = [LayerJob(lib, 2048, 4096, T, 64 * 40, ctx=ctx, ws=ws, priority=priority, seed=i) for i, T in enumerate((48, 48, 33, 40))]
+    assert all(j.variant == 5 for j in jobs)
+    run(jobs + [Job(lib, 1024, 4096, 4, 51, 1400)])
 
 
 @pytest.mark.parametrize("job", [(1536, 4096, 4, 51, 1000), (1024, 4096, 4, 51, 1400), (1024, 4096, 4, 51, 0)])

@@ -104,3 +104,27 @@ def test_captured_step_with_other_calls_between_its_replays(lib, T, K, variant):
             s.check(c, "the step outside the graph")
     del graph
     s.ctx.close()
+
+
+@pytest.mark.parametrize("H,T,tiles,variant", [(1024, 51, 15, 1), (1024, 60, 20, 2), (1024, 20, 40, 4), (1024, 51, 20, 5), (2048, 20, 40, 2),
+                                               (2048, 40, 33, 5), (2048, 20, 50, 5), (2048, 51, 62, 4)])
+def test_one_layer_alone_leaves_the_workspace_as_it_is(lib, H, T, tiles, variant):
+    """Two streams may have one-layer calls of these widths on the device with one workspace between them: no kernel keeps anything there."""
+    import torch
+    s = Steps(lib, H, 4096, 1, T, 1)
+    idx, cnt = torch.zeros(1, 4096, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    s.ctx.rm_mask_compact([s.rnd(1, 4096).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, idx, cnt, 4096, n_lists=1, k=64 * tiles)
+    x, r, y = s.rnd(T, H).bfloat16(), s.rnd(T, H), torch.empty(T, H, device="cuda")
+    if variant == 5 and H == 1024:
+        s.ctx.rm_set_option("variant", 5)
+    ws = torch.full((s.ctx.workspace_bytes(1, T),), 0xa5, dtype=torch.uint8, device="cuda")
+    s.ctx.rm_sparse_mlp(s.layers[0], x, r, idx, cnt, y, ws=ws)
+    assert s.ctx.rm_get_info("last_variant") == variant
+    assert s.ctx.rm_device_status() == 0
+    assert bool((ws == 0xa5).all())
+    s.ctx.rm_set_option("path", 1)
+    want = torch.empty_like(y)
+    s.ctx.rm_sparse_mlp(s.layers[0], x, r, idx, cnt, want)
+    # (fp32 sums in another order, hidden values to 17 bits)
+    assert float((y - want).norm() / (want - r).norm()) <= 1e-4
+    s.ctx.close()

@@ -1556,16 +1556,12 @@ int launch_fused_ws(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, c
     return RM_OK;
 }
 
-// Shared memory that keeps a second CTA off the SM (of the 228 KB)
-constexpr int ALONE_BYTES = 116 * 1024;
-
 template <int NTOK, int HS, bool PIPE, int OCC = HS == 128 && !PIPE ? 2 : 1, bool LATE = false>
 int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cudaStream_t s) {
     using S = Smem<NTOK, HS, PIPE, OCC>;
     const bool eq4 = a.anchor_mode != RM_ANCHOR_NONE || a.gate != nullptr;
     auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE> : fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>;
-    int smem = S::total_bytes(a.T);
-    if (OCC == 1 && smem < ALONE_BYTES) smem = ALONE_BYTES;
+    const int smem = S::total_bytes(a.T);
     static rm_smem_configured configured = {};
     if (!configured.covers(ctx->device, smem)) {
         RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
@@ -1695,13 +1691,11 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     const long long tiles = per_episode > 0 ? (long long)((per_episode + NT - 1) / NT) * la.B : 0;
     // Variant.  H = 1024: the lean kernel (112 KB and at most 128 registers: two CTAs per SM, so a cluster's exchange waits are
     // covered by its SM-mate and consecutive layers overlap); measured, 33 of its clusters are co-resident, two more than
-    // twice the number the occupancy query reports for one CTA per SM.  Where no second CTA would fit the SM (more than 52 tokens), and
-    // where all clusters of a launch, in a stack those of the layer behind it too, find SMs of their own, it is built for one
-    // CTA per SM: nothing shares an SM by chance, values stay in registers, and outgoing sums have an area of their own.  us, two per
-    // SM / one, 6 layers: T = 8, 7 tiles 41.7 / 39.3; T = 32, 7 tiles 45.5 / 43.3; T = 51, 7 tiles 55.9 / 53.9, 12 tiles 57.8 / 63.7
-    // (two layers no longer fit side by side); T = 60, 12 tiles 69.0 / 67.0; T = 64, 7 tiles 62.6 / 58.3, 12 tiles 72.6 / 68.4;
-    // with Eq. 4 T = 20, 7 tiles 46.6 / 44.2; one layer alone, T = 51, 12 tiles 11.9 / 11.6.
-    // Its clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers 88.0 / 80.5.
+    // twice the number the occupancy query reports for one CTA per SM.  Where no second CTA would fit the SM (more than 52 tokens) it is
+    // built for one: registers and a staging area of its own.  Built so for few tiles of fewer tokens too, it keeps other streams
+    // off its SMs and gains nothing alone (us, two per SM with LATE / one per SM: 6 layers of 7 tiles, T = 20 36.2 / 36.3, T = 51 51.7 /
+    // 50.8, on 4 streams at once 50.2 / 92.5 and 74.5 / 119.9; one layer of 15 tiles of 51 tokens 11.1 / 11.0, on 4 streams 19.4 / 36.1).
+    // Of more than 52 tokens the clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers 88.0 / 80.5.
     // H = 2048 (one CTA per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
     // which runs the phases of consecutive tiles concurrently.  One layer alone of up to 52 tokens: the two-tile variant (us, warp-
     // specialised / two-tile, T = 40: 18 tiles 18.0 / 17.8, 27 18.8 / 18.2; T = 16: 36 tiles 19.9 / 19.0).
@@ -1713,7 +1707,6 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
         if (ctx->g.H == 1024) variant = !two_per_sm && tiles > ctx->fused_clusters ? 2 : 1;
         else variant = tiles > 0 && tiles <= cap ? 1 : tiles > 0 && la.x && la.T <= 52 ? 2 : 3;
     }
-    const bool alone = !two_per_sm || (tiles > 0 && tiles <= (la.x ? ctx->fused_clusters : ctx->fused_clusters / 2));
     if (variant == 3) {
         const int fits_t = ctx->g.H == 1024 ? SmemWS<64, 128>::total_bytes(la.T) : SmemWS<64, 256>::total_bytes(la.T);
         if (fits_t > 232448) variant = 2;
@@ -1739,8 +1732,7 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     if (ctx->g.H == 1024) {
         if (pipe)
             return small_t ? launch_fused<32, 128, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, true>(ctx, a, nc, pdl, s);
-        if (alone)
-            return small_t ? launch_fused<32, 128, false, 1>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 1>(ctx, a, nc, pdl, s);
+        if (!two_per_sm) return launch_fused<64, 128, false, 1>(ctx, a, nc, pdl, s);        // (more than 52 tokens)
         if (tiles > 0 && tiles <= nc)
             return small_t ? launch_fused<32, 128, false, 2, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 2, true>(ctx, a, nc, pdl, s);
         return small_t ? launch_fused<32, 128, false>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false>(ctx, a, nc, pdl, s);

@@ -1,5 +1,5 @@
-"""The lean layer kernel built for one CTA per SM: lists of one tile, up to as many tiles as leave room for the next layer's clusters,
-one more (the kernel for two CTAs per SM again), and chunks of more than 52 tokens, where it takes every launch."""
+"""The lean layer kernel: lists of one tile, up to a cluster's one tile and more, and chunks of more than 52 tokens, where it is built for
+one CTA per SM."""
 import pytest
 
 from test_gpu_edges import step_case

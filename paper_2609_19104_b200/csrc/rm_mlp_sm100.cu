@@ -1703,15 +1703,18 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     int cap = two_per_sm ? 2 * ctx->fused_clusters + 2 : ctx->fused_clusters;
     if (ctx->max_clusters_override > 0) cap = ctx->max_clusters_override;
     int variant = ctx->variant_override >= 5 ? 0 : ctx->variant_override;    // 5 and above: a call that the named kernel does not cover
+    // (the two-tile kernel's buffers fit the 227 KB of an SM, at 2048 columns up to 52 tokens)
+    const bool small_t = la.T <= 32, two_tile_fits = ctx->g.H == 1024 || small_t || Smem<64, 256, true>::total_bytes(la.T) <= 232448;
     if (variant == 0) {
         if (ctx->g.H == 1024) variant = !two_per_sm && tiles > ctx->fused_clusters ? 2 : 1;
-        else variant = tiles > 0 && tiles <= cap ? 1 : tiles > 0 && la.x && la.T <= 52 ? 2 : 3;
+        else variant = tiles > 0 && tiles <= cap ? 1 : tiles > 0 && la.x && two_tile_fits ? 2 : 3;
     }
     if (variant == 3) {
         const int fits_t = ctx->g.H == 1024 ? SmemWS<64, 128>::total_bytes(la.T) : SmemWS<64, 256>::total_bytes(la.T);
         if (fits_t > 232448) variant = 2;
         else if (ctx->max_clusters_override <= 0 || cap > ctx->fused_clusters) cap = ctx->fused_clusters;
     }
+    if (variant == 2 && !two_tile_fits) variant = 1;
     if (variant == 2 && ctx->max_clusters_override <= 0) cap = ctx->fused_clusters;      // one CTA per SM
     // Clusters: no more than the cap, and when the tile count is known, the fewest that keep the longest run of
     // tiles per cluster as short as the cap allows (40 tiles under a cap of 32: 20 clusters of 2, not 32 of 1 or 2).
@@ -1721,7 +1724,6 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
         const long long run = (tiles + cap - 1) / cap;
         nc = variant == 3 ? (int)(tiles < cap ? tiles : cap) : (int)((tiles + run - 1) / run);
     }
-    const bool small_t = la.T <= 32;
     ctx->last_variant = variant;
     if (variant == 3) {
         if (ctx->g.H == 1024)
@@ -1737,13 +1739,11 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
             return small_t ? launch_fused<32, 128, false, 2, true>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false, 2, true>(ctx, a, nc, pdl, s);
         return small_t ? launch_fused<32, 128, false>(ctx, a, nc, pdl, s) : launch_fused<64, 128, false>(ctx, a, nc, pdl, s);
     }
-    // H = 2048: the two-tile variant when its buffers fit the 227 KB of an SM (they do up to T = 60), else serial
-    const bool fits = Smem<64, 256, true>::total_bytes(la.T) <= 232448;
     const bool late = tiles > 0 && tiles <= nc;
     if (small_t) {
         if (pipe) return launch_fused<32, 256, true>(ctx, a, nc, pdl, s);
         return late ? launch_fused<32, 256, false, 1, true>(ctx, a, nc, pdl, s) : launch_fused<32, 256, false>(ctx, a, nc, pdl, s);
     }
-    if (pipe && fits) return launch_fused<64, 256, true>(ctx, a, nc, pdl, s);
+    if (pipe) return launch_fused<64, 256, true>(ctx, a, nc, pdl, s);
     return late ? launch_fused<64, 256, false, 1, true>(ctx, a, nc, pdl, s) : launch_fused<64, 256, false>(ctx, a, nc, pdl, s);
 }

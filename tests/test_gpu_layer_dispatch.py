@@ -6,7 +6,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("H,T,borders", [
     (1024, 60, [(15, 1), (16, 2), (30, 2), (31, 4)]), (2048, 16, [(15, 1), (16, 2), (59, 2), (60, 4)]),
-    (2048, 32, [(45, 2), (46, 5), (59, 5), (60, 4)]), (2048, 33, [(30, 2), (31, 5), (59, 5), (60, 4)]), (2048, 61, [(30, 2), (31, 5)])])
+    (2048, 32, [(45, 2), (46, 5), (59, 5), (60, 4)]), (2048, 33, [(30, 2), (31, 5), (59, 5), (60, 4)]),
+    (2048, 52, [(15, 1), (16, 2), (30, 2)]), (2048, 53, [(15, 1), (16, 1), (30, 1), (31, 5)]), (2048, 61, [(30, 1), (31, 5)])])
 def test_borders_of_one_layer(lib, H, T, borders):
     import torch
     I = 3968
@@ -19,12 +20,13 @@ def test_borders_of_one_layer(lib, H, T, borders):
         idx, cnt = torch.zeros(I, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
         ctx.rm_mask_compact([rnd(1, I).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, idx, cnt, I, n_lists=1, k=64 * tiles - 5)
         outs = []
-        for variant in (0, 1, 0):
+        other = 1 if kernel != 1 else 2 if H == 1024 or T <= 52 else 5          # (another kernel than the chosen one)
+        for variant in (0, other, 0):
             ctx.rm_set_option("variant", variant)
             y = r.clone() if len(outs) == 2 else torch.empty_like(r)           # (the last one in place)
             outs.append(ctx.rm_sparse_mlp(layer, x, y if len(outs) == 2 else r, idx, cnt, y))
-            if variant == 0:
-                assert ctx.rm_get_info("last_variant") == kernel, (tiles, ctx.rm_get_info("last_variant"))
+            last = ctx.rm_get_info("last_variant")
+            assert last == kernel if variant == 0 else last != kernel, (tiles, variant, last)
         for out in outs:
             # (one layer on the same bf16 input: only the order of fp32 sums of hidden values to 17 bits differs)
             assert torch.isfinite(out).all() and float((out - outs[1]).norm() / (outs[1] - r).norm()) <= 1e-4, tiles

@@ -276,8 +276,12 @@ int64_t rm_launch_count(const rm_ctx* ctx);
  *                         no records of more than 64 tokens; chosen by itself for widths and chunk lengths that the others
  *                         do not take), 7 = the sweep kernel (dense
  *                         steps of one episode in one launch)
- *   "stream_min_tiles"    launches with at least this many 64-neuron tiles use variant 4 when the variant is chosen
- *                         per launch (default 33 at H = 1024, 31 at H = 2048)
+ *   "stream_min_tiles"    launches with at least this many 64-neuron tiles (of all episodes together) use variant 4 when the variant is
+ *                         chosen per launch and the call is not one for variants 5 to 7; half as many do in steps of H = 1024
+ *                         with more than 52 tokens and no anchor state or gate, anchor steps and updates may need more.
+ *                         Unless set: 33 at H = 1024, 31 at H = 2048, and in one-layer calls 31 at H = 1024 with more than 52
+ *                         tokens and 60 at H = 2048 (with variant 5 below that from 31 tiles on, 46 with 17 to 32 tokens, and
+ *                         none with fewer; a value that is set keeps one-layer calls off variant 5)
  *   "persist_max_batch"   largest B for which the whole-step kernel may be chosen per call (default 1)
  *   "persist_prefetch_kb" whole-step kernel: KB of weight rows a CTA may ask into L2 ahead of its loaders (default 0:
  *                         measured slower than no prefetch)                                                    */

@@ -59,7 +59,7 @@ inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool eq4, 
     if (ctx->variant_override == 5) return true;
     if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b) return false;
     const long long K = masked ? rm_effective_count_hint(ctx) : ctx->g.I, tiles = (K + 63) / 64;
-    if (!steps) return ctx->g.H == 2048 && T > 16 && tiles >= (T > 32 ? 31 : 46) && tiles < 60;
+    if (!steps) return ctx->g.H == 2048 && ctx->stream_min_tiles == 0 && T > 16 && tiles >= (T > 32 ? 31 : 46) && tiles < 60;
     if (K <= 0) return ctx->g.H == 2048;
     if (ctx->g.H == 2048) {
         if (tiles <= (eq4 || T <= 55 ? 15 : 13)) return false;
@@ -105,7 +105,11 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 
 // The streaming variant (whole tiles per CTA): a tile costs an SM ~16 us at H = 1024 (its gathers run at ~20 bytes per clock,
 // its adds at 16), however few tiles there are; the cluster kernels, which spread a tile over 8 SMs, win while every cluster
-// has a single tile (stream_min_tiles, see rm_create).  `masked` says whether a count is in play.
+// has a single tile.  Measured crossover, us a step of 18 layers and 51 tokens, lean / streaming kernel (the lean kernel's time steps up
+// with every round of its 32 (H = 1024) or 15 (H = 2048) co-resident clusters): H = 1024: 32 tiles 269 / 291, 36 tiles 363 / 293 (20
+// tokens: 285 / 251), 46 tiles 408 / 294.  H = 2048: up to 30 tiles 360 to 380 / ~470, 32 tiles 531 / 475, 52 tiles 658 / 491.
+// The option stream_min_tiles, when set, stands for these lines, and for a single layer's (which it then keeps off the whole-step kernel).
+// `masked` says whether a count is in play.
 // With the anchor state of Eq. 4 the tiles do more (the anchor step adds two boxes per block and stores h_anchor, an update step reads
 // it), in the layer kernels beside other tiles.  us per 6 layers, 4 episodes, streaming / layer kernels:
 //   anchor step, H = 1024, T = 20: 40 tiles 111 / 106, 44 112 / 125     T = 51: 56 158 / 150, 60 159 / 171     T = 60: 32 169 / 186
@@ -123,8 +127,9 @@ inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_
     if (per_episode <= 0) return false;
     const long long tiles = (long long)((per_episode + 63) / 64) * B;
     const bool wide = ctx->g.H == 2048, once = !wide && !rm_fused_two_per_sm(ctx, T);
-    int least = !eq4 && once ? (ctx->stream_min_tiles + 1) / 2 : ctx->stream_min_tiles, eq4_least = 0;
-    if (!steps) least = once ? ctx->stream_min_tiles - 2 : wide && T <= 32 ? ctx->stream_min_tiles + 29 : ctx->stream_min_tiles;
+    const int line = ctx->stream_min_tiles > 0 ? ctx->stream_min_tiles : wide ? 31 : 33;
+    int least = !eq4 && once ? line / 2 + line % 2 : line, eq4_least = 0;
+    if (!steps && ctx->stream_min_tiles == 0) least = wide ? (T <= 32 ? 60 : line) : once ? 31 : line;
     if (anchor_mode == RM_ANCHOR_WRITE) eq4_least = wide ? (T > 52 ? 53 : 0) : T <= 32 ? 41 : once ? 0 : 57;
     if (anchor_mode == RM_ANCHOR_UPDATE && wide && T <= 32) eq4_least = 64;
     return tiles >= (least > eq4_least ? least : eq4_least);
@@ -150,11 +155,7 @@ int rm_create(rm_ctx** out, const rm_model_desc* desc) {
     c->g.Hs = desc->H / RM_NS;
     c->launches = 0;
     c->status_detail = 0;
-    // Measured crossover with the cluster kernels, us a step of 18 layers and 51 tokens, lean / streaming kernel.  The lean
-    // kernel's time steps up with every round of its 32 (H = 1024) or 15 (H = 2048) co-resident clusters.  H = 1024: 32 tiles 269 / 291,
-    // 36 tiles 363 / 293 (20 tokens: 285 / 251), 46 tiles 408 / 294.  H = 2048: up to 30 tiles 360 to 380 / ~470, 32 tiles
-    // 531 / 475, 52 tiles 658 / 491.
-    c->stream_min_tiles = desc->H == 2048 ? 31 : 33;
+    c->stream_min_tiles = 0;
     c->d_status = nullptr;
     int major = 0;                         // (two attributes: cudaGetDeviceProperties takes milliseconds)
     if (cudaGetDevice(&c->device) != cudaSuccess ||

@@ -48,7 +48,7 @@ struct rm_ctx {
     int count_hint_seen;                   // k of the last top-k / group compaction through this context (0: none yet)
     int max_clusters_override;             // > 0: cap on clusters per launch
     int l2_prefetch;                       // L2 prefetch distance (tiles) of the warp-specialised kernel
-    int stream_min_tiles;                  // launches with at least this many 64-neuron tiles use the streaming variant
+    int stream_min_tiles;                  // option: launches with at least this many 64-neuron tiles use the streaming variant (0: not set)
     int variant_override;                  // 0 auto, 1 lean kernel, 2 kernel with a dedicated staging buffer
     int last_variant;                      // kernel family of the last layer or step launched (see rm_get_info)
     // whole-step kernel (rm_mlp_persist.cu)

@@ -32,3 +32,32 @@ def test_borders_of_one_layer(lib, H, T, borders):
             assert torch.isfinite(out).all() and float((out - outs[1]).norm() / (outs[1] - r).norm()) <= 1e-4, tiles
     assert ctx.rm_device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("H,T,tiles,unset", [(2048, 20, 40, 2), (2048, 40, 40, 5), (1024, 60, 20, 2), (1024, 40, 20, 1)])
+def test_streaming_threshold_of_one_layer_is_the_option_when_it_is_set(lib, H, T, tiles, unset):
+    """From 1 (everything) to the largest int (nothing), on one layer and on a step of one."""
+    import torch
+    I = 2624
+    g = torch.Generator(device="cuda").manual_seed(H + T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    ctx = lib.Context(1, H, I, T)
+    layer = ctx.rm_pack_weights(*[(0.64 / H ** 0.5 * rnd(*s)).bfloat16() for s in ((I, H), (I, H), (H, I))])
+    x, r = rnd(T, H).bfloat16(), rnd(T, H)
+    idx, cnt = torch.zeros(1, I, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ctx.rm_mask_compact([rnd(1, I).abs()], lib.RM_SRC_SCORE_F32, lib.RM_REDUCE_TOPK, idx, cnt, I, n_lists=1, k=64 * tiles - 5)
+    want = None
+    for value in (None, 1, tiles, 2 * tiles + 1, 2 ** 31 - 1):
+        if value is not None:
+            ctx.rm_set_option("stream_min_tiles", value)
+        y = ctx.rm_sparse_mlp(layer, x, r, idx, cnt, torch.empty_like(r))
+        kernel = ctx.rm_get_info("last_variant")
+        assert kernel == unset if value is None else (kernel == 4) == (value <= tiles), (value, kernel)
+        want = y if want is None else want
+        # (fp32 sums in another order, hidden values to 17 bits)
+        assert torch.isfinite(y).all() and float((y - want).norm() / (want - r).norm()) <= 1e-4, value
+    ctx.rm_set_option("persist_max_batch", 0)
+    ctx.rm_action_expert_step([layer], r.view(1, T, H), idx, cnt, I, torch.empty_like(r))
+    assert ctx.rm_get_info("last_variant") != 4
+    assert ctx.rm_device_status() == 0
+    ctx.close()

@@ -53,13 +53,14 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 // `steps`: a whole stack (false: the one-layer entry, which pays the kernel's set-up for a single layer, and only where a streaming
 // tile takes longer still; H = 2048, us, whole-step / streaming / two-tile kernel:
 //   T =  8: 36 tiles 24.4/23.6/18.7   45: 25.1/23.6/22.2     T = 32: 36: 22.6/24.5/20.0   48: 23.0/24.7/23.8   57: 24.1/24.7/24.1
-//   T = 48: 30 tiles 20.9/27.0/20.5   33: 21.0/27.0/22.2   57: 22.4/27.2/26.9   63: 29.7/27.4/30.0     T = 64: 33: 21.3/27.5/26.8   57: 22.4/27.5/33.0).
+//   T = 48: 30 tiles 20.9/27.0/20.5   33: 21.0/27.0/22.2   57: 22.4/27.2/26.9   63: 29.7/27.4/30.0     T = 64: 33: 21.3/27.5/26.8   57: 22.4/27.5/33.0;
+// up to 4 tiles of 64 to a cluster: its tile is one of 256).
 inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool eq4, bool steps) {
     if (ctx->path == 1 || !rm_persist_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 5) return true;
     if ((ctx->variant_override != 0 && ctx->variant_override != 7) || B > ctx->persist_max_b) return false;
     const long long K = masked ? rm_effective_count_hint(ctx) : ctx->g.I, tiles = (K + 63) / 64;
-    if (!steps) return ctx->g.H == 2048 && ctx->stream_min_tiles == 0 && T > 16 && tiles >= (T > 32 ? 31 : 46) && tiles < 60;
+    if (!steps) return ctx->g.H == 2048 && ctx->stream_min_tiles == 0 && T > 16 && tiles >= (T > 32 ? 31 : 46) && tiles < 4 * ctx->persist_clusters;
     if (K <= 0) return ctx->g.H == 2048;
     if (ctx->g.H == 2048) {
         if (tiles <= (eq4 || T <= 55 ? 15 : 13)) return false;
@@ -129,7 +130,7 @@ inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_
     const bool wide = ctx->g.H == 2048, once = !wide && !rm_fused_two_per_sm(ctx, T);
     const int line = ctx->stream_min_tiles > 0 ? ctx->stream_min_tiles : wide ? 31 : 33;
     int least = !eq4 && once ? line / 2 + line % 2 : line, eq4_least = 0;
-    if (!steps && ctx->stream_min_tiles == 0) least = wide ? (T <= 32 ? 60 : line) : once ? 31 : line;
+    if (!steps && ctx->stream_min_tiles == 0) least = wide ? (T <= 32 ? 4 * ctx->fused_clusters : line) : once ? 2 * ctx->fused_clusters + 1 : line;
     if (anchor_mode == RM_ANCHOR_WRITE) eq4_least = wide ? (T > 52 ? 53 : 0) : T <= 32 ? 41 : once ? 0 : 57;
     if (anchor_mode == RM_ANCHOR_UPDATE && wide && T <= 32) eq4_least = 64;
     return tiles >= (least > eq4_least ? least : eq4_least);

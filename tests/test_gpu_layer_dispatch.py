@@ -1,5 +1,10 @@
 """Which kernel the one-layer entry takes follows width, chunk length and list length; at the borders both sides agree."""
+import numpy as np
 import pytest
+
+import oracle
+from paper_2609_19104_b200 import workloads as wl
+from harness import Model, assert_close, dev, dev_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -61,3 +66,44 @@ def test_streaming_threshold_of_one_layer_is_the_option_when_it_is_set(lib, H, T
     assert ctx.rm_get_info("last_variant") != 4
     assert ctx.rm_device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("T,tiles,kernel", [(48, 33, 5), (48, 57, 5), (20, 57, 5), (64, 33, 5), (20, 36, 2), (52, 16, 2), (60, 30, 1)])
+def test_one_wide_layer_against_the_oracle(lib, T, tiles, kernel):
+    """2048 columns: dense with records, a list without a residual, a compact layer, and a list far longer than the hint."""
+    import torch
+    H, I = 2048, 64 * tiles - 5
+    w = wl.Workload(97, "wide-layer", 1, H, I, T, 1.0 / np.sqrt(H), 1, 0.5)
+    model = Model(lib, w)
+    ctx, x, r = model.ctx, wl.step_input(w, 0), wl.residual_input(w)
+    W = model.Wg[0], model.Wu[0], model.Wd[0]
+
+    def call(idx, cnt, residual, **kw):
+        y = torch.full((T, H), 7.0, device="cuda")
+        return ctx.rm_sparse_mlp(kw.pop("layer", model.packed[0]), dev_bf16(x), None if residual is None else dev(residual), idx, cnt, y, **kw).cpu().numpy()
+
+    rec, scale = torch.zeros(I, device="cuda"), (1.0 + np.arange(I) % 3).astype(np.float32)
+    got = call(None, None, r, record_out=rec, record_scale=dev(scale))
+    assert ctx.rm_get_info("last_variant") == kernel
+    want, want_rec = oracle.dense_mlp(x, *W, r, scale=scale, return_record=True)
+    assert_close(got, want, "dense")
+    assert np.all(np.abs(rec.cpu().numpy() - want_rec) <= 2e-2 + 1e-2 * np.abs(want_rec))
+
+    lists = [np.flatnonzero(wl.uniform(wl.tensor_key(13, 97, 0, 2, i), I) < d).astype(np.int32) for i, d in enumerate((0.95, 0.4))]
+    for sel, hint in ((lists[0], I), (lists[1], I), (np.arange(I, dtype=np.int32), I // 4)):     # (the hint decides on the kernel)
+        ctx.rm_set_option("count_hint", hint)
+        idx, cnt = np.zeros((I + 3) // 4 * 4, np.int32), dev(np.array([sel.size], np.int32))
+        idx[:sel.size] = sel
+        got = call(dev(idx), cnt, None)
+        assert hint < I or ctx.rm_get_info("last_variant") == kernel
+        assert_close(got, oracle.masked_mlp(x, *W, None, sel), f"{sel.size} neurons, hint {hint}")
+    ctx.rm_set_option("count_hint", I)
+    sel = lists[0]
+    idx[:sel.size], cnt = sel, dev(np.array([sel.size], np.int32))
+    compact = torch.full((ctx.packed_layer_bytes() // 2,), 0x7FC0, dtype=torch.int16, device="cuda").view(torch.uint8)      # (NaN behind the rows)
+    ctx.rm_gather_weights(model.packed[0], dev(idx), cnt, I, compact_out=compact)
+    got = call(None, cnt, r, layer=compact)
+    assert ctx.rm_get_info("last_variant") == kernel
+    assert_close(got, oracle.masked_mlp(x, *W, r, sel), "compact layer")
+    assert ctx.rm_device_status() == 0
+    model.close()

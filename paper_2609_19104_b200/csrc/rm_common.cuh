@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "rmuscle.h"
@@ -74,13 +75,28 @@ extern int rm_last_cuda_error;            // cudaError_t of the last failed runt
     } while (0)
 
 // Dynamic shared-memory size a kernel has been configured for, per device: cudaFuncSetAttribute applies to the
-// current device only, and one process may hold contexts on several devices.  (A race between two threads costs a
-// redundant call, nothing else.)
+// current device only, and one process may hold contexts on several devices.  The attribute replaces the value that was
+// there, so it is only ever raised, and by one thread at a time: a smaller size of another thread's first call, set between this
+// thread's call and its launch, would make the launch fail.
 struct rm_smem_configured {
-    int bytes[64];
-    bool covers(int device, int need) const { return device >= 0 && device < 64 && bytes[device] >= need; }
-    void set(int device, int need) { if (device >= 0 && device < 64) bytes[device] = need; }
+    std::atomic<int> bytes[64];
+    std::mutex mutex;
+    bool covers(int device, int need) const { return device >= 0 && device < 64 && bytes[device].load(std::memory_order_acquire) >= need; }
+    template <class F>
+    int raise(int device, int need, F set) {                   // set(): configures for `need` bytes, returns an rm_status
+        if (covers(device, need)) return RM_OK;
+        std::lock_guard<std::mutex> lock(mutex);
+        if (covers(device, need)) return RM_OK;
+        const int rc = set();
+        if (rc == RM_OK && device >= 0 && device < 64) bytes[device].store(need, std::memory_order_release);
+        return rc;
+    }
 };
+template <class K>
+int rm_set_smem(K kernel, int bytes) {
+    RM_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    return RM_OK;
+}
 
 static inline bool rm_aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -434,10 +434,8 @@ template <int MODE>
 int launch_gemm(rm_ctx* ctx, const CtxGemmArgs& a, dim3 grid, const CUtensorMap& t0, const CUtensorMap& t1, const CUtensorMap& tb, cudaStream_t s) {
     using S = SmemCtx<MODE>;
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, S::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(ctx_gemm_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-        configured.set(ctx->device, S::TOTAL);
-    }
+    const int set = configured.raise(ctx->device, S::TOTAL, [] { return rm_set_smem(ctx_gemm_kernel<MODE>, S::TOTAL); });
+    if (set != RM_OK) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(CT);

@@ -89,10 +89,8 @@ int launch_gather(rm_ctx* ctx, const GatherArgs& a, cudaStream_t s) {
     const int smem = DEPTH * 6 * g.H + 128;
     if (smem > 227 * 1024) return RM_ERR_UNSUPPORTED;
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, smem)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(gather_read_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        configured.set(ctx->device, smem);
-    }
+    const int set = configured.raise(ctx->device, smem, [&] { return rm_set_smem(gather_read_kernel, smem); });
+    if (set != RM_OK) return set;
     gather_read_kernel<<<ctx->sm_count > 0 ? ctx->sm_count : 148, GT, smem, s>>>(a);
     ctx->launches++;
     RM_CUDA_TRY(cudaGetLastError());

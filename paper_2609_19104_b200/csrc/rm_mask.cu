@@ -389,9 +389,9 @@ __global__ void __launch_bounds__(MASK_THREADS, 1) mask_compact_kernel(const __g
 template <int E>
 int launch_mask(rm_ctx* ctx, const MaskParams& p, int n_lists, size_t smem, cudaStream_t s) {
     static rm_smem_configured configured = {};
-    if (smem + sizeof(MaskShared) > 48 * 1024 && !configured.covers(ctx->device, (int)smem)) {     // (48 KB, the static part included, need no asking)
-        RM_CUDA_TRY(cudaFuncSetAttribute(mask_compact_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        configured.set(ctx->device, (int)smem);
+    if (smem + sizeof(MaskShared) > 48 * 1024) {              // (48 KB, the static part included, need no asking)
+        const int set = configured.raise(ctx->device, (int)smem, [&] { return rm_set_smem(mask_compact_kernel<E>, (int)smem); });
+        if (set != RM_OK) return set;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_lists * p.cluster);

@@ -1328,10 +1328,8 @@ int query_clusters(int* out) {
 template <int HS8, bool EQ4>
 int launch(rm_ctx* ctx, const PArgs& a, const CUtensorMap& tmXext, int n_clusters, cudaStream_t s) {
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, Geo<HS8>::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(step_kernel<HS8, EQ4>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<HS8>::TOTAL));
-        configured.set(ctx->device, Geo<HS8>::TOTAL);
-    }
+    const int set = configured.raise(ctx->device, Geo<HS8>::TOTAL, [] { return rm_set_smem(step_kernel<HS8, EQ4>, Geo<HS8>::TOTAL); });
+    if (set != RM_OK) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_clusters * CS);
     cfg.blockDim = dim3(NTHREADS);

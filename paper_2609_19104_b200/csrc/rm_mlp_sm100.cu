@@ -1529,11 +1529,11 @@ int launch_fused_ws(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, c
     auto kern = eq4 ? fused_layer_ws_kernel<NTOK, HS, true> : fused_layer_ws_kernel<NTOK, HS, false>;
     const int smem = S::total_bytes(a.T);
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, smem)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_ws_kernel<NTOK, HS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_ws_kernel<NTOK, HS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        configured.set(ctx->device, smem);
-    }
+    const int set = configured.raise(ctx->device, smem, [&] {
+        const int rc = rm_set_smem(fused_layer_ws_kernel<NTOK, HS, true>, smem);
+        return rc != RM_OK ? rc : rm_set_smem(fused_layer_ws_kernel<NTOK, HS, false>, smem);
+    });
+    if (set != RM_OK) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_clusters * CS);
     cfg.blockDim = dim3(WT);
@@ -1563,11 +1563,11 @@ int launch_fused(rm_ctx* ctx, const FusedArgs& a, int n_clusters, bool pdl, cuda
     auto kern = eq4 ? fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE> : fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>;
     const int smem = S::total_bytes(a.T);
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, smem)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        RM_CUDA_TRY(cudaFuncSetAttribute(fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        configured.set(ctx->device, smem);
-    }
+    const int set = configured.raise(ctx->device, smem, [&] {
+        const int rc = rm_set_smem(fused_layer_kernel<NTOK, HS, PIPE, true, OCC, LATE>, smem);
+        return rc != RM_OK ? rc : rm_set_smem(fused_layer_kernel<NTOK, HS, PIPE, false, OCC, LATE>, smem);
+    });
+    if (set != RM_OK) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_clusters * CS);
     cfg.blockDim = dim3(FT);

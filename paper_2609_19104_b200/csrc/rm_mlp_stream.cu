@@ -698,15 +698,16 @@ int launch_tiles(rm_ctx* ctx, const StreamArgs& a, int n_ctas, bool dependent, c
         else kern = eq4 ? stream_tile_kernel<NTOK, true, false, 1> : stream_tile_kernel<NTOK, false, false, 1>;
     }
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, S::TOTAL)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, true, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+    const int set = configured.raise(ctx->device, S::TOTAL, [] {
+        int rc = rm_set_smem(stream_tile_kernel<NTOK, false, true, CL>, S::TOTAL);
         if (CL == 1) {
-            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, true, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
-            RM_CUDA_TRY(cudaFuncSetAttribute(stream_tile_kernel<NTOK, false, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::TOTAL));
+            if (rc == RM_OK) rc = rm_set_smem(stream_tile_kernel<NTOK, true, true, 1>, S::TOTAL);
+            if (rc == RM_OK) rc = rm_set_smem(stream_tile_kernel<NTOK, true, false, 1>, S::TOTAL);
+            if (rc == RM_OK) rc = rm_set_smem(stream_tile_kernel<NTOK, false, false, 1>, S::TOTAL);
         }
-        configured.set(ctx->device, S::TOTAL);
-    }
+        return rc;
+    });
+    if (set != RM_OK) return set;
     CUtensorMap tmW, tmX, tmOut, tmYa;
     int rc = make_map(&tmW, a.packed, (uint64_t)a.I, (uint64_t)3 * a.H, NT);       // used without a list only
     if (rc != RM_OK) return rc;

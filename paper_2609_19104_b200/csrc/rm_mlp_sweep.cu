@@ -491,10 +491,8 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 template <int HS, bool EQ4>
 int launch(rm_ctx* ctx, const WArgs& a, const WMaps& maps, int G, cudaStream_t s) {
     static rm_smem_configured configured = {};
-    if (!configured.covers(ctx->device, SMEM)) {
-        RM_CUDA_TRY(cudaFuncSetAttribute(sweep_kernel<HS, EQ4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
-        configured.set(ctx->device, SMEM);
-    }
+    const int set = configured.raise(ctx->device, SMEM, [] { return rm_set_smem(sweep_kernel<HS, EQ4>, SMEM); });
+    if (set != RM_OK) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(G);
     cfg.blockDim = dim3(NTHREADS);

@@ -134,8 +134,11 @@ int rm_launch_pack(rm_ctx* ctx, const void* Wg, const void* Wu, const void* Wd, 
     const rm_geom& g = ctx->g;
     dim3 grid((g.I + 31) / 32, RM_NS);
     size_t smem = (size_t)g.Hs * 33 * sizeof(__nv_bfloat16);
-    if (smem > 48 * 1024)
-        RM_CUDA_TRY(cudaFuncSetAttribute(pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) {
+        static rm_smem_configured configured = {};
+        const int set = configured.raise(ctx->device, (int)smem, [&] { return rm_set_smem(pack_kernel, (int)smem); });
+        if (set != RM_OK) return set;
+    }
     pack_kernel<<<grid, 256, smem, s>>>(static_cast<const __nv_bfloat16*>(Wg), static_cast<const __nv_bfloat16*>(Wu),
                                         static_cast<const __nv_bfloat16*>(Wd), static_cast<__nv_bfloat16*>(packed), g);
     ctx->launches++;

@@ -207,6 +207,7 @@ struct Smem {
     static constexpr int OFF_HT = OFF_DN + DN_STAGE;         // per buffer: hi tile, then lo tile
     static constexpr int OFF_HS = OFF_HT + NB * 2 * HT_HALF; // per buffer: this CTA's h atom (1 KB hi, 1 KB lo)
     static constexpr int OFF_SS = OFF_HS + NB * 2048;        // [CS][64] floats: row sums of squares per source CTA
+    static constexpr int OFF_SS2 = OFF_HT + (NB - 1) * 2 * HT_HALF;  // the same of a second tile of another episode (see xprep)
     static constexpr int OFF_N = OFF_SS + CS * 64 * 4;       // [2][64] neuron ids of two consecutive tiles
     static constexpr int OFF_PREF = OFF_N + 2 * NT * 4;      // [MAXB+1] tile prefix, [MAXB] counts
     static constexpr int OFF_BAR = ((OFF_PREF + (2 * MAXB + 1) * 4 + 7) / 8) * 8;
@@ -253,15 +254,15 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* gbase = smem_dyn + (base - smem_u32(smem_dyn));
     const uint32_t sX = base + S::OFF_X, sGU = base + S::OFF_GU, sDN = base + S::OFF_DN, sHT = base + S::OFF_HT;
-    const uint32_t sP = base + S::OFF_P, sSS = base + S::OFF_SS;
-    const float* gSS = reinterpret_cast<const float*>(gbase + S::OFF_SS);
+    const uint32_t sP = base + S::OFF_P;
     int* gN = reinterpret_cast<int*>(gbase + S::OFF_N);
     int* gPref = reinterpret_cast<int*>(gbase + S::OFF_PREF);
     int* gCnt = gPref + MAXB + 1;
     // mbarriers: MMA completion (gate/up per buffer, down) and arrival of the exchanges (partial sums and h per
     // buffer, sums of squares)
     const uint32_t bar0 = base + S::OFF_BAR;
-    const uint32_t bar_dn = bar0 + 48, bar_s = bar0 + 56, s_tmem = bar0 + 64;
+    const uint32_t bar_dn = bar0 + 48, s_tmem = bar0 + 64;
+    auto bar_s = [&](bool second) { return bar0 + (second ? 72 : 56); };
     auto bar_gu = [&](int pb) { return bar0 + 8 * pb; };
     auto bar_p = [&](int pb) { return bar0 + 16 + 8 * pb; };
     auto bar_h = [&](int pb) { return bar0 + 32 + 8 * pb; };
@@ -284,7 +285,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     if (tid == 0) {
         for (int pb = 0; pb < 2; ++pb) { mbar_init(bar_gu(pb), 1); mbar_init(bar_p(pb), 1); mbar_init(bar_h(pb), 1); }
         mbar_init(bar_dn, 1);
-        mbar_init(bar_s, 1);
+        for (int sb = 0; sb < NB; ++sb) mbar_init(bar_s(sb == 1), 1);
         fence_mbar_init();
         int acc = 0;
         const int cap = (int)(a.list_cap < (int64_t)a.I ? a.list_cap : (int64_t)a.I);
@@ -443,7 +444,11 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
     };
 
     // ---- phase: x slice of episode b -> bf16, 128-byte-swizzled K-major operand tile (cluster-collective)
-    auto xprep = [&](int b) {
+    // `second`: for the second of two tiles in flight.  Nothing has made this CTA wait until its peers have read the first one's sums of
+    // squares, so these have a place and a barrier of their own: the h buffer of this tile, which its h can reach only once this CTA has
+    // sent its partial sums.  (In front of later tiles, as with one tile at a time, lies a wait for an h that every peer sends behind
+    // its reads.  Room of its own would take 60 tokens beyond 196 KB, the last step of the SM's split but one: 80.6 -> 83.5 us.)
+    auto xprep = [&](int b, bool second) {
         cur_b = b;
         constexpr int CPP = HS / PARTS;                    // columns per thread
         const int t = tid / PARTS, part = tid % PARTS;
@@ -483,10 +488,11 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             for (int d = 1; d < PARTS; d <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, d);
             if (!pdl_fired) { pdl_launch_dependents(); pdl_fired = true; }   // the residual slice has arrived
             // all-gather of the row sums of squares: the PARTS lanes of a row share the 8 destinations
-            if (tid == 0) mbar_arrive_expect_tx(bar_s, CS * NTOK * 4);
+            const uint32_t ss_off = second ? S::OFF_SS2 : S::OFF_SS, ss_bar = bar_s(second);
+            if (tid == 0) mbar_arrive_expect_tx(ss_bar, CS * NTOK * 4);
 #pragma unroll
             for (int dst = part; dst < CS; dst += PARTS)
-                st_async_f32(map_to_rank(sSS + (j * 64 + t) * 4, dst), ss, map_to_rank(bar_s, dst));
+                st_async_f32(map_to_rank(base + ss_off + (j * 64 + t) * 4, dst), ss, map_to_rank(ss_bar, dst));
             // residual: token row t of this episode is added by exactly one of the clusters that work on the
             // episode, from the values already in registers, while the exchange is in flight
             if (a.add_residual && t < T && add_row) {
@@ -496,8 +502,9 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
                 for (int i = 0; i < CPP / 4; ++i)
                     add_residual4(ya_update, gate, H, a.r_out + row + col + 4 * i, row, col + 4 * i, b, v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             }
-            wait_bar(bar_s, par_s);
-            par_s ^= 1;
+            wait_bar(ss_bar, second ? 0 : par_s);
+            par_s ^= second ? 0 : 1;
+            const float* gSS = reinterpret_cast<const float*>(gbase + ss_off);
             float tot = 0.f;
 #pragma unroll
             for (int src = 0; src < CS; ++src) tot += gSS[src * 64 + t];
@@ -525,7 +532,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             mbar_arrive_expect_tx(bar_p(buf_of(i)), p_tx_bytes(i));
             mbar_arrive_expect_tx(bar_h(buf_of(i)), CS * 2048);
         }
-        if (tr.b != cur_b) xprep(tr.b);
+        if (tr.b != cur_b) xprep(tr.b, PIPE && i == 1);
     };
 
     // ---- phase: gate/up partial products of tile i over this CTA's column slice (operands are in shared memory
@@ -818,11 +825,7 @@ __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
             const TileRef tr = tile_ref(g_lo + i);
             const bool more = i + 1 < n_tiles;
             if (more) {
-                const TileRef nx = tile_ref(g_lo + i + 1);
-                // The x of a second tile of another episode: its sums of squares go where the first one's still lie, and nothing so far has
-                // made this CTA wait for its peers to have read those.  (From the third tile on h of the tile before the last one has.)
-                if (i == 0 && nx.b != tr.b) cluster_sync();
-                open_tile(i + 1, nx);
+                open_tile(i + 1, tile_ref(g_lo + i + 1));
                 if (i == 0) cp_async_wait<0>(); else cp_async_wait<1>();      // gate/up rows of tile i+1 have landed
                 fence_proxy_async_smem();
                 __syncthreads();

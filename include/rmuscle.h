@@ -268,9 +268,10 @@ int64_t rm_launch_count(const rm_ctx* ctx);
  *   "l2_prefetch"         warp-specialised kernel: number of tiles ahead for which the weights are pulled into L2
  *                         (0 = off, the default)
  *   "variant"             tcgen05 kernel variant: 0 = choose per launch, 1 = lean (one tile at a time, two CTAs per
- *                         SM at H = 1024), 2 = two tiles in flight per cluster, 3 = warp-specialised (the phases
+ *                         SM at H = 1024 and up to 52 tokens), 2 = two tiles in flight per cluster, 3 = warp-specialised (the phases
  *                         of consecutive tiles run concurrently; for clusters that walk many tiles), 4 = streaming
- *                         (no clusters: every CTA owns whole tiles; for launches with many tiles), 5 = the whole-step
+ *                         (no clusters: every CTA owns whole tiles; for launches with many tiles; one layer takes the fewest SMs
+ *                         so, which counts where several streams have such calls at once), 5 = the whole-step
  *                         kernel (every layer of a step in one launch; B <= 16; calls it does not cover are chosen per
  *                         launch), 6 = the slice kernel (every layer of a step in one launch, H up to 2048, any T, but
  *                         no records of more than 64 tokens; chosen by itself for widths and chunk lengths that the others

@@ -23,38 +23,42 @@ inline bool use_fused(const rm_ctx* ctx, int B, int T) {
 }
 
 // The whole-step kernel (variant 5).  Chosen by itself where it is measured ahead of the per-layer kernels (single episodes).
-// Its time per layer is ~10 us at H = 1024 and ~14 us at H = 2048, with little growth in K or T (chains between CTAs); the
+// Its time per layer is ~11 us at H = 1024 and ~15 us at H = 2048, with little growth in K or T (chains between CTAs); the
 // lean per-layer kernel's grows with T (tiles of 32 or 64 token columns; T > 52: one CTA per SM) and by a step at every
 // 64-neuron tile that makes a cluster's run longer; the streaming kernel's by a step at every wave of tiles over the SMs.
-// us per step of 6 layers, whole-step / per-layer kernels (s: streaming), by T:
-//   H = 1024  K =  500: 8: 61/42    32: 63/45    52: 65/56    56: 65/63    64: 66/67
-//                  900: 8: 61/44    32: 64/47    52: 65/59    56: 65/71    64: 66/76
-//                 1024: 8: 63/47    32: 66/54    48: 68/68    52: 68/68    64: 69/103
-//                 1280: 8: 64/54    32: 67/59    33: 67/69    52: 69/77    64: 70/109
-//                 1900: 8: 66/64    32: 69/69    33: 69/78    52: 71/86
-//                 2048: 8: 67/66    32: 70/72    33: 71/81    52: 72/90
-//   H = 2048  K =  500: 8: 82/54    32: 88/62    48: 91/77    64: 93/84
-//                  960: 8: 83/65    32: 88/74    48: 91/88    56: 92/93    64: 94/97
-//                 1024: 8: 85/86    32: 90/95    48: 93/110   64: 95/126
-//                 4600: 8: 142/144s 32: 148/152s 51: 153/167s
-//                 4900: 8: 147/143s 32: 154/152s 51: 158/167s
-//                 6100: 8: 158/146s 32: 166/157s 40: 167/168s 64: 171/171s
-//                 6500: 8: 161/146s 32: 170/159s 40: 172/170s 64: 175/173s
-//                 9400: 8: 223/167s 32: 233/198s 64: 238/216s   (10000, beyond a wave of 148 tiles: 225/272s, 239/329s)
-// with the anchor update (Eq. 4), whose sums the streaming kernel is slow at (4600: 148/224s):
-//   H = 1024  K =  600: 8: 66/46    32: 72/50    51: 75/63    60: 76/72    64: 78/76
-//                  900: 8: 68/47    32: 74/52    51: 78/65    60: 79/78    64: 81/83
-//                 1400: 8: 73/59    32: 80/66    40: 82/81    51: 83/86    64: 86/125
-//                 2048: 8: 76/70    32: 83/77    33: 83/90
-//   H = 2048  K =  960: 8: 92/71    32: 104/82   64: 117/112       1100: 8: 93/93   33: 107/112
+// us per step of 6 layers, whole-step / per-layer kernels (s: streaming), by T (I = 4096 and 16384):
+//   H = 1024  K =  500: 8: 62/35    32: 64/40    52: 66/53    56: 66/59    64: 67/62
+//                  900: 8: 62/37    32: 65/43    52: 66/55    56: 67/67    64: 67/70
+//                 1024: 8: 65/42    32: 67/48    48: 68/63    52: 69/63    64: 69/84
+//                 1152: 33: 67/62   48: 69/70    52: 69/70    64: 70/98s
+//                 1280: 8: 66/47    32: 68/54    33: 68/65    52: 69/72    64: 70/98s
+//                 1900: 8: 68/55    32: 70/63    33: 70/72    52: 72/82
+//                 2048: 8: 70/58    32: 72/65    33: 72/74    52: 73/85
+//   H = 2048  K =  500: 8: 83/50    32: 88/61    48: 91/73    64: 94/80
+//                  960: 8: 84/60    32: 89/69    48: 92/83    56: 93/87    64: 95/90
+//                 1024: 8: 86/85    32: 91/94    48: 94/108   64: 97/119
+//                 4600: 8: 144/137s 32: 150/147s 51: 154/161s
+//                 4900: 8: 149/139s 32: 155/148s 51: 158/161s
+//                 6100: 8: 158/141s 32: 165/151s 40: 167/162s 64: 171/165s
+//                 6500: 8: 162/141s 32: 168/152s 40: 170/163s 64: 174/166s
+//                 9400: 8: 223/157s 32: 231/194s 64: 237/207s   (10000, beyond a wave of 148 tiles: 225/265s, 239/324s)
+// with the anchor update (Eq. 4), whose sums the streaming kernel is slow at:
+//   H = 1024  K =  600: 8: 67/41    32: 72/46    51: 74/59    60: 75/68    64: 76/70
+//                  900: 8: 68/42    32: 73/48    51: 74/61    60: 75/74    64: 76/76
+//                 1400: 8: 71/51    32: 77/59    40: 78/73    51: 78/79    64: 80/95
+//                 2048: 8: 76/62    32: 82/70    33: 81/83
+//   H = 2048  K =  960: 8: 92/63    32: 103/75   64: 116/106      1100: 8: 94/88   32: 107/97
 // So, in tiles of 64 neurons, with K the caller's count hint (the whole layer for a dense pass): up to the bounds below the
-// layer kernels; from the bounds of H = 2048 up to one wave the streaming kernel.  Without a hint the whole-step kernel at
+// layer kernels; from the bounds of H = 2048 up to one wave the streaming kernel.  The bounds were drawn where the columns crossed when
+// the layer kernels took 3 to 8 us more; they now lie a few tiles on the low side (H = 1024: 16 to 24 tiles of 33 to 52
+// tokens, 30 and more of up to 32).  Without a hint the whole-step kernel at
 // H = 2048 (it adapts to the counts on the device), the lean kernel at H = 1024.  Batches stay with the streaming kernel.
 // `steps`: a whole stack (false: the one-layer entry, which pays the kernel's set-up for a single layer, and only where a streaming
-// tile takes longer still; H = 2048, us, whole-step / streaming / two-tile kernel:
-//   T =  8: 36 tiles 24.4/23.6/18.7   45: 25.1/23.6/22.2     T = 32: 36: 22.6/24.5/20.0   48: 23.0/24.7/23.8   57: 24.1/24.7/24.1
-//   T = 48: 30 tiles 20.9/27.0/20.5   33: 21.0/27.0/22.2   57: 22.4/27.2/26.9   63: 29.7/27.4/30.0     T = 64: 33: 21.3/27.5/26.8   57: 22.4/27.5/33.0;
-// up to 4 tiles of 64 to a cluster: its tile is one of 256).
+// tile takes longer still; H = 2048, us, whole-step / streaming / two-tile kernel (T = 64: the lean kernel in its place):
+//   T =  8: 36 tiles 20.8/22.8/17.5   57: 22.7/22.8/20.9     T = 32: 36: 18.3/24.0/19.2   48: 19.2/24.0/23.2   57: 19.6/24.0/23.3
+//   T = 48: 30 tiles 18.4/26.1/17.8   33: 18.6/26.2/22.2   57: 19.9/26.2/27.0   63: 26.9/26.2/31.3     T = 64: 33: 18.5/26.3/26.2   57: 19.8/26.3/32.3;
+// up to 4 tiles of 64 to a cluster: its tile is one of 256).  It takes 120 SMs for that time, the streaming kernel one per tile:
+// calls on several streams overlap less (33 tiles of 48 tokens, us a round of 1 / 2 / 4 streams: 18.8/34.4/68 against 26.2/27.2/35).
 inline bool use_persist(const rm_ctx* ctx, int B, int T, bool masked, bool eq4, bool steps) {
     if (ctx->path == 1 || !rm_persist_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 5) return true;
@@ -113,13 +117,16 @@ inline void slice_buffers(const rm_ctx* ctx, rm_step_args& sa, void* ws, int B, 
 // `masked` says whether a count is in play.
 // With the anchor state of Eq. 4 the tiles do more (the anchor step adds two boxes per block and stores h_anchor, an update step reads
 // it), in the layer kernels beside other tiles.  us per 6 layers, 4 episodes, streaming / layer kernels:
-//   anchor step, H = 1024, T = 20: 40 tiles 111 / 106, 44 112 / 125     T = 51: 56 158 / 150, 60 159 / 171     T = 60: 32 169 / 186
-//                H = 2048, T = 20: 32 tiles 190 / 212     T = 51: 32 278 / 287     T = 56: 48 288 / 248, 56 289 / 289, 64 290 / 330
-//   update step, H = 1024, T = 20: 36 tiles 96 / 104      T = 51: 36 116 / 147
-//                H = 2048, T = 8: 32 tiles 189 / 171, 52 195 / 185     T = 20: 32 193 / 179, 52 196 / 193     T = 51: 32 219 / 245
-// Where the lean kernel fits an SM only once (H = 1024, T > 52), its clusters walk two tiles from 17 tiles on: half the threshold
-// (2 episodes of 60 tokens, 3600 neurons, us per 6 layers, lean / streaming: 10 tiles 68 / 101, 18 tiles 114 / 102).  One layer
-// alone has the two-tile variant there (T = 56, 18 tiles 15.0 / 17.8 us, 30 16.3 / 17.9), at H = 2048 up to 59 tiles with short chunks.
+//   anchor step, H = 1024, T = 20: 40 tiles 112 / 100, 44 116 / 116     T = 51: 56 168 / 144, 60 168 / 158     T = 60: 32 162 / 137
+//                H = 2048, T = 20: 32 tiles 219 / 201     T = 51: 32 307 / 279     T = 56: 48 315 / 240, 56 316 / 277, 64 312 / 318
+//   update step, H = 1024, T = 20: 36 tiles 115 / 99     T = 51: 36 132 / 149
+//                H = 2048, T = 8: 32 tiles 218 / 170, 52 219 / 180, 64 217 / 220     T = 20: 32 219 / 177, 52 217 / 188     T = 51: 32 236 / 248
+// Where the lean kernel fits an SM only once (H = 1024, T > 52), clusters walk two tiles from 16 tiles on: half the threshold.  The
+// two-tile kernel takes those launches; 2 episodes of 60 tokens, us per 6 layers, streaming / two-tile / lean kernel: 16 tiles 97 / 80 / 89,
+// 18 97 / 93 / 104, 20 97 / 82 / 91, 28 98 / 89 / 99, 32 98 / 115 / 132 (from 17 to 30 tiles half the threshold is on the low side); with
+// the gate alone 18 99 / 96 / 107, 32 100 / 118 / 135; update steps 16 115 / 88 / 97, 18 116 / 107 / 117, 32 129 / 134 / 151; anchor steps 32
+// 162 / 137 / 151.  One layer alone: T = 56, 18 tiles 17.0 / 13.7, 30 17.1 / 14.2, 31 17.2 / 17.0; at H = 2048 the two-tile kernel
+// takes up to 59 tiles of short chunks.
 inline bool use_stream(const rm_ctx* ctx, bool masked, int B, int T, int anchor_mode = RM_ANCHOR_NONE, bool eq4 = false, bool steps = true) {
     if (ctx->path == 1 || !rm_stream_supported(ctx, B, T)) return false;
     if (ctx->variant_override == 4) return true;

@@ -168,7 +168,7 @@ __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, int line, 
 
 // The same accumulator, scaled by the gate, laid out in shared memory as [128-column block][token][128 columns] for
 // the copy engine's bulk add (one box of the [B, T, H] tensor map per block).  In line in the layer kernel, where it is on every
-// layer's chain (out of line: 10 tiles, 6 layers, T = 20 / 32 / 51 39.1 -> 40.2, 41.8 -> 42.9, 54.1 -> 54.8 us), out of line in the other.
+// layer's chain (out of line 6 layers of 10 tiles take 1 us more of 37 to 52), out of line in the other.
 template <int NTOK, int HS>
 __device__ __forceinline__ void stage_partial(float* __restrict__ stage, const float* __restrict__ gate, uint32_t tmem_d2,
                                            int wrow, int lane, int c0_first, int c0_step, int T, int col_base) {
@@ -237,9 +237,10 @@ struct TileRef {
 // EQ4 = false compiles the anchor-relative update and the output gate out (the zero-fill step pays nothing for them)
 // OCC: CTAs per SM that the registers allow.  LATE: a tile's outgoing partial sums always lie in the gate/up stage, which is refilled
 // only once they have been read -- for launches whose clusters have one tile each as far as the host knows.  (The code that sends
-// rows from registers otherwise costs registers where it is not used.)  A layer is a chain of latencies, and instructions on it
-// count: with this, the integer division of the residual's share and the first tile's bounds before the dependency wait, and one
-// rsqrt for a root and a division, 6 layers of 10 tiles take, T = 20 / 32 / 51, 40.4 / 43.0 / 55.6 us instead of 43.7 / 46.1 / 57.0.
+// rows from registers otherwise costs registers where it is not used.)  A layer is a chain of latencies, and instructions on it count:
+// LATE, the residual's share (an integer division) and the first tile's bounds worked out in front of the dependency wait, and one rsqrt
+// for a root and a division are worth 2.5 to 4 us of a step of 6 layers of 10 tiles (T = 20 / 32 / 51: 37.0 / 40.5 / 52.5 us, without
+// them 41.1 / 43.6 / 55.0).
 template <int NTOK, int HS, bool PIPE, bool EQ4, int OCC, bool LATE>
 __global__ void __launch_bounds__(FT, OCC) fused_layer_kernel(const FusedArgs a,
                                                                                                const __grid_constant__ CUtensorMap tmOut) {
@@ -1698,10 +1699,11 @@ int rm_launch_layer_fused(rm_ctx* ctx, const rm_layer_args& la, float* zero_buf,
     // built for one: registers and a staging area of its own.  Built so for few tiles of fewer tokens too, it keeps other streams
     // off its SMs and gains nothing alone (us, two per SM with LATE / one per SM: 6 layers of 7 tiles, T = 20 36.2 / 36.3, T = 51 51.7 /
     // 50.8, on 4 streams at once 50.2 / 92.5 and 74.5 / 119.9; one layer of 15 tiles of 51 tokens 11.1 / 11.0, on 4 streams 19.4 / 36.1).
-    // Of more than 52 tokens the clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers 88.0 / 80.5.
+    // Of more than 52 tokens the clusters walk a second tile from 16 tiles on, which the two-tile variant overlaps: T = 60, 16 tiles, 6 layers, us,
+    // lean / two-tile 89 / 80 (with the gate alone 90 / 82, an update step 97 / 88, an anchor step 100 / 95).
     // H = 2048 (one CTA per SM either way): the lean kernel while every cluster gets a single tile, else the warp-specialised kernel,
     // which runs the phases of consecutive tiles concurrently.  One layer alone of up to 52 tokens: the two-tile variant (us, warp-
-    // specialised / two-tile, T = 40: 18 tiles 18.0 / 17.8, 27 18.8 / 18.2; T = 16: 36 tiles 19.9 / 19.0).
+    // specialised / two-tile, T = 48: 24 tiles 18.8 / 17.6, 30 18.9 / 17.8; T = 16: 36 tiles 19.6 / 17.9).
     const bool two_per_sm = rm_fused_two_per_sm(ctx, la.T);
     int cap = two_per_sm ? 2 * ctx->fused_clusters + 2 : ctx->fused_clusters;
     if (ctx->max_clusters_override > 0) cap = ctx->max_clusters_override;
